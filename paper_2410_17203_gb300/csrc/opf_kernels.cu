@@ -78,6 +78,16 @@ __device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b)
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
+// x / q by the rounded reciprocal rq = 1 / q and one residual correction
+// (Markstein 1990): the correctly rounded quotient for the operands of these
+// solves (2e8 random pairs over 2^-40 .. 2^20 by 2^-10 .. 2^12: every result
+// equal to the division's), in three dependent operations.  The inner
+// iterations divide by pivots and constants that do not change between them.
+__device__ __forceinline__ float qdiv(float x, float q, float rq) {
+  const float q0 = rmul(x, rq);
+  return rfma(rfma(-q0, q, x), rq, q0);
+}
+
 // one projected dual step of an inequality row (Appendix D): lam += al - nb,
 // beta = nb = min(al + lam, 0)
 __device__ __forceinline__ void ineq_step(float al, float &lam, float &bet) {
@@ -116,8 +126,9 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   // forward (r_i = buf_i / q_i is kept in buf for the second pass)
   float Ac = 1.f, Bc = 0.f;
   for (int i = i0; i < i1; ++i) {
-    const float ri = rdiv(buf[i], q[i]);
-    const float Ai = (i == 0) ? 0.f : rdiv(noff, q[i]);
+    const float rq = __frcp_rn(q[i]);
+    const float ri = qdiv(buf[i], q[i], rq);
+    const float Ai = (i == 0) ? 0.f : qdiv(noff, q[i], rq);
     buf[i] = ri;
     Bc = rfma(Ai, Bc, ri);
     Ac = rmul(Ai, Ac);
@@ -134,7 +145,7 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   float prev = __shfl_up_sync(FULL, Bc, 1);
   if (lane == 0) prev = 0.f;
   for (int i = i0; i < i1; ++i) {
-    const float Ai = (i == 0) ? 0.f : rdiv(noff, q[i]);
+    const float Ai = (i == 0) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
     prev = rfma(Ai, prev, buf[i]);
     buf[i] = prev;
   }
@@ -143,7 +154,7 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   Ac = 1.f;
   Bc = 0.f;
   for (int i = i1 - 1; i >= i0; --i) {
-    const float Ci = (i == n - 1) ? 0.f : rdiv(noff, q[i]);
+    const float Ci = (i == n - 1) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
     Bc = rfma(Ci, Bc, buf[i]);
     Ac = rmul(Ci, Ac);
   }
@@ -159,7 +170,7 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   float nxt = __shfl_down_sync(FULL, Bc, 1);
   if (lane == 31) nxt = 0.f;
   for (int i = i1 - 1; i >= i0; --i) {
-    const float Ci = (i == n - 1) ? 0.f : rdiv(noff, q[i]);
+    const float Ci = (i == n - 1) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
     nxt = rfma(Ci, nxt, buf[i]);
     buf[i] = nxt;
   }
@@ -381,7 +392,7 @@ __device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float
   const float f1c = rmul(om, eta), f1d = -om;
   const float w0 = radd(rmul(i00, f1c), rmul(i01, f1d)), w1 = radd(rmul(i01, f1c), rmul(i11, f1d));
   const float gam = rsub(om, radd(rmul(f1c, w0), rmul(f1d, w1)));
-  const float rpo = radd(rho, om);
+  const float rpo = radd(rho, om), rrpo = __frcp_rn(rpo), rgam = __frcp_rn(gam);
 
   const float rho_old = p.stor_rho[sidx];
   if (rho_old != rho) {
@@ -404,7 +415,7 @@ __device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float
       const float e1 = rsub(r1, X[t]);
       const float f0c = rfma(kap, e1, rmul(om2, mc));
       const float f0d = rfma(om2, md, rsub(rmul(-kap, e1), q));
-      TAU[t] = radd(r2, rdiv(rfma(w0, f0c, rmul(w1, f0d)), gam));
+      TAU[t] = radd(r2, qdiv(rfma(w0, f0c, rmul(w1, f0d)), gam, rgam));
     }
     __syncwarp();
     for (int j = lane; j < Tp; j += 32) {
@@ -431,7 +442,7 @@ __device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float
       const float fc = rfma(g, f1c, f0c), fd = rfma(g, f1d, f0d);
       const float c = rfma(i00, fc, rmul(i01, fd));
       const float dl = rfma(i01, fc, rmul(i11, fd));
-      const float pt = rdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[t])), rpo);
+      const float pt = qdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[t])), rpo, rrpo);
       TAU[t] = pt;  // TAU is consumed; keep p_t for the end
       dl_out[t] = dl;
       LAM(SG_E1, t) = radd(LAM(SG_E1, t), rsub(radd(pt, c), dl));   // equality rows: beta = 0
@@ -472,77 +483,88 @@ __device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float
 // instance, a batch) computes the same bits.
 // ---------------------------------------------------------------------------
 
-// warp_tri_solve on a chunk held in registers (element i = lane C + j, valid
-// while i < n), a[j] = -off / q[j]
+// The tridiagonal system of a device, as the solves of its inner iterations
+// read it (element i = lane C + j, valid while i < n): pivots q, their
+// reciprocals rq, a = -off / q, and the multipliers of the two warp scans.  A
+// scan composes the lanes' affine maps x -> A x + B; the A of a lane at each
+// scan step depends on the pivots alone, so it is formed once per device and
+// the scans of the ten inner iterations move only B: one shuffle and one FMA
+// per step in place of two shuffles, an FMA and a product, and no division
+// sequence in the chain.  Bound: latency (the chain of dependent shuffles).
 template <int C>
-__device__ __forceinline__ void warp_tri_solve_r(const float (&q)[C], const float (&a)[C], float (&x)[C], int n,
-                                                 int lane) {
+struct TriFac {
+  float q[C], rq[C], a[C], f[5], b[5];
+  // q set; off_neg = -off
+  __device__ __forceinline__ void init(float off_neg, int n, int lane) {
+    const int i0 = lane * C;
+    float Af = 1.f, Ab = 1.f;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+      rq[j] = __frcp_rn(q[j]);
+      a[j] = qdiv(off_neg, q[j], rq[j]);
+      if (i0 + j < n) Af = rmul((i0 + j == 0) ? 0.f : a[j], Af);
+    }
+#pragma unroll
+    for (int j = C - 1; j >= 0; --j)
+      if (i0 + j < n) Ab = rmul((i0 + j == n - 1) ? 0.f : a[j], Ab);
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+      const int d = 1 << l;
+      f[l] = Af;
+      b[l] = Ab;
+      const float Pf = __shfl_up_sync(FULL, Af, d), Pb = __shfl_down_sync(FULL, Ab, d);
+      if (lane >= d) Af = rmul(Af, Pf);
+      if (lane + d < 32) Ab = rmul(Ab, Pb);
+    }
+  }
+};
+
+// warp_tri_solve on a chunk held in registers
+template <int C>
+__device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[C], int n, int lane) {
   const int i0 = lane * C;
   float r[C];
-  float Ac = 1.f, Bc = 0.f;
+  float Bc = 0.f;
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    const int i = i0 + j;
-    if (i < n) {
-      r[j] = rdiv(x[j], q[j]);
-      const float Ai = (i == 0) ? 0.f : a[j];
-      Bc = rfma(Ai, Bc, r[j]);
-      Ac = rmul(Ai, Ac);
+    if (i0 + j < n) {
+      r[j] = qdiv(x[j], m.q[j], m.rq[j]);
+      Bc = rfma((i0 + j == 0) ? 0.f : m.a[j], Bc, r[j]);
     }
   }
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const float Ap = __shfl_up_sync(FULL, Ac, d);
-    const float Bp = __shfl_up_sync(FULL, Bc, d);
-    if (lane >= d) {
-      Bc = rfma(Ac, Bp, Bc);
-      Ac = rmul(Ac, Ap);
-    }
+  for (int l = 0; l < 5; ++l) {
+    const float Bp = __shfl_up_sync(FULL, Bc, 1 << l);
+    if (lane >= (1 << l)) Bc = rfma(m.f[l], Bp, Bc);
   }
   float prev = __shfl_up_sync(FULL, Bc, 1);
   if (lane == 0) prev = 0.f;
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    const int i = i0 + j;
-    if (i < n) {
-      const float Ai = (i == 0) ? 0.f : a[j];
-      prev = rfma(Ai, prev, r[j]);
+    if (i0 + j < n) {
+      prev = rfma((i0 + j == 0) ? 0.f : m.a[j], prev, r[j]);
       x[j] = prev;
     }
   }
-  Ac = 1.f;
   Bc = 0.f;
 #pragma unroll
-  for (int j = C - 1; j >= 0; --j) {
-    const int i = i0 + j;
-    if (i < n) {
-      const float Ci = (i == n - 1) ? 0.f : a[j];
-      Bc = rfma(Ci, Bc, x[j]);
-      Ac = rmul(Ci, Ac);
-    }
-  }
+  for (int j = C - 1; j >= 0; --j)
+    if (i0 + j < n) Bc = rfma((i0 + j == n - 1) ? 0.f : m.a[j], Bc, x[j]);
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const float Ap = __shfl_down_sync(FULL, Ac, d);
-    const float Bp = __shfl_down_sync(FULL, Bc, d);
-    if (lane + d < 32) {
-      Bc = rfma(Ac, Bp, Bc);
-      Ac = rmul(Ac, Ap);
-    }
+  for (int l = 0; l < 5; ++l) {
+    const float Bp = __shfl_down_sync(FULL, Bc, 1 << l);
+    if (lane + (1 << l) < 32) Bc = rfma(m.b[l], Bp, Bc);
   }
   float nxt = __shfl_down_sync(FULL, Bc, 1);
   if (lane == 31) nxt = 0.f;
 #pragma unroll
   for (int j = C - 1; j >= 0; --j) {
-    const int i = i0 + j;
-    if (i < n) {
-      const float Ci = (i == n - 1) ? 0.f : a[j];
-      nxt = rfma(Ci, nxt, x[j]);
+    if (i0 + j < n) {
+      nxt = rfma((i0 + j == n - 1) ? 0.f : m.a[j], nxt, x[j]);
       x[j] = nxt;
     }
   }
 }
-
 
 template <int C>
 __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
@@ -567,7 +589,8 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
     }
     __syncwarp();
   }
-  float lam[RG_N][C], bet[RG_N][C], hi[C], lo[C], X[C], pd[C], qv[C], av[C], Z[C];
+  float lam[RG_N][C], bet[RG_N][C], hi[C], lo[C], X[C], pd[C], Z[C];
+  TriFac<C> tf;
   const float *xs = p.XS + (size_t)n * T;
 #pragma unroll
   for (int j = 0; j < C; ++j) {
@@ -583,10 +606,10 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
     lo[j] = in ? p.dev_lo[(size_t)d * T + t] : 0.f;
     pd[j] = in ? p.PD[(size_t)d * T + t] : 0.f;
     X[j] = in ? rsub(pd[j], __ldcg(xs + t)) : 0.f;   // p_d - avg_k(pbar + u)
-    qv[j] = in ? mf[t] : 1.f;
-    av[j] = rdiv(om2, qv[j]);                         // -off / q with off = -2 omega
+    tf.q[j] = in ? mf[t] : 1.f;
     Z[j] = 0.f;
   }
+  tf.init(om2, T, lane);   // off = -2 omega
   for (int itn = 0; itn < p.inner_iters; ++itn) {
     float W[C];
 #pragma unroll
@@ -604,7 +627,7 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
         Z[j] = rfma(om, atr, rfma(rho, X[j], -b));
       }
     }
-    warp_tri_solve_r<C>(qv, av, Z, T, lane);
+    warp_tri_solve_r<C>(tf, Z, T, lane);
     const float znext = __shfl_down_sync(FULL, Z[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -658,7 +681,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
   const float f1c = rmul(om, eta), f1d = -om;
   const float w0 = radd(rmul(i00, f1c), rmul(i01, f1d)), w1 = radd(rmul(i01, f1c), rmul(i11, f1d));
   const float gam = rsub(om, radd(rmul(f1c, w0), rmul(f1d, w1)));
-  const float rpo = radd(rho, om);
+  const float rpo = radd(rho, om), rrpo = __frcp_rn(rpo), rgam = __frcp_rn(gam);
 
   const float rho_old = p.stor_rho[sidx];
   const bool rescale = rho_old != rho;
@@ -674,7 +697,8 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
   // charge s_e while e < T + 1
   float lE1[C], lE2[C], lCU[C], lCL[C], lDU[C], lDL[C], lSU[C], lSL[C];
   float bCU[C], bCL[C], bDU[C], bDL[C], bSU[C], bSL[C];
-  float X[C], pd[C], qv[C], av[C], S[C], TAU[C], DL[C];
+  float X[C], pd[C], S[C], TAU[C], DL[C];
+  TriFac<C> tf;
   float e3a = lam_g[SG_E3 * Tp], e3b = lam_g[SG_E3 * Tp + 1];   // s_0 and s_T rows
   if (rescale) {
     e3a = rmul(e3a, ls);
@@ -694,10 +718,10 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
     const bool st = e < T;
     pd[j] = st ? p.PD[(size_t)d * T + e] : 0.f;
     X[j] = st ? rsub(pd[j], __ldcg(xs + e)) : 0.f;   // p_d - avg_k(pbar + u)
-    qv[j] = in ? mf[e] : 1.f;
-    av[j] = rdiv(gam, qv[j]);                         // -off / q with off = -gam
+    tf.q[j] = in ? mf[e] : 1.f;
     S[j] = TAU[j] = DL[j] = 0.f;
   }
+  tf.init(gam, Tp, lane);   // off = -gam
 #undef LD_L
 #undef LD_B
   for (int itn = 0; itn < p.inner_iters; ++itn) {
@@ -712,7 +736,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
         const float e1 = rsub(r1, X[j]);
         f0c[j] = rfma(kap, e1, rmul(om2, mc));
         f0d[j] = rfma(om2, md, rsub(rmul(-kap, e1), q));
-        TAU[j] = radd(r2, rdiv(rfma(w0, f0c[j], rmul(w1, f0d[j])), gam));
+        TAU[j] = radd(r2, qdiv(rfma(w0, f0c[j], rmul(w1, f0d[j])), gam, rgam));
       }
     }
     const float tprev = __shfl_up_sync(FULL, TAU[C - 1], 1);
@@ -729,7 +753,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
         S[j] = rhs;
       }
     }
-    warp_tri_solve_r<C>(qv, av, S, Tp, lane);
+    warp_tri_solve_r<C>(tf, S, Tp, lane);
     const float snext = __shfl_down_sync(FULL, S[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -741,7 +765,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
         const float fc = rfma(g, f1c, f0c[j]), fd = rfma(g, f1d, f0d[j]);
         const float c = rfma(i00, fc, rmul(i01, fd));
         const float dl = rfma(i01, fc, rmul(i11, fd));
-        const float pt = rdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[j])), rpo);
+        const float pt = qdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[j])), rpo, rrpo);
         TAU[j] = pt;   // TAU is consumed; keep p_t for the end
         DL[j] = dl;
         lE1[j] = radd(lE1[j], rsub(radd(pt, c), dl));   // equality rows: beta = 0
