@@ -354,6 +354,7 @@ void carve(opf_ctx *c, Arena &a) {
   p.DSM = a.take<float>((size_t)c->N * T);
   p.DSQ = a.take<float>((size_t)c->N * T);
   p.partials = a.take<double>((size_t)c->plan.node_grid * opfk::NSLOT);
+  p.done = a.take<unsigned>(1);
   p.xsum = c->slice ? a.take<double>(slice_exchange_len(c)) : nullptr;
 }
 
@@ -365,6 +366,7 @@ opf_status init_scalars(opf_ctx *c) {
   sc.sv = 1.0;
   sc.v_fresh = 1;
   sc.stall_ref = HUGE_VAL;
+  opfk::set_iter(c->P, sc);
   CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return OPF_OK;
@@ -856,9 +858,9 @@ opf_status opf_iterate(opf_ctx *c, int32_t n_iters, double rho) {
   // after the caller's earlier work on its stream ...
   CK(cudaEventRecord(c->ev_in, c->stream));
   CK(cudaStreamWaitEvent(c->s_main, c->ev_in, 0));
-  if (rho > 0 && opfk_set_rho_launch(c->P.sc, rho, c->s_main) != 0) return fail(OPF_ECUDA, "set_rho launch failed");
+  if (rho > 0 && opfk_set_rho_launch(c->P, rho, c->s_main) != 0) return fail(OPF_ECUDA, "set_rho launch failed");
   if (n_iters > 0) {
-    if (opfk_begin_launch(c->P.sc, n_iters, 1, c->s_main) != 0) return fail(OPF_ECUDA, "begin launch failed");
+    if (opfk_begin_launch(c->P, n_iters, 1, c->s_main) != 0) return fail(OPF_ECUDA, "begin launch failed");
     for (int i = 0; i < n_iters / kGraphIters; ++i) CK(cudaGraphLaunch(c->g_many, c->s_main));
     for (int i = 0; i < n_iters % kGraphIters; ++i) CK(cudaGraphLaunch(c->g_one, c->s_main));
   }
@@ -905,8 +907,8 @@ opf_status opf_slice_begin(opf_ctx *c, int32_t n_iters, double rho) {
   if (rho > 0 && !std::isfinite(rho)) return fail(OPF_EINVAL, "rho must be finite");
   opf_status s = slice_in(c);
   if (s != OPF_OK) return s;
-  if (rho > 0 && opfk_set_rho_launch(c->P.sc, rho, c->s_main) != 0) return fail(OPF_ECUDA, "set_rho launch failed");
-  if (opfk_begin_launch(c->P.sc, n_iters, 1, c->s_main) != 0) return fail(OPF_ECUDA, "begin launch failed");
+  if (rho > 0 && opfk_set_rho_launch(c->P, rho, c->s_main) != 0) return fail(OPF_ECUDA, "set_rho launch failed");
+  if (opfk_begin_launch(c->P, n_iters, 1, c->s_main) != 0) return fail(OPF_ECUDA, "begin launch failed");
   return slice_out(c);
 }
 
@@ -956,9 +958,9 @@ opf_status opf_get_info(opf_ctx *c, opf_info *info) {
   info->tolerance = c->tol;
   {
     const opfk::IterPlan &pl = c->plan;
-    info->kernels_per_iteration = (pl.xs_grid > 0) + (pl.inner_grid > 0) + 1 +
-                                  pl.n_slabs * ((pl.line_grid > 0 && c->L > 0) + 1 +
-                                                (pl.lean_grid > 0 && c->opt.alpha == 1.0)) + 1;
+    // a slice's decisions are a launch of their own (opf_slice_finish)
+    info->kernels_per_iteration =
+        (pl.xs_grid > 0) + (pl.inner_grid > 0) + 1 + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
   }
   info->N = c->N;
   info->L = c->L;
@@ -1635,6 +1637,7 @@ opf_status opf_set_state(opf_ctx *c, int32_t on_device, const opf_state *src) {
   sc.frozen_at = 0;
   sc.stall_ref = HUGE_VAL;
   sc.stall_it = sc.it;
+  opfk::set_iter(c->P, sc);
   CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->host_status = 0;
@@ -1686,6 +1689,7 @@ opf_status opf_set_state_from_nodes(opf_ctx *c, int32_t on_device, const float *
   sc.frozen_at = 0;
   sc.stall_ref = HUGE_VAL;
   sc.stall_it = sc.it;
+  opfk::set_iter(c->P, sc);
   CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->host_status = 0;

@@ -37,6 +37,23 @@ constexpr int BLOCK = 256;
 // clamps (fminf/fmaxf) would otherwise turn a NaN input into a finite bound.
 enum { SL_PP = 0, SL_PT = 1, SL_DP = 2, SL_DT = 3, SL_NF = 4, NSLOT = 5 };
 
+// The scalars of the current iteration in the form the iteration kernels read
+// them: two 16-byte loads per thread, with no barrier, conversion or 64-bit
+// remainder in front of a kernel's first load of the state.  Every writer of
+// DevScalars keeps it in step (set_iter).
+struct alignas(16) Iter {
+  float frp, frt, fsu, fsv;   // penalties, pending rescales of u and v
+  float rho_dev;              // rho' = (K+1) rho_p
+  int old;                    // buffer of the previous iterate (it & 1)
+  int flags;                  // ITF_*
+  int pad;
+};
+enum {
+  ITF_SKIP = 1,      // stopped in this call (passed stopping test, stall) or a sticky error: return at once
+  ITF_RES = 2,       // the residuals are read (stopping test, adaptation, end of the call)
+  ITF_VFRESH = 4     // V1/V2 already hold the current v
+};
+
 // Scalars that persist on the device between launches.
 struct DevScalars {
   double rho_p, rho_th;  // penalties in force for the next iteration
@@ -60,6 +77,7 @@ struct DevScalars {
   int stalled;
   int pad0;
   long long hist_n;      // residual-history rows written (ring of Params::hist_cap rows)
+  Iter cur;              // the next iteration's scalars (set_iter)
 };
 
 // Battery group offsets inside lam/beta rows of stride Tp = T + 1.
@@ -123,6 +141,7 @@ struct Params {
   // scratch
   double *partials;  // [node_grid][NSLOT] per-CTA residual partial sums of the node kernel
   int node_grid;     // CTAs of the node kernel (partial-sum slots)
+  unsigned *done;    // CTAs of the node kernel that have finished this iteration (0 between iterations)
   int dsum_lean;     // IterPlan::dsum_lean
   DevScalars *sc;
   // options
@@ -157,11 +176,37 @@ __host__ __device__ __forceinline__ size_t nidx(const Params &p, int k, int n, i
   return ((size_t)n * p.Kp + k) * p.T + t;
 }
 
+// whether the penalties may still change after iteration itn (1-based):
+// adaptation on, within opf_options.adapt_until, not fixed by the stall rule
+__host__ __device__ __forceinline__ bool adapting(const Params &p, const DevScalars &sc, long long itn) {
+  return p.adapt_every > 0 && (p.adapt_until <= 0 || itn <= p.adapt_until) && sc.frozen_at == 0;
+}
+// iteration itn adapts the penalties (Section 3.5, every adapt_every iterations)
+__host__ __device__ __forceinline__ bool adapt_at(const Params &p, const DevScalars &sc, long long itn) {
+  return adapting(p, sc, itn) && itn % p.adapt_every == 0;
+}
+// iteration itn forms its residuals
+__host__ __device__ __forceinline__ bool res_at(const Params &p, const DevScalars &sc, long long itn) {
+  return adapt_at(p, sc, itn) || (p.eps > 0 && p.check_every > 0 && itn % p.check_every == 0) || itn >= sc.it_last;
+}
+// the next iteration's scalars from the persistent ones
+__host__ __device__ __forceinline__ void set_iter(const Params &p, DevScalars &sc) {
+  Iter r;
+  r.frp = (float)sc.rho_p;
+  r.frt = (float)sc.rho_th;
+  r.fsu = (float)sc.su;
+  r.fsv = (float)sc.sv;
+  r.rho_dev = (float)(p.Kp_glob * sc.rho_p);
+  r.old = (int)(sc.it & 1);
+  r.flags = ((sc.status != 0 || sc.stop != 0) ? ITF_SKIP : 0) | (res_at(p, sc, sc.it + 1) ? ITF_RES : 0) |
+            (sc.v_fresh ? ITF_VFRESH : 0);
+  r.pad = 0;
+  sc.cur = r;
+}
+
 // Launch configuration of one iteration's kernels.
 struct IterPlan {
   int line_grid, node_grid, xs_grid, inner_grid, dsum_grid;  // 0: the kernel has no work
-  int lean_grid;   // residual-free node pass (T % 4 == 0 and plain ADMM only)
-  int n_slabs, slab_k;  // contingency slabs of the line / node kernels, slab_k contingencies each
   size_t inner_smem;
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
   int dsum_lean;   // 1: the passes without residuals sum device powers themselves (dsum only where
@@ -171,8 +216,7 @@ struct IterPlan {
 // A batch of instances: the CTA schedules of each batch kernel, concatenated
 // in one array of (instance, block within the instance, blocks of the
 // instance, 0), in the order of BatchKernel.
-enum BatchKernel { BK_XS4, BK_XS1, BK_INNER, BK_DSUM2, BK_DSUM1, BK_LINE4, BK_LINE1, BK_NODE4, BK_NODE1,
-                   BK_DECIDE, BK_COUNT };
+enum BatchKernel { BK_XS4, BK_XS1, BK_INNER, BK_DSUM2, BK_DSUM1, BK_LINE4, BK_LINE1, BK_NODE4, BK_NODE1, BK_COUNT };
 struct BatchPlan {
   int count[BK_COUNT];
   int offset[BK_COUNT];
@@ -200,12 +244,12 @@ int opf_record_error(int s, const char *msg);
 int opfk_plan(const opfk::Params &p, opfk::IterPlan *plan);
 // Start a call of n iterations: the residuals are formed at its last one;
 // clear_stop restarts a context that stopped (opf_iterate, not batches).
-int opfk_begin_launch(opfk::DevScalars *sc, long long n, int clear_stop, void *stream);
+int opfk_begin_launch(const opfk::Params &p, long long n, int clear_stop, void *stream);
 int opfk_begin_batch_launch(const opfk::Params *d_params, int n_inst, long long n, void *stream);
-// Enqueue one iteration: xs, inner, dsum, the node kernels and decide on
-// main_stream, the line kernels on aux_stream (forked after the previous
-// iteration; each slab joined before its node kernel).  Works under stream
-// capture.
+// Enqueue one iteration: xs, inner, dsum and the node kernel (whose last CTA
+// takes the decisions) on main_stream, the line kernel on aux_stream (forked
+// after the previous iteration, joined before the node kernel).  Works under
+// stream capture.
 int opfk_iteration_enqueue(const opfk::Params &p, const opfk::IterPlan &plan, void *main_stream,
                            void *aux_stream, void *ev_fork, void *ev_join);
 // Schedules of the batch kernels for n instances (host parameter copies and
@@ -236,7 +280,7 @@ int opfk_export_lines_launch(const opfk::Params &p, int cur, float *p_line, floa
 int opfk_export_pdev_launch(const opfk::Params &p, float *out, void *stream);
 int opfk_export_nodes_launch(const opfk::Params &p, int cur, float *u, float *theta_node,
                              float *price, void *stream);
-int opfk_set_rho_launch(opfk::DevScalars *sc, double rho, void *stream);
+int opfk_set_rho_launch(const opfk::Params &p, double rho, void *stream);
 // Contingency slices: the local half of one iteration (devices from the
 // exchanged sums, line proxes, node sums, then this slice's sums into the
 // exchange buffer) and the decisions from the exchanged sums; `prime`

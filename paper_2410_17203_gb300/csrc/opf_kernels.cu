@@ -45,11 +45,10 @@ namespace opfk {
 constexpr int WARPS = BLOCK / 32;
 constexpr int ST_NONFINITE = 5;  // opf_status value set on the device
 constexpr int NODE_VW = 4;       // time steps per node item
-constexpr int NODE_MIN_CTAS = 2; // resident CTAs per SM the node kernel is compiled for
+constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is compiled for (64 registers)
+constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
+constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
 constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items)
-constexpr int N_SLABS = 1;       // contingency slabs per iteration (line / node overlap)
-constexpr int NODE_LEAN_CTAS = 4;  // resident CTAs per SM of the residual-free node pass
-constexpr int NODE_LEAN_NB = 2;    // line terminals it gathers together
 constexpr int REG_T = 127;         // longest horizon of the register-resident inner ADMM (T + 1 <= 4 x 32)
 
 // shared floats per warp of the shared-memory inner ADMM: 3 (T+1) for the
@@ -1032,16 +1031,17 @@ __device__ __forceinline__ void line_item(const Params &p, int old, int nw, int 
 // terminal codes come four at a time so that a node's row loads issue
 // together.
 // ---------------------------------------------------------------------------
-// res = 0: the iteration's residuals are not read, so the node sums skip the
+// RES false: the iteration's residuals are not read, so the node sums skip the
 // inputs only they need (old p and theta_bar rows, the device Welford state)
 // and their accumulation; the relaxed variant always needs the mean change.
+// NB: line terminals gathered together.
 // ILD: where the pass forms no residuals, whether it sums the device powers
 // itself (0 never, 1 always, 2 as Params::dsum_lean says)
-template <int VW, bool RELAX, int NB = 4, int ILD = 2>
+template <int VW, bool RELAX, bool RES, int NB, int ILD>
 __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int k, int n, int toff, float fsu,
-                                          float *acc, bool res) {
+                                          float *acc) {
   const int T = p.T;
-  if constexpr (RELAX) res = true;
+  constexpr bool res = RES || RELAX;
   // level 1: the node record, the node's old rows and its device sums
   const int4 r0 = p.nrec[3 * n], r1 = p.nrec[3 * n + 1], r2 = p.nrec[3 * n + 2];
   const float cp = __int_as_float(r0.x), ct = __int_as_float(r0.y);
@@ -1173,51 +1173,17 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   stv_cs<VW>(p.THBAR[nw] + on, tbar);
 }
 
-// ---------------------------------------------------------------------------
-// the persistent iteration kernel
-// ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// the scalars of the current iteration, read once per CTA.  A context that
-// stopped in this call (passed stopping test) or holds a sticky error makes
-// every kernel return at once.
-// ---------------------------------------------------------------------------
-struct Iter {
-  float frp, frt, fsu, fsv, rho_dev;
-  int old, nw, v_fresh, skip;
-  int res;   // this iteration's residuals are read (stopping test, adaptation, end of the call)
-};
-
-// whether the penalties may still change after iteration itn (1-based):
-// adaptation on, within opf_options.adapt_until, not fixed by the stall rule
-__device__ __forceinline__ bool adapting(const Params &p, const DevScalars &sc, long long itn) {
-  return p.adapt_every > 0 && (p.adapt_until <= 0 || itn <= p.adapt_until) && sc.frozen_at == 0;
-}
-// iteration itn adapts the penalties (Section 3.5, every adapt_every iterations)
-__device__ __forceinline__ bool adapt_at(const Params &p, const DevScalars &sc, long long itn) {
-  return adapting(p, sc, itn) && itn % p.adapt_every == 0;
-}
-
-__device__ __forceinline__ Iter iter_scalars(const Params &p) {
-  __shared__ Iter s;
-  if (threadIdx.x == 0) {
-    const DevScalars sc = *p.sc;
+// the current iteration's scalars (the same two loads in every thread)
+__device__ __forceinline__ Iter load_iter(const Params &p) {
+  union {
     Iter r;
-    r.frp = (float)sc.rho_p;
-    r.frt = (float)sc.rho_th;
-    r.fsu = (float)sc.su;
-    r.fsv = (float)sc.sv;
-    r.rho_dev = (float)(p.Kp_glob * sc.rho_p);   // rho' = (K+1) rho_p
-    r.old = (int)(sc.it & 1);
-    r.nw = r.old ^ 1;
-    r.v_fresh = sc.v_fresh;
-    r.skip = (sc.status != 0 || sc.stop != 0) ? 1 : 0;
-    const long long itn = sc.it + 1;
-    r.res = adapt_at(p, sc, itn) || (p.eps > 0 && p.check_every > 0 && itn % p.check_every == 0) ||
-            itn >= sc.it_last;
-    s = r;
-  }
-  __syncthreads();
-  return s;
+    int4 v[2];
+  } x;
+  static_assert(sizeof(Iter) == 32, "Iter is loaded as two int4");
+  const int4 *s = reinterpret_cast<const int4 *>(&p.sc->cur);
+  x.v[0] = s[0];
+  x.v[1] = s[1];
+  return x.r;
 }
 
 // ---------------------------------------------------------------------------
@@ -1227,8 +1193,8 @@ __device__ __forceinline__ Iter iter_scalars(const Params &p) {
 // ---------------------------------------------------------------------------
 template <int VW>
 __device__ __forceinline__ void xs_body(const Params &p, unsigned bid, unsigned nblk) {
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   const int T = p.T, TV = T / VW, Kp = p.Kp;
   const float kpf = (float)p.Kp_glob, rkp = __frcp_rn(kpf);
   const size_t KT = (size_t)Kp * T;    // a node's K+1 rows are contiguous
@@ -1310,8 +1276,8 @@ __device__ __forceinline__ void ramp_r(const Params &p, int r, float rho, int la
 // ---------------------------------------------------------------------------
 template <int C, bool MIXED>
 __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem) {
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int T = p.T;
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
@@ -1355,11 +1321,11 @@ __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsign
 // ---------------------------------------------------------------------------
 template <int VW>
 __device__ __forceinline__ void dsum_body(const Params &p, unsigned bid, unsigned nblk) {
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   // with dsum_lean the node passes that form no residuals sum the device
   // powers themselves
-  if (p.dsum_lean && !q.res && p.alpha == 1.f) return;
+  if (p.dsum_lean && !(q.flags & ITF_RES) && p.alpha == 1.f) return;
   const int T = p.T, TV = T / VW;
   const unsigned n_items = (unsigned)p.N * (unsigned)TV;
   for (unsigned item = bid * BLOCK + threadIdx.x; item < n_items; item += nblk * BLOCK) {
@@ -1390,76 +1356,23 @@ __device__ __forceinline__ void dsum_body(const Params &p, unsigned bid, unsigne
 // line: step 1 for every (contingency, line, VW time steps)
 // ---------------------------------------------------------------------------
 template <int VW>
-__device__ __forceinline__ void line_body(const Params &p, int k0, int k1, unsigned bid) {
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
+__device__ __forceinline__ void line_body(const Params &p, unsigned bid) {
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   const int L = p.L, TV = p.T / VW;
-  const unsigned n = (unsigned)(k1 - k0) * (unsigned)L * (unsigned)TV;
+  const unsigned n = (unsigned)p.Kp * (unsigned)L * (unsigned)TV;
   // each CTA takes LINE_IPT consecutive blocks of BLOCK items, so CTAs are
   // short-lived and the device kernels' CTAs find room beside them
   const unsigned base = bid * (unsigned)(BLOCK * LINE_IPT) + threadIdx.x;
   // items (line, contingency, step block): a line's K+1 rows are contiguous
-  const int KK = k1 - k0;
+  const int Kp = p.Kp;
   Idx3 ix, dx;
-  ix.set(base, KK, TV);
-  dx.set(BLOCK, KK, TV);
+  ix.set(base, Kp, TV);
+  dx.set(BLOCK, Kp, TV);
 #pragma unroll 1
-  for (int j = 0; j < LINE_IPT; ++j, ix.step(dx, KK, TV)) {
+  for (int j = 0; j < LINE_IPT; ++j, ix.step(dx, Kp, TV)) {
     if (base + (unsigned)(j * BLOCK) < n)
-      line_item<VW>(p, q.old, q.nw, k0 + ix.b, ix.a, ix.c * VW, q.frp, q.frt, q.fsu, q.fsv, q.v_fresh);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// node: step 3 for every (contingency, node, VW time steps), and the CTA's
-// residual partial sums: FP32 per thread, FP64 across warps
-// ---------------------------------------------------------------------------
-// LEAN: the variant for iterations that form no residuals (it returns at
-// once on the others); the general variant returns at once on those when a
-// lean launch covers them.
-template <int VW, bool RELAX, bool LEAN = false, int ILD = 2>
-__device__ __forceinline__ void node_body(const Params &p, int k0, int k1, int first, unsigned bid,
-                                          unsigned nblk, bool lean_split = false) {
-  __shared__ double red[WARPS][NSLOT];
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
-  if constexpr (LEAN) {
-    if (q.res) return;
-  } else {
-    if (lean_split && !q.res) return;
-  }
-  const int N = p.N, TV = p.T / VW;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const unsigned n = (unsigned)(k1 - k0) * (unsigned)N * (unsigned)TV;
-  const unsigned stride = nblk * BLOCK;
-  unsigned item = bid * BLOCK + threadIdx.x;
-  float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  // items (node, contingency, step block): a node's K+1 rows are contiguous,
-  // and so are the K+1 rows of each line it gathers
-  const int KK = k1 - k0;
-  Idx3 ix, dx;
-  ix.set(item, KK, TV);
-  dx.set(stride, KK, TV);
-  for (; item < n; item += stride, ix.step(dx, KK, TV))
-    node_item<VW, RELAX, LEAN ? NODE_LEAN_NB : 4, ILD>(p, q.old, q.nw, k0 + ix.b, ix.a, ix.c * VW, q.fsu, acc,
-                                                  LEAN ? false : q.res != 0);
-  if constexpr (!LEAN) {
-    if (!q.res) return;   // nothing reads this iteration's partial sums
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-      float v = acc[s];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) red[wib][s] = (double)v;
-    }
-    __syncthreads();
-    // the slabs of one iteration run in order on one stream: the first one
-    // sets the CTA's partial sums, the others add to them
-    if (threadIdx.x < NSLOT) {
-      double v = first ? 0.0 : p.partials[(size_t)bid * NSLOT + threadIdx.x];
-      for (int w = 0; w < WARPS; ++w) v += red[w][threadIdx.x];
-      p.partials[(size_t)bid * NSLOT + threadIdx.x] = v;
-    }
+      line_item<VW>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.frp, q.frt, q.fsu, q.fsv, q.flags & ITF_VFRESH);
   }
 }
 
@@ -1469,7 +1382,8 @@ __device__ __forceinline__ void node_body(const Params &p, int k0, int k1, int f
 // adaptive penalty (Section 3.5); advances the iteration counter.
 // ---------------------------------------------------------------------------
 // the node kernel's n_part CTA partial sums reduced in FP64 and a fixed
-// order; thread 0 returns true with the totals
+// order; thread 0 returns true with the totals (written by other CTAs of the
+// same launch: read past L1)
 __device__ __forceinline__ bool reduce_partials(const Params &p, int n_part, double tot[NSLOT],
                                                 double (*red)[NSLOT]) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1477,7 +1391,7 @@ __device__ __forceinline__ bool reduce_partials(const Params &p, int n_part, dou
   for (int s = 0; s < NSLOT; ++s) tot[s] = 0.0;
   for (int b = threadIdx.x; b < n_part; b += BLOCK) {
 #pragma unroll
-    for (int s = 0; s < NSLOT; ++s) tot[s] += p.partials[(size_t)b * NSLOT + s];
+    for (int s = 0; s < NSLOT; ++s) tot[s] += __ldcg(p.partials + (size_t)b * NSLOT + s);
   }
 #pragma unroll
   for (int s = 0; s < NSLOT; ++s) {
@@ -1497,11 +1411,8 @@ __device__ __forceinline__ bool reduce_partials(const Params &p, int n_part, dou
   return true;
 }
 
-__device__ __forceinline__ void decide_body(const Params &p, int n_part) {
-  __shared__ double red[WARPS][NSLOT];
-  const Iter q = iter_scalars(p);
-  if (q.skip) return;
-  if (!q.res) {
+__device__ __forceinline__ void decide_body(const Params &p, int n_part, bool res, double (*red)[NSLOT]) {
+  if (!res) {
     // nothing reads this iteration's residuals (a non-finite value is caught
     // at the next iteration that forms them): advance
     if (threadIdx.x == 0) {
@@ -1510,6 +1421,7 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part) {
       sc.sv = 1.0;
       sc.it = sc.it + 1;
       sc.v_fresh = 0;
+      set_iter(p, sc);
       *p.sc = sc;
     }
     return;
@@ -1594,7 +1506,74 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part) {
   sc.rho_th = nrt;
   sc.it = itn;
   sc.v_fresh = 0;
+  set_iter(p, sc);
   *p.sc = sc;
+}
+
+// ---------------------------------------------------------------------------
+// node: step 3 for every (contingency, node, VW time steps); where the
+// residuals are read, the CTA's partial sums (FP32 per thread, FP64 across
+// warps); then the last CTA to finish takes the decisions and advances the
+// iteration (a slice's decisions wait for the exchange: opf_slice_finish).
+// One launch serves both kinds of iteration and the decisions: as three
+// kernels (a residual-free pass, a general one and the decisions, each
+// returning at once when not due) an iteration of 2k buses spent about 5 of
+// its 36 us on their launches.  At 64 registers (four CTAs per SM, what the
+// residual-free pass wants) the general pass gathers one terminal at a time.
+// ---------------------------------------------------------------------------
+template <int VW, bool RELAX, int ILD>
+__device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk) {
+  __shared__ double red[WARPS][NSLOT];
+  __shared__ int s_last;
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
+  const bool res = q.flags & ITF_RES;
+  const int N = p.N, TV = p.T / VW, Kp = p.Kp;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const unsigned n = (unsigned)Kp * (unsigned)N * (unsigned)TV;
+  const unsigned stride = nblk * BLOCK;
+  unsigned item = bid * BLOCK + threadIdx.x;
+  float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  // items (node, contingency, step block): a node's K+1 rows are contiguous,
+  // and so are the K+1 rows of each line it gathers
+  Idx3 ix, dx;
+  ix.set(item, Kp, TV);
+  dx.set(stride, Kp, TV);
+  if (res || RELAX) {
+    for (; item < n; item += stride, ix.step(dx, Kp, TV))
+      node_item<VW, RELAX, true, RELAX ? 4 : NODE_RES_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+  } else {
+    for (; item < n; item += stride, ix.step(dx, Kp, TV))
+      node_item<VW, RELAX, false, NODE_LEAN_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+  }
+  if (res) {
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s) {
+      float v = acc[s];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) red[wib][s] = (double)v;
+    }
+    __syncthreads();
+    if (threadIdx.x < NSLOT) {
+      double v = 0.0;
+      for (int w = 0; w < WARPS; ++w) v += red[w][threadIdx.x];
+      p.partials[(size_t)bid * NSLOT + threadIdx.x] = v;
+    }
+  }
+  if (p.slice) return;
+  // the count is taken after every thread of the CTA has read the scalars and
+  // (res) its partial sums are written; the last CTA alone goes on
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(p.done, 1u) == nblk - 1;
+    if (s_last) *p.done = 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  decide_body(p, (int)nblk, res, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -1616,25 +1595,24 @@ template <int VW>
 __global__ void __launch_bounds__(BLOCK) dsum_kernel(Params p) { dsum_body<VW>(p, blockIdx.x, gridDim.x); }
 
 template <int VW>
-__global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p, int k0, int k1) {
-  line_body<VW>(p, k0, k1, blockIdx.x);
+__global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p) {
+  line_body<VW>(p, blockIdx.x);
 }
 
 // the over-relaxed variant carries more per-terminal state: it takes the
-// registers of one CTA per SM rather than spill
-template <int VW, bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_MIN_CTAS) node_kernel(Params p, int k0, int k1, int first) {
-  node_body<VW, RELAX>(p, k0, k1, first, blockIdx.x, gridDim.x, !RELAX && VW == NODE_VW);
+// registers of one CTA per SM rather than spill; ILD: the plan's dsum_lean
+template <int VW, bool RELAX, int ILD>
+__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel(Params p) {
+  node_body<VW, RELAX, ILD>(p, blockIdx.x, gridDim.x);
 }
 
-// the residual-free node pass: fewer live values, more CTAs per SM
-// ILD: the plan's dsum_lean, fixed at compile time for this pass
-template <int ILD>
-__global__ void __launch_bounds__(BLOCK, NODE_LEAN_CTAS) node_kernel_lean(Params p, int k0, int k1, int first) {
-  node_body<NODE_VW, false, true, ILD>(p, k0, k1, first, blockIdx.x, gridDim.x);
+// a slice's decisions, from the exchanged sums
+__global__ void __launch_bounds__(BLOCK) decide_kernel(Params p) {
+  __shared__ double red[WARPS][NSLOT];
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
+  decide_body(p, 0, q.flags & ITF_RES, red);
 }
-
-__global__ void __launch_bounds__(BLOCK) decide_kernel(Params p, int n_part) { decide_body(p, n_part); }
 
 // A contingency slice's contributions to the exchange (after its node
 // sums): sum over its k of pbar + u at every node with devices, the same of
@@ -1654,8 +1632,7 @@ __global__ void __launch_bounds__(BLOCK) slice_sums_kernel(Params p, int prime) 
     const int old = (int)(sc.it & 1);
     s_buf = current ? old : old ^ 1;
     s_with_u = current || adapt_at(p, sc, itn);
-    s_res = !current && ((p.adapt_every > 0 && adapt_at(p, sc, itn)) ||
-                         (p.eps > 0 && p.check_every > 0 && itn % p.check_every == 0) || itn >= sc.it_last);
+    s_res = !current && res_at(p, sc, itn);
   }
   __syncthreads();
   const int T = p.T, Kp = p.Kp;
@@ -1732,22 +1709,15 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, cons
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  line_body<VW>(p, 0, p.Kp, bid);
+  line_body<VW>(p, bid);
 }
 
 template <int VW, bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_MIN_CTAS) node_kernel_b(const Params *ps, const int4 *sched) {
+__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched) {
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  node_body<VW, RELAX>(p, 0, p.Kp, 1, bid, nblk);
-}
-
-__global__ void __launch_bounds__(BLOCK) decide_kernel_b(const Params *ps, const int4 *sched) {
-  __shared__ Params sp;
-  unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  decide_body(p, p.node_grid);
+  node_body<VW, RELAX, 2>(p, bid, nblk);
 }
 
 // A line's terminal values from its stored (p, mid) at contingency k:
@@ -1963,30 +1933,38 @@ __global__ void export_pdev_kernel(Params p, float *out) {
     out[i] = rx ? fmaf(c, p.DPD[i], p.PD[i]) : p.PD[i];
 }
 
-__global__ void begin_kernel(DevScalars *sc, long long n, int clear_stop) {
+__global__ void begin_kernel(Params p, long long n, int clear_stop) {
+  DevScalars sc = *p.sc;
   if (clear_stop) {
-    sc->stop = 0;
-    if (sc->stalled) {   // a new call after a stall restarts the stall window
-      sc->stalled = 0;
-      sc->stall_ref = HUGE_VAL;
-      sc->stall_it = sc->it;
+    sc.stop = 0;
+    if (sc.stalled) {   // a new call after a stall restarts the stall window
+      sc.stalled = 0;
+      sc.stall_ref = HUGE_VAL;
+      sc.stall_it = sc.it;
     }
   }
-  sc->it_last = sc->it + n;
+  sc.it_last = sc.it + n;
+  set_iter(p, sc);
+  *p.sc = sc;
 }
 
 __global__ void begin_batch_kernel(const Params *ps, int n_inst, long long n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_inst) ps[i].sc->it_last = ps[i].sc->it + n;
+  if (i >= n_inst) return;
+  DevScalars sc = *ps[i].sc;
+  sc.it_last = sc.it + n;
+  set_iter(ps[i], sc);
+  *ps[i].sc = sc;
 }
 
-__global__ void set_rho_kernel(DevScalars *sc, double rho) {
-  DevScalars s = *sc;
+__global__ void set_rho_kernel(Params p, double rho) {
+  DevScalars s = *p.sc;
   s.su *= s.rho_p / rho;
   s.sv *= s.rho_th / rho;
   s.rho_p = rho;
   s.rho_th = rho;
-  *sc = s;
+  set_iter(p, s);
+  *p.sc = s;
 }
 
 static size_t inner_smem(int T) { return (size_t)WARPS * warp_smem_floats(T) * sizeof(float); }
@@ -2014,26 +1992,16 @@ int opfk_plan(const Params &p, IterPlan *plan) {
       cudaFuncSetAttribute(inner_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism) != cudaSuccess)
     return -1;
   const bool vn = (p.T % NODE_VW == 0);
-  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false>, 0) : resident_grid(node_kernel<1, false>, 0);
-  const int gl = vn ? resident_grid(node_kernel_lean<0>, 0) : 0;
+  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false, 0>, 0) : resident_grid(node_kernel<1, false, 0>, 0);
   const int gx = v4 ? resident_grid(xs_kernel<4>, 0) : resident_grid(xs_kernel<1>, 0);
   const int gd = v2 ? resident_grid(dsum_kernel<2>, 0) : resident_grid(dsum_kernel<1>, 0);
   if (gn < 1 || gx < 1 || gd < 1) return -1;
-  // contingency slabs: the node sums of slab s run beside the line proxes of
-  // slab s + 1, so the latency-bound node pass overlaps the bandwidth-bound
-  // line pass; a few slabs keep the launch count low
-  int ns = std::min(N_SLABS, p.Kp);
-  int G = (p.Kp + ns - 1) / ns;
-  ns = (p.Kp + G - 1) / G;
-  plan->n_slabs = ns;
-  plan->slab_k = G;
   const long long tvl = p.T / (v4 ? 4 : 1), tvn = p.T / (vn ? NODE_VW : 1);
-  const long long nl = (long long)G * p.L * tvl, nn = (long long)G * p.N * tvn;
+  const long long nl = (long long)p.Kp * p.L * tvl, nn = (long long)p.Kp * p.N * tvn;
   const long long nx = (long long)p.n_dnode * (p.T / (v4 ? 4 : 1));
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
   plan->line_grid = (int)((nl + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT));
   plan->node_grid = (int)std::min<long long>(gn, (nn + BLOCK - 1) / BLOCK);
-  plan->lean_grid = vn ? (int)std::min<long long>(gl, (nn + BLOCK - 1) / BLOCK) : 0;
   plan->xs_grid = (int)std::min<long long>(gx, (nx + BLOCK - 1) / BLOCK);
   plan->inner_grid = (n_inner + WARPS - 1) / WARPS;
   {
@@ -2085,9 +2053,8 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
                              void *ev_fork, void *ev_join, bool slice) {
   cudaStream_t sm = (cudaStream_t)main_stream, sa = (cudaStream_t)aux_stream;
   const bool v4 = (p.T % 4 == 0), v2 = (p.T % 2 == 0);
-  // The line proxes of slab s (aux stream) read only the previous iterate;
-  // the node sums of slab s (main stream) follow them and the device
-  // kernels, and run beside the line proxes of slab s + 1.
+  // The line proxes (aux stream) read only the previous iterate; the node
+  // sums (main stream) follow them and the device kernels.
   if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
   if (plan.xs_grid > 0) {
@@ -2105,30 +2072,24 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
   }
   if (v2) dsum_kernel<2><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
   else dsum_kernel<1><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
-  for (int s = 0; s < plan.n_slabs; ++s) {
-    const int k0 = s * plan.slab_k, k1 = std::min(p.Kp, k0 + plan.slab_k);
-    if (plan.line_grid > 0 && p.L > 0) {
-      const int lg = (int)(((long long)(k1 - k0) * p.L * (p.T / (v4 ? 4 : 1)) + (long long)BLOCK * LINE_IPT - 1) /
-                           ((long long)BLOCK * LINE_IPT));
-      if (v4) line_kernel<4><<<lg, BLOCK, 0, sa>>>(p, k0, k1);
-      else line_kernel<1><<<lg, BLOCK, 0, sa>>>(p, k0, k1);
-      if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
-      if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
-    }
-    const bool vn = p.T % NODE_VW == 0, rx = p.alpha != 1.f;
-    if (vn && !rx) {
-      // one of the two returns at once: the general pass forms residuals,
-      // the lean one runs the iterations that need none
-      node_kernel<NODE_VW, false><<<plan.node_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
-      if (p.dsum_lean) node_kernel_lean<1><<<plan.lean_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
-      else node_kernel_lean<0><<<plan.lean_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
-    }
-    else if (!rx) node_kernel<1, false><<<plan.node_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
-    else if (vn) node_kernel<NODE_VW, true><<<plan.node_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
-    else node_kernel<1, true><<<plan.node_grid, BLOCK, 0, sm>>>(p, k0, k1, s == 0);
+  if (plan.line_grid > 0) {
+    if (v4) line_kernel<4><<<plan.line_grid, BLOCK, 0, sa>>>(p);
+    else line_kernel<1><<<plan.line_grid, BLOCK, 0, sa>>>(p);
+  }
+  if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
+  if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
+  const bool vn = p.T % NODE_VW == 0;
+  if (p.alpha != 1.f) {
+    if (vn) node_kernel<NODE_VW, true, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
+    else node_kernel<1, true, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
+  } else if (vn) {
+    if (p.dsum_lean) node_kernel<NODE_VW, false, 1><<<plan.node_grid, BLOCK, 0, sm>>>(p);
+    else node_kernel<NODE_VW, false, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
+  } else {
+    if (p.dsum_lean) node_kernel<1, false, 1><<<plan.node_grid, BLOCK, 0, sm>>>(p);
+    else node_kernel<1, false, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
   }
   if (slice) slice_sums_kernel<<<aux_grid((long long)p.n_dnode * p.T), BLOCK, 0, sm>>>(p, 0);
-  else decide_kernel<<<1, BLOCK, 0, sm>>>(p, plan.node_grid);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2143,7 +2104,7 @@ int opfk_slice_local_enqueue(const Params &p, const IterPlan &plan, void *main_s
 }
 
 int opfk_slice_finish_enqueue(const Params &p, void *stream) {
-  decide_kernel<<<1, BLOCK, 0, (cudaStream_t)stream>>>(p, p.node_grid);
+  decide_kernel<<<1, BLOCK, 0, (cudaStream_t)stream>>>(p);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2202,9 +2163,6 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           break;
         case BK_NODE4: case BK_NODE1:
           if ((kind == BK_NODE4) == vn) blocks = plans[i].node_grid;
-          break;
-        case BK_DECIDE:
-          blocks = 1;
           break;
       }
       // the grid-stride phases take any block count: `div` puts more work in
@@ -2286,7 +2244,6 @@ int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPl
     if (bp.count[BK_NODE4]) node_kernel_b<4, true><<<bp.count[BK_NODE4], BLOCK, 0, sm>>>(d_params, at(BK_NODE4));
     if (bp.count[BK_NODE1]) node_kernel_b<1, true><<<bp.count[BK_NODE1], BLOCK, 0, sm>>>(d_params, at(BK_NODE1));
   }
-  if (bp.count[BK_DECIDE]) decide_kernel_b<<<bp.count[BK_DECIDE], BLOCK, 0, sm>>>(d_params, at(BK_DECIDE));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2328,8 +2285,8 @@ int opfk_export_lines_launch(const Params &p, int cur, float *pl, float *a1, flo
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int opfk_begin_launch(DevScalars *sc, long long n, int clear_stop, void *stream) {
-  begin_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(sc, n, clear_stop);
+int opfk_begin_launch(const Params &p, long long n, int clear_stop, void *stream) {
+  begin_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(p, n, clear_stop);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2350,7 +2307,7 @@ int opfk_export_nodes_launch(const Params &p, int cur, float *u, float *theta, f
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int opfk_set_rho_launch(DevScalars *sc, double rho, void *stream) {
-  set_rho_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(sc, rho);
+int opfk_set_rho_launch(const Params &p, double rho, void *stream) {
+  set_rho_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(p, rho);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
