@@ -334,6 +334,7 @@ void carve(opf_ctx *c, Arena &a) {
   p.dnode_ptr = a.take<int>(c->n_dnode + 1);
   p.dnode_dev = a.take<int>(c->n_closed);
   p.dnode_keep = a.take<int>(c->n_dnode);
+  p.crec = a.take<int4>(c->n_dnode);
   p.dev_a = a.take<float>(c->S);
   p.dev_b = a.take<float>(c->S);
   p.dev_lo = a.take<float>(ST);
@@ -620,6 +621,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   // nodes with devices (avg_k(pbar + u) is formed once per node), their
   // closed-form devices, and whether inner-ADMM devices need the average
   std::vector<int> dnode_ids, dnode_ptr(1, 0), dnode_dev, dnode_keep;
+  std::vector<int4> crec;
   for (int n = 0; n < N; ++n) {
     if (dptr[n + 1] == dptr[n]) continue;
     int keep = 0;
@@ -628,6 +630,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
       else keep = 1;
     }
     dnode_ids.push_back(n);
+    if ((int)dnode_dev.size() > dnode_ptr.back()) crec.push_back(make_int4(n, dnode_ptr.back(), (int)dnode_dev.size(), 0));
     dnode_ptr.push_back((int)dnode_dev.size());
     dnode_keep.push_back(keep);
   }
@@ -667,6 +670,8 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
     q.n_stor = c->n_stor;
     q.n_hvdc = c->H;
     q.S = S;
+    q.n_cnode = (int)crec.size();
+    q.slice = slice ? 1 : 0;
     if (opfk_plan(q, &c->plan) != 0) {
       delete c;
       return fail(OPF_ECUDA, "occupancy query for the iteration kernels failed");
@@ -722,7 +727,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   p.n_hvdc = c->H;
   p.hvdc0 = G + D + c->B;
   p.node_grid = c->plan.node_grid;
-  p.dsum_lean = c->plan.dsum_lean;
+  p.n_cnode = (int)crec.size();
   p.eps = opt.eps;
   p.mu = opt.mu;
   p.gamma = opt.gamma;
@@ -795,6 +800,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   up(p.dnode_ptr, dnode_ptr);
   up(p.dnode_dev, dnode_dev);
   up(p.dnode_keep, dnode_keep);
+  up(p.crec, crec);
   up(p.dev_a, dev_a);
   up(p.dev_b, dev_b);
   up(p.dev_lo, lo);
@@ -958,9 +964,10 @@ opf_status opf_get_info(opf_ctx *c, opf_info *info) {
   info->tolerance = c->tol;
   {
     const opfk::IterPlan &pl = c->plan;
-    // a slice's decisions are a launch of their own (opf_slice_finish)
-    info->kernels_per_iteration =
-        (pl.xs_grid > 0) + (pl.inner_grid > 0) + 1 + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
+    // devices (one launch, or averages, inner ADMM and sums), lines, nodes; a
+    // slice's decisions are a launch of their own (opf_slice_finish)
+    const int dev = pl.fused ? (pl.dev_inner + pl.dev_closed > 0) : (pl.xs_grid > 0) + (pl.inner_grid > 0) + 1;
+    info->kernels_per_iteration = dev + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
   }
   info->N = c->N;
   info->L = c->L;

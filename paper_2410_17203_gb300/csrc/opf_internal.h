@@ -123,6 +123,9 @@ struct Params {
   // nodes with devices; per node its closed-form devices and whether it has
   // inner-ADMM devices, whose input avg_k(pbar + u) is then kept in XS
   const int *dnode_ids, *dnode_ptr, *dnode_dev, *dnode_keep;
+  // nodes with closed-form devices: (node, first and one past the last entry of dnode_dev, 0)
+  const int4 *crec;
+  int n_cnode;
   float *XS;  // [N][T], avg_k(pbar + u) of the previous iterate at kept nodes
   const float *dev_a, *dev_b;
   const float *dev_lo, *dev_hi;  // [S][T]
@@ -142,7 +145,6 @@ struct Params {
   double *partials;  // [node_grid][NSLOT] per-CTA residual partial sums of the node kernel
   int node_grid;     // CTAs of the node kernel (partial-sum slots)
   unsigned *done;    // CTAs of the node kernel that have finished this iteration (0 between iterations)
-  int dsum_lean;     // IterPlan::dsum_lean
   DevScalars *sc;
   // options
   double eps, mu, gamma, tol;
@@ -206,17 +208,18 @@ __host__ __device__ __forceinline__ void set_iter(const Params &p, DevScalars &s
 
 // Launch configuration of one iteration's kernels.
 struct IterPlan {
-  int line_grid, node_grid, xs_grid, inner_grid, dsum_grid;  // 0: the kernel has no work
+  int line_grid, node_grid;            // 0: the kernel has no work
+  int fused;                           // 1: one device kernel; 0: averages, inner ADMM and device sums apart
+  int dev_inner, dev_closed;           // fused: CTAs of the device kernel for inner-ADMM and closed-form devices
+  int xs_grid, inner_grid, dsum_grid;  // not fused
   size_t inner_smem;
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
-  int dsum_lean;   // 1: the passes without residuals sum device powers themselves (dsum only where
-                   // residuals are formed); for instances whose device chain the line pass cannot hide
 };
 
 // A batch of instances: the CTA schedules of each batch kernel, concatenated
 // in one array of (instance, block within the instance, blocks of the
 // instance, 0), in the order of BatchKernel.
-enum BatchKernel { BK_XS4, BK_XS1, BK_INNER, BK_DSUM2, BK_DSUM1, BK_LINE4, BK_LINE1, BK_NODE4, BK_NODE1, BK_COUNT };
+enum BatchKernel { BK_INNER, BK_CLOSED, BK_LINE4, BK_LINE1, BK_NODE4, BK_NODE1, BK_COUNT };
 struct BatchPlan {
   int count[BK_COUNT];
   int offset[BK_COUNT];
@@ -226,8 +229,8 @@ struct BatchPlan {
 };
 // How a batch schedule lays out CTAs: instances in `order` (NULL: as given),
 // each instance's CTAs of a phase contiguous or dealt round-robin across
-// instances, and `div` times fewer CTAs for the grid-stride phases (xs,
-// inner, dsum), each doing proportionally more work.
+// instances, and `div` times fewer CTAs for the grid-stride phases (devices,
+// node sums), each doing proportionally more work.
 struct BatchLayout {
   const int *order;
   int interleave;
@@ -246,8 +249,8 @@ int opfk_plan(const opfk::Params &p, opfk::IterPlan *plan);
 // clear_stop restarts a context that stopped (opf_iterate, not batches).
 int opfk_begin_launch(const opfk::Params &p, long long n, int clear_stop, void *stream);
 int opfk_begin_batch_launch(const opfk::Params *d_params, int n_inst, long long n, void *stream);
-// Enqueue one iteration: xs, inner, dsum and the node kernel (whose last CTA
-// takes the decisions) on main_stream, the line kernel on aux_stream (forked
+// Enqueue one iteration: the device kernel (or xs, inner and dsum) and the
+// node kernel (whose last CTA takes the decisions) on main_stream, the line kernel on aux_stream (forked
 // after the previous iteration, joined before the node kernel).  Works under
 // stream capture.
 int opfk_iteration_enqueue(const opfk::Params &p, const opfk::IterPlan &plan, void *main_stream,

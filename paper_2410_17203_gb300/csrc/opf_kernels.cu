@@ -49,6 +49,9 @@ constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is comp
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
 constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items)
+constexpr int DEVB = 128;        // threads per CTA of the device kernel (its inner-ADMM warps spread over more SMs)
+constexpr int DEV_WARPS = DEVB / 32;
+constexpr int CLOSED_LANES4 = 2, CLOSED_LANES1 = 8;   // lanes per closed-form item: the classes of ksum2 / ksum8
 constexpr int REG_T = 127;         // longest horizon of the register-resident inner ADMM (T + 1 <= 4 x 32)
 
 // shared floats per warp of the shared-memory inner ADMM: 3 (T+1) for the
@@ -176,60 +179,156 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   __syncwarp();
 }
 
-// sums over contingencies k of two node arrays (pbar + u and u; u_o may be
-// NULL, giving 0) at one (node, t) offset o, with 8 independent loads in
-// flight per step
-__device__ __forceinline__ void ksum(const float *pbar_o, const float *u_o, size_t o, size_t stride, int Kp,
-                                     float &sp, float &sq) {
-  float a[8], b[8];
+// ---------------------------------------------------------------------------
+// VW consecutive time steps per thread (4 -> 128-bit accesses when T % 4 == 0)
+// ---------------------------------------------------------------------------
+template <int VW>
+struct FV {
+  float v[VW];
+};
+
+template <int VW>
+__device__ __forceinline__ FV<VW> ldv(const float *p) {
+  FV<VW> r;
+  if constexpr (VW == 4) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
+  } else if constexpr (VW == 2) {
+    const float2 t = *reinterpret_cast<const float2 *>(p);
+    r.v[0] = t.x; r.v[1] = t.y;
+  } else {
+    r.v[0] = *p;
+  }
+  return r;
+}
+
+// streaming load (read once per iteration: evict first)
+template <int VW>
+__device__ __forceinline__ FV<VW> ldv_cs(const float *p) {
+  FV<VW> r;
+  if constexpr (VW == 4) {
+    const float4 t = __ldcs(reinterpret_cast<const float4 *>(p));
+    r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
+  } else if constexpr (VW == 2) {
+    const float2 t = __ldcs(reinterpret_cast<const float2 *>(p));
+    r.v[0] = t.x; r.v[1] = t.y;
+  } else {
+    r.v[0] = __ldcs(p);
+  }
+  return r;
+}
+
+template <int VW>
+__device__ __forceinline__ void stv(float *p, const FV<VW> &r) {
+  if constexpr (VW == 4) {
+    *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+  } else if constexpr (VW == 2) {
+    *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
+  } else {
+    *p = r.v[0];
+  }
+}
+
+// streaming store (not read again in this iteration: evict first)
+template <int VW>
+__device__ __forceinline__ void stv_cs(float *p, const FV<VW> &r) {
+  if constexpr (VW == 4) {
+    __stcs(reinterpret_cast<float4 *>(p), make_float4(r.v[0], r.v[1], r.v[2], r.v[3]));
+  } else if constexpr (VW == 2) {
+    __stcs(reinterpret_cast<float2 *>(p), make_float2(r.v[0], r.v[1]));
+  } else {
+    __stcs(p, r.v[0]);
+  }
+}
+
+// x / c given r = 1/c rounded to nearest: one FMA correction step gives the
+// correctly rounded quotient for these well-scaled operands (a plain x * r
+// would carry the rounding bias of r into every node average, iteration
+// after iteration).
+__device__ __forceinline__ float div_rn(float x, float c, float r) {
+  const float q = x * r;
+  return fmaf(fmaf(-q, c, x), r, q);
+}
+
+// Sums over contingencies k of a node array (o: its offset of k = 0; rows T
+// floats apart).  The order of each sum is fixed, so that every form of the
+// device averages (one thread here, a group of lanes in closed_body) agrees
+// bit for bit: ksum2 adds two partial sums, over even and odd k; ksum8 eight,
+// over k mod 8 while whole groups of eight last, the rest going to the first.
+template <int VW>
+__device__ __forceinline__ FV<VW> ksum2(const float *a, size_t o, int T, int Kp) {
+  FV<VW> c[2];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) { a[j] = 0.f; b[j] = 0.f; }
+  for (int e = 0; e < VW; ++e) c[0].v[e] = c[1].v[e] = 0.f;
+  const float *r = a + o;
   int k = 0;
-  for (; k + 8 <= Kp; k += 8) {
+#pragma unroll 4
+  for (; k + 2 <= Kp; k += 2, r += 2 * (size_t)T) {
+    const FV<VW> x = ldv<VW>(r), y = ldv<VW>(r + T);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      a[j] += pbar_o[(size_t)(k + j) * stride + o];
-      b[j] += u_o ? u_o[(size_t)(k + j) * stride + o] : 0.f;
+    for (int e = 0; e < VW; ++e) {
+      c[0].v[e] += x.v[e];
+      c[1].v[e] += y.v[e];
     }
   }
-  for (; k < Kp; ++k) {
-    a[0] += pbar_o[(size_t)k * stride + o];
-    b[0] += u_o ? u_o[(size_t)k * stride + o] : 0.f;
-  }
-  sp = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-  sq = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+  FV<VW> s;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) s.v[e] = 0.f;
+  if (k < Kp) s = ldv<VW>(r);
+#pragma unroll
+  for (int e = 0; e < VW; ++e) s.v[e] = (c[0].v[e] + s.v[e]) + c[1].v[e];
+  return s;
 }
 
-// The same sums for four consecutive time steps (o 16-byte aligned): one
-// 128-bit load per row, two rows of each array in flight per step.
-__device__ __forceinline__ void ksum4(const float *pbar_o, const float *u_o, size_t o, size_t stride, int Kp,
-                                      float4 &sp, float4 &sq) {
-  float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
+__device__ __forceinline__ float ksum8(const float *a, size_t o, int T, int Kp) {
+  float c[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) c[j] = 0.f;
+  const float *r = a + o;
   int k = 0;
-  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (; k + 2 <= Kp; k += 2) {
-    const float4 x0 = *reinterpret_cast<const float4 *>(pbar_o + (size_t)k * stride + o);
-    const float4 x1 = *reinterpret_cast<const float4 *>(pbar_o + (size_t)(k + 1) * stride + o);
-    const float4 y0 = u_o ? *reinterpret_cast<const float4 *>(u_o + (size_t)k * stride + o) : z;
-    const float4 y1 = u_o ? *reinterpret_cast<const float4 *>(u_o + (size_t)(k + 1) * stride + o) : z;
-    a0.x += x0.x; a0.y += x0.y; a0.z += x0.z; a0.w += x0.w;
-    a1.x += x1.x; a1.y += x1.y; a1.z += x1.z; a1.w += x1.w;
-    b0.x += y0.x; b0.y += y0.y; b0.z += y0.z; b0.w += y0.w;
-    b1.x += y1.x; b1.y += y1.y; b1.z += y1.z; b1.w += y1.w;
+#pragma unroll 1
+  for (; k + 8 <= Kp; k += 8, r += 8 * (size_t)T) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) c[j] += r[j * (size_t)T];
   }
-  if (k < Kp) {
-    const float4 x = *reinterpret_cast<const float4 *>(pbar_o + (size_t)k * stride + o);
-    const float4 y = u_o ? *reinterpret_cast<const float4 *>(u_o + (size_t)k * stride + o) : z;
-    a0.x += x.x; a0.y += x.y; a0.z += x.z; a0.w += x.w;
-    b0.x += y.x; b0.y += y.y; b0.z += y.z; b0.w += y.w;
-  }
-  sp = make_float4(a0.x + a1.x, a0.y + a1.y, a0.z + a1.z, a0.w + a1.w);
-  sq = make_float4(b0.x + b1.x, b0.y + b1.y, b0.z + b1.z, b0.w + b1.w);
+  float x[7];   // the rest together in flight
+#pragma unroll
+  for (int j = 0; j < 7; ++j) x[j] = k + j < Kp ? r[j * (size_t)T] : 0.f;
+#pragma unroll
+  for (int j = 0; j < 7; ++j)
+    if (k + j < Kp) c[0] += x[j];
+  return ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
 }
 
-// X[t] = p_d[t] - avg_k(pbar + u) at the device's node n, t in [0, T), by
-// one warp (Section 3.2 step 2 input); the average was formed this iteration
-// by the node-average items into XS
+// avg_k(pbar + s u) = (sum_k PU + (s - 1) sum_k u) / (K+1) from the two sums
+// (Section 3.2 step 2)
+__device__ __forceinline__ float avg_of(const Params &p, float sm1, float sp, float sq) {
+  const float kpf = (float)p.Kp_glob;
+  return div_rn(fmaf(sm1, sq, sp), kpf, __frcp_rn(kpf));
+}
+
+// the average at node n, steps t0 .. t0 + VW - 1; u is read only while a
+// penalty rescale s != 1 is pending.  Horizons of whole 4-step blocks sum in
+// the order of ksum2, others (one step at a time) in that of ksum8.
+template <int VW>
+__device__ __forceinline__ FV<VW> node_avg(const Params &p, const Iter &q, int n, int t0) {
+  const size_t o = (size_t)n * p.Kp * p.T + t0;   // a node's K+1 rows are contiguous
+  const float sm1 = q.fsu - 1.f;
+  FV<VW> sp, sq;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) sq.v[e] = 0.f;
+  if (VW > 1 || p.T % 4 == 0) {
+    sp = ksum2<VW>(p.PU[q.old], o, p.T, p.Kp);
+    if (sm1 != 0.f) sq = ksum2<VW>(p.U[q.old], o, p.T, p.Kp);
+  } else {
+    sp.v[0] = ksum8(p.PU[q.old], o, p.T, p.Kp);
+    if (sm1 != 0.f) sq.v[0] = ksum8(p.U[q.old], o, p.T, p.Kp);
+  }
+#pragma unroll
+  for (int e = 0; e < VW; ++e) sp.v[e] = avg_of(p, sm1, sp.v[e], sq.v[e]);
+  return sp;
+}
+
 // Over-relaxation (Section 3.6) in the form kept on the device: the stored
 // schedules are the relaxed P = alpha p + (1 - alpha) P_prev, whose node
 // averages are the copies' complements (z = P - avg_n P, xi = avg_n Theta);
@@ -238,11 +337,36 @@ __device__ __forceinline__ float relaxed(float alpha, float pnew, float pold) {
   return rfma(alpha, pnew, rmul(rsub(1.f, alpha), pold));
 }
 
-__device__ __forceinline__ void device_x(const Params &p, int n, const float *pd, float *X, int lane) {
+// X[t] = p_d[t] - avg_k(pbar + u) at the device's node n, t in [0, T), by one
+// warp (Section 3.2 step 2 input).  AVG: the warp forms the average itself;
+// else xs_kernel left it in XS.
+template <bool AVG>
+__device__ __forceinline__ void device_x(const Params &p, const Iter &q, int n, const float *pd, float *X, int lane) {
   const int T = p.T;
   const float *xs = p.XS + (size_t)n * T;
-  for (int t = lane; t < T; t += 32) X[t] = rsub(pd[t], __ldcg(xs + t));
+  for (int t = lane; t < T; t += 32) X[t] = rsub(pd[t], AVG ? node_avg<1>(p, q, n, t).v[0] : __ldcg(xs + t));
   __syncwarp();
+}
+
+// the averages of a lane's C consecutive steps from t0 (0 beyond T)
+template <int C, bool AVG>
+__device__ __forceinline__ void lane_avg(const Params &p, const Iter &q, int n, int t0, float (&xs)[C]) {
+  const int T = p.T;
+  if constexpr (AVG && (C == 2 || C == 4)) {
+    if (T % 4 == 0) {   // the lane's rows as one 64- or 128-bit load
+      if (t0 < T) {
+        const FV<C> a = node_avg<C>(p, q, n, t0);
+#pragma unroll
+        for (int j = 0; j < C; ++j) xs[j] = a.v[j];
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    xs[j] = 0.f;
+    if (t0 + j < T) xs[j] = AVG ? node_avg<1>(p, q, n, t0 + j).v[0] : __ldcg(p.XS + (size_t)n * T + t0 + j);
+  }
 }
 
 // The warp's inner-ADMM state (lam, beta) lives in shared memory during the
@@ -273,8 +397,10 @@ __device__ __forceinline__ void stage_out(float *lam_g, float *bet_g, const floa
 // Rows: p_t <= pmax_t, -p_t <= -pmin_t, p_{t+1} - p_t <= R, p_t - p_{t+1} <= R.
 // x-update matrix (2a + rho + 2 omega) I + 2 omega D'D is tridiagonal.
 // ---------------------------------------------------------------------------
-__device__ void ramp_prox(const Params &p, int r, float rho, float *sm, float *state_sh, int lane) {
+template <bool AVG>
+__device__ void ramp_prox(const Params &p, const Iter &q, int r, float *sm, float *state_sh, int lane) {
   const int T = p.T;
+  const float rho = q.rho_dev;
   const int d = p.ramp_ids[r];
   const int n = p.dev_node[d];
   const float a = p.dev_a[d], b = p.dev_b[d], R = p.ramp_R[r];
@@ -302,7 +428,7 @@ __device__ void ramp_prox(const Params &p, int r, float rho, float *sm, float *s
     }
     __syncwarp();
   }
-  device_x(p, n, pd, X, lane);   // p_d - avg_k(pbar + u)
+  device_x<AVG>(p, q, n, pd, X, lane);   // p_d - avg_k(pbar + u)
   for (int itn = 0; itn < p.inner_iters; ++itn) {
     for (int t = lane; t < T - 1; t += 32)
       W[t] = rsub(rsub(bet[RG_RU * T + t], lam[RG_RU * T + t]), rsub(bet[RG_RD * T + t], lam[RG_RD * T + t]));
@@ -342,15 +468,18 @@ __device__ void ramp_prox(const Params &p, int r, float rho, float *sm, float *s
 // terminal i, p2 = clip((x2 - x1) / 2, -u, u) and p1 = -p2 (the minimiser
 // of the two squared distances over p1 + p2 = 0, clipped to the limit)
 // ---------------------------------------------------------------------------
-__device__ void hvdc_prox(const Params &p, int h, int lane) {
+template <bool AVG>
+__device__ void hvdc_prox(const Params &p, const Iter &q, int h, int lane) {
   const int T = p.T;
   const int d1 = p.hvdc0 + 2 * h, d2 = d1 + 1;
   const float u = p.hvdc_u[h];
-  const float *xs1 = p.XS + (size_t)p.dev_node[d1] * T, *xs2 = p.XS + (size_t)p.dev_node[d2] * T;
+  const int m1 = p.dev_node[d1], m2 = p.dev_node[d2];
+  const float *xs1 = p.XS + (size_t)m1 * T, *xs2 = p.XS + (size_t)m2 * T;
   float *pd1 = p.PD + (size_t)d1 * T, *pd2 = p.PD + (size_t)d2 * T;
   for (int t = lane; t < T; t += 32) {
     const float q1 = pd1[t], q2 = pd2[t];
-    const float x1 = q1 - __ldcg(xs1 + t), x2 = q2 - __ldcg(xs2 + t);
+    const float x1 = q1 - (AVG ? node_avg<1>(p, q, m1, t).v[0] : __ldcg(xs1 + t));
+    const float x2 = q2 - (AVG ? node_avg<1>(p, q, m2, t).v[0] : __ldcg(xs2 + t));
     const float f = fminf(fmaxf(0.5f * (x2 - x1), -u), u);
     const float r1 = relaxed(p.alpha, -f, q1), r2 = relaxed(p.alpha, f, q2);
     p.DPD[(size_t)d1 * T + t] = r1 - q1;
@@ -366,8 +495,10 @@ __device__ void hvdc_prox(const Params &p, int h, int lane) {
 // (c_t, delta_t) per step (a 2x2 Schur complement), leaving a tridiagonal
 // system of size T + 1 in the state of charge s.
 // ---------------------------------------------------------------------------
-__device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float *state_sh, int lane) {
+template <bool AVG>
+__device__ void stor_prox(const Params &p, const Iter &it, int sidx, float *sm, float *state_sh, int lane) {
   const int T = p.T, Tp = T + 1;
+  const float rho = it.rho_dev;
   const int d = p.stor_ids[sidx];
   const int n = p.dev_node[d];
   const float eta = p.stor_eff[sidx], Pm = p.stor_P[sidx], Em = rmul(p.stor_dur[sidx], Pm);
@@ -403,7 +534,7 @@ __device__ void stor_prox(const Params &p, int sidx, float rho, float *sm, float
     }
     __syncwarp();
   }
-  device_x(p, n, pd, X, lane);   // p_d - avg_k(pbar + u)
+  device_x<AVG>(p, it, n, pd, X, lane);   // p_d - avg_k(pbar + u)
 #define LAM(g, t) lam[(g) * Tp + (t)]
 #define BET(g, t) bet[(g) * Tp + (t)]
   for (int itn = 0; itn < p.inner_iters; ++itn) {
@@ -565,9 +696,10 @@ __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[
   }
 }
 
-template <int C>
-__device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
+template <int C, bool AVG>
+__device__ void ramp_prox_r(const Params &p, const Iter &q, int r, int lane) {
   const int T = p.T, t0 = lane * C;
+  const float rho = q.rho_dev;
   const int d = p.ramp_ids[r];
   const int n = p.dev_node[d];
   const float a = p.dev_a[d], b = p.dev_b[d], R = p.ramp_R[r];
@@ -590,7 +722,7 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
   }
   float lam[RG_N][C], bet[RG_N][C], hi[C], lo[C], X[C], pd[C], Z[C];
   TriFac<C> tf;
-  const float *xs = p.XS + (size_t)n * T;
+  lane_avg<C, AVG>(p, q, n, t0, X);
 #pragma unroll
   for (int j = 0; j < C; ++j) {
     const int t = t0 + j;
@@ -604,7 +736,7 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
     hi[j] = in ? p.dev_hi[(size_t)d * T + t] : 0.f;
     lo[j] = in ? p.dev_lo[(size_t)d * T + t] : 0.f;
     pd[j] = in ? p.PD[(size_t)d * T + t] : 0.f;
-    X[j] = in ? rsub(pd[j], __ldcg(xs + t)) : 0.f;   // p_d - avg_k(pbar + u)
+    X[j] = in ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
     tf.q[j] = in ? mf[t] : 1.f;
     Z[j] = 0.f;
   }
@@ -659,9 +791,10 @@ __device__ void ramp_prox_r(const Params &p, int r, float rho, int lane) {
   }
 }
 
-template <int C>
-__device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
+template <int C, bool AVG>
+__device__ void stor_prox_r(const Params &p, const Iter &it, int sidx, int lane) {
   const int T = p.T, Tp = T + 1, t0 = lane * C;
+  const float rho = it.rho_dev;
   const int d = p.stor_ids[sidx];
   const int n = p.dev_node[d];
   const float eta = p.stor_eff[sidx], Pm = p.stor_P[sidx], Em = rmul(p.stor_dur[sidx], Pm);
@@ -703,7 +836,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
     e3a = rmul(e3a, ls);
     e3b = rmul(e3b, ls);
   }
-  const float *xs = p.XS + (size_t)n * T;
+  lane_avg<C, AVG>(p, it, n, t0, X);
 #define LD_L(arr, g) arr[j] = in ? (rescale ? rmul(lam_g[(g) * Tp + e], ls) : lam_g[(g) * Tp + e]) : 0.f
 #define LD_B(arr, g) arr[j] = in ? bet_g[(g) * Tp + e] : 0.f
 #pragma unroll
@@ -716,7 +849,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
     LD_B(bSU, SG_SU); LD_B(bSL, SG_SL);
     const bool st = e < T;
     pd[j] = st ? p.PD[(size_t)d * T + e] : 0.f;
-    X[j] = st ? rsub(pd[j], __ldcg(xs + e)) : 0.f;   // p_d - avg_k(pbar + u)
+    X[j] = st ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
     tf.q[j] = in ? mf[e] : 1.f;
     S[j] = TAU[j] = DL[j] = 0.f;
   }
@@ -812,68 +945,6 @@ __device__ void stor_prox_r(const Params &p, int sidx, float rho, int lane) {
 #undef ST_B
 }
 
-// ---------------------------------------------------------------------------
-// VW consecutive time steps per thread (4 -> 128-bit accesses when T % 4 == 0)
-// ---------------------------------------------------------------------------
-template <int VW>
-struct FV {
-  float v[VW];
-};
-
-template <int VW>
-__device__ __forceinline__ FV<VW> ldv(const float *p) {
-  FV<VW> r;
-  if constexpr (VW == 4) {
-    const float4 t = *reinterpret_cast<const float4 *>(p);
-    r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
-  } else if constexpr (VW == 2) {
-    const float2 t = *reinterpret_cast<const float2 *>(p);
-    r.v[0] = t.x; r.v[1] = t.y;
-  } else {
-    r.v[0] = *p;
-  }
-  return r;
-}
-
-// streaming load (read once per iteration: evict first)
-template <int VW>
-__device__ __forceinline__ FV<VW> ldv_cs(const float *p) {
-  FV<VW> r;
-  if constexpr (VW == 4) {
-    const float4 t = __ldcs(reinterpret_cast<const float4 *>(p));
-    r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
-  } else if constexpr (VW == 2) {
-    const float2 t = __ldcs(reinterpret_cast<const float2 *>(p));
-    r.v[0] = t.x; r.v[1] = t.y;
-  } else {
-    r.v[0] = __ldcs(p);
-  }
-  return r;
-}
-
-template <int VW>
-__device__ __forceinline__ void stv(float *p, const FV<VW> &r) {
-  if constexpr (VW == 4) {
-    *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
-  } else if constexpr (VW == 2) {
-    *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
-  } else {
-    *p = r.v[0];
-  }
-}
-
-// streaming store (not read again in this iteration: evict first)
-template <int VW>
-__device__ __forceinline__ void stv_cs(float *p, const FV<VW> &r) {
-  if constexpr (VW == 4) {
-    __stcs(reinterpret_cast<float4 *>(p), make_float4(r.v[0], r.v[1], r.v[2], r.v[3]));
-  } else if constexpr (VW == 2) {
-    __stcs(reinterpret_cast<float2 *>(p), make_float2(r.v[0], r.v[1]));
-  } else {
-    __stcs(p, r.v[0]);
-  }
-}
-
 // one-pass sum of squared deviations from the mean (Welford)
 template <int VW>
 struct Welf {
@@ -921,15 +992,6 @@ struct Welf2 {
     }
   }
 };
-
-// x / c given r = 1/c rounded to nearest: one FMA correction step gives the
-// correctly rounded quotient for these well-scaled operands (a plain x * r
-// would carry the rounding bias of r into every node average, iteration
-// after iteration).
-__device__ __forceinline__ float div_rn(float x, float c, float r) {
-  const float q = x * r;
-  return fmaf(fmaf(-q, c, x), r, q);
-}
 
 // Index (a, b, c) of a row-major [.][B][C] item space, advanced by a fixed
 // stride with carries instead of 64-bit divisions per item.
@@ -1035,9 +1097,9 @@ __device__ __forceinline__ void line_item(const Params &p, int old, int nw, int 
 // inputs only they need (old p and theta_bar rows, the device Welford state)
 // and their accumulation; the relaxed variant always needs the mean change.
 // NB: line terminals gathered together.
-// ILD: where the pass forms no residuals, whether it sums the device powers
-// itself (0 never, 1 always, 2 as Params::dsum_lean says)
-template <int VW, bool RELAX, bool RES, int NB, int ILD>
+// ILD: the pass sums the node's device powers (and the Welford state of their
+// changes) itself; else dsum_kernel has left them in DSP, DSM and DSQ.
+template <int VW, bool RELAX, bool RES, int NB, bool ILD>
 __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int k, int n, int toff, float fsu,
                                           float *acc) {
   const int T = p.T;
@@ -1051,28 +1113,30 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   FV<VW> go;
   if (res) go = ldv_cs<VW>(p.THBAR[old] + on);
   // device terminals first: the sum and the Welford state after them, the
-  // same in every contingency -- from dsum_kernel, or (dsum_lean, where no
-  // residuals are formed) summed here over the node's devices in its order
+  // same in every contingency, in the order of dcsr_idx
   FV<VW> sp, st;
-  if (res || ILD == 0 || (ILD == 2 && !p.dsum_lean)) {
-    sp = ldv<VW>(p.DSP + os);
-  } else {
-#pragma unroll
-    for (int e = 0; e < VW; ++e) sp.v[e] = 0.f;
-    for (int j = r2.w; j < r2.w + r2.z; ++j) {
-      const FV<VW> pd = ldv<VW>(p.PD + (size_t)p.dcsr_idx[j] * T + toff);
-#pragma unroll
-      for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
-    }
-  }
   Welf<VW> wdp, wth;
   Welf2<VW> wrx;   // RELAX: (Theta_new, Theta_new - Theta_old) over the line terminals
   if constexpr (RELAX) wrx.reset();
-  if (res) {
-    const FV<VW> m = ldv<VW>(p.DSM + os), q = ldv<VW>(p.DSQ + os);
-    wdp.n = (float)r2.z;
+  if constexpr (!ILD) {
+    sp = ldv<VW>(p.DSP + os);
+    if constexpr (res) {
+      const FV<VW> m = ldv<VW>(p.DSM + os), q = ldv<VW>(p.DSQ + os);
+      wdp.n = (float)r2.z;
 #pragma unroll
-    for (int e = 0; e < VW; ++e) { wdp.mean[e] = m.v[e]; wdp.m2[e] = q.v[e]; }
+      for (int e = 0; e < VW; ++e) { wdp.mean[e] = m.v[e]; wdp.m2[e] = q.v[e]; }
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < VW; ++e) sp.v[e] = 0.f;
+    if constexpr (res) wdp.reset();
+    for (int j = r2.w; j < r2.w + r2.z; ++j) {
+      const size_t od = (size_t)p.dcsr_idx[j] * T + toff;
+      const FV<VW> pd = ldv<VW>(p.PD + od);
+#pragma unroll
+      for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
+      if constexpr (res) wdp.add(ldv<VW>(p.DPD + od).v);
+    }
   }
   wth.reset();
 #pragma unroll
@@ -1186,6 +1250,24 @@ __device__ __forceinline__ Iter load_iter(const Params &p) {
   return x.r;
 }
 
+// closed-form prox of device d at VW time steps, given the average there
+// (Section 4.2, weight (K+1) rho_p)
+template <int VW>
+__device__ __forceinline__ void closed_prox(const Params &p, const Iter &q, int d, int t0, const FV<VW> &xs) {
+  const size_t od = (size_t)d * p.T + t0;
+  const float den = 2.f * p.dev_a[d] + q.rho_dev, rden = __frcp_rn(den), bd = p.dev_b[d];
+  const FV<VW> pd = ldv<VW>(p.PD + od), lo = ldv<VW>(p.dev_lo + od), hi = ldv<VW>(p.dev_hi + od);
+  FV<VW> pn, dp;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) {
+    const float x = pd.v[e] - xs.v[e];                 // p_d - avg_k(pbar + u)
+    pn.v[e] = relaxed(p.alpha, fminf(fmaxf(div_rn(q.rho_dev * x - bd, den, rden), lo.v[e]), hi.v[e]), pd.v[e]);
+    dp.v[e] = pn.v[e] - pd.v[e];
+  }
+  stv<VW>(p.DPD + od, dp);
+  stv<VW>(p.PD + od, pn);
+}
+
 // ---------------------------------------------------------------------------
 // xs: avg_k(pbar + u) at each node with devices, one (node, VW time steps)
 // item per thread; the node's closed-form devices are updated on the spot
@@ -1195,86 +1277,119 @@ template <int VW>
 __device__ __forceinline__ void xs_body(const Params &p, unsigned bid, unsigned nblk) {
   const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
-  const int T = p.T, TV = T / VW, Kp = p.Kp;
-  const float kpf = (float)p.Kp_glob, rkp = __frcp_rn(kpf);
-  const size_t KT = (size_t)Kp * T;    // a node's K+1 rows are contiguous
-  // avg_k(pbar + s u) = (sum_k PU + (s - 1) sum_k u) / (K+1); u is read only
-  // while a penalty rescale s != 1 is pending
-  const float *Uo = p.U[q.old], *Wo = p.PU[q.old];
-  const bool rescale = q.fsu != 1.f;
-  const float sm1 = q.fsu - 1.f;
+  const int T = p.T, TV = p.T / VW;
   const unsigned n_xv = (unsigned)p.n_dnode * (unsigned)TV;
   for (unsigned item = bid * BLOCK + threadIdx.x; item < n_xv; item += nblk * BLOCK) {
-    const int ci = (int)(item / (unsigned)TV), t0 = (int)(item % (unsigned)TV) * VW;
-    const size_t on = (size_t)p.dnode_ids[ci] * T + t0, ok = (size_t)p.dnode_ids[ci] * KT + t0;
+    const int ci = (int)(item / (unsigned)TV), t0 = (int)(item % (unsigned)TV) * VW, n = p.dnode_ids[ci];
+    const size_t on = (size_t)n * T + t0;
     FV<VW> xs;
     if (p.slice) {
       // a contingency slice: the sums over every slice's k, exchanged
+      const float kpf = (float)p.Kp_glob, rkp = __frcp_rn(kpf), sm1 = q.fsu - 1.f;
       const double *esp = p.xsum + (size_t)ci * T + t0, *esq = p.xsum + (size_t)(p.n_dnode + ci) * T + t0;
 #pragma unroll
       for (int e = 0; e < VW; ++e) xs.v[e] = div_rn(fmaf(sm1, (float)esq[e], (float)esp[e]), kpf, rkp);
-    } else if constexpr (VW == 4) {
-      float4 sp, sq;
-      ksum4(Wo, rescale ? Uo : nullptr, ok, T, Kp, sp, sq);   // sum_k PU, sum_k u
-      xs.v[0] = div_rn(fmaf(sm1, sq.x, sp.x), kpf, rkp);
-      xs.v[1] = div_rn(fmaf(sm1, sq.y, sp.y), kpf, rkp);
-      xs.v[2] = div_rn(fmaf(sm1, sq.z, sp.z), kpf, rkp);
-      xs.v[3] = div_rn(fmaf(sm1, sq.w, sp.w), kpf, rkp);
     } else {
-      float sp, sq;
-      ksum(Wo, rescale ? Uo : nullptr, ok, T, Kp, sp, sq);
-      xs.v[0] = div_rn(fmaf(sm1, sq, sp), kpf, rkp);
+      xs = node_avg<VW>(p, q, n, t0);
     }
     if (p.dnode_keep[ci]) stv<VW>(p.XS + on, xs);
-    for (int j = p.dnode_ptr[ci]; j < p.dnode_ptr[ci + 1]; ++j) {
-      const int d = p.dnode_dev[j];
-      const size_t od = (size_t)d * T + t0;
-      const float den = 2.f * p.dev_a[d] + q.rho_dev, rden = __frcp_rn(den), bd = p.dev_b[d];
-      const FV<VW> pd = ldv<VW>(p.PD + od), lo = ldv<VW>(p.dev_lo + od), hi = ldv<VW>(p.dev_hi + od);
-      FV<VW> pn, dp;
-#pragma unroll
-      for (int e = 0; e < VW; ++e) {
-        const float x = pd.v[e] - xs.v[e];                 // p_d - avg_k(pbar + u)
-        pn.v[e] = relaxed(p.alpha, fminf(fmaxf(div_rn(q.rho_dev * x - bd, den, rden), lo.v[e]), hi.v[e]),
-                          pd.v[e]);
-        dp.v[e] = pn.v[e] - pd.v[e];
-      }
-      stv<VW>(p.DPD + od, dp);
-      stv<VW>(p.PD + od, pn);
-    }
+    for (int j = p.dnode_ptr[ci]; j < p.dnode_ptr[ci + 1]; ++j) closed_prox<VW>(p, q, p.dnode_dev[j], t0, xs);
   }
 }
 
-// the register path at the device's own chunk (cs, cr <= C)
-template <int C>
-__device__ __forceinline__ void stor_r(const Params &p, int sidx, float rho, int lane, int cs) {
-  if constexpr (C > 1) {
+// ---------------------------------------------------------------------------
+// closed: the closed-form devices of the nodes that have some, a group of
+// lanes per (node, VW time steps): each lane sums one class of contingencies
+// (the order of ksum2 at VW = 4, of ksum8 at VW = 1), then they share the
+// node's devices.  With one thread per item the row loads, a few in flight at
+// a time, were most of the 5 us that this phase took in front of the inner
+// ADMM at 2k buses.
+// ---------------------------------------------------------------------------
+// the group's sums over k (every lane returns the total)
+template <int VW, int G>
+__device__ __forceinline__ FV<VW> group_ksum(const float *r, int T, int Kp, int c, unsigned gmask) {
+  FV<VW> s;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) s.v[e] = 0.f;
+  const int whole = G == 8 ? (Kp & ~7) : Kp;
+#pragma unroll 4
+  for (int k = c; k < whole; k += G) {
+    const FV<VW> x = ldv<VW>(r + (size_t)k * T);
+#pragma unroll
+    for (int e = 0; e < VW; ++e) s.v[e] += x.v[e];
+  }
+  if (G == 8 && c == 0) {
+    for (int k = whole; k < Kp; ++k) {
+      const FV<VW> x = ldv<VW>(r + (size_t)k * T);
+#pragma unroll
+      for (int e = 0; e < VW; ++e) s.v[e] += x.v[e];
+    }
+  }
+#pragma unroll
+  for (int m = 1; m < G; m <<= 1)
+#pragma unroll
+    for (int e = 0; e < VW; ++e) s.v[e] += __shfl_xor_sync(gmask, s.v[e], m);
+  return s;
+}
+
+template <int VW>
+__device__ __forceinline__ void closed_body(const Params &p, unsigned bid, unsigned nblk) {
+  constexpr int G = VW == 4 ? CLOSED_LANES4 : CLOSED_LANES1;
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
+  const int T = p.T, TV = T / VW, Kp = p.Kp, c = threadIdx.x & (G - 1);
+  const unsigned gmask = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
+  const float sm1 = q.fsu - 1.f;
+  const unsigned n = (unsigned)p.n_cnode * (unsigned)TV, step = (nblk * blockDim.x) / G;
+  for (unsigned item = (bid * blockDim.x + threadIdx.x) / G; item < n; item += step) {
+    const int t0 = (int)(item % (unsigned)TV) * VW;
+    const int4 r = p.crec[item / (unsigned)TV];   // node, its first and one past its last entry of dnode_dev
+    const int d0 = r.y + c < r.z ? p.dnode_dev[r.y + c] : -1;
+    const size_t o = (size_t)r.x * Kp * T + t0;
+    FV<VW> xs = group_ksum<VW, G>(p.PU[q.old] + o, T, Kp, c, gmask), sq;
+#pragma unroll
+    for (int e = 0; e < VW; ++e) sq.v[e] = 0.f;
+    if (sm1 != 0.f) sq = group_ksum<VW, G>(p.U[q.old] + o, T, Kp, c, gmask);
+#pragma unroll
+    for (int e = 0; e < VW; ++e) xs.v[e] = avg_of(p, sm1, xs.v[e], sq.v[e]);
+    if (d0 >= 0) closed_prox<VW>(p, q, d0, t0, xs);
+    for (int j = r.y + c + G; j < r.z; j += G) closed_prox<VW>(p, q, p.dnode_dev[j], t0, xs);
+  }
+}
+
+// the register path at the device's own chunk (cs, cr <= C; ONLY: cs = C and
+// cr is C or C - 1, as for one instance)
+template <int C, bool AVG, bool ONLY>
+__device__ __forceinline__ void stor_r(const Params &p, const Iter &q, int sidx, int lane, int cs) {
+  if constexpr (C > 1 && !ONLY) {
     if (cs < C) {
-      stor_r<C - 1>(p, sidx, rho, lane, cs);
+      stor_r<C - 1, AVG, false>(p, q, sidx, lane, cs);
       return;
     }
   }
-  stor_prox_r<C>(p, sidx, rho, lane);
+  stor_prox_r<C, AVG>(p, q, sidx, lane);
 }
 
-template <int C>
-__device__ __forceinline__ void ramp_r(const Params &p, int r, float rho, int lane, int cr) {
+template <int C, bool AVG, bool ONLY>
+__device__ __forceinline__ void ramp_r(const Params &p, const Iter &q, int r, int lane, int cr) {
   if constexpr (C > 1) {
     if (cr < C) {
-      ramp_r<C - 1>(p, r, rho, lane, cr);
+      if constexpr (ONLY) ramp_prox_r<C - 1, AVG>(p, q, r, lane);
+      else ramp_r<C - 1, AVG, false>(p, q, r, lane, cr);
       return;
     }
   }
-  ramp_prox_r<C>(p, r, rho, lane);
+  ramp_prox_r<C, AVG>(p, q, r, lane);
 }
 
 // ---------------------------------------------------------------------------
-// inner: one warp per battery, then per ramp-limited generator (Appendix D).
-// C > 0: the register path, for horizons of at most REG_T steps (chunks of
-// at most C); C = 0: the shared-memory path.  MIXED (batches): the
-// instance's horizon chooses, beyond REG_T the shared-memory path.
+// inner: one warp per battery, then per ramp-limited generator (Appendix D),
+// then per HVDC link.  C > 0: the register path, for horizons of at most
+// REG_T steps (chunks of at most C); C = 0: the shared-memory path.  MIXED
+// (batches): the instance's horizon chooses, beyond REG_T the shared-memory
+// path.  AVG: each warp forms its node's average over contingencies.
 // ---------------------------------------------------------------------------
-template <int C, bool MIXED>
+template <int C, bool MIXED, bool AVG>
 __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem) {
   const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
@@ -1294,21 +1409,21 @@ __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsign
     if (w < p.n_stor) {
       if constexpr (HAS_REG) {
         if (reg) {
-          stor_r<C>(p, w, q.rho_dev, lane, cs);
+          stor_r<C, AVG, !MIXED>(p, q, w, lane, cs);
           continue;
         }
       }
-      if constexpr (HAS_SMEM) stor_prox(p, w, q.rho_dev, wsm, state_sh, lane);
+      if constexpr (HAS_SMEM) stor_prox<AVG>(p, q, w, wsm, state_sh, lane);
     } else if (w < p.n_stor + p.n_ramp) {
       if constexpr (HAS_REG) {
         if (reg) {
-          ramp_r<C>(p, w - p.n_stor, q.rho_dev, lane, cr);
+          ramp_r<C, AVG, !MIXED>(p, q, w - p.n_stor, lane, cr);
           continue;
         }
       }
-      if constexpr (HAS_SMEM) ramp_prox(p, w - p.n_stor, q.rho_dev, wsm, state_sh, lane);
+      if constexpr (HAS_SMEM) ramp_prox<AVG>(p, q, w - p.n_stor, wsm, state_sh, lane);
     } else {
-      hvdc_prox(p, w - p.n_stor - p.n_ramp, lane);
+      hvdc_prox<AVG>(p, q, w - p.n_stor - p.n_ramp, lane);
     }
   }
 }
@@ -1316,16 +1431,12 @@ __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsign
 // ---------------------------------------------------------------------------
 // dsum: per (node, VW time steps), the sum of the node's device powers and
 // the Welford state of their changes, in device order (the node sums of
-// every contingency start from it), on the iterations that form residuals
-// (and every iteration of the over-relaxed form)
+// every contingency start from it)
 // ---------------------------------------------------------------------------
 template <int VW>
 __device__ __forceinline__ void dsum_body(const Params &p, unsigned bid, unsigned nblk) {
   const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
-  // with dsum_lean the node passes that form no residuals sum the device
-  // powers themselves
-  if (p.dsum_lean && !(q.flags & ITF_RES) && p.alpha == 1.f) return;
   const int T = p.T, TV = T / VW;
   const unsigned n_items = (unsigned)p.N * (unsigned)TV;
   for (unsigned item = bid * BLOCK + threadIdx.x; item < n_items; item += nblk * BLOCK) {
@@ -1521,7 +1632,7 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part, bool re
 // its 36 us on their launches.  At 64 registers (four CTAs per SM, what the
 // residual-free pass wants) the general pass gathers one terminal at a time.
 // ---------------------------------------------------------------------------
-template <int VW, bool RELAX, int ILD>
+template <int VW, bool RELAX, bool ILD>
 __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk) {
   __shared__ double red[WARPS][NSLOT];
   __shared__ int s_last;
@@ -1588,7 +1699,19 @@ __global__ void __launch_bounds__(BLOCK) xs_kernel(Params p) { xs_body<VW>(p, bl
 template <int C>
 __global__ void __launch_bounds__(BLOCK) inner_kernel(Params p) {
   extern __shared__ float smem[];
-  inner_body<C, false>(p, blockIdx.x, gridDim.x, smem);
+  inner_body<C, false, false>(p, blockIdx.x, gridDim.x, smem);
+}
+
+// Every device of an iteration in one launch (step 2): the first inner_blocks
+// CTAs take the inner-ADMM devices and links, the others the closed-form
+// ones.  Each forms its node's average itself, so nothing runs in front of
+// the inner ADMM, the longest chain of the phase; nodes with several
+// inner-ADMM devices form it once per device.
+template <int C, int VW>
+__global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks) {
+  extern __shared__ float smem[];
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, false, true>(p, blockIdx.x, inner_blocks, smem);
+  else closed_body<VW>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
 }
 
 template <int VW>
@@ -1600,8 +1723,8 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p) {
 }
 
 // the over-relaxed variant carries more per-terminal state: it takes the
-// registers of one CTA per SM rather than spill; ILD: the plan's dsum_lean
-template <int VW, bool RELAX, int ILD>
+// registers of one CTA per SM rather than spill; ILD: device sums in the pass
+template <int VW, bool RELAX, bool ILD>
 __global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel(Params p) {
   node_body<VW, RELAX, ILD>(p, blockIdx.x, gridDim.x);
 }
@@ -1643,10 +1766,9 @@ __global__ void __launch_bounds__(BLOCK) slice_sums_kernel(Params p, int prime) 
   for (long long i = (long long)blockIdx.x * BLOCK + threadIdx.x; i < (long long)p.n_dnode * T;
        i += (long long)gridDim.x * BLOCK) {
     const int ci = (int)(i / T), t = (int)(i % T);
-    float sp, sq;
-    ksum(W, with_u ? U : nullptr, (size_t)p.dnode_ids[ci] * KT + t, T, Kp, sp, sq);
-    esp[i] = (double)sp;
-    esq[i] = (double)sq;
+    const size_t o = (size_t)p.dnode_ids[ci] * KT + t;
+    esp[i] = (double)ksum8(W, o, T, Kp);
+    esq[i] = with_u ? (double)ksum8(U, o, T, Kp) : 0.0;
   }
   if (blockIdx.x == 0) {
     double tot[NSLOT];
@@ -1668,40 +1790,26 @@ __device__ __forceinline__ const Params &batch_params(const Params *ps, const in
   static_assert(sizeof(Params) % 4 == 0, "Params is copied as 32-bit words");
   const int *src = reinterpret_cast<const int *>(ps + e.x);
   int *dst = reinterpret_cast<int *>(&sp);
-  for (int i = threadIdx.x; i < (int)(sizeof(Params) / 4); i += BLOCK) dst[i] = src[i];
+  for (int i = threadIdx.x; i < (int)(sizeof(Params) / 4); i += blockDim.x) dst[i] = src[i];
   __syncthreads();
   bid = (unsigned)e.y;
   nblk = (unsigned)e.z;
   return sp;
 }
 
-template <int VW>
-__global__ void __launch_bounds__(BLOCK) xs_kernel_b(const Params *ps, const int4 *sched) {
-  __shared__ Params sp;
-  unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  xs_body<VW>(p, bid, nblk);
-}
-
-// batches keep the GPU full of inner-ADMM warps: on the shared-memory path
-// alone 64 registers, 4 CTAs per SM; C: the largest register chunk of the
-// batch's instances (0: every horizon beyond REG_T), any longer horizon on
-// the shared-memory path
+// the devices of every instance: the first inner_blocks CTAs of the schedule
+// take inner-ADMM devices, the others closed-form ones.  C: the largest
+// register chunk of the batch's instances (0: every horizon beyond REG_T),
+// any longer horizon on the shared-memory path
 template <int C>
-__global__ void __launch_bounds__(BLOCK, C == 0 ? 4 : 1) inner_kernel_b(const Params *ps, const int4 *sched) {
+__global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks) {
   extern __shared__ float smem[];
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  inner_body<C, true>(p, bid, nblk, smem);
-}
-
-template <int VW>
-__global__ void __launch_bounds__(BLOCK) dsum_kernel_b(const Params *ps, const int4 *sched) {
-  __shared__ Params sp;
-  unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  dsum_body<VW>(p, bid, nblk);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0), true>(p, bid, nblk, smem);
+  else if (p.T % 4 == 0) closed_body<4>(p, bid, nblk);
+  else closed_body<1>(p, bid, nblk);
 }
 
 template <int VW>
@@ -1717,7 +1825,7 @@ __global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel_b(co
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  node_body<VW, RELAX, 2>(p, bid, nblk);
+  node_body<VW, RELAX, true>(p, bid, nblk);
 }
 
 // A line's terminal values from its stored (p, mid) at contingency k:
@@ -1967,7 +2075,7 @@ __global__ void set_rho_kernel(Params p, double rho) {
   *p.sc = s;
 }
 
-static size_t inner_smem(int T) { return (size_t)WARPS * warp_smem_floats(T) * sizeof(float); }
+static size_t inner_smem(int T, int warps) { return (size_t)warps * warp_smem_floats(T) * sizeof(float); }
 
 }  // namespace opfk
 
@@ -1983,67 +2091,64 @@ static int resident_grid(F fn, size_t smem) {
   return nb * sms;
 }
 
+// dynamic shared memory of the device kernels, set on each of them
+template <class F>
+static bool allow_smem(F fn, size_t smem) {
+  return smem <= 48 * 1024 ||
+         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+}
+
 int opfk_plan(const Params &p, IterPlan *plan) {
   const bool v4 = (p.T % 4 == 0), v2 = (p.T % 2 == 0);
   // the inner ADMM in registers up to REG_T steps, else in shared memory
   const int ic = inner_chunk(p.T);
-  const size_t ism = ic ? 0 : inner_smem(p.T);
-  if (ism > 48 * 1024 &&
-      cudaFuncSetAttribute(inner_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism) != cudaSuccess)
-    return -1;
   const bool vn = (p.T % NODE_VW == 0);
-  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false, 0>, 0) : resident_grid(node_kernel<1, false, 0>, 0);
+  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false, false>, 0) : resident_grid(node_kernel<1, false, false>, 0);
   const int gx = v4 ? resident_grid(xs_kernel<4>, 0) : resident_grid(xs_kernel<1>, 0);
   const int gd = v2 ? resident_grid(dsum_kernel<2>, 0) : resident_grid(dsum_kernel<1>, 0);
   if (gn < 1 || gx < 1 || gd < 1) return -1;
   const long long tvl = p.T / (v4 ? 4 : 1), tvn = p.T / (vn ? NODE_VW : 1);
   const long long nl = (long long)p.Kp * p.L * tvl, nn = (long long)p.Kp * p.N * tvn;
-  const long long nx = (long long)p.n_dnode * (p.T / (v4 ? 4 : 1));
+  const long long nx = (long long)p.n_dnode * tvl;
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
   plan->line_grid = (int)((nl + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT));
   plan->node_grid = (int)std::min<long long>(gn, (nn + BLOCK - 1) / BLOCK);
-  plan->xs_grid = (int)std::min<long long>(gx, (nx + BLOCK - 1) / BLOCK);
-  plan->inner_grid = (n_inner + WARPS - 1) / WARPS;
-  {
-    // The inner-ADMM kernel is latency-bound (one warp per device through its
-    // ten Appendix D iterations) and runs beside the bandwidth-bound line
-    // kernel, whose CTAs it displaces.  When the line pass is long enough to
-    // hide it, fewer CTAs walking the devices in several rounds leave the
-    // line kernel more of the GPU.  The estimates: the line pass moves about
-    // 32 bytes per (line, contingency, step) at 6.5 TB/s; a round of devices
-    // takes about 0.13 T microseconds from registers, 0.45 T in shared memory.
-    // Registers: the fewest CTAs whose rounds fit in half the line pass (10k
-    // buses, T = 96, K = 50, 3,000 devices, in ms per iteration: 375 CTAs
-    // 0.706, 76 CTAs 0.706, 38 0.698, 25 0.696, 19 0.704, 12 0.851).  Shared
-    // memory: one CTA on every other SM while its rounds fit in 70 % of it
-    // (0.741 -> 0.706 at the same size).
-    const double line_us = (double)p.Kp * p.L * p.T * 32.0 / 6.5e6;
-    plan->dsum_lean = 0;
-    if (ic) {
-      const int max_rounds = (int)std::floor(0.5 * line_us / (0.13 * p.T));
-      if (max_rounds >= 2) plan->inner_grid = (plan->inner_grid + max_rounds - 1) / max_rounds;
-      // a line pass too short to hide the device chain (xs, inner, dsum):
-      // shorten the chain by summing device powers in the node passes that
-      // form no residuals (2k buses, T = 24: 35.5 -> 34.0 us per iteration;
-      // at 10k, where the chain is hidden, the extra loads of the node pass
-      // cost more than dsum: 0.697 -> 0.701 ms)
-      else plan->dsum_lean = 1;
-    } else {
-      int dev = 0, sms = 0;
-      if (cudaGetDevice(&dev) == cudaSuccess &&
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms >= 2) {
-        const int half = sms / 2;
-        if (plan->inner_grid > half) {
-          const double rounds = std::ceil((double)plan->inner_grid / half);
-          if (rounds * 0.45 * p.T <= 0.7 * line_us) plan->inner_grid = half;
-        }
-      }
-    }
+  plan->inner_c = ic;
+  // One device kernel beside the line kernel, or three (averages, inner ADMM,
+  // device sums)?  The inner ADMM is latency-bound, one warp per device.  When
+  // the line pass is long enough to hide it, few CTAs walking the devices in
+  // several rounds leave the line kernel more of the GPU, and the averages and
+  // sums, formed once per node, are hidden as well.  Otherwise the devices are
+  // the critical path: one launch, every device at once, averages formed where
+  // they are used, device sums in the node pass.  The estimates: the line pass
+  // moves about 32 bytes per (line, contingency, step) at 6.5 TB/s; a round of
+  // devices takes about 5 + 0.08 T microseconds from registers, 0.45 T in
+  // shared memory.  At 10k buses, T = 96, K = 50 (3,000 devices), ms per
+  // iteration by CTAs of the inner kernel: 375 0.706, 76 0.706, 38 0.698, 25
+  // 0.696, 19 0.704, 12 0.851: the fewest whose rounds fit in half the line
+  // pass; device sums in the node pass 0.701 against 0.697.  At 2k buses,
+  // T = 24, K = 20: three device kernels 31.7 us per iteration, one 25.2.
+  const double line_us = (double)p.Kp * p.L * p.T * 32.0 / 6.5e6;
+  const int one_round = (n_inner + WARPS - 1) / WARPS;
+  const double round_us = ic ? 5.0 + 0.08 * p.T : 0.45 * p.T;
+  const int max_rounds = (int)std::floor((ic ? 0.5 : 0.7) * line_us / round_us);
+  plan->fused = !p.slice && max_rounds < 2;
+  plan->xs_grid = plan->dsum_grid = plan->inner_grid = plan->dev_inner = plan->dev_closed = 0;
+  if (plan->fused) {
+    const size_t ism = ic ? 0 : inner_smem(p.T, DEV_WARPS);
+    if (!allow_smem(dev_kernel<0, 4>, ism) || !allow_smem(dev_kernel<0, 1>, ism)) return -1;
+    plan->inner_smem = ism;
+    plan->dev_inner = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
+    plan->dev_closed = (int)std::min<long long>(4096, ((long long)p.n_cnode * tvl * (v4 ? CLOSED_LANES4 : CLOSED_LANES1) + DEVB - 1) / DEVB);
+    return 0;
   }
+  const size_t ism = ic ? 0 : inner_smem(p.T, WARPS);
+  if (!allow_smem(inner_kernel<0>, ism)) return -1;
+  plan->inner_smem = ism;
+  plan->inner_grid = max_rounds >= 2 ? (one_round + max_rounds - 1) / max_rounds : one_round;
+  plan->xs_grid = (int)std::min<long long>(gx, (nx + BLOCK - 1) / BLOCK);
   const long long nd = (long long)p.N * (p.T / (v2 ? 2 : 1));
   plan->dsum_grid = (int)std::min<long long>(gd, (nd + BLOCK - 1) / BLOCK);
-  plan->inner_smem = ism;
-  plan->inner_c = ic;
   return 0;
 }
 
@@ -2057,38 +2162,55 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
   // sums (main stream) follow them and the device kernels.
   if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
-  if (plan.xs_grid > 0) {
-    if (v4) xs_kernel<4><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
-    else xs_kernel<1><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
-  }
-  if (plan.inner_grid > 0) {
-    switch (plan.inner_c) {
-      case 1: inner_kernel<1><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-      case 2: inner_kernel<2><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-      case 3: inner_kernel<3><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-      case 4: inner_kernel<4><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-      default: inner_kernel<0><<<plan.inner_grid, BLOCK, plan.inner_smem, sm>>>(p); break;
+  if (plan.fused) {
+    const int ni = plan.dev_inner, g = ni + plan.dev_closed;
+    if (g > 0) {
+#define DEV_LAUNCH(C)                                                             \
+  if (v4) dev_kernel<C, 4><<<g, DEVB, plan.inner_smem, sm>>>(p, ni);              \
+  else dev_kernel<C, 1><<<g, DEVB, plan.inner_smem, sm>>>(p, ni);                 \
+  break
+      switch (plan.inner_c) {
+        case 1: DEV_LAUNCH(1);
+        case 2: DEV_LAUNCH(2);
+        case 3: DEV_LAUNCH(3);
+        case 4: DEV_LAUNCH(4);
+        default: DEV_LAUNCH(0);
+      }
+#undef DEV_LAUNCH
     }
+  } else {
+    if (plan.xs_grid > 0) {
+      if (v4) xs_kernel<4><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
+      else xs_kernel<1><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
+    }
+    if (plan.inner_grid > 0) {
+      switch (plan.inner_c) {
+        case 1: inner_kernel<1><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
+        case 2: inner_kernel<2><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
+        case 3: inner_kernel<3><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
+        case 4: inner_kernel<4><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
+        default: inner_kernel<0><<<plan.inner_grid, BLOCK, plan.inner_smem, sm>>>(p); break;
+      }
+    }
+    if (v2) dsum_kernel<2><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
+    else dsum_kernel<1><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
   }
-  if (v2) dsum_kernel<2><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
-  else dsum_kernel<1><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
   if (plan.line_grid > 0) {
     if (v4) line_kernel<4><<<plan.line_grid, BLOCK, 0, sa>>>(p);
     else line_kernel<1><<<plan.line_grid, BLOCK, 0, sa>>>(p);
   }
   if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
-  const bool vn = p.T % NODE_VW == 0;
-  if (p.alpha != 1.f) {
-    if (vn) node_kernel<NODE_VW, true, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-    else node_kernel<1, true, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-  } else if (vn) {
-    if (p.dsum_lean) node_kernel<NODE_VW, false, 1><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-    else node_kernel<NODE_VW, false, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-  } else {
-    if (p.dsum_lean) node_kernel<1, false, 1><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-    else node_kernel<1, false, 0><<<plan.node_grid, BLOCK, 0, sm>>>(p);
-  }
+  const bool vn = p.T % NODE_VW == 0, rx = p.alpha != 1.f;
+  const int g = plan.node_grid;
+#define NODE_LAUNCH(RX, ILD)                                           \
+  if (vn) node_kernel<NODE_VW, RX, ILD><<<g, BLOCK, 0, sm>>>(p);       \
+  else node_kernel<1, RX, ILD><<<g, BLOCK, 0, sm>>>(p)
+  if (rx && plan.fused) { NODE_LAUNCH(true, true); }
+  else if (rx) { NODE_LAUNCH(true, false); }
+  else if (plan.fused) { NODE_LAUNCH(false, true); }
+  else { NODE_LAUNCH(false, false); }
+#undef NODE_LAUNCH
   if (slice) slice_sums_kernel<<<aux_grid((long long)p.n_dnode * p.T), BLOCK, 0, sm>>>(p, 0);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -2138,24 +2260,21 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     for (int j = 0; j < n; ++j) {
       const int i = lay.order ? lay.order[j] : j;
       const Params &p = hp[i];
-      const bool v4 = (p.T % 4 == 0), v2 = (p.T % 2 == 0), vn = (p.T % NODE_VW == 0);
-      const long long tv4 = p.T / (v4 ? 4 : 1), tv2 = p.T / (v2 ? 2 : 1);
+      const bool v4 = (p.T % 4 == 0), vn = (p.T % NODE_VW == 0);
+      const long long tv4 = p.T / (v4 ? 4 : 1);
       const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
       long long blocks = 0;
       switch (kind) {
-        case BK_XS4: case BK_XS1:
-          if ((kind == BK_XS4) == v4) blocks = ((long long)p.n_dnode * tv4 + BLOCK - 1) / BLOCK;
-          break;
         case BK_INNER:
-          blocks = (n_inner + WARPS - 1) / WARPS;
+          blocks = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
           if (blocks) {
             const int ic = inner_chunk(p.T);
             if (ic) ic_max = std::max(ic_max, ic);
-            else ism = std::max(ism, inner_smem(p.T));   // the shared-memory path
+            else ism = std::max(ism, inner_smem(p.T, DEV_WARPS));   // the shared-memory path
           }
           break;
-        case BK_DSUM2: case BK_DSUM1:
-          if ((kind == BK_DSUM2) == v2) blocks = ((long long)p.N * tv2 + BLOCK - 1) / BLOCK;
+        case BK_CLOSED:
+          blocks = ((long long)p.n_cnode * tv4 * (v4 ? CLOSED_LANES4 : CLOSED_LANES1) + DEVB - 1) / DEVB;
           break;
         case BK_LINE4: case BK_LINE1:
           if ((kind == BK_LINE4) == v4 && p.L > 0)
@@ -2168,8 +2287,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
       // the grid-stride phases take any block count: `div` puts more work in
       // each CTA (for the node phase the caller sets the instance's partial-sum
       // count to the same number, batch_node_blocks)
-      if (blocks > 0 && (kind == BK_XS4 || kind == BK_XS1 || kind == BK_INNER || kind == BK_DSUM2 ||
-                         kind == BK_DSUM1 || kind == BK_NODE4 || kind == BK_NODE1))
+      if (blocks > 0 && (kind == BK_INNER || kind == BK_CLOSED || kind == BK_NODE4 || kind == BK_NODE1))
         blocks = (blocks + div - 1) / div;
       nb[j] = blocks;
       most = std::max(most, blocks);
@@ -2192,16 +2310,9 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
   bp->relax = (n > 0 && hp[0].alpha != 1.f) ? 1 : 0;
   for (int i = 0; i < n; ++i)
     if ((hp[i].alpha != 1.f) != (bp->relax != 0)) return -2;   // one node kernel for every instance
-  if (ism > 48 * 1024) {
-    const int a = (int)ism;
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (cudaFuncSetAttribute(inner_kernel_b<0>, at, a) != cudaSuccess ||
-        cudaFuncSetAttribute(inner_kernel_b<1>, at, a) != cudaSuccess ||
-        cudaFuncSetAttribute(inner_kernel_b<2>, at, a) != cudaSuccess ||
-        cudaFuncSetAttribute(inner_kernel_b<3>, at, a) != cudaSuccess ||
-        cudaFuncSetAttribute(inner_kernel_b<4>, at, a) != cudaSuccess)
-      return -1;
-  }
+  if (!allow_smem(dev_kernel_b<0>, ism) || !allow_smem(dev_kernel_b<1>, ism) || !allow_smem(dev_kernel_b<2>, ism) ||
+      !allow_smem(dev_kernel_b<3>, ism) || !allow_smem(dev_kernel_b<4>, ism))
+    return -1;
   *sched_len = len;
   return 0;
 }
@@ -2221,21 +2332,18 @@ int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPl
   if (bp.count[BK_LINE4]) line_kernel_b<4><<<bp.count[BK_LINE4], BLOCK, 0, sa>>>(d_params, at(BK_LINE4));
   if (bp.count[BK_LINE1]) line_kernel_b<1><<<bp.count[BK_LINE1], BLOCK, 0, sa>>>(d_params, at(BK_LINE1));
   if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
-  if (bp.count[BK_XS4]) xs_kernel_b<4><<<bp.count[BK_XS4], BLOCK, 0, sm>>>(d_params, at(BK_XS4));
-  if (bp.count[BK_XS1]) xs_kernel_b<1><<<bp.count[BK_XS1], BLOCK, 0, sm>>>(d_params, at(BK_XS1));
-  if (bp.count[BK_INNER]) {
+  static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
+  const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED];
+  if (nd) {
     const int4 *si = at(BK_INNER);
-    const int nb = bp.count[BK_INNER];
     switch (bp.inner_c) {
-      case 1: inner_kernel_b<1><<<nb, BLOCK, bp.inner_smem, sm>>>(d_params, si); break;
-      case 2: inner_kernel_b<2><<<nb, BLOCK, bp.inner_smem, sm>>>(d_params, si); break;
-      case 3: inner_kernel_b<3><<<nb, BLOCK, bp.inner_smem, sm>>>(d_params, si); break;
-      case 4: inner_kernel_b<4><<<nb, BLOCK, bp.inner_smem, sm>>>(d_params, si); break;
-      default: inner_kernel_b<0><<<nb, BLOCK, bp.inner_smem, sm>>>(d_params, si); break;
+      case 1: dev_kernel_b<1><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
+      case 2: dev_kernel_b<2><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
+      case 3: dev_kernel_b<3><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
+      case 4: dev_kernel_b<4><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
+      default: dev_kernel_b<0><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
     }
   }
-  if (bp.count[BK_DSUM2]) dsum_kernel_b<2><<<bp.count[BK_DSUM2], BLOCK, 0, sm>>>(d_params, at(BK_DSUM2));
-  if (bp.count[BK_DSUM1]) dsum_kernel_b<1><<<bp.count[BK_DSUM1], BLOCK, 0, sm>>>(d_params, at(BK_DSUM1));
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
   if (!bp.relax) {
     if (bp.count[BK_NODE4]) node_kernel_b<4, false><<<bp.count[BK_NODE4], BLOCK, 0, sm>>>(d_params, at(BK_NODE4));
