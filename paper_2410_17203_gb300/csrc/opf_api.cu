@@ -727,6 +727,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   p.n_hvdc = c->H;
   p.hvdc0 = G + D + c->B;
   p.node_grid = c->plan.node_grid;
+  p.line_ipt = c->plan.line_ipt;
   p.n_cnode = (int)crec.size();
   p.eps = opt.eps;
   p.mu = opt.mu;

@@ -46,7 +46,7 @@ struct alignas(16) Iter {
   float rho_dev;              // rho' = (K+1) rho_p
   int old;                    // buffer of the previous iterate (it & 1)
   int flags;                  // ITF_*
-  int pad;
+  int left;                   // iterations before the next one that forms residuals (0: this one)
 };
 enum {
   ITF_SKIP = 1,      // stopped in this call (passed stopping test, stall) or a sticky error: return at once
@@ -91,6 +91,7 @@ struct Params {
   int n_dnode, n_ramp, n_stor;
   int n_hvdc, hvdc0;                     // HVDC links; device id of the first link's terminal 1
   // lines (internal numbering)
+  int line_ipt;                  // IterPlan::line_ipt
   const int *line_n1, *line_n2;  // internal node of terminal 1 (from) and terminal 2 (to)
   const float *line_b, *line_u;
   const int *out_line;  // [Kp], internal index of the outaged line, -1 = none
@@ -200,15 +201,27 @@ __host__ __device__ __forceinline__ void set_iter(const Params &p, DevScalars &s
   r.fsv = (float)sc.sv;
   r.rho_dev = (float)(p.Kp_glob * sc.rho_p);
   r.old = (int)(sc.it & 1);
-  r.flags = ((sc.status != 0 || sc.stop != 0) ? ITF_SKIP : 0) | (res_at(p, sc, sc.it + 1) ? ITF_RES : 0) |
+  // the first of the next iterations it + 1 .. it_last that forms residuals:
+  // the call's last one, a stopping test, or an adaptation
+  long long left = sc.it_last - (sc.it + 1);
+  if (p.eps > 0 && p.check_every > 0) {
+    const long long c = p.check_every - 1 - sc.it % p.check_every;
+    if (c < left) left = c;
+  }
+  if (p.adapt_every > 0) {
+    const long long a = p.adapt_every - 1 - sc.it % p.adapt_every;
+    if (a < left && adapting(p, sc, sc.it + 1 + a)) left = a;
+  }
+  r.left = (int)(left > 0 ? left : 0);   // a call has at most 2^31 - 1 iterations
+  r.flags = ((sc.status != 0 || sc.stop != 0) ? ITF_SKIP : 0) | (r.left == 0 ? ITF_RES : 0) |
             (sc.v_fresh ? ITF_VFRESH : 0);
-  r.pad = 0;
   sc.cur = r;
 }
 
 // Launch configuration of one iteration's kernels.
 struct IterPlan {
   int line_grid, node_grid;            // 0: the kernel has no work
+  int line_ipt;                        // line items per thread
   int fused;                           // 1: one device kernel; 0: averages, inner ADMM and device sums apart
   int dev_inner, dev_closed;           // fused: CTAs of the device kernel for inner-ADMM and closed-form devices
   int xs_grid, inner_grid, dsum_grid;  // not fused

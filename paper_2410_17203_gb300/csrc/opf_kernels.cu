@@ -49,6 +49,7 @@ constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is comp
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
 constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items)
+constexpr long long LINE_SHORT = 1 << 20;   // ... one, up to this many items
 constexpr int DEVB = 128;        // threads per CTA of the device kernel (its inner-ADMM warps spread over more SMs)
 constexpr int DEV_WARPS = DEVB / 32;
 constexpr int CLOSED_LANES4 = 2, CLOSED_LANES1 = 8;   // lanes per closed-form item: the classes of ksum2 / ksum8
@@ -1126,7 +1127,8 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
 #pragma unroll
       for (int e = 0; e < VW; ++e) { wdp.mean[e] = m.v[e]; wdp.m2[e] = q.v[e]; }
     }
-  } else {
+  }
+  if constexpr (ILD) {
 #pragma unroll
     for (int e = 0; e < VW; ++e) sp.v[e] = 0.f;
     if constexpr (res) wdp.reset();
@@ -1236,6 +1238,8 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   stv_cs<VW>(p.PU[nw] + on, pu);
   stv_cs<VW>(p.THBAR[nw] + on, tbar);
 }
+
+__device__ __forceinline__ void prefetch_l1(const void *a) { asm volatile("prefetch.global.L1 [%0];" ::"l"(a)); }
 
 // the current iteration's scalars (the same two loads in every thread)
 __device__ __forceinline__ Iter load_iter(const Params &p) {
@@ -1468,20 +1472,26 @@ __device__ __forceinline__ void dsum_body(const Params &p, unsigned bid, unsigne
 // ---------------------------------------------------------------------------
 template <int VW>
 __device__ __forceinline__ void line_body(const Params &p, unsigned bid) {
-  const Iter q = load_iter(p);
-  if (q.flags & ITF_SKIP) return;
-  const int L = p.L, TV = p.T / VW;
+  const int L = p.L, TV = p.T / VW, ipt = p.line_ipt;
   const unsigned n = (unsigned)p.Kp * (unsigned)L * (unsigned)TV;
-  // each CTA takes LINE_IPT consecutive blocks of BLOCK items, so CTAs are
+  // each CTA takes line_ipt consecutive blocks of BLOCK items, so CTAs are
   // short-lived and the device kernels' CTAs find room beside them
-  const unsigned base = bid * (unsigned)(BLOCK * LINE_IPT) + threadIdx.x;
+  const unsigned base = bid * (unsigned)(BLOCK * ipt) + threadIdx.x;
   // items (line, contingency, step block): a line's K+1 rows are contiguous
   const int Kp = p.Kp;
   Idx3 ix, dx;
   ix.set(base, Kp, TV);
   dx.set(BLOCK, Kp, TV);
+  if (base < n) {   // static: requested beside the scalars
+    prefetch_l1(p.line_n1 + ix.a);
+    prefetch_l1(p.line_n2 + ix.a);
+    prefetch_l1(p.line_b + ix.a);
+    prefetch_l1(p.line_u + ix.a);
+  }
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
 #pragma unroll 1
-  for (int j = 0; j < LINE_IPT; ++j, ix.step(dx, Kp, TV)) {
+  for (int j = 0; j < ipt; ++j, ix.step(dx, Kp, TV)) {
     if (base + (unsigned)(j * BLOCK) < n)
       line_item<VW>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.frp, q.frt, q.fsu, q.fsv, q.flags & ITF_VFRESH);
   }
@@ -1522,21 +1532,32 @@ __device__ __forceinline__ bool reduce_partials(const Params &p, int n_part, dou
   return true;
 }
 
-__device__ __forceinline__ void decide_body(const Params &p, int n_part, bool res, double (*red)[NSLOT]) {
-  if (!res) {
-    // nothing reads this iteration's residuals (a non-finite value is caught
-    // at the next iteration that forms them): advance
-    if (threadIdx.x == 0) {
-      DevScalars sc = *p.sc;
-      sc.su = 1.0;
-      sc.sv = 1.0;
-      sc.it = sc.it + 1;
-      sc.v_fresh = 0;
-      set_iter(p, sc);
-      *p.sc = sc;
-    }
-    return;
-  }
+// An iteration whose residuals nobody reads (a non-finite value is caught at
+// the next one that forms them): one thread advances the counter with stores
+// alone.  Reading the scalars back and forming the next iteration's from them
+// (FP64 conversions, 64-bit remainders) at the end of every iteration took
+// about 3 us.
+__device__ __forceinline__ void advance(const Params &p) {
+  union {
+    Iter r;
+    int4 v[2];
+  } x;
+  const Iter q = load_iter(p);
+  x.r = q;
+  x.r.fsu = x.r.fsv = 1.f;
+  x.r.old = q.old ^ 1;
+  x.r.left = q.left - 1;
+  x.r.flags = x.r.left == 0 ? ITF_RES : 0;
+  int4 *d = reinterpret_cast<int4 *>(&p.sc->cur);
+  d[0] = x.v[0];
+  d[1] = x.v[1];
+  atomicAdd(reinterpret_cast<unsigned long long *>(&p.sc->it), 1ull);
+  p.sc->su = 1.0;
+  p.sc->sv = 1.0;
+  p.sc->v_fresh = 0;
+}
+
+__device__ __forceinline__ void decide_body(const Params &p, int n_part, double (*red)[NSLOT]) {
   double tot[NSLOT];
   if (p.slice) {
     // a contingency slice: the residual sums of every slice, exchanged
@@ -1636,20 +1657,21 @@ template <int VW, bool RELAX, bool ILD>
 __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk) {
   __shared__ double red[WARPS][NSLOT];
   __shared__ int s_last;
-  const Iter q = load_iter(p);
-  if (q.flags & ITF_SKIP) return;
-  const bool res = q.flags & ITF_RES;
   const int N = p.N, TV = p.T / VW, Kp = p.Kp;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const unsigned n = (unsigned)Kp * (unsigned)N * (unsigned)TV;
   const unsigned stride = nblk * BLOCK;
   unsigned item = bid * BLOCK + threadIdx.x;
-  float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
   // items (node, contingency, step block): a node's K+1 rows are contiguous,
   // and so are the K+1 rows of each line it gathers
   Idx3 ix, dx;
   ix.set(item, Kp, TV);
   dx.set(stride, Kp, TV);
+  if (item < n) prefetch_l1(p.nrec + 3 * ix.a);   // static: requested beside the scalars
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
+  const bool res = q.flags & ITF_RES;
+  float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if (res || RELAX) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
       node_item<VW, RELAX, true, RELAX ? 4 : NODE_RES_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
@@ -1677,14 +1699,19 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   // (res) its partial sums are written; the last CTA alone goes on
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(p.done, 1u) == nblk - 1;
-    if (s_last) *p.done = 0;
+    if (res) __threadfence();
+    const bool last = atomicAdd(p.done, 1u) == nblk - 1;
+    s_last = last;
+    if (last) {
+      *p.done = 0;
+      if (!res) advance(p);
+    }
   }
+  if (!res) return;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  decide_body(p, (int)nblk, res, red);
+  decide_body(p, (int)nblk, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -1734,7 +1761,8 @@ __global__ void __launch_bounds__(BLOCK) decide_kernel(Params p) {
   __shared__ double red[WARPS][NSLOT];
   const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
-  decide_body(p, 0, q.flags & ITF_RES, red);
+  if (q.flags & ITF_RES) decide_body(p, 0, red);
+  else if (threadIdx.x == 0) advance(p);
 }
 
 // A contingency slice's contributions to the exchange (after its node
@@ -2111,7 +2139,8 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   const long long nl = (long long)p.Kp * p.L * tvl, nn = (long long)p.Kp * p.N * tvn;
   const long long nx = (long long)p.n_dnode * tvl;
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
-  plan->line_grid = (int)((nl + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT));
+  plan->line_ipt = nl <= LINE_SHORT ? 1 : LINE_IPT;
+  plan->line_grid = (int)((nl + (long long)BLOCK * plan->line_ipt - 1) / ((long long)BLOCK * plan->line_ipt));
   plan->node_grid = (int)std::min<long long>(gn, (nn + BLOCK - 1) / BLOCK);
   plan->inner_c = ic;
   // One device kernel beside the line kernel, or three (averages, inner ADMM,
@@ -2278,7 +2307,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           break;
         case BK_LINE4: case BK_LINE1:
           if ((kind == BK_LINE4) == v4 && p.L > 0)
-            blocks = ((long long)p.Kp * p.L * tv4 + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT);
+            blocks = plans[i].line_grid;
           break;
         case BK_NODE4: case BK_NODE1:
           if ((kind == BK_NODE4) == vn) blocks = plans[i].node_grid;
