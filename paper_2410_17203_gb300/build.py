@@ -45,7 +45,7 @@ def build(verbose=False, extra_flags=()):
     """Compile and link; returns the path of the shared library."""
     os.makedirs(BUILD, exist_ok=True)
     os.makedirs(os.path.dirname(LIB), exist_ok=True)
-    common = [nvcc(), "-std=c++17", "-O3", ARCH, "-lineinfo", "-Xcompiler", "-fPIC",
+    common = [nvcc(), "-std=c++17", "-O3", ARCH, "-lineinfo", "-split-compile=0", "-Xcompiler", "-fPIC",
               "-I", INCLUDE, "-I", CSRC, *extra_flags]
     objs = [os.path.join(BUILD, s.replace(".cu", ".o")) for s in SOURCES]
     jobs = [common + ["-c", os.path.join(CSRC, s), "-o", o] for s, o in zip(SOURCES, objs)]

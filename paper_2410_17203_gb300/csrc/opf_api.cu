@@ -339,6 +339,8 @@ void carve(opf_ctx *c, Arena &a) {
   p.dev_b = a.take<float>(c->S);
   p.dev_lo = a.take<float>(ST);
   p.dev_hi = a.take<float>(ST);
+  p.irec = a.take<int2>((size_t)c->n_stor + c->n_ramp);
+  p.ipar = a.take<float4>((size_t)c->n_stor + c->n_ramp);
   p.ramp_ids = a.take<int>(c->n_ramp);
   p.ramp_R = a.take<float>(c->n_ramp);
   p.stor_ids = a.take<int>(c->n_stor);
@@ -806,6 +808,20 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   up(p.dev_b, dev_b);
   up(p.dev_lo, lo);
   up(p.dev_hi, hi);
+  {
+    std::vector<int2> irec;
+    std::vector<float4> ipar;
+    for (size_t b = 0; b < stor.size(); ++b) {
+      irec.push_back(make_int2(stor[b], dev_node_int[stor[b]]));
+      ipar.push_back(make_float4(seff[b], sP[b], sdur[b], scost[b]));
+    }
+    for (size_t r = 0; r < ramp.size(); ++r) {
+      irec.push_back(make_int2(ramp[r], dev_node_int[ramp[r]]));
+      ipar.push_back(make_float4(dev_a[ramp[r]], dev_b[ramp[r]], rampR[r], 0.f));
+    }
+    up(p.irec, irec);
+    up(p.ipar, ipar);
+  }
   up(p.ramp_ids, ramp);
   up(p.ramp_R, rampR);
   up(p.stor_ids, stor);
@@ -967,7 +983,7 @@ opf_status opf_get_info(opf_ctx *c, opf_info *info) {
     const opfk::IterPlan &pl = c->plan;
     // devices (one launch, or averages, inner ADMM and sums), lines, nodes; a
     // slice's decisions are a launch of their own (opf_slice_finish)
-    const int dev = pl.fused ? (pl.dev_inner + pl.dev_closed > 0) : (pl.xs_grid > 0) + (pl.inner_grid > 0) + 1;
+    const int dev = (pl.dev_inner + pl.dev_closed > 0) + (pl.fused ? 0 : (pl.xs_grid > 0) + 1);
     info->kernels_per_iteration = dev + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
   }
   info->N = c->N;

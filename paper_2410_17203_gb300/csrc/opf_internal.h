@@ -130,6 +130,11 @@ struct Params {
   float *XS;  // [N][T], avg_k(pbar + u) of the previous iterate at kept nodes
   const float *dev_a, *dev_b;
   const float *dev_lo, *dev_hi;  // [S][T]
+  // inner-ADMM devices in the order of their warps (batteries, ramp-limited
+  // generators): (device, node) and a battery's (efficiency, power, duration,
+  // cost) or a generator's (a, b, ramp limit, 0)
+  const int2 *irec;
+  const float4 *ipar;
   // ramp-limited generators
   const int *ramp_ids;
   const float *ramp_R;
@@ -223,8 +228,8 @@ struct IterPlan {
   int line_grid, node_grid;            // 0: the kernel has no work
   int line_ipt;                        // line items per thread
   int fused;                           // 1: one device kernel; 0: averages, inner ADMM and device sums apart
-  int dev_inner, dev_closed;           // fused: CTAs of the device kernel for inner-ADMM and closed-form devices
-  int xs_grid, inner_grid, dsum_grid;  // not fused
+  int dev_inner, dev_closed;           // CTAs of the device kernel for inner-ADMM and (fused) closed-form devices
+  int xs_grid, dsum_grid;              // not fused: averages with closed-form devices, device sums
   size_t inner_smem;
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
 };

@@ -53,7 +53,10 @@ constexpr long long LINE_SHORT = 1 << 20;   // ... one, up to this many items
 constexpr int DEVB = 128;        // threads per CTA of the device kernel (its inner-ADMM warps spread over more SMs)
 constexpr int DEV_WARPS = DEVB / 32;
 constexpr int CLOSED_LANES4 = 2, CLOSED_LANES1 = 8;   // lanes per closed-form item: the classes of ksum2 / ksum8
-constexpr int REG_T = 127;         // longest horizon of the register-resident inner ADMM (T + 1 <= 4 x 32)
+constexpr int REG_C = 8;           // largest chunk of the register-resident inner ADMM ...
+constexpr int REG_T = 32 * REG_C - 1;   // ... its longest horizon (T + 1 <= 32 C)
+constexpr int BATCH_C = 4;         // the same in batches, whose kernels hold every chunk up to theirs
+constexpr int BATCH_REG_T = 32 * BATCH_C - 1;
 
 // shared floats per warp of the shared-memory inner ADMM: 3 (T+1) for the
 // work arrays, plus room for one device's (lam, beta) while the horizon is
@@ -64,8 +67,8 @@ __host__ __device__ inline int warp_smem_floats(int T) {
 }
 
 // register chunk of the inner ADMM at horizon T: a battery's T + 1 elements
-// over 32 lanes (1 .. 4); 0 beyond REG_T (the shared-memory path)
-__host__ __device__ inline int inner_chunk(int T) { return T <= REG_T ? (T + 32) >> 5 : 0; }
+// over 32 lanes (1 .. REG_C); 0 beyond longest (the shared-memory path)
+__host__ __device__ inline int inner_chunk(int T, int longest = REG_T) { return T <= longest ? (T + 32) >> 5 : 0; }
 
 // ---------------------------------------------------------------------------
 // The inner ADMM (Appendix D) writes every product, sum and quotient with its
@@ -251,6 +254,21 @@ __device__ __forceinline__ float div_rn(float x, float c, float r) {
   return fmaf(fmaf(-q, c, x), r, q);
 }
 
+__device__ __forceinline__ void prefetch_l1(const void *a) { asm volatile("prefetch.global.L1 [%0];" ::"l"(a)); }
+
+// the current iteration's scalars (the same two loads in every thread)
+__device__ __forceinline__ Iter load_iter(const Params &p) {
+  union {
+    Iter r;
+    int4 v[2];
+  } x;
+  static_assert(sizeof(Iter) == 32, "Iter is loaded as two int4");
+  const int4 *s = reinterpret_cast<const int4 *>(&p.sc->cur);
+  x.v[0] = s[0];
+  x.v[1] = s[1];
+  return x.r;
+}
+
 // Sums over contingencies k of a node array (o: its offset of k = 0; rows T
 // floats apart).  The order of each sum is fixed, so that every form of the
 // device averages (one thread here, a group of lanes in closed_body) agrees
@@ -263,7 +281,8 @@ __device__ __forceinline__ FV<VW> ksum2(const float *a, size_t o, int T, int Kp)
   for (int e = 0; e < VW; ++e) c[0].v[e] = c[1].v[e] = 0.f;
   const float *r = a + o;
   int k = 0;
-#pragma unroll 4
+  constexpr int U = VW == 1 ? 8 : VW == 2 ? 4 : 2;   // 16 values in flight
+#pragma unroll U
   for (; k + 2 <= Kp; k += 2, r += 2 * (size_t)T) {
     const FV<VW> x = ldv<VW>(r), y = ldv<VW>(r + T);
 #pragma unroll
@@ -339,22 +358,22 @@ __device__ __forceinline__ float relaxed(float alpha, float pnew, float pold) {
 }
 
 // X[t] = p_d[t] - avg_k(pbar + u) at the device's node n, t in [0, T), by one
-// warp (Section 3.2 step 2 input).  AVG: the warp forms the average itself;
+// warp (Section 3.2 step 2 input).  avg: the warp forms the average itself;
 // else xs_kernel left it in XS.
-template <bool AVG>
-__device__ __forceinline__ void device_x(const Params &p, const Iter &q, int n, const float *pd, float *X, int lane) {
+__device__ __forceinline__ void device_x(const Params &p, const Iter &q, int n, const float *pd, float *X, int lane,
+                                         bool avg) {
   const int T = p.T;
   const float *xs = p.XS + (size_t)n * T;
-  for (int t = lane; t < T; t += 32) X[t] = rsub(pd[t], AVG ? node_avg<1>(p, q, n, t).v[0] : __ldcg(xs + t));
+  for (int t = lane; t < T; t += 32) X[t] = rsub(pd[t], avg ? node_avg<1>(p, q, n, t).v[0] : __ldcg(xs + t));
   __syncwarp();
 }
 
 // the averages of a lane's C consecutive steps from t0 (0 beyond T)
-template <int C, bool AVG>
-__device__ __forceinline__ void lane_avg(const Params &p, const Iter &q, int n, int t0, float (&xs)[C]) {
+template <int C>
+__device__ __forceinline__ void lane_avg(const Params &p, const Iter &q, int n, int t0, float (&xs)[C], bool avg) {
   const int T = p.T;
-  if constexpr (AVG && (C == 2 || C == 4)) {
-    if (T % 4 == 0) {   // the lane's rows as one 64- or 128-bit load
+  if constexpr (C == 2 || C == 4) {
+    if (avg && T % 4 == 0) {   // the lane's rows as one 64- or 128-bit load
       if (t0 < T) {
         const FV<C> a = node_avg<C>(p, q, n, t0);
 #pragma unroll
@@ -366,7 +385,7 @@ __device__ __forceinline__ void lane_avg(const Params &p, const Iter &q, int n, 
 #pragma unroll
   for (int j = 0; j < C; ++j) {
     xs[j] = 0.f;
-    if (t0 + j < T) xs[j] = AVG ? node_avg<1>(p, q, n, t0 + j).v[0] : __ldcg(p.XS + (size_t)n * T + t0 + j);
+    if (t0 + j < T) xs[j] = avg ? node_avg<1>(p, q, n, t0 + j).v[0] : __ldcg(p.XS + (size_t)n * T + t0 + j);
   }
 }
 
@@ -398,8 +417,9 @@ __device__ __forceinline__ void stage_out(float *lam_g, float *bet_g, const floa
 // Rows: p_t <= pmax_t, -p_t <= -pmin_t, p_{t+1} - p_t <= R, p_t - p_{t+1} <= R.
 // x-update matrix (2a + rho + 2 omega) I + 2 omega D'D is tridiagonal.
 // ---------------------------------------------------------------------------
-template <bool AVG>
-__device__ void ramp_prox(const Params &p, const Iter &q, int r, float *sm, float *state_sh, int lane) {
+__device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, int lane, bool avg) {
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   const int T = p.T;
   const float rho = q.rho_dev;
   const int d = p.ramp_ids[r];
@@ -429,7 +449,7 @@ __device__ void ramp_prox(const Params &p, const Iter &q, int r, float *sm, floa
     }
     __syncwarp();
   }
-  device_x<AVG>(p, q, n, pd, X, lane);   // p_d - avg_k(pbar + u)
+  device_x(p, q, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
   for (int itn = 0; itn < p.inner_iters; ++itn) {
     for (int t = lane; t < T - 1; t += 32)
       W[t] = rsub(rsub(bet[RG_RU * T + t], lam[RG_RU * T + t]), rsub(bet[RG_RD * T + t], lam[RG_RD * T + t]));
@@ -469,8 +489,9 @@ __device__ void ramp_prox(const Params &p, const Iter &q, int r, float *sm, floa
 // terminal i, p2 = clip((x2 - x1) / 2, -u, u) and p1 = -p2 (the minimiser
 // of the two squared distances over p1 + p2 = 0, clipped to the limit)
 // ---------------------------------------------------------------------------
-template <bool AVG>
-__device__ void hvdc_prox(const Params &p, const Iter &q, int h, int lane) {
+__device__ void hvdc_prox(const Params &p, int h, int lane, bool avg) {
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
   const int T = p.T;
   const int d1 = p.hvdc0 + 2 * h, d2 = d1 + 1;
   const float u = p.hvdc_u[h];
@@ -479,8 +500,8 @@ __device__ void hvdc_prox(const Params &p, const Iter &q, int h, int lane) {
   float *pd1 = p.PD + (size_t)d1 * T, *pd2 = p.PD + (size_t)d2 * T;
   for (int t = lane; t < T; t += 32) {
     const float q1 = pd1[t], q2 = pd2[t];
-    const float x1 = q1 - (AVG ? node_avg<1>(p, q, m1, t).v[0] : __ldcg(xs1 + t));
-    const float x2 = q2 - (AVG ? node_avg<1>(p, q, m2, t).v[0] : __ldcg(xs2 + t));
+    const float x1 = q1 - (avg ? node_avg<1>(p, q, m1, t).v[0] : __ldcg(xs1 + t));
+    const float x2 = q2 - (avg ? node_avg<1>(p, q, m2, t).v[0] : __ldcg(xs2 + t));
     const float f = fminf(fmaxf(0.5f * (x2 - x1), -u), u);
     const float r1 = relaxed(p.alpha, -f, q1), r2 = relaxed(p.alpha, f, q2);
     p.DPD[(size_t)d1 * T + t] = r1 - q1;
@@ -496,8 +517,9 @@ __device__ void hvdc_prox(const Params &p, const Iter &q, int h, int lane) {
 // (c_t, delta_t) per step (a 2x2 Schur complement), leaving a tridiagonal
 // system of size T + 1 in the state of charge s.
 // ---------------------------------------------------------------------------
-template <bool AVG>
-__device__ void stor_prox(const Params &p, const Iter &it, int sidx, float *sm, float *state_sh, int lane) {
+__device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh, int lane, bool avg) {
+  const Iter it = load_iter(p);
+  if (it.flags & ITF_SKIP) return;
   const int T = p.T, Tp = T + 1;
   const float rho = it.rho_dev;
   const int d = p.stor_ids[sidx];
@@ -535,7 +557,7 @@ __device__ void stor_prox(const Params &p, const Iter &it, int sidx, float *sm, 
     }
     __syncwarp();
   }
-  device_x<AVG>(p, it, n, pd, X, lane);   // p_d - avg_k(pbar + u)
+  device_x(p, it, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
 #define LAM(g, t) lam[(g) * Tp + (t)]
 #define BET(g, t) bet[(g) * Tp + (t)]
   for (int itn = 0; itn < p.inner_iters; ++itn) {
@@ -697,33 +719,21 @@ __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[
   }
 }
 
-template <int C, bool AVG>
-__device__ void ramp_prox_r(const Params &p, const Iter &q, int r, int lane) {
+// The state that does not depend on the iteration's scalars is requested
+// first, with them; the contingency rows of the node and the box follow when
+// the device's record arrives, so the ten inner iterations wait for two rounds
+// of loads.
+template <int C>
+__device__ void ramp_prox_r(const Params &p, int r, int lane, bool avg) {
   const int T = p.T, t0 = lane * C;
-  const float rho = q.rho_dev;
-  const int d = p.ramp_ids[r];
-  const int n = p.dev_node[d];
-  const float a = p.dev_a[d], b = p.dev_b[d], R = p.ramp_R[r];
-  const float om = rho, om2 = rmul(2.f, om);
+  const int2 ids = p.irec[p.n_stor + r];           // device, node
+  const float4 par = p.ipar[p.n_stor + r];         // a, b, ramp limit
   float *const lam_g = p.ramp_lam + (size_t)r * RG_N * T;
   float *const bet_g = p.ramp_beta + (size_t)r * RG_N * T;
   float *mf = p.ramp_q + (size_t)r * T;
-  // keep the unscaled inner duals omega * lam when omega changes; refactor
-  // (2a + rho + 2 omega) I + 2 omega D'D
   const float rho_old = p.ramp_rho[r];
-  const bool rescale = rho_old != rho;
-  const float ls = (rho_old == 0.f) ? 1.f : rdiv(fabsf(rho_old), rho);
-  if (rescale) {
-    if (lane == 0) {
-      const float base = radd(rmul(2.f, a), rho);
-      tri_factor(mf, T, radd(base, rmul(4.f, om)), radd(base, rmul(6.f, om)), -om2);
-      p.ramp_rho[r] = rho;
-    }
-    __syncwarp();
-  }
   float lam[RG_N][C], bet[RG_N][C], hi[C], lo[C], X[C], pd[C], Z[C];
   TriFac<C> tf;
-  lane_avg<C, AVG>(p, q, n, t0, X);
 #pragma unroll
   for (int j = 0; j < C; ++j) {
     const int t = t0 + j;
@@ -732,15 +742,43 @@ __device__ void ramp_prox_r(const Params &p, const Iter &q, int r, int lane) {
     for (int g = 0; g < RG_N; ++g) {
       lam[g][j] = in ? lam_g[g * T + t] : 0.f;
       bet[g][j] = in ? bet_g[g * T + t] : 0.f;
-      if (rescale) lam[g][j] = rmul(lam[g][j], ls);
     }
-    hi[j] = in ? p.dev_hi[(size_t)d * T + t] : 0.f;
-    lo[j] = in ? p.dev_lo[(size_t)d * T + t] : 0.f;
-    pd[j] = in ? p.PD[(size_t)d * T + t] : 0.f;
-    X[j] = in ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
     tf.q[j] = in ? mf[t] : 1.f;
     Z[j] = 0.f;
   }
+  const Iter q = load_iter(p);
+  if (q.flags & ITF_SKIP) return;
+  const int d = ids.x, n = ids.y;
+  const float a = par.x, b = par.y, R = par.z;
+  const float rho = q.rho_dev, om = rho, om2 = rmul(2.f, om);
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    const int t = t0 + j;
+    const bool in = t < T;
+    hi[j] = in ? p.dev_hi[(size_t)d * T + t] : 0.f;
+    lo[j] = in ? p.dev_lo[(size_t)d * T + t] : 0.f;
+    pd[j] = in ? p.PD[(size_t)d * T + t] : 0.f;
+  }
+  lane_avg<C>(p, q, n, t0, X, avg);
+  // keep the unscaled inner duals omega * lam when omega changes; refactor
+  // (2a + rho + 2 omega) I + 2 omega D'D
+  if (rho_old != rho) {
+    const float ls = (rho_old == 0.f) ? 1.f : rdiv(fabsf(rho_old), rho);
+    if (lane == 0) {
+      const float base = radd(rmul(2.f, a), rho);
+      tri_factor(mf, T, radd(base, rmul(4.f, om)), radd(base, rmul(6.f, om)), -om2);
+      p.ramp_rho[r] = rho;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+#pragma unroll
+      for (int g = 0; g < RG_N; ++g) lam[g][j] = rmul(lam[g][j], ls);
+      tf.q[j] = t0 + j < T ? mf[t0 + j] : 1.f;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < C; ++j) X[j] = t0 + j < T ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
   tf.init(om2, T, lane);   // off = -2 omega
   for (int itn = 0; itn < p.inner_iters; ++itn) {
     float W[C];
@@ -792,18 +830,47 @@ __device__ void ramp_prox_r(const Params &p, const Iter &q, int r, int lane) {
   }
 }
 
-template <int C, bool AVG>
-__device__ void stor_prox_r(const Params &p, const Iter &it, int sidx, int lane) {
+template <int C>
+__device__ void stor_prox_r(const Params &p, int sidx, int lane, bool avg) {
   const int T = p.T, Tp = T + 1, t0 = lane * C;
-  const float rho = it.rho_dev;
-  const int d = p.stor_ids[sidx];
-  const int n = p.dev_node[d];
-  const float eta = p.stor_eff[sidx], Pm = p.stor_P[sidx], Em = rmul(p.stor_dur[sidx], Pm);
-  const float q = p.stor_cost[sidx];
-  const float om = rho, om2 = rmul(2.f, om);
+  const int2 ids = p.irec[sidx];                   // device, node
+  const float4 par = p.ipar[sidx];                 // efficiency, power, duration, cost
   float *const lam_g = p.stor_lam + (size_t)sidx * SG_N * Tp;
   float *const bet_g = p.stor_beta + (size_t)sidx * SG_N * Tp;
   float *mf = p.stor_q + (size_t)sidx * Tp;
+  const float rho_old = p.stor_rho[sidx];
+  // element e = t0 + j: step t = e of (p, c, delta) while e < T, state of
+  // charge s_e while e < T + 1
+  float lE1[C], lE2[C], lCU[C], lCL[C], lDU[C], lDL[C], lSU[C], lSL[C];
+  float bCU[C], bCL[C], bDU[C], bDL[C], bSU[C], bSL[C];
+  float X[C], pd[C], S[C], TAU[C], DL[C];
+  TriFac<C> tf;
+  float e3a = lam_g[SG_E3 * Tp], e3b = lam_g[SG_E3 * Tp + 1];   // s_0 and s_T rows
+#define LD_L(arr, g) arr[j] = in ? lam_g[(g) * Tp + e] : 0.f
+#define LD_B(arr, g) arr[j] = in ? bet_g[(g) * Tp + e] : 0.f
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    const int e = t0 + j;
+    const bool in = e < Tp;
+    LD_L(lE1, SG_E1); LD_L(lE2, SG_E2); LD_L(lCU, SG_CU); LD_L(lCL, SG_CL);
+    LD_L(lDU, SG_DU); LD_L(lDL, SG_DL); LD_L(lSU, SG_SU); LD_L(lSL, SG_SL);
+    LD_B(bCU, SG_CU); LD_B(bCL, SG_CL); LD_B(bDU, SG_DU); LD_B(bDL, SG_DL);
+    LD_B(bSU, SG_SU); LD_B(bSL, SG_SL);
+    tf.q[j] = in ? mf[e] : 1.f;
+    S[j] = TAU[j] = DL[j] = 0.f;
+  }
+#undef LD_L
+#undef LD_B
+  const Iter it = load_iter(p);
+  if (it.flags & ITF_SKIP) return;
+  const int d = ids.x, n = ids.y;
+#pragma unroll
+  for (int j = 0; j < C; ++j) pd[j] = t0 + j < T ? p.PD[(size_t)d * T + t0 + j] : 0.f;
+  lane_avg<C>(p, it, n, t0, X, avg);
+  const float rho = it.rho_dev;
+  const float eta = par.x, Pm = par.y, Em = rmul(par.z, Pm);
+  const float q = par.w;
+  const float om = rho, om2 = rmul(2.f, om);
 
   // 2x2 block of (c, delta) after eliminating p; constants of the reduction
   const float kap = rdiv(rmul(rho, om), radd(rho, om));
@@ -816,47 +883,27 @@ __device__ void stor_prox_r(const Params &p, const Iter &it, int sidx, int lane)
   const float gam = rsub(om, radd(rmul(f1c, w0), rmul(f1d, w1)));
   const float rpo = radd(rho, om), rrpo = __frcp_rn(rpo), rgam = __frcp_rn(gam);
 
-  const float rho_old = p.stor_rho[sidx];
-  const bool rescale = rho_old != rho;
-  const float ls = (rho_old == 0.f) ? 1.f : rdiv(fabsf(rho_old), rho);
-  if (rescale) {
+  if (rho_old != rho) {
+    const float ls = (rho_old == 0.f) ? 1.f : rdiv(fabsf(rho_old), rho);
     if (lane == 0) {
       tri_factor(mf, Tp, radd(gam, rmul(3.f, om)), radd(rmul(2.f, gam), om2), -gam);
       p.stor_rho[sidx] = rho;
     }
     __syncwarp();
-  }
-  // element e = t0 + j: step t = e of (p, c, delta) while e < T, state of
-  // charge s_e while e < T + 1
-  float lE1[C], lE2[C], lCU[C], lCL[C], lDU[C], lDL[C], lSU[C], lSL[C];
-  float bCU[C], bCL[C], bDU[C], bDL[C], bSU[C], bSL[C];
-  float X[C], pd[C], S[C], TAU[C], DL[C];
-  TriFac<C> tf;
-  float e3a = lam_g[SG_E3 * Tp], e3b = lam_g[SG_E3 * Tp + 1];   // s_0 and s_T rows
-  if (rescale) {
     e3a = rmul(e3a, ls);
     e3b = rmul(e3b, ls);
-  }
-  lane_avg<C, AVG>(p, it, n, t0, X);
-#define LD_L(arr, g) arr[j] = in ? (rescale ? rmul(lam_g[(g) * Tp + e], ls) : lam_g[(g) * Tp + e]) : 0.f
-#define LD_B(arr, g) arr[j] = in ? bet_g[(g) * Tp + e] : 0.f
 #pragma unroll
-  for (int j = 0; j < C; ++j) {
-    const int e = t0 + j;
-    const bool in = e < Tp;
-    LD_L(lE1, SG_E1); LD_L(lE2, SG_E2); LD_L(lCU, SG_CU); LD_L(lCL, SG_CL);
-    LD_L(lDU, SG_DU); LD_L(lDL, SG_DL); LD_L(lSU, SG_SU); LD_L(lSL, SG_SL);
-    LD_B(bCU, SG_CU); LD_B(bCL, SG_CL); LD_B(bDU, SG_DU); LD_B(bDL, SG_DL);
-    LD_B(bSU, SG_SU); LD_B(bSL, SG_SL);
-    const bool st = e < T;
-    pd[j] = st ? p.PD[(size_t)d * T + e] : 0.f;
-    X[j] = st ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
-    tf.q[j] = in ? mf[e] : 1.f;
-    S[j] = TAU[j] = DL[j] = 0.f;
+    for (int j = 0; j < C; ++j) {
+      lE1[j] = rmul(lE1[j], ls); lE2[j] = rmul(lE2[j], ls);
+      lCU[j] = rmul(lCU[j], ls); lCL[j] = rmul(lCL[j], ls);
+      lDU[j] = rmul(lDU[j], ls); lDL[j] = rmul(lDL[j], ls);
+      lSU[j] = rmul(lSU[j], ls); lSL[j] = rmul(lSL[j], ls);
+      tf.q[j] = t0 + j < Tp ? mf[t0 + j] : 1.f;
+    }
   }
+#pragma unroll
+  for (int j = 0; j < C; ++j) X[j] = t0 + j < T ? rsub(pd[j], X[j]) : 0.f;   // p_d - avg_k(pbar + u)
   tf.init(gam, Tp, lane);   // off = -gam
-#undef LD_L
-#undef LD_B
   for (int itn = 0; itn < p.inner_iters; ++itn) {
     float f0c[C], f0d[C];
 #pragma unroll
@@ -1239,21 +1286,6 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   stv_cs<VW>(p.THBAR[nw] + on, tbar);
 }
 
-__device__ __forceinline__ void prefetch_l1(const void *a) { asm volatile("prefetch.global.L1 [%0];" ::"l"(a)); }
-
-// the current iteration's scalars (the same two loads in every thread)
-__device__ __forceinline__ Iter load_iter(const Params &p) {
-  union {
-    Iter r;
-    int4 v[2];
-  } x;
-  static_assert(sizeof(Iter) == 32, "Iter is loaded as two int4");
-  const int4 *s = reinterpret_cast<const int4 *>(&p.sc->cur);
-  x.v[0] = s[0];
-  x.v[1] = s[1];
-  return x.r;
-}
-
 // closed-form prox of device d at VW time steps, given the average there
 // (Section 4.2, weight (K+1) rho_p)
 template <int VW>
@@ -1363,45 +1395,44 @@ __device__ __forceinline__ void closed_body(const Params &p, unsigned bid, unsig
 
 // the register path at the device's own chunk (cs, cr <= C; ONLY: cs = C and
 // cr is C or C - 1, as for one instance)
-template <int C, bool AVG, bool ONLY>
-__device__ __forceinline__ void stor_r(const Params &p, const Iter &q, int sidx, int lane, int cs) {
+template <int C, bool ONLY>
+__device__ __forceinline__ void stor_r(const Params &p, int sidx, int lane, int cs, bool avg) {
   if constexpr (C > 1 && !ONLY) {
     if (cs < C) {
-      stor_r<C - 1, AVG, false>(p, q, sidx, lane, cs);
+      stor_r<C - 1, false>(p, sidx, lane, cs, avg);
       return;
     }
   }
-  stor_prox_r<C, AVG>(p, q, sidx, lane);
+  stor_prox_r<C>(p, sidx, lane, avg);
 }
 
-template <int C, bool AVG, bool ONLY>
-__device__ __forceinline__ void ramp_r(const Params &p, const Iter &q, int r, int lane, int cr) {
+template <int C, bool ONLY>
+__device__ __forceinline__ void ramp_r(const Params &p, int r, int lane, int cr, bool avg) {
   if constexpr (C > 1) {
     if (cr < C) {
-      if constexpr (ONLY) ramp_prox_r<C - 1, AVG>(p, q, r, lane);
-      else ramp_r<C - 1, AVG, false>(p, q, r, lane, cr);
+      if constexpr (ONLY) ramp_prox_r<C - 1>(p, r, lane, avg);
+      else ramp_r<C - 1, false>(p, r, lane, cr, avg);
       return;
     }
   }
-  ramp_prox_r<C, AVG>(p, q, r, lane);
+  ramp_prox_r<C>(p, r, lane, avg);
 }
 
 // ---------------------------------------------------------------------------
 // inner: one warp per battery, then per ramp-limited generator (Appendix D),
 // then per HVDC link.  C > 0: the register path, for horizons of at most
 // REG_T steps (chunks of at most C); C = 0: the shared-memory path.  MIXED
-// (batches): the instance's horizon chooses, beyond REG_T the shared-memory
-// path.  AVG: each warp forms its node's average over contingencies.
+// (batches): the instance's horizon chooses, beyond BATCH_REG_T the
+// shared-memory path.  avg: each warp forms its node's average over
+// contingencies (else it is in XS).
 // ---------------------------------------------------------------------------
-template <int C, bool MIXED, bool AVG>
-__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem) {
-  const Iter q = load_iter(p);
-  if (q.flags & ITF_SKIP) return;
+template <int C, bool MIXED>
+__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem, bool avg) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int T = p.T;
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
   constexpr bool HAS_SMEM = C == 0 || MIXED, HAS_REG = C > 0;
-  const bool reg = HAS_REG && (!HAS_SMEM || T <= REG_T);
+  const bool reg = HAS_REG && (!HAS_SMEM || T <= BATCH_REG_T);
   float *wsm = nullptr, *state_sh = nullptr;
   if (HAS_SMEM && !reg) {
     const int wfl = warp_smem_floats(T);
@@ -1413,21 +1444,21 @@ __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsign
     if (w < p.n_stor) {
       if constexpr (HAS_REG) {
         if (reg) {
-          stor_r<C, AVG, !MIXED>(p, q, w, lane, cs);
+          stor_r<C, !MIXED>(p, w, lane, cs, avg);
           continue;
         }
       }
-      if constexpr (HAS_SMEM) stor_prox<AVG>(p, q, w, wsm, state_sh, lane);
+      if constexpr (HAS_SMEM) stor_prox(p, w, wsm, state_sh, lane, avg);
     } else if (w < p.n_stor + p.n_ramp) {
       if constexpr (HAS_REG) {
         if (reg) {
-          ramp_r<C, AVG, !MIXED>(p, q, w - p.n_stor, lane, cr);
+          ramp_r<C, !MIXED>(p, w - p.n_stor, lane, cr, avg);
           continue;
         }
       }
-      if constexpr (HAS_SMEM) ramp_prox<AVG>(p, q, w - p.n_stor, wsm, state_sh, lane);
+      if constexpr (HAS_SMEM) ramp_prox(p, w - p.n_stor, wsm, state_sh, lane, avg);
     } else {
-      hvdc_prox<AVG>(p, q, w - p.n_stor - p.n_ramp, lane);
+      hvdc_prox(p, w - p.n_stor - p.n_ramp, lane, avg);
     }
   }
 }
@@ -1723,22 +1754,19 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
 template <int VW>
 __global__ void __launch_bounds__(BLOCK) xs_kernel(Params p) { xs_body<VW>(p, blockIdx.x, gridDim.x); }
 
-template <int C>
-__global__ void __launch_bounds__(BLOCK) inner_kernel(Params p) {
-  extern __shared__ float smem[];
-  inner_body<C, false, false>(p, blockIdx.x, gridDim.x, smem);
-}
-
 // Every device of an iteration in one launch (step 2): the first inner_blocks
 // CTAs take the inner-ADMM devices and links, the others the closed-form
 // ones.  Each forms its node's average itself, so nothing runs in front of
 // the inner ADMM, the longest chain of the phase; nodes with several
-// inner-ADMM devices form it once per device.
-template <int C, int VW>
-__global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks) {
+// inner-ADMM devices form it once per device.  Where the averages and the
+// closed-form devices are a kernel of their own (avg false), only the first
+// part is launched.
+template <int C>
+__global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks, bool avg) {
   extern __shared__ float smem[];
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, false, true>(p, blockIdx.x, inner_blocks, smem);
-  else closed_body<VW>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, blockIdx.x, inner_blocks, smem, avg);
+  else if (p.T % 4 == 0) closed_body<4>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
+  else closed_body<1>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
 }
 
 template <int VW>
@@ -1827,15 +1855,15 @@ __device__ __forceinline__ const Params &batch_params(const Params *ps, const in
 
 // the devices of every instance: the first inner_blocks CTAs of the schedule
 // take inner-ADMM devices, the others closed-form ones.  C: the largest
-// register chunk of the batch's instances (0: every horizon beyond REG_T),
-// any longer horizon on the shared-memory path
+// register chunk of the batch's instances (0: every horizon beyond
+// BATCH_REG_T), any longer horizon on the shared-memory path (the same bits)
 template <int C>
 __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks) {
   extern __shared__ float smem[];
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0), true>(p, bid, nblk, smem);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true);
   else if (p.T % 4 == 0) closed_body<4>(p, bid, nblk);
   else closed_body<1>(p, bid, nblk);
 }
@@ -2153,28 +2181,26 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // moves about 32 bytes per (line, contingency, step) at 6.5 TB/s; a round of
   // devices takes about 5 + 0.08 T microseconds from registers, 0.45 T in
   // shared memory.  At 10k buses, T = 96, K = 50 (3,000 devices), ms per
-  // iteration by CTAs of the inner kernel: 375 0.706, 76 0.706, 38 0.698, 25
-  // 0.696, 19 0.704, 12 0.851: the fewest whose rounds fit in half the line
-  // pass; device sums in the node pass 0.701 against 0.697.  At 2k buses,
+  // iteration by warps of the inner kernel: 3,000 0.706, 608 0.706, 304 0.698,
+  // 200 0.696, 152 0.704, 96 0.851: the fewest whose rounds fit in half the
+  // line pass; device sums in the node pass 0.701 against 0.697.  At 2k buses,
   // T = 24, K = 20: three device kernels 31.7 us per iteration, one 25.2.
   const double line_us = (double)p.Kp * p.L * p.T * 32.0 / 6.5e6;
-  const int one_round = (n_inner + WARPS - 1) / WARPS;
+  const int one_round = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
   const double round_us = ic ? 5.0 + 0.08 * p.T : 0.45 * p.T;
   const int max_rounds = (int)std::floor((ic ? 0.5 : 0.7) * line_us / round_us);
+  const size_t ism = ic ? 0 : inner_smem(p.T, DEV_WARPS);
+  if (!allow_smem(dev_kernel<0>, ism)) return -1;
+  plan->inner_smem = ism;
   plan->fused = !p.slice && max_rounds < 2;
-  plan->xs_grid = plan->dsum_grid = plan->inner_grid = plan->dev_inner = plan->dev_closed = 0;
+  plan->xs_grid = plan->dsum_grid = plan->dev_closed = 0;
+  plan->dev_inner = one_round;
   if (plan->fused) {
-    const size_t ism = ic ? 0 : inner_smem(p.T, DEV_WARPS);
-    if (!allow_smem(dev_kernel<0, 4>, ism) || !allow_smem(dev_kernel<0, 1>, ism)) return -1;
-    plan->inner_smem = ism;
-    plan->dev_inner = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
-    plan->dev_closed = (int)std::min<long long>(4096, ((long long)p.n_cnode * tvl * (v4 ? CLOSED_LANES4 : CLOSED_LANES1) + DEVB - 1) / DEVB);
+    plan->dev_closed = (int)std::min<long long>(
+        4096, ((long long)p.n_cnode * tvl * (v4 ? CLOSED_LANES4 : CLOSED_LANES1) + DEVB - 1) / DEVB);
     return 0;
   }
-  const size_t ism = ic ? 0 : inner_smem(p.T, WARPS);
-  if (!allow_smem(inner_kernel<0>, ism)) return -1;
-  plan->inner_smem = ism;
-  plan->inner_grid = max_rounds >= 2 ? (one_round + max_rounds - 1) / max_rounds : one_round;
+  if (max_rounds >= 2) plan->dev_inner = (one_round + max_rounds - 1) / max_rounds;
   plan->xs_grid = (int)std::min<long long>(gx, (nx + BLOCK - 1) / BLOCK);
   const long long nd = (long long)p.N * (p.T / (v2 ? 2 : 1));
   plan->dsum_grid = (int)std::min<long long>(gd, (nd + BLOCK - 1) / BLOCK);
@@ -2191,36 +2217,22 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
   // sums (main stream) follow them and the device kernels.
   if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
-  if (plan.fused) {
-    const int ni = plan.dev_inner, g = ni + plan.dev_closed;
-    if (g > 0) {
-#define DEV_LAUNCH(C)                                                             \
-  if (v4) dev_kernel<C, 4><<<g, DEVB, plan.inner_smem, sm>>>(p, ni);              \
-  else dev_kernel<C, 1><<<g, DEVB, plan.inner_smem, sm>>>(p, ni);                 \
-  break
-      switch (plan.inner_c) {
-        case 1: DEV_LAUNCH(1);
-        case 2: DEV_LAUNCH(2);
-        case 3: DEV_LAUNCH(3);
-        case 4: DEV_LAUNCH(4);
-        default: DEV_LAUNCH(0);
-      }
+  if (!plan.fused && plan.xs_grid > 0) {
+    if (v4) xs_kernel<4><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
+    else xs_kernel<1><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
+  }
+  const int ni = plan.dev_inner, nd = ni + plan.dev_closed;
+  const bool avg = plan.fused;
+  if (nd > 0) {
+#define DEV_LAUNCH(C) case C: dev_kernel<C><<<nd, DEVB, plan.inner_smem, sm>>>(p, ni, avg); break
+    static_assert(REG_C == 8, "the chunks launched below");
+    switch (plan.inner_c) {
+      DEV_LAUNCH(0); DEV_LAUNCH(1); DEV_LAUNCH(2); DEV_LAUNCH(3); DEV_LAUNCH(4);
+      DEV_LAUNCH(5); DEV_LAUNCH(6); DEV_LAUNCH(7); DEV_LAUNCH(8);
+    }
 #undef DEV_LAUNCH
-    }
-  } else {
-    if (plan.xs_grid > 0) {
-      if (v4) xs_kernel<4><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
-      else xs_kernel<1><<<plan.xs_grid, BLOCK, 0, sm>>>(p);
-    }
-    if (plan.inner_grid > 0) {
-      switch (plan.inner_c) {
-        case 1: inner_kernel<1><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-        case 2: inner_kernel<2><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-        case 3: inner_kernel<3><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-        case 4: inner_kernel<4><<<plan.inner_grid, BLOCK, 0, sm>>>(p); break;
-        default: inner_kernel<0><<<plan.inner_grid, BLOCK, plan.inner_smem, sm>>>(p); break;
-      }
-    }
+  }
+  if (!plan.fused) {
     if (v2) dsum_kernel<2><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
     else dsum_kernel<1><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
   }
@@ -2297,7 +2309,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
         case BK_INNER:
           blocks = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
           if (blocks) {
-            const int ic = inner_chunk(p.T);
+            const int ic = inner_chunk(p.T, BATCH_REG_T);
             if (ic) ic_max = std::max(ic_max, ic);
             else ism = std::max(ism, inner_smem(p.T, DEV_WARPS));   // the shared-memory path
           }

@@ -1,0 +1,61 @@
+"""The forms of the device phase against the oracle and against each other:
+the register-resident inner ADMM at the edges of its chunks of steps per lane
+and the shared-memory form beyond them, one device kernel or separate
+averages and sums, one instance or a batch."""
+import numpy as np
+import pytest
+
+from gridgen import make_case, scale_case
+from helpers import compare_states
+from oracle import Oracle, OracleOptions
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_2410_17203_gb300 import load_library
+    load_library()
+
+
+@pytest.mark.parametrize("T", [2, 31, 32, 63, 64, 127, 128, 159, 160, 255, 256])
+def test_inner_chunks_match_oracle(T):
+    """A battery holds T + 1 elements and a ramp-limited generator T: their
+    chunk sizes change at T = 31 / 32, 63 / 64 and so on; 255 is the longest
+    horizon in registers.  12 iterations include one change of the penalty."""
+    from paper_2410_17203_gb300 import Solver
+    case = make_case(scale_case(20, T, 2, seed=500 + T, stor_per_node=0.2, n_hvdc=1))
+    opts = dict(adapt_every=10, eps=0.0)
+    s = Solver(case, opts)
+    s.iterate(12)
+    o = Oracle(case, OracleOptions(**opts))
+    o.iterate(12, stop=False)
+    compare_states(s.state(), o)
+    s.close()
+
+
+@pytest.mark.parametrize("n, T, K, alpha", [
+    (60, 1, 9, 1.0), (60, 31, 10, 1.0), (40, 128, 3, 1.0), (30, 255, 2, 1.5), (60, 7, 22, 1.5),
+    # a line pass long enough to hide the devices: averages and device sums are kernels of their own
+    (2600, 160, 24, 1.0), (2600, 160, 24, 1.5), (3000, 121, 24, 1.0),
+])
+def test_single_instance_and_batch_agree_bit_for_bit(n, T, K, alpha):
+    """A batch forms every average where it is used, sums device powers in the
+    node pass and takes horizons beyond 127 steps through shared memory."""
+    from paper_2410_17203_gb300 import Solver, opf_batch_create, opf_batch_destroy, opf_batch_iterate
+    case = make_case(scale_case(n, T, K, seed=7))
+    opts = dict(adapt_every=10, eps=0.0, alpha=alpha)
+    single, member = Solver(case, opts), Solver(case, opts)
+    single.iterate(13)
+    b = opf_batch_create([member.h])
+    try:
+        opf_batch_iterate(b, 13)
+        x, y = single.state(), member.state()
+        for k in x:
+            np.testing.assert_array_equal(x[k], y[k], err_msg=k)
+    finally:
+        opf_batch_destroy(b)
+        single.close()
+        member.close()
