@@ -46,6 +46,7 @@ constexpr int WARPS = BLOCK / 32;
 constexpr int ST_NONFINITE = 5;  // opf_status value set on the device
 constexpr int NODE_VW = 4;       // time steps per node item
 constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is compiled for (64 registers)
+constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
 constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items)
@@ -1015,6 +1016,24 @@ struct Welf {
   }
 };
 
+// the mean alone (the same bits as Welf's)
+template <int VW>
+struct WelfMean {
+  float n;
+  float mean[VW];
+  __device__ __forceinline__ void reset() {
+    n = 0.f;
+#pragma unroll
+    for (int e = 0; e < VW; ++e) mean[e] = 0.f;
+  }
+  __device__ __forceinline__ void add(const float *x) {
+    n += 1.f;
+    const float r = __frcp_rn(n);
+#pragma unroll
+    for (int e = 0; e < VW; ++e) mean[e] = fmaf(x[e] - mean[e], r, mean[e]);
+  }
+};
+
 // one-pass sums of two series over a node's terminals (Welford with the
 // co-moment): means, centred second moments and sum (x - mean_x)(y - mean_y)
 template <int VW>
@@ -1143,7 +1162,8 @@ __device__ __forceinline__ void line_item(const Params &p, int old, int nw, int 
 // ---------------------------------------------------------------------------
 // RES false: the iteration's residuals are not read, so the node sums skip the
 // inputs only they need (old p and theta_bar rows, the device Welford state)
-// and their accumulation; the relaxed variant always needs the mean change.
+// and their accumulation; the relaxed variant still needs the mean change of p
+// (its u update), so it reads the old p rows and keeps that mean alone.
 // NB: line terminals gathered together.
 // ILD: the pass sums the node's device powers (and the Welford state of their
 // changes) itself; else dsum_kernel has left them in DSP, DSM and DSQ.
@@ -1151,7 +1171,7 @@ template <int VW, bool RELAX, bool RES, int NB, bool ILD>
 __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int k, int n, int toff, float fsu,
                                           float *acc) {
   const int T = p.T;
-  constexpr bool res = RES || RELAX;
+  constexpr bool dp = RES || RELAX;   // the change of p is read
   // level 1: the node record, the node's old rows and its device sums
   const int4 r0 = p.nrec[3 * n], r1 = p.nrec[3 * n + 1], r2 = p.nrec[3 * n + 2];
   const float cp = __int_as_float(r0.x), ct = __int_as_float(r0.y);
@@ -1159,16 +1179,23 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   const size_t on = nidx(p, k, n, toff), os = (size_t)n * T + toff;
   const FV<VW> uo = ldv_cs<VW>(p.U[old] + on);
   FV<VW> go;
-  if (res) go = ldv_cs<VW>(p.THBAR[old] + on);
+  if constexpr (RES) go = ldv_cs<VW>(p.THBAR[old] + on);
   // device terminals first: the sum and the Welford state after them, the
   // same in every contingency, in the order of dcsr_idx
   FV<VW> sp, st;
   Welf<VW> wdp, wth;
   Welf2<VW> wrx;   // RELAX: (Theta_new, Theta_new - Theta_old) over the line terminals
-  if constexpr (RELAX) wrx.reset();
+  WelfMean<VW> wm; // RELAX without residuals: the mean change of p
+  if constexpr (RELAX && RES) wrx.reset();
   if constexpr (!ILD) {
     sp = ldv<VW>(p.DSP + os);
-    if constexpr (res) {
+    if constexpr (RELAX && !RES) {
+      const FV<VW> m = ldv<VW>(p.DSM + os);
+      wm.n = (float)r2.z;
+#pragma unroll
+      for (int e = 0; e < VW; ++e) wm.mean[e] = m.v[e];
+    }
+    if constexpr (RES) {
       const FV<VW> m = ldv<VW>(p.DSM + os), q = ldv<VW>(p.DSQ + os);
       wdp.n = (float)r2.z;
 #pragma unroll
@@ -1178,13 +1205,15 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   if constexpr (ILD) {
 #pragma unroll
     for (int e = 0; e < VW; ++e) sp.v[e] = 0.f;
-    if constexpr (res) wdp.reset();
+    if constexpr (RES) wdp.reset();
+    if constexpr (RELAX && !RES) wm.reset();
     for (int j = r2.w; j < r2.w + r2.z; ++j) {
       const size_t od = (size_t)p.dcsr_idx[j] * T + toff;
       const FV<VW> pd = ldv<VW>(p.PD + od);
 #pragma unroll
       for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
-      if constexpr (res) wdp.add(ldv<VW>(p.DPD + od).v);
+      if constexpr (RES) wdp.add(ldv<VW>(p.DPD + od).v);
+      else if constexpr (RELAX) wm.add(ldv<VW>(p.DPD + od).v);
     }
   }
   wth.reset();
@@ -1196,13 +1225,14 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   const int lout = p.out_line[k];
   int4 c4 = r1;
   for (int j = r2.x - 4;;) {
-    const int code4[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll 1
     for (int half = 0; half < 4; half += NB) {
-    int code[NB];
-#pragma unroll
-    for (int q = 0; q < NB; ++q) code[q] = code4[half + q];
-    FV<VW> pn[NB], po[NB], mq[NB], mo[RELAX ? NB : 1];
+    // the next NB codes; the rest move up (an indexed array of the four would
+    // live in local memory)
+    const int code[4] = {c4.x, c4.y, c4.z, c4.w};
+    c4 = NB == 1 ? make_int4(code[1], code[2], code[3], 0) : make_int4(code[2], code[3], 0, 0);
+    static_assert(NB == 1 || NB == 2 || NB == 4, "codes taken together");
+    FV<VW> pn[NB], po[NB], mq[NB], mo[RELAX && RES ? NB : 1];
     float bq[NB];
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
@@ -1210,9 +1240,9 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
         const int l = code[q] >> 1;
         const size_t ol = (size_t)l * lrow + kb;
         pn[q] = ldv<VW>(p.P[nw] + ol);
-        if (res) po[q] = ldv<VW>(p.P[old] + ol);   // kept in L2 for the line's other end
+        if constexpr (dp) po[q] = ldv<VW>(p.P[old] + ol);   // kept in L2 for the line's other end
         mq[q] = ldv<VW>(p.MID[nw] + ol);
-        if constexpr (RELAX) mo[q] = ldv<VW>(p.MID[old] + ol);
+        if constexpr (RELAX && RES) mo[q] = ldv<VW>(p.MID[old] + ol);
         bq[q] = p.line_b[l];
       }
     }
@@ -1224,21 +1254,23 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
         float dpo[VW], th[VW], dth[VW];
 #pragma unroll
         for (int e = 0; e < VW; ++e) {
-          const float pv = act ? pn[q].v[e] : 0.f, pov = (act && res) ? po[q].v[e] : 0.f;
+          const float pv = act ? pn[q].v[e] : 0.f, pov = (act && dp) ? po[q].v[e] : 0.f;
           const float h = act ? div_rn(pn[q].v[e], tb, rtb) : pn[q].v[e];
           th[e] = t2 ? mq[q].v[e] - h : mq[q].v[e] + h;
           sp.v[e] += t2 ? pv : -pv;
           st.v[e] += th[e];
           dpo[e] = t2 ? pv - pov : pov - pv;
-          if constexpr (RELAX) {
+          if constexpr (RELAX && RES) {
             const float ho = act ? div_rn(po[q].v[e], tb, rtb) : po[q].v[e];
             dth[e] = th[e] - (t2 ? mo[q].v[e] - ho : mo[q].v[e] + ho);
           }
         }
-        if (res) {
+        if constexpr (RES) {
           wdp.add(dpo);
           if constexpr (RELAX) wrx.add(th, dth);
           else wth.add(th);
+        } else if constexpr (RELAX) {
+          wm.add(dpo);
         }
       }
     }
@@ -1252,8 +1284,13 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
   for (int e = 0; e < VW; ++e) {
     pb.v[e] = div_rn(sp.v[e], cp, rcp);                      // Eq. (average-op)
     tbar.v[e] = ct > 0.f ? div_rn(st.v[e], ct, rct) : 0.f;
-    if (!res) {
-      un.v[e] = fsu * uo.v[e] + pb.v[e];                     // u += pbar
+    if constexpr (!RES) {
+      if constexpr (RELAX) {
+        const float a = p.alpha;
+        un.v[e] = fsu * uo.v[e] + fmaf(a, pb.v[e], (1.f - a) * wm.mean[e]);
+      } else {
+        un.v[e] = fsu * uo.v[e] + pb.v[e];                   // u += pbar
+      }
       continue;
     }
     const float dt = tbar.v[e] - go.v[e];
@@ -1703,9 +1740,9 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   if (q.flags & ITF_SKIP) return;
   const bool res = q.flags & ITF_RES;
   float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  if (res || RELAX) {
+  if (res) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
-      node_item<VW, RELAX, true, RELAX ? 4 : NODE_RES_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+      node_item<VW, RELAX, true, NODE_RES_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
   } else {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
       node_item<VW, RELAX, false, NODE_LEAN_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
@@ -1777,10 +1814,12 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p) {
   line_body<VW>(p, blockIdx.x);
 }
 
-// the over-relaxed variant carries more per-terminal state: it takes the
-// registers of one CTA per SM rather than spill; ILD: device sums in the pass
+// The over-relaxed variant reads one more row per terminal and carries the mean
+// change of p: three CTAs per SM at 80 registers (1k buses, T = 48, K = 20,
+// alpha = 1.5, us per iteration: two 28.6, three 26.9, four 28.3; 39.8 when
+// every iteration carried the residual sums).  ILD: device sums in the pass.
 template <int VW, bool RELAX, bool ILD>
-__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel(Params p) {
+__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel(Params p) {
   node_body<VW, RELAX, ILD>(p, blockIdx.x, gridDim.x);
 }
 
@@ -1877,7 +1916,7 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, cons
 }
 
 template <int VW, bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? 1 : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched) {
+__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched) {
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);

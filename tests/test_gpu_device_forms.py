@@ -59,3 +59,22 @@ def test_single_instance_and_batch_agree_bit_for_bit(n, T, K, alpha):
         opf_batch_destroy(b)
         single.close()
         member.close()
+
+
+@pytest.mark.parametrize("T", [24, 7])
+def test_relaxed_split_launches_equal_one_launch(T):
+    """The over-relaxed node pass without residual sums (all but the last
+    iteration of a call and the adaptation iterations) gives the iterate of
+    the pass with them bit for bit, wherever the calls end."""
+    from paper_2410_17203_gb300 import Solver
+    case = make_case(scale_case(90, T, 3, seed=41))
+    opts = dict(adapt_every=10, eps=0.0, alpha=1.5)
+    a, b = Solver(case, opts), Solver(case, opts)
+    a.iterate(33)
+    for n in (1, 1, 4, 9, 3, 15):
+        b.iterate(n)
+    x, y = a.state(), b.state()
+    for k in x:
+        np.testing.assert_array_equal(x[k], y[k], err_msg=k)
+    a.close()
+    b.close()
