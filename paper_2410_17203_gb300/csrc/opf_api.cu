@@ -280,6 +280,11 @@ std::vector<int> rcm_order(int N, const std::vector<int> &ptr, const std::vector
 // nodes with devices, then the residual partial sums
 size_t slice_exchange_len(const opf_ctx *c) { return (size_t)2 * c->n_dnode * c->T + opfk::NSLOT; }
 
+// floats of the exported inner-ADMM state (opf_info.inner_len)
+int64_t inner_len(const opf_ctx *c) {
+  return (int64_t)c->n_ramp * 2 * (4 * (int64_t)c->T - 2) + (int64_t)c->n_stor * 2 * (8 * (int64_t)c->T + 4);
+}
+
 // The arena layout; called once with a null base to size it.
 void carve(opf_ctx *c, Arena &a) {
   Params &p = c->P;
@@ -994,8 +999,7 @@ opf_status opf_get_info(opf_ctx *c, opf_info *info) {
   info->J = 2 * c->L + c->S;
   info->n_ramp = c->n_ramp;
   info->n_stor = c->n_stor;
-  info->inner_len = (int64_t)c->n_ramp * 2 * (4 * (int64_t)c->T - 2) +
-                    (int64_t)c->n_stor * 2 * (8 * (int64_t)c->T + 4);
+  info->inner_len = inner_len(c);
   info->device_bytes = (int64_t)c->arena_bytes;
   info->stalled = sc.stalled;
   info->frozen_at = sc.frozen_at;
@@ -1032,42 +1036,20 @@ opf_status opf_history(opf_ctx *c, int32_t max_rows, double *rows, int32_t *n_ro
 
 namespace {
 
-// canonical inner-state entry -> (device array, index)
-struct InnerEntry {
-  int arr;     // 0 ramp_lam, 1 ramp_beta, 2 stor_lam, 3 stor_beta, -1 always zero
-  size_t idx;
-};
-
-std::vector<InnerEntry> inner_layout(const opf_ctx *c) {
-  const int T = c->T, Tp = T + 1;
-  std::vector<InnerEntry> v;
-  for (int r = 0; r < c->n_ramp; ++r) {
-    const size_t base = (size_t)r * opfk::RG_N * T;
-    std::vector<size_t> rows;
-    for (int t = 0; t < T; ++t) rows.push_back(base + opfk::RG_UP * T + t);
-    for (int t = 0; t < T; ++t) rows.push_back(base + opfk::RG_LO * T + t);
-    for (int t = 0; t < T - 1; ++t) rows.push_back(base + opfk::RG_RU * T + t);
-    for (int t = 0; t < T - 1; ++t) rows.push_back(base + opfk::RG_RD * T + t);
-    for (size_t x : rows) v.push_back({0, x});
-    for (size_t x : rows) v.push_back({1, x});
+// zero the inner-ADMM state (factors are rebuilt on first use)
+opf_status zero_inner(opf_ctx *c) {
+  const size_t nr = (size_t)c->n_ramp * opfk::RG_N * c->T, ns = (size_t)c->n_stor * opfk::SG_N * (c->T + 1);
+  if (nr) {
+    CK(cudaMemsetAsync(c->P.ramp_lam, 0, nr * 4, c->stream));
+    CK(cudaMemsetAsync(c->P.ramp_beta, 0, nr * 4, c->stream));
+    CK(cudaMemsetAsync(c->P.ramp_rho, 0, c->n_ramp * 4, c->stream));
   }
-  for (int b = 0; b < c->n_stor; ++b) {
-    const size_t base = (size_t)b * opfk::SG_N * Tp;
-    std::vector<std::pair<size_t, bool>> rows;  // (device index, equality row)
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_E1 * Tp + t, true});
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_E2 * Tp + t, true});
-    rows.push_back({base + opfk::SG_E3 * Tp + 0, true});
-    rows.push_back({base + opfk::SG_E3 * Tp + 1, true});
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_CU * Tp + t, false});
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_CL * Tp + t, false});
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_DU * Tp + t, false});
-    for (int t = 0; t < T; ++t) rows.push_back({base + opfk::SG_DL * Tp + t, false});
-    for (int t = 0; t < Tp; ++t) rows.push_back({base + opfk::SG_SU * Tp + t, false});
-    for (int t = 0; t < Tp; ++t) rows.push_back({base + opfk::SG_SL * Tp + t, false});
-    for (auto &x : rows) v.push_back({2, x.first});
-    for (auto &x : rows) v.push_back({x.second ? -1 : 3, x.first});
+  if (ns) {
+    CK(cudaMemsetAsync(c->P.stor_lam, 0, ns * 4, c->stream));
+    CK(cudaMemsetAsync(c->P.stor_beta, 0, ns * 4, c->stream));
+    CK(cudaMemsetAsync(c->P.stor_rho, 0, c->n_stor * 4, c->stream));
   }
-  return v;
+  return OPF_OK;
 }
 
 // Destination for an export: the caller's device buffer, or a device staging
@@ -1519,7 +1501,7 @@ opf_status opf_get_state(opf_ctx *c, int32_t on_device, const opf_state *dst) {
   float *lines[5] = {dst->p_line, dst->th1, dst->th2, dst->v1, dst->v2};
   DevTmp tmp;
   if (!on_device || (relax && dst->p_dev)) {
-    size_t n = (dst->u ? KNT : 0) + ST;
+    size_t n = (dst->u ? KNT : 0) + ST + (dst->inner ? (size_t)inner_len(c) : 0);
     for (float *x : lines) n += x ? KLT : 0;
     if ((s = alloc_tmp(tmp, n)) != OPF_OK) return s;
   }
@@ -1551,30 +1533,11 @@ opf_status opf_get_state(opf_ctx *c, int32_t on_device, const opf_state *dst) {
       if (lines[j]) CK(cudaMemcpyAsync(lines[j], stg[j], KLT * 4, cudaMemcpyDeviceToHost, c->stream));
     if (dst->u) CK(cudaMemcpyAsync(dst->u, ustg, KNT * 4, cudaMemcpyDeviceToHost, c->stream));
   }
-  if (dst->inner) {
-    auto lay = inner_layout(c);
-    const size_t nr = (size_t)c->n_ramp * opfk::RG_N * c->T, ns = (size_t)c->n_stor * opfk::SG_N * (c->T + 1);
-    std::vector<float> rl(nr), rb(nr), sl(ns), sb(ns);
-    if (nr) {
-      CK(cudaMemcpyAsync(rl.data(), c->P.ramp_lam, nr * 4, cudaMemcpyDeviceToHost, c->stream));
-      CK(cudaMemcpyAsync(rb.data(), c->P.ramp_beta, nr * 4, cudaMemcpyDeviceToHost, c->stream));
-    }
-    if (ns) {
-      CK(cudaMemcpyAsync(sl.data(), c->P.stor_lam, ns * 4, cudaMemcpyDeviceToHost, c->stream));
-      CK(cudaMemcpyAsync(sb.data(), c->P.stor_beta, ns * 4, cudaMemcpyDeviceToHost, c->stream));
-    }
-    CK(cudaStreamSynchronize(c->stream));
-    std::vector<float> flat(lay.size());
-    for (size_t i = 0; i < lay.size(); ++i) {
-      const auto &e = lay[i];
-      flat[i] = e.arr == 0 ? rl[e.idx] : e.arr == 1 ? rb[e.idx] : e.arr == 2 ? sl[e.idx] : e.arr == 3 ? sb[e.idx] : 0.f;
-    }
-    if (on_device) {
-      CK(cudaMemcpyAsync(dst->inner, flat.data(), flat.size() * 4, cudaMemcpyHostToDevice, c->stream));
-      CK(cudaStreamSynchronize(c->stream));
-    } else {
-      std::memcpy(dst->inner, flat.data(), flat.size() * 4);
-    }
+  if (dst->inner && inner_len(c) > 0) {
+    const int64_t n = inner_len(c);
+    float *istg = on_device ? dst->inner : cursor + (dst->u ? KNT : 0);
+    if (opfk_inner_export_launch(c->P, istg, n, c->stream) != 0) return fail(OPF_ECUDA, "export launch failed");
+    if (!on_device) CK(cudaMemcpyAsync(dst->inner, istg, n * 4, cudaMemcpyDeviceToHost, c->stream));
   }
   CK(cudaStreamSynchronize(c->stream));
   return OPF_OK;
@@ -1589,10 +1552,11 @@ opf_status opf_set_state(opf_ctx *c, int32_t on_device, const opf_state *src) {
   if ((s = read_scalars(c, &sc)) != OPF_OK) return s;
   const int cur = (int)(sc.it & 1);
   const float *lines[5] = {src->p_line, src->th1, src->th2, src->v1, src->v2};
-  const float *dsrc[5], *usrc = src->u;
+  const float *dsrc[5], *usrc = src->u, *isrc = src->inner;
+  const int64_t n_inner = src->inner ? inner_len(c) : 0;
   DevTmp tmp;
   if (!on_device) {
-    size_t n = src->u ? KNT : 0;
+    size_t n = (src->u ? KNT : 0) + (size_t)n_inner;
     for (const float *x : lines) n += x ? KLT : 0;
     if ((s = alloc_tmp(tmp, n)) != OPF_OK) return s;
     float *cursor = tmp.p;
@@ -1607,6 +1571,11 @@ opf_status opf_set_state(opf_ctx *c, int32_t on_device, const opf_state *src) {
     if (src->u) {
       CK(cudaMemcpyAsync(cursor, src->u, KNT * 4, cudaMemcpyHostToDevice, c->stream));
       usrc = cursor;
+      cursor += KNT;
+    }
+    if (n_inner > 0) {
+      CK(cudaMemcpyAsync(cursor, src->inner, n_inner * 4, cudaMemcpyHostToDevice, c->stream));
+      isrc = cursor;
     }
   } else {
     for (int j = 0; j < 5; ++j) dsrc[j] = lines[j];
@@ -1619,36 +1588,10 @@ opf_status opf_set_state(opf_ctx *c, int32_t on_device, const opf_state *src) {
   else
     CK(cudaMemsetAsync(c->P.PD, 0, ST * 4, c->stream));
   // inner duals: scaled for the current penalty; factors rebuilt on first use
-  const float rho_dev = (float)(c->Kp_glob * sc.rho_p);
-  const size_t nr = (size_t)c->n_ramp * opfk::RG_N * c->T, ns = (size_t)c->n_stor * opfk::SG_N * (c->T + 1);
-  std::vector<float> rl(nr, 0.f), rb(nr, 0.f), sl(ns, 0.f), sb(ns, 0.f);
-  if (src->inner) {
-    auto lay = inner_layout(c);
-    std::vector<float> flat(lay.size());
-    if (on_device) {
-      CK(cudaMemcpy(flat.data(), src->inner, flat.size() * 4, cudaMemcpyDeviceToHost));
-    } else {
-      std::memcpy(flat.data(), src->inner, flat.size() * 4);
-    }
-    for (size_t i = 0; i < lay.size(); ++i) {
-      const auto &e = lay[i];
-      if (e.arr == 0) rl[e.idx] = flat[i];
-      else if (e.arr == 1) rb[e.idx] = flat[i];
-      else if (e.arr == 2) sl[e.idx] = flat[i];
-      else if (e.arr == 3) sb[e.idx] = flat[i];
-    }
-  }
-  std::vector<float> rr(c->n_ramp, src->inner ? -rho_dev : 0.f), sr(c->n_stor, src->inner ? -rho_dev : 0.f);
-  if (nr) {
-    CK(cudaMemcpyAsync(c->P.ramp_lam, rl.data(), nr * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->P.ramp_beta, rb.data(), nr * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->P.ramp_rho, rr.data(), rr.size() * 4, cudaMemcpyHostToDevice, c->stream));
-  }
-  if (ns) {
-    CK(cudaMemcpyAsync(c->P.stor_lam, sl.data(), ns * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->P.stor_beta, sb.data(), ns * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->P.stor_rho, sr.data(), sr.size() * 4, cudaMemcpyHostToDevice, c->stream));
-  }
+  if ((s = zero_inner(c)) != OPF_OK) return s;
+  if (n_inner > 0 &&
+      opfk_inner_import_launch(c->P, isrc, n_inner, -(float)(c->Kp_glob * sc.rho_p), c->stream) != 0)
+    return fail(OPF_ECUDA, "import launch failed");
   if (opfk_project_v_launch(c->P, cur, c->stream) != 0) return fail(OPF_ECUDA, "project_v launch failed");
   if (opfk_node_average_launch(c->P, cur, c->stream) != 0) return fail(OPF_ECUDA, "node_average launch failed");
   sc.su = 1.0;
@@ -1691,18 +1634,8 @@ opf_status opf_set_state_from_nodes(opf_ctx *c, int32_t on_device, const float *
     return fail(OPF_ECUDA, "start launch failed");
   // device powers and the inner duals from zero (factors rebuilt on first use)
   const size_t ST = (size_t)c->S * c->T;
-  const size_t nr = (size_t)c->n_ramp * opfk::RG_N * c->T, ns = (size_t)c->n_stor * opfk::SG_N * (c->T + 1);
   CK(cudaMemsetAsync(c->P.PD, 0, ST * 4, c->stream));
-  if (nr) {
-    CK(cudaMemsetAsync(c->P.ramp_lam, 0, nr * 4, c->stream));
-    CK(cudaMemsetAsync(c->P.ramp_beta, 0, nr * 4, c->stream));
-    CK(cudaMemsetAsync(c->P.ramp_rho, 0, c->n_ramp * 4, c->stream));
-  }
-  if (ns) {
-    CK(cudaMemsetAsync(c->P.stor_lam, 0, ns * 4, c->stream));
-    CK(cudaMemsetAsync(c->P.stor_beta, 0, ns * 4, c->stream));
-    CK(cudaMemsetAsync(c->P.stor_rho, 0, c->n_stor * 4, c->stream));
-  }
+  if ((s = zero_inner(c)) != OPF_OK) return s;
   if (opfk_node_average_launch(c->P, cur, c->stream) != 0) return fail(OPF_ECUDA, "node_average launch failed");
   sc.su = 1.0;
   sc.sv = 1.0;

@@ -289,6 +289,11 @@ int opfk_batch_enqueue(const opfk::Params *d_params, const int *d_sched, const o
 int opfk_import_launch(const opfk::Params &p, int cur, const float *p_line, const float *th1,
                        const float *th2, const float *v1, const float *v2, const float *u,
                        void *stream);
+// The inner-ADMM state between the device arrays and the caller's layout
+// (device pointers, n = opf_info.inner_len); an import wants the arrays
+// zeroed and sets the penalty its duals are scaled for (rho, negative).
+int opfk_inner_export_launch(const opfk::Params &p, float *out, long long n, void *stream);
+int opfk_inner_import_launch(const opfk::Params &p, const float *in, long long n, float rho, void *stream);
 int opfk_node_average_launch(const opfk::Params &p, int cur, void *stream);
 // Starting state from node rows [T][N][stride] (price / price_scale, angle),
 // caller numbering; u = -price * u_scale

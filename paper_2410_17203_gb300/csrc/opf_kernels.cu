@@ -1977,6 +1977,56 @@ __global__ void import_kernel(Params p, int cur, const float *pl, const float *a
   }
 }
 
+// Entry i of the exported inner-ADMM state (opf_get_info's layout: per
+// ramp-limited generator, then per battery, lambda then beta over the
+// constraint rows): its place in the device arrays, nullptr for a battery's
+// equality rows' beta (always 0).
+__device__ __forceinline__ float *inner_slot(const Params &p, long long i) {
+  const int T = p.T, Tp = T + 1, mr = 4 * T - 2, ms = 8 * T + 4;
+  const long long nr = (long long)p.n_ramp * 2 * mr;
+  if (i < nr) {
+    const int r = (int)(i / (2 * mr));
+    int x = (int)(i - (long long)r * 2 * mr);
+    float *a = x < mr ? p.ramp_lam : p.ramp_beta;
+    if (x >= mr) x -= mr;
+    // rows p <= pmax, -p <= -pmin (T each), ramp up, ramp down (T - 1 each)
+    const int g = x < 2 * T ? x / T : RG_RU + (x - 2 * T) / (T - 1);
+    const int t = x < 2 * T ? x % T : (x - 2 * T) % (T - 1);
+    return a + ((size_t)r * RG_N + g) * T + t;
+  }
+  i -= nr;
+  const int b = (int)(i / (2 * ms));
+  int x = (int)(i - (long long)b * 2 * ms);
+  const bool beta = x >= ms;
+  if (beta) x -= ms;
+  float *a = (beta ? p.stor_beta : p.stor_lam) + (size_t)b * SG_N * Tp;
+  if (x < 2 * T + 2) {   // p + c - delta = 0, soc dynamics (T each), s_1 = 0, s_{T+1} = 0
+    if (beta) return nullptr;
+    return x < 2 * T ? a + (x / T) * Tp + x % T : a + SG_E3 * Tp + (x - 2 * T);
+  }
+  x -= 2 * T + 2;        // limits of c and delta (T each), of s (T + 1 each)
+  return x < 4 * T ? a + (SG_CU + x / T) * Tp + x % T : a + (SG_SU + (x - 4 * T) / Tp) * Tp + (x - 4 * T) % Tp;
+}
+
+__global__ void inner_export_kernel(Params p, float *out, long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const float *s = inner_slot(p, i);
+    out[i] = s ? *s : 0.f;
+  }
+}
+
+// the arrays were zeroed; rho: the penalty the duals are scaled for, negative
+// so that the factors are rebuilt on first use
+__global__ void inner_import_kernel(Params p, const float *in, long long n, float rho) {
+  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long i = i0; i < n; i += (long long)gridDim.x * blockDim.x) {
+    float *s = inner_slot(p, i);
+    if (s) *s = in[i];
+  }
+  for (long long i = i0; i < (long long)p.n_ramp + p.n_stor; i += (long long)gridDim.x * blockDim.x)
+    (i < p.n_ramp ? p.ramp_rho[i] : p.stor_rho[i - p.n_ramp]) = rho;
+}
+
 // A starting state from node rows in the caller's numbering, rows[(t N + n)
 // stride + 0] = price / price_scale and [+ 1] = node angle: u_k = -price /
 // (rho_p (K+1)) in every contingency (prices are -rho_p sum_k u_k), every
@@ -2453,6 +2503,16 @@ int opfk_start_from_nodes_launch(const Params &p, int cur, const float *rows, in
                                  float u_scale, void *stream) {
   start_from_nodes_kernel<<<aux_grid((long long)p.Kp * (p.L + p.N) * p.T), 256, 0, (cudaStream_t)stream>>>(
       p, cur, rows, stride, price_scale, u_scale);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int opfk_inner_export_launch(const Params &p, float *out, long long n, void *stream) {
+  inner_export_kernel<<<aux_grid(n), 256, 0, (cudaStream_t)stream>>>(p, out, n);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int opfk_inner_import_launch(const Params &p, const float *in, long long n, float rho, void *stream) {
+  inner_import_kernel<<<aux_grid(n), 256, 0, (cudaStream_t)stream>>>(p, in, n, rho);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -78,3 +78,35 @@ def test_relaxed_split_launches_equal_one_launch(T):
         np.testing.assert_array_equal(x[k], y[k], err_msg=k)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 7, 24])
+def test_inner_state_round_trip(T):
+    """The inner-ADMM duals through opf_get_state / opf_set_state, host and
+    device buffers: bit for bit the same, zero for a battery's equality rows'
+    beta, and in the layout from which the oracle continues alike."""
+    import torch
+    from paper_2410_17203_gb300 import Solver, opf_get_state, opf_set_state, state_shapes
+    case = make_case(scale_case(40, T, 2, seed=60 + T, stor_per_node=0.1))
+    opts = dict(adapt_every=0, eps=0.0, rho_p=2.0)
+    a, b, c = (Solver(case, opts) for _ in range(3))
+    a.iterate(15)
+    x = a.state()
+    b.set_state(x)
+    np.testing.assert_array_equal(b.state()["inner"], x["inner"])
+    dev = {k: torch.from_numpy(v).cuda() for k, v in x.items()}
+    opf_set_state(c.h, dev, on_device=True)
+    out = {k: torch.full(s, np.nan, dtype=torch.float32, device="cuda") for k, s in state_shapes(c.info).items()}
+    opf_get_state(c.h, on_device=True, out=out)
+    np.testing.assert_array_equal(out["inner"].cpu().numpy(), x["inner"])
+    nr, ns = a.info["n_ramp"] * 2 * (4 * T - 2), 8 * T + 4
+    stor = x["inner"][nr:].reshape(a.info["n_stor"], 2, ns)
+    assert not stor[:, 1, :2 * T + 2].any() and stor[:, 0].any()
+    o = Oracle(case, OracleOptions(**opts))
+    o.load_state(x)
+    o.iterate(3, stop=False)
+    for s in (b, c):
+        s.iterate(3)
+        compare_states(s.state(), o)
+        s.close()
+    a.close()
