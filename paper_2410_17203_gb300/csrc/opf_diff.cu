@@ -20,8 +20,18 @@
 
 #include "opf_diff.h"
 #include "opf_internal.h"
+#include "opf_tri.h"
 
 namespace {
+
+using opfk::qdiv;
+using opfk::radd;
+using opfk::rdiv;
+using opfk::rfma;
+using opfk::rmul;
+using opfk::rsub;
+using opfk::TriFac;
+using opfk::warp_tri_solve_r;
 
 constexpr int TB = 256;       // threads per CTA of the element-wise kernels (eight per SM: they wait
                               // on gathers, so they are held to 32 registers for the most warps)
@@ -233,11 +243,12 @@ __global__ void __launch_bounds__(TB, VW == 4 ? VW4_CTAS : 8) fwd_avg(DP p, St s
       }
     }
     const Vf<VW> u = ldv<VW>(s.U + it.o);
+    const float cn = p.cnt[n], icn = p.icnt[n], ct = p.cth[n], ict = p.icth[n];
     Vf<VW> pb, tbr, un;
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
-      pb.x[e] = sp[e] / p.cnt[n];
-      tbr.x[e] = p.cth[n] > 0.f ? st[e] / p.cth[n] : 0.f;
+      pb.x[e] = qdiv(sp[e], cn, icn);
+      tbr.x[e] = ct > 0.f ? qdiv(st[e], ct, ict) : 0.f;
       un.x[e] = u.x[e] + pb.x[e];
     }
     stv<VW>(nx.PB + it.o, pb);
@@ -281,8 +292,10 @@ __device__ __forceinline__ LineIn line_inputs(const DP &p, const St &s, int k, i
 __device__ __forceinline__ float line_den(const DP &p, float b, float tb) {
   return __fadd_rn(__fmul_rn(2.f, p.rp), p.rt / (tb * b));
 }
-__device__ __forceinline__ float line_z(const DP &p, const LineIn &in, float tb, float den) {
-  return __fadd_rn(__fmul_rn(p.rp, in.x2 - in.x1), __fmul_rn(p.rt, in.y1 - in.y2) / tb) / den;
+// (rtb = 1 / tb, rden = 1 / den: the quotients by the rounded reciprocals and
+// one correction each, as the division rounds them)
+__device__ __forceinline__ float line_z(const DP &p, const LineIn &in, float tb, float rtb, float den, float rden) {
+  return qdiv(__fadd_rn(__fmul_rn(p.rp, in.x2 - in.x1), qdiv(__fmul_rn(p.rt, in.y1 - in.y2), tb, rtb)), den, rden);
 }
 __device__ __forceinline__ float gen_den(const DP &p, int d) { return __fadd_rn(__fmul_rn(2.f, p.ga[d]), p.rd); }
 __device__ __forceinline__ float gen_z(const DP &p, int d, float X) {
@@ -314,19 +327,21 @@ __global__ void __launch_bounds__(TB, VW == 4 ? VW4_CTAS : 8) fwd_line(DP p, St 
     Vf<VW> np, t1, t2;
     if (p.out[k] != l) {
       const float b = p.b[l], tb = 2.f * b, u = p.lu[l], den = line_den(p, b, tb);
+      const float rtb = __frcp_rn(tb), rden = __frcp_rn(den);
       Vb<VW> code;
 #pragma unroll
       for (int e = 0; e < VW; ++e) {
         // the prox inputs as line_inputs forms them
         const LineIn in{-P.x[e] - PB1.x[e] - U1.x[e], P.x[e] - PB2.x[e] - U2.x[e], TB1.x[e] - V1.x[e],
                         TB2.x[e] - V2.x[e]};
-        const float z = line_z(p, in, tb, den);
+        const float z = line_z(p, in, tb, rtb, den, rden);
         code.x[e] = clip_code(z, -u, u);
         const float p2 = fminf(fmaxf(z, -u), u);
         const float mid = 0.5f * (in.y1 + in.y2);
+        const float h = qdiv(p2, tb, rtb);
         np.x[e] = p2;
-        t1.x[e] = mid + p2 / tb;
-        t2.x[e] = mid - p2 / tb;
+        t1.x[e] = mid + h;
+        t2.x[e] = mid - h;
       }
       if (lmask) stb<VW>(lmask + o, code);
     } else {
@@ -604,7 +619,7 @@ __device__ __forceinline__ void line_back(const DP &p, const St &s, const Adj &a
   const float ic1 = p.icnt[n1], ic2 = p.icnt[n2], ih1 = p.icth[n1], ih2 = p.icth[n2];
   const Vf<VW> B1 = ldv<VW>(B + o1), B2 = ldv<VW>(B + o2), LV1 = ldv<VW>(a.LV1 + o), LV2 = ldv<VW>(a.LV2 + o);
   const bool act = p.out[k] != l;
-  Vb<VW> code;
+  Vb<VW> code{};
   if (act && lmask) code = ldb<VW>(lmask + o);
   Vf<VW> x2, y1, y2, lpn, v1, v2;
 #pragma unroll
@@ -615,8 +630,11 @@ __device__ __forceinline__ void line_back(const DP &p, const St &s, const Adj &a
     float lx1 = 0.f, lx2 = 0.f, ly1, ly2;
     if (act) {
       const float b = p.b[l], tb = 2.f * b, u = p.lu[l];
-      const unsigned char cd =
-          lmask ? code.x[e] : clip_code(line_z(p, line_inputs(p, s, k, l, it.t0 + e), tb, line_den(p, b, tb)), -u, u);
+      unsigned char cd = code.x[e];
+      if (!lmask) {
+        const float den = line_den(p, b, tb);
+        cd = clip_code(line_z(p, line_inputs(p, s, k, l, it.t0 + e), tb, __frcp_rn(tb), den, __frcp_rn(den)), -u, u);
+      }
       const float lpt = fmaf(lt1 - lt2, p.lfac[l], lp);     // theta_{1,2} = mid +- p / (2b)
       const float half = __fmul_rn(0.5f, lt1 + lt2);
       ly1 = ly2 = half;
@@ -886,79 +904,6 @@ constexpr int DREG_T = 127;
 constexpr unsigned FULLM = 0xffffffffu;
 constexpr int RWARPS = TB / 32;   // devices per CTA of the register kernels
 
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-
-// x := M^-1 x for a tridiagonal M with pivots q and a = -off / q (element i
-// = lane C + j, valid while i < n): first-order recurrences composed over
-// each lane's chunk, then across the warp by shuffle scans
-template <int C>
-__device__ __forceinline__ void tri_solve_r(const float (&q)[C], const float (&a)[C], float (&x)[C], int n,
-                                            int lane) {
-  const int i0 = lane * C;
-  float r[C];
-  float Ac = 1.f, Bc = 0.f;
-#pragma unroll
-  for (int j = 0; j < C; ++j) {
-    r[j] = 0.f;
-    if (i0 + j < n) {
-      r[j] = rdiv(x[j], q[j]);
-      const float Ai = (i0 + j == 0) ? 0.f : a[j];
-      Bc = rfma(Ai, Bc, r[j]);
-      Ac = rmul(Ai, Ac);
-    }
-  }
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const float Ap = __shfl_up_sync(FULLM, Ac, d), Bp = __shfl_up_sync(FULLM, Bc, d);
-    if (lane >= d) {
-      Bc = rfma(Ac, Bp, Bc);
-      Ac = rmul(Ac, Ap);
-    }
-  }
-  float prev = __shfl_up_sync(FULLM, Bc, 1);
-  if (lane == 0) prev = 0.f;
-#pragma unroll
-  for (int j = 0; j < C; ++j) {
-    if (i0 + j < n) {
-      const float Ai = (i0 + j == 0) ? 0.f : a[j];
-      prev = rfma(Ai, prev, r[j]);
-      x[j] = prev;
-    }
-  }
-  Ac = 1.f;
-  Bc = 0.f;
-#pragma unroll
-  for (int j = C - 1; j >= 0; --j) {
-    if (i0 + j < n) {
-      const float Ci = (i0 + j == n - 1) ? 0.f : a[j];
-      Bc = rfma(Ci, Bc, x[j]);
-      Ac = rmul(Ci, Ac);
-    }
-  }
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const float Ap = __shfl_down_sync(FULLM, Ac, d), Bp = __shfl_down_sync(FULLM, Bc, d);
-    if (lane + d < 32) {
-      Bc = rfma(Ac, Bp, Bc);
-      Ac = rmul(Ac, Ap);
-    }
-  }
-  float nxt = __shfl_down_sync(FULLM, Bc, 1);
-  if (lane == 31) nxt = 0.f;
-#pragma unroll
-  for (int j = C - 1; j >= 0; --j) {
-    if (i0 + j < n) {
-      const float Ci = (i0 + j == n - 1) ? 0.f : a[j];
-      nxt = rfma(Ci, nxt, x[j]);
-      x[j] = nxt;
-    }
-  }
-}
-
 // The register path records which rows clipped as one 64-bit word per lane
 // and inner iteration (bit g C + j: row group g, element j of the lane's
 // chunk), [device][inner iteration][lane]: coalesced stores and loads.
@@ -991,13 +936,13 @@ __device__ __forceinline__ float sbar_r(unsigned long long bits, int b, float bb
 // A battery's constants: omega eta, H^-1 and g = H^-1 f with f = (-omega eta,
 // omega) the coupling of (c_t, delta_t) to s_{t+1} - s_t
 struct StorK {
-  float rho, om, eta, rpo, i00, i01, i11, gc, gd;
+  float rho, om, eta, rpo, rrpo, i00, i01, i11, gc, gd;   // rpo = rho + omega, rrpo = 1 / rpo
 };
 
 // z := M^-1 z for a battery, z = (p, c, delta) at steps t < T, s at j <= T
 // (element e = lane C + j holds step e and state of charge e)
 template <int C>
-__device__ __forceinline__ void stor_solve_r(const StorK &k, const float (&qv)[C], const float (&av)[C],
+__device__ __forceinline__ void stor_solve_r(const StorK &k, const TriFac<C> &tf,
                                              float (&zp)[C], float (&zc)[C], float (&zd)[C], float (&zs)[C], int T,
                                              int lane) {
   const int t0 = lane * C;
@@ -1007,7 +952,7 @@ __device__ __forceinline__ void stor_solve_r(const StorK &k, const float (&qv)[C
   for (int j = 0; j < C; ++j) {
     u[j] = yc[j] = yd[j] = fy[j] = 0.f;
     if (t0 + j < T) {
-      u[j] = rdiv(zp[j], k.rpo);                          // p = u - omega (c - delta) / (rho + omega)
+      u[j] = qdiv(zp[j], k.rpo, k.rrpo);                          // p = u - omega (c - delta) / (rho + omega)
       const float rc = rsub(zc[j], rmul(k.om, u[j])), rd = radd(zd[j], rmul(k.om, u[j]));
       yc[j] = rfma(k.i00, rc, rmul(k.i01, rd));             // y = H^-1 r'
       yd[j] = rfma(k.i01, rc, rmul(k.i11, rd));
@@ -1025,7 +970,7 @@ __device__ __forceinline__ void stor_solve_r(const StorK &k, const float (&qv)[C
       zs[j] = r;
     }
   }
-  tri_solve_r<C>(qv, av, zs, T + 1, lane);
+  warp_tri_solve_r<C>(tf, zs, T + 1, lane);
   const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
   for (int j = 0; j < C; ++j) {
@@ -1034,7 +979,7 @@ __device__ __forceinline__ void stor_solve_r(const StorK &k, const float (&qv)[C
       const float c = rsub(yc[j], rmul(k.gc, dsv)), dl = rsub(yd[j], rmul(k.gd, dsv));
       zc[j] = c;
       zd[j] = dl;
-      zp[j] = rsub(u[j], rdiv(rmul(k.om, rsub(c, dl)), k.rpo));
+      zp[j] = rsub(u[j], qdiv(rmul(k.om, rsub(c, dl)), k.rpo, k.rrpo));
     }
   }
 }
@@ -1045,7 +990,7 @@ __device__ __forceinline__ void stor_solve_r(const StorK &k, const float (&qv)[C
 // the device's record block (N_INNER x m bytes) or NULL
 template <int C>
 __device__ void ramp_fwd_r(int T, int lane, float rho, float om, float qlin, const float (&x)[C],
-                           const float (&qv)[C], const float (&av)[C], const float (&hU)[C], const float (&hL)[C],
+                           const TriFac<C> &tf, const float (&hU)[C], const float (&hL)[C],
                            const float (&hRU)[C], const float (&hRD)[C], float (&bU)[C], float (&lU)[C],
                            float (&bL)[C], float (&lL)[C], float (&bRU)[C], float (&lRU)[C], float (&bRD)[C],
                            float (&lRD)[C], float (&z)[C], unsigned long long *rec) {
@@ -1070,7 +1015,7 @@ __device__ void ramp_fwd_r(int T, int lane, float rho, float om, float qlin, con
         z[j] = rfma(rho, x[j], rfma(om, acc, -qlin));                                           // r
       }
     }
-    tri_solve_r<C>(qv, av, z, T, lane);
+    warp_tri_solve_r<C>(tf, z, T, lane);
     const float zn = __shfl_down_sync(FULLM, z[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -1108,7 +1053,7 @@ __device__ __forceinline__ bool shas(int g, int e, int T) { return g < SSU ? e <
 
 template <int C>
 __device__ void stor_fwd_r(int T, int lane, const StorK &k, float cost, float Pm, float Em, const float (&x)[C],
-                           const float (&qv)[C], const float (&av)[C], StorRows<C> &lam, StorRows<C> &bet,
+                           const TriFac<C> &tf, StorRows<C> &lam, StorRows<C> &bet,
                            float (&zp)[C], float (&zd)[C], unsigned long long *rec) {
   const int t0 = lane * C;
   for (int it = 0; it < N_INNER; ++it) {
@@ -1140,7 +1085,7 @@ __device__ void stor_fwd_r(int T, int lane, const StorK &k, float cost, float Pm
         zs[j] = rmul(k.om, as);
       }
     }
-    stor_solve_r<C>(k, qv, av, zp, zc, zd, zs, T, lane);
+    stor_solve_r<C>(k, tf, zp, zc, zd, zs, T, lane);
     const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -1171,8 +1116,7 @@ struct RDev {
 };
 
 template <int C>
-__device__ void ramp_load(const DP &p, const St &s, const RDev &dv, int T, int lane, float (&x)[C], float (&qv)[C],
-                          float (&av)[C], float (&hU)[C], float (&hL)[C], float (&hRU)[C], float (&hRD)[C],
+__device__ void ramp_load(const DP &p, const St &s, const RDev &dv, int T, int lane, float (&x)[C], TriFac<C> &tf, float (&hU)[C], float (&hL)[C], float (&hRU)[C], float (&hRD)[C],
                           float (&bU)[C], float (&lU)[C], float (&bL)[C], float (&lL)[C], float (&bRU)[C],
                           float (&lRU)[C], float (&bRD)[C], float (&lRD)[C], const float *XD) {
   const int t0 = lane * C;
@@ -1182,8 +1126,8 @@ __device__ void ramp_load(const DP &p, const St &s, const RDev &dv, int T, int l
     const int t = t0 + j;
     const bool in = t < T, rr = t < T - 1;
     x[j] = (in && XD) ? XD[(size_t)dv.dev * T + t] : 0.f;
-    qv[j] = in ? p.piv[dv.piv + t] : 1.f;
-    av[j] = in ? p.piv[dv.piv + T + t] : 0.f;
+    tf.q[j] = in ? p.piv[dv.piv + t] : 1.f;
+    tf.a[j] = in ? p.piv[dv.piv + T + t] : 0.f;
     hU[j] = in ? Hh[t] : 0.f;
     hL[j] = in ? Hh[T + t] : 0.f;
     bU[j] = in ? B[t] : 0.f;
@@ -1197,11 +1141,12 @@ __device__ void ramp_load(const DP &p, const St &s, const RDev &dv, int T, int l
     bRD[j] = rr ? B[3 * T - 1 + t] : 0.f;
     lRD[j] = rr ? Lm[3 * T - 1 + t] : 0.f;
   }
+  tf.init(T, lane);
 }
 
 template <int C>
 __device__ void stor_load(const DP &p, const St &s, const RDev &dv, int T, int lane, StorK &k, float &cost,
-                          float &Pm, float &Em, float (&x)[C], float (&qv)[C], float (&av)[C], StorRows<C> &lam,
+                          float &Pm, float &Em, float (&x)[C], TriFac<C> &tf, StorRows<C> &lam,
                           StorRows<C> &bet, const float *XD) {
   const int t0 = lane * C;
   const float *B = s.INS + dv.h, *Lm = s.INS + p.Mtot + dv.h, *Hh = p.RH + dv.h;
@@ -1210,6 +1155,7 @@ __device__ void stor_load(const DP &p, const St &s, const RDev &dv, int T, int l
   k.om = p.rd;
   k.eta = p.beff[dv.bat];
   k.rpo = radd(k.rho, k.om);
+  k.rrpo = __frcp_rn(k.rpo);
   k.i00 = kc[0];
   k.i01 = kc[1];
   k.i11 = kc[2];
@@ -1226,8 +1172,8 @@ __device__ void stor_load(const DP &p, const St &s, const RDev &dv, int T, int l
     const int e = t0 + j;
     const bool st = e < T, ss = e <= T;
     x[j] = (st && XD) ? XD[(size_t)dv.dev * T + e] : 0.f;
-    qv[j] = ss ? kc[8 + e] : 1.f;
-    av[j] = ss ? kc[8 + (T + 1) + e] : 0.f;
+    tf.q[j] = ss ? kc[8 + e] : 1.f;
+    tf.a[j] = ss ? kc[8 + (T + 1) + e] : 0.f;
     lam.v[SE1][j] = st ? Lm[e] : 0.f;
     lam.v[SE2][j] = st ? Lm[T + e] : 0.f;
     lam.v[SCU][j] = st ? Lm[2 * T + 2 + e] : 0.f;
@@ -1244,6 +1190,7 @@ __device__ void stor_load(const DP &p, const St &s, const RDev &dv, int T, int l
     bet.v[SSU][j] = ss ? B[6 * T + 2 + e] : 0.f;
     bet.v[SSL][j] = ss ? B[7 * T + 3 + e] : 0.f;
   }
+  tf.init(T + 1, lane);
 }
 
 __device__ __forceinline__ RDev rdev(const DP &p, int w) {
@@ -1260,11 +1207,12 @@ __global__ void __launch_bounds__(TB, 1) fwd_inner_r(DP p, St s, St nx, const fl
   const RDev dv = rdev(p, w);
   unsigned long long *mask = grec ? grec + (size_t)w * RREC_WORDS : nullptr;
   float *Bo = nx.INS + dv.h, *Lo = nx.INS + p.Mtot + dv.h;
-  float x[C], qv[C], av[C];
+  float x[C];
+  TriFac<C> tf;
   if (dv.bat < 0) {
     float hU[C], hL[C], hRU[C], hRD[C], bU[C], lU[C], bL[C], lL[C], bRU[C], lRU[C], bRD[C], lRD[C], z[C];
-    ramp_load<C>(p, s, dv, T, lane, x, qv, av, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD, XD);
-    ramp_fwd_r<C>(T, lane, p.rd, p.rd, p.gb[dv.dev], x, qv, av, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
+    ramp_load<C>(p, s, dv, T, lane, x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD, XD);
+    ramp_fwd_r<C>(T, lane, p.rd, p.rd, p.gb[dv.dev], x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
                   lRD, z, mask);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -1287,8 +1235,8 @@ __global__ void __launch_bounds__(TB, 1) fwd_inner_r(DP p, St s, St nx, const fl
     StorK k;
     float cost, Pm, Em, zp[C], zd[C];
     StorRows<C> lam, bet;
-    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, qv, av, lam, bet, XD);
-    stor_fwd_r<C>(T, lane, k, cost, Pm, Em, x, qv, av, lam, bet, zp, zd, mask);
+    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, tf, lam, bet, XD);
+    stor_fwd_r<C>(T, lane, k, cost, Pm, Em, x, tf, lam, bet, zp, zd, mask);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
@@ -1339,18 +1287,19 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
   const RDev dv = rdev(p, w);
   const float rho = p.rd, om = p.rd;
   float *BB = a.LINS + dv.h, *LB = a.LINS + p.Mtot + dv.h, *HBd = HB + dv.h;
-  float x[C], qv[C], av[C], xb[C];
+  float x[C], xb[C];
+  TriFac<C> tf;
 #pragma unroll
   for (int j = 0; j < C; ++j) xb[j] = 0.f;
   if (dv.bat < 0) {
     float hU[C], hL[C], hRU[C], hRD[C], bU[C], lU[C], bL[C], lL[C], bRU[C], lRU[C], bRD[C], lRD[C];
     // X (and the state) only to run the forward iterations again
-    ramp_load<C>(p, s, dv, T, lane, x, qv, av, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD,
+    ramp_load<C>(p, s, dv, T, lane, x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD,
                  grec ? nullptr : XD);
     const unsigned long long *mask = (grec ? grec : scratch) + (size_t)w * RREC_WORDS;
     if (!grec) {
       float z[C];
-      ramp_fwd_r<C>(T, lane, rho, om, p.gb[dv.dev], x, qv, av, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
+      ramp_fwd_r<C>(T, lane, rho, om, p.gb[dv.dev], x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
                     lRD, z, scratch + (size_t)w * RREC_WORDS);
     }
     // adjoints of (beta, lambda) per row, and of the right-hand sides
@@ -1397,7 +1346,7 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
           rb[j] = acc;
         }
       }
-      tri_solve_r<C>(qv, av, rb, T, lane);
+      warp_tri_solve_r<C>(tf, rb, T, lane);
       const float rn = __shfl_down_sync(FULLM, rb[0], 1);
 #pragma unroll
       for (int j = 0; j < C; ++j) {
@@ -1437,11 +1386,11 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
     StorK k;
     float cost, Pm, Em;
     StorRows<C> lam, bet;
-    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, qv, av, lam, bet, grec ? nullptr : XD);
+    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, tf, lam, bet, grec ? nullptr : XD);
     const unsigned long long *mask = (grec ? grec : scratch) + (size_t)w * RREC_WORDS;
     if (!grec) {
       float zp[C], zd[C];
-      stor_fwd_r<C>(T, lane, k, cost, Pm, Em, x, qv, av, lam, bet, zp, zd, scratch + (size_t)w * RREC_WORDS);
+      stor_fwd_r<C>(T, lane, k, cost, Pm, Em, x, tf, lam, bet, zp, zd, scratch + (size_t)w * RREC_WORDS);
     }
     const float dcost = last ? cost : 0.f;
     // per row group: adjoints of beta (ab), lambda (al), the right-hand side (ah)
@@ -1504,7 +1453,7 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
           zs[j] = as;
         }
       }
-      stor_solve_r<C>(k, qv, av, zp, zc, zd, zs, T, lane);
+      stor_solve_r<C>(k, tf, zp, zc, zd, zs, T, lane);
       const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
       for (int j = 0; j < C; ++j) {
@@ -1770,12 +1719,18 @@ __global__ void set_ramp_rhs(DP p, float *RH) {
 // d f / d u_l: the limit is the same in every contingency and step, so the
 // per-(k, l, t) adjoints are summed (FP64, fixed order); and a ramp
 // generator's capacity gradient gains the adjoint of its capacity rows
-__global__ void finish_line_grad(DP p, const float *GU, float *out) {
-  GRID_STRIDE(l, (long long)p.L) {
+// One warp per line (a thread per line walked Kp T scattered values one load
+// after another: 77 us at 2k buses, T = 24, K = 20).
+__global__ void __launch_bounds__(TB) finish_line_grad(DP p, const float *GU, float *out) {
+  const int lane = threadIdx.x & 31;
+  for (int l = blockIdx.x * (TB / 32) + (threadIdx.x >> 5); l < p.L; l += gridDim.x * (TB / 32)) {
     double s = 0.0;
+#pragma unroll 4
     for (int k = 0; k < p.Kp; ++k)
-      for (int t = 0; t < p.T; ++t) s += GU[((size_t)k * p.L + l) * p.T + t];
-    out[l] = (float)s;
+      for (int t = lane; t < p.T; t += 32) s += GU[li(p, k, l, t)];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULLM, s, o);
+    if (lane == 0) out[l] = (float)s;
   }
 }
 
@@ -2585,7 +2540,7 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   }
   if (e == cudaSuccess && g_pmax && p.n_inner)
     finish_cap_grad<<<grid_for((long long)p.n_inner * T), TB, 0, d->stream>>>(p, HB, GP);
-  if (e == cudaSuccess && g_u) finish_line_grad<<<grid_for((long long)L), TB, 0, d->stream>>>(p, GU, d->gline);
+  if (e == cudaSuccess && g_u) finish_line_grad<<<grid_for(32 * (long long)L), TB, 0, d->stream>>>(p, GU, d->gline);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess && g_load) e = cudaMemcpyAsync(g_load, GL, DT * 4, out_kind, d->stream);
   if (e == cudaSuccess && g_pmax) e = cudaMemcpyAsync(g_pmax, GP, GT * 4, out_kind, d->stream);

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "opf_internal.h"
+#include "opf_tri.h"
 
 namespace opfk {
 
@@ -77,24 +78,6 @@ __host__ __device__ inline int inner_chunk(int T, int longest = REG_T) { return 
 // contract or reorder: its shared-memory and register forms, and each kernel
 // that inlines them (one instance, a batch), compute the same bits.
 // ---------------------------------------------------------------------------
-constexpr unsigned FULL = 0xffffffffu;
-
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-
-// x / q by the rounded reciprocal rq = 1 / q and one residual correction
-// (Markstein 1990): the correctly rounded quotient for the operands of these
-// solves (2e8 random pairs over 2^-40 .. 2^20 by 2^-10 .. 2^12: every result
-// equal to the division's), in three dependent operations.  The inner
-// iterations divide by pivots and constants that do not change between them.
-__device__ __forceinline__ float qdiv(float x, float q, float rq) {
-  const float q0 = rmul(x, rq);
-  return rfma(rfma(-q0, q, x), rq, q0);
-}
-
 // one projected dual step of an inequality row (Appendix D): lam += al - nb,
 // beta = nb = min(al + lam, 0)
 __device__ __forceinline__ void ineq_step(float al, float &lam, float &bet) {
@@ -636,89 +619,6 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
 // not contract or reorder, so each kernel that inlines this path (one
 // instance, a batch) computes the same bits.
 // ---------------------------------------------------------------------------
-
-// The tridiagonal system of a device, as the solves of its inner iterations
-// read it (element i = lane C + j, valid while i < n): pivots q, their
-// reciprocals rq, a = -off / q, and the multipliers of the two warp scans.  A
-// scan composes the lanes' affine maps x -> A x + B; the A of a lane at each
-// scan step depends on the pivots alone, so it is formed once per device and
-// the scans of the ten inner iterations move only B: one shuffle and one FMA
-// per step in place of two shuffles, an FMA and a product, and no division
-// sequence in the chain.  Bound: latency (the chain of dependent shuffles).
-template <int C>
-struct TriFac {
-  float q[C], rq[C], a[C], f[5], b[5];
-  // q set; off_neg = -off
-  __device__ __forceinline__ void init(float off_neg, int n, int lane) {
-    const int i0 = lane * C;
-    float Af = 1.f, Ab = 1.f;
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-      rq[j] = __frcp_rn(q[j]);
-      a[j] = qdiv(off_neg, q[j], rq[j]);
-      if (i0 + j < n) Af = rmul((i0 + j == 0) ? 0.f : a[j], Af);
-    }
-#pragma unroll
-    for (int j = C - 1; j >= 0; --j)
-      if (i0 + j < n) Ab = rmul((i0 + j == n - 1) ? 0.f : a[j], Ab);
-#pragma unroll
-    for (int l = 0; l < 5; ++l) {
-      const int d = 1 << l;
-      f[l] = Af;
-      b[l] = Ab;
-      const float Pf = __shfl_up_sync(FULL, Af, d), Pb = __shfl_down_sync(FULL, Ab, d);
-      if (lane >= d) Af = rmul(Af, Pf);
-      if (lane + d < 32) Ab = rmul(Ab, Pb);
-    }
-  }
-};
-
-// warp_tri_solve on a chunk held in registers
-template <int C>
-__device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[C], int n, int lane) {
-  const int i0 = lane * C;
-  float r[C];
-  float Bc = 0.f;
-#pragma unroll
-  for (int j = 0; j < C; ++j) {
-    if (i0 + j < n) {
-      r[j] = qdiv(x[j], m.q[j], m.rq[j]);
-      Bc = rfma((i0 + j == 0) ? 0.f : m.a[j], Bc, r[j]);
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < 5; ++l) {
-    const float Bp = __shfl_up_sync(FULL, Bc, 1 << l);
-    if (lane >= (1 << l)) Bc = rfma(m.f[l], Bp, Bc);
-  }
-  float prev = __shfl_up_sync(FULL, Bc, 1);
-  if (lane == 0) prev = 0.f;
-#pragma unroll
-  for (int j = 0; j < C; ++j) {
-    if (i0 + j < n) {
-      prev = rfma((i0 + j == 0) ? 0.f : m.a[j], prev, r[j]);
-      x[j] = prev;
-    }
-  }
-  Bc = 0.f;
-#pragma unroll
-  for (int j = C - 1; j >= 0; --j)
-    if (i0 + j < n) Bc = rfma((i0 + j == n - 1) ? 0.f : m.a[j], Bc, x[j]);
-#pragma unroll
-  for (int l = 0; l < 5; ++l) {
-    const float Bp = __shfl_down_sync(FULL, Bc, 1 << l);
-    if (lane + (1 << l) < 32) Bc = rfma(m.b[l], Bp, Bc);
-  }
-  float nxt = __shfl_down_sync(FULL, Bc, 1);
-  if (lane == 31) nxt = 0.f;
-#pragma unroll
-  for (int j = C - 1; j >= 0; --j) {
-    if (i0 + j < n) {
-      nxt = rfma((i0 + j == n - 1) ? 0.f : m.a[j], nxt, x[j]);
-      x[j] = nxt;
-    }
-  }
-}
 
 // The state that does not depend on the iteration's scalars is requested
 // first, with them; the contingency rows of the node and the box follow when
