@@ -125,24 +125,6 @@ constexpr int KL = 8;
 
 __device__ __forceinline__ unsigned group_mask() { return 0xFFu << ((threadIdx.x & 31) & ~(KL - 1)); }
 
-// sum over the contingencies of V (and W, when not NULL) at node n, step t,
-// split over the group's lanes (lane j = threadIdx.x % KL)
-__device__ __forceinline__ float ksum(const DP &p, const float *V, const float *W, int n, int t) {
-  const int j = threadIdx.x & (KL - 1);
-  float s = 0.f;
-  if (W) {
-#pragma unroll 3
-    for (int k = j; k < p.Kp; k += KL) s += V[ni(p, k, n, t)] + W[ni(p, k, n, t)];
-  } else {
-#pragma unroll 3
-    for (int k = j; k < p.Kp; k += KL) s += V[ni(p, k, n, t)];
-  }
-  const unsigned gm = group_mask();
-#pragma unroll
-  for (int o = KL / 2; o > 0; o >>= 1) s += __shfl_xor_sync(gm, s, o);
-  return s;
-}
-
 // ---------------------------------------------------------------------------
 // forward (Section 3.2)
 // ---------------------------------------------------------------------------
@@ -358,9 +340,50 @@ __global__ void __launch_bounds__(TB, VW == 4 ? VW4_CTAS : 8) fwd_line(DP p, St 
   }
 }
 
-// a device's prox input X = p_d - avg_k(pbar + u) (every lane of the group)
-__device__ __forceinline__ float dev_x(const DP &p, const St &s, int d, int t) {
-  return s.PD[(size_t)d * p.T + t] - ksum(p, s.PB, s.U, p.dnode[d], t) / (float)p.Kp;
+// The device kernels take VW steps per lane group: the sum over contingencies
+// of V (and W, when not NULL), split over the group's lanes (lane j =
+// threadIdx.x % KL), and a device's prox input X = p_d - avg_k(pbar + u), at
+// steps t0 .. t0 + VW - 1; each step is summed in the same order whatever VW
+template <int VW>
+__device__ __forceinline__ Vf<VW> ksumv(const DP &p, const float *V, const float *W, int n, int t0) {
+  const int j = threadIdx.x & (KL - 1);
+  Vf<VW> s;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) s.x[e] = 0.f;
+#pragma unroll 3
+  for (int k = j; k < p.Kp; k += KL) {
+    const Vf<VW> v = ldv<VW>(V + ni(p, k, n, t0));
+    if (W) {
+      const Vf<VW> w = ldv<VW>(W + ni(p, k, n, t0));
+#pragma unroll
+      for (int e = 0; e < VW; ++e) s.x[e] += v.x[e] + w.x[e];
+    } else {
+#pragma unroll
+      for (int e = 0; e < VW; ++e) s.x[e] += v.x[e];
+    }
+  }
+  const unsigned gm = group_mask();
+#pragma unroll
+  for (int o = KL / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int e = 0; e < VW; ++e) s.x[e] += __shfl_xor_sync(gm, s.x[e], o);
+  return s;
+}
+template <int VW>
+__device__ __forceinline__ Vf<VW> dev_xv(const DP &p, const St &s, int d, int t0) {
+  const Vf<VW> pd = ldv<VW>(s.PD + (size_t)d * p.T + t0), k = ksumv<VW>(p, s.PB, s.U, p.dnode[d], t0);
+  Vf<VW> r;
+#pragma unroll
+  for (int e = 0; e < VW; ++e) r.x[e] = pd.x[e] - k.x[e] / (float)p.Kp;
+  return r;
+}
+// device item i of a [S][T / VW] field: device d, first step t0, offset
+// d T + t0 = i VW
+template <int VW>
+__device__ __forceinline__ void dev_item(unsigned i, int T, int &d, int &t0) {
+  const unsigned TV = (unsigned)(T / VW);
+  d = (int)(i / TV);
+  t0 = (int)(i - (unsigned)d * TV) * VW;
 }
 
 // the HVDC partner of terminal d (its index), or -1
@@ -375,42 +398,73 @@ __device__ __forceinline__ int hvdc_partner(const DP &p, int d) {
 // evaluates its link's prox p2 = clip((x2 - x1)/2, -u, u), p1 = -p2.
 // dmask (optional): the iteration's record of where each closed-form
 // device's unclipped power lay
-__global__ void __launch_bounds__(TB, 8) fwd_dev(DP p, St s, St nx, float *XD, unsigned char *dmask) {
-  GROUP_STRIDE(i, (long long)p.S * p.T) {
-    const int d = (int)(i / (unsigned)p.T), t = (int)(i - (unsigned)d * (unsigned)p.T), d2 = hvdc_partner(p, d);
-    const float X = dev_x(p, s, d, t), Xo = d2 < 0 ? 0.f : dev_x(p, s, d2, t);
+// (XD NULL: the inner-ADMM devices form theirs themselves).
+template <int VW>
+__device__ __forceinline__ void closed_part(const DP &p, const St &s, const St &nx, float *XD, unsigned char *dmask,
+                                            unsigned bid, unsigned nb) {
+  GROUP_STRIDE_B(i, (long long)p.S * (p.T / VW), bid, nb) {
+    int d, t0;
+    dev_item<VW>(i, p.T, d, t0);
+    const int kind = p.kind[d];
+    if (kind == 1 && !XD) continue;
+    const int d2 = hvdc_partner(p, d);
+    const Vf<VW> X = dev_xv<VW>(p, s, d, t0);
+    Vf<VW> Xo{};
+    if (d2 >= 0) Xo = dev_xv<VW>(p, s, d2, t0);
     if (threadIdx.x & (KL - 1)) continue;   // the group's first lane writes
-    if (p.kind[d] == 1) {
-      XD[i] = X;
+    const size_t o0 = (size_t)i * VW;
+    Vf<VW> r;
+    Vb<VW> code;
+    bool mask = dmask != nullptr;
+    if (kind == 1) {
+      stv<VW>(XD + o0, X);
       continue;
     }
-    if (p.kind[d] == 2) {
-      const int e = d - (p.G + p.D + p.B), h = e >> 1;
-      const float x1 = (e & 1) ? Xo : X, x2 = (e & 1) ? X : Xo;
-      const float z = 0.5f * (x2 - x1), u = p.hvdc_u[h];
-      if (dmask) dmask[i] = clip_code(z, -u, u);
-      const float f = fminf(fmaxf(z, -u), u);
-      nx.PD[i] = (e & 1) ? f : -f;
-      continue;
-    }
-    float r;
-    if (d < p.G) {
-      const float z = gen_z(p, d, X);
-      if (dmask) dmask[i] = clip_code(z, p.gpmin[i], p.gpmax[i]);
-      r = fminf(fmaxf(z, p.gpmin[i]), p.gpmax[i]);
+    if (kind == 2) {
+      const int e2 = d - (p.G + p.D + p.B), h = e2 >> 1;
+      const float u = p.hvdc_u[h];
+#pragma unroll
+      for (int e = 0; e < VW; ++e) {
+        const float x1 = (e2 & 1) ? Xo.x[e] : X.x[e], x2 = (e2 & 1) ? X.x[e] : Xo.x[e];
+        const float z = 0.5f * (x2 - x1);
+        code.x[e] = clip_code(z, -u, u);
+        const float f = fminf(fmaxf(z, -u), u);
+        r.x[e] = (e2 & 1) ? f : -f;
+      }
+    } else if (d < p.G) {
+      const Vf<VW> lo = ldv<VW>(p.gpmin + o0), hi = ldv<VW>(p.gpmax + o0);
+#pragma unroll
+      for (int e = 0; e < VW; ++e) {
+        const float z = gen_z(p, d, X.x[e]);
+        code.x[e] = clip_code(z, lo.x[e], hi.x[e]);
+        r.x[e] = fminf(fmaxf(z, lo.x[e]), hi.x[e]);
+      }
     } else {
-      const int e = d - p.G;
-      const size_t o = (size_t)e * p.T + t;
-      if (p.voll[e] < 0.f) {
-        r = -p.load_p[o];
+      const int l = d - p.G;
+      const Vf<VW> P = ldv<VW>(p.load_p + (size_t)l * p.T + t0);
+      if (p.voll[l] < 0.f) {
+        mask = false;
+#pragma unroll
+        for (int e = 0; e < VW; ++e) r.x[e] = -P.x[e];
       } else {
-        const float z = load_z(p, e, X);
-        if (dmask) dmask[i] = clip_code(z, -p.load_p[o], 0.f);
-        r = fminf(fmaxf(z, -p.load_p[o]), 0.f);
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+          const float z = load_z(p, l, X.x[e]);
+          code.x[e] = clip_code(z, -P.x[e], 0.f);
+          r.x[e] = fminf(fmaxf(z, -P.x[e]), 0.f);
+        }
       }
     }
-    nx.PD[i] = r;
+    if (mask) stb<VW>(dmask + o0, code);
+    stv<VW>(nx.PD + o0, r);
   }
+}
+
+// the device phase of the horizons beyond the register path: closed-form
+// devices and the inputs of the inner ADMM (fwd_inner follows)
+template <int VW>
+__global__ void __launch_bounds__(TB, VW == 4 ? VW4_CTAS : 8) fwd_dev(DP p, St s, St nx, float *XD, unsigned char *dmask) {
+  closed_part<VW>(p, s, nx, XD, dmask, blockIdx.x, gridDim.x);
 }
 
 // One device's inner problem as the kernels read it: constraint rows in CSR
@@ -728,44 +782,8 @@ __device__ __forceinline__ void dev_back(const DP &p, float *LX, float *GL, floa
   LX[i] = lx;
 }
 
-// The reverse device kernels on VW steps per lane group: ksum and dev_x for
-// steps t0 .. t0 + VW - 1, each step summed in the same order as the
-// one-step forms (so the results are the same step by step), and
-// add_node_kv: lpd + the sum over contingencies of V at device d's node
-// divided by the node's terminal count (the k-average's adjoint)
-template <int VW>
-__device__ __forceinline__ Vf<VW> ksumv(const DP &p, const float *V, const float *W, int n, int t0) {
-  const int j = threadIdx.x & (KL - 1);
-  Vf<VW> s;
-#pragma unroll
-  for (int e = 0; e < VW; ++e) s.x[e] = 0.f;
-#pragma unroll 3
-  for (int k = j; k < p.Kp; k += KL) {
-    const Vf<VW> v = ldv<VW>(V + ni(p, k, n, t0));
-    if (W) {
-      const Vf<VW> w = ldv<VW>(W + ni(p, k, n, t0));
-#pragma unroll
-      for (int e = 0; e < VW; ++e) s.x[e] += v.x[e] + w.x[e];
-    } else {
-#pragma unroll
-      for (int e = 0; e < VW; ++e) s.x[e] += v.x[e];
-    }
-  }
-  const unsigned gm = group_mask();
-#pragma unroll
-  for (int o = KL / 2; o > 0; o >>= 1)
-#pragma unroll
-    for (int e = 0; e < VW; ++e) s.x[e] += __shfl_xor_sync(gm, s.x[e], o);
-  return s;
-}
-template <int VW>
-__device__ __forceinline__ Vf<VW> dev_xv(const DP &p, const St &s, int d, int t0) {
-  const Vf<VW> pd = ldv<VW>(s.PD + (size_t)d * p.T + t0), k = ksumv<VW>(p, s.PB, s.U, p.dnode[d], t0);
-  Vf<VW> r;
-#pragma unroll
-  for (int e = 0; e < VW; ++e) r.x[e] = pd.x[e] - k.x[e] / (float)p.Kp;
-  return r;
-}
+// lpd + the sum over contingencies of V at device d's node divided by the
+// node's terminal count (the k-average's adjoint)
 template <int VW>
 __device__ __forceinline__ Vf<VW> add_node_kv(const DP &p, const float *V, int d, int t0, const Vf<VW> &lpd) {
   const int n = p.dnode[d];
@@ -774,15 +792,6 @@ __device__ __forceinline__ Vf<VW> add_node_kv(const DP &p, const float *V, int d
 #pragma unroll
   for (int e = 0; e < VW; ++e) r.x[e] = fmaf(k.x[e], p.icnt[n], lpd.x[e]);
   return r;
-}
-
-// device item i of a [S][T / VW] field: device d, first step t0, offset
-// d T + t0 = i VW
-template <int VW>
-__device__ __forceinline__ void dev_item(unsigned i, int T, int &d, int &t0) {
-  const unsigned TV = (unsigned)(T / VW);
-  d = (int)(i / TV);
-  t0 = (int)(i - (unsigned)d * TV) * VW;
 }
 
 template <int VW>
@@ -1198,21 +1207,58 @@ __device__ __forceinline__ RDev rdev(const DP &p, int w) {
   return RDev{di.dev, di.h, di.bat, di.piv};
 }
 
-// step 2 for the inner-ADMM devices from registers, one warp per device
+// X = p_d - avg_k(pbar + u) at a lane's C steps (0 beyond T), by one thread in
+// the order of ksumv: eight partial sums over k mod 8, met as its butterfly
+// meets them
 template <int C>
-__global__ void __launch_bounds__(TB, 1) fwd_inner_r(DP p, St s, St nx, const float *XD, float *DEL,
-                                                     unsigned long long *grec) {
+__device__ __forceinline__ void lane_x(const DP &p, const St &s, int d, int t0, float (&x)[C]) {
+  const int n = p.dnode[d], T = p.T;
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    x[j] = 0.f;
+    if (t0 + j < T) {
+      const float pd = s.PD[(size_t)d * T + t0 + j];
+      const float *V = s.PB + ni(p, 0, n, t0 + j), *W = s.U + ni(p, 0, n, t0 + j);
+      const size_t kn = (size_t)p.N * T;
+      float c[KL];
+#pragma unroll
+      for (int q = 0; q < KL; ++q) c[q] = 0.f;
+      for (int k = 0; k < p.Kp; k += KL) {
+#pragma unroll
+        for (int q = 0; q < KL; ++q)
+          if (k + q < p.Kp) c[q] += V[(size_t)(k + q) * kn] + W[(size_t)(k + q) * kn];
+      }
+      static_assert(KL == 8, "the pattern of ksumv's butterfly");
+      const float sum = ((c[0] + c[4]) + (c[2] + c[6])) + ((c[1] + c[5]) + (c[3] + c[7]));
+      x[j] = pd - sum / (float)p.Kp;
+    }
+  }
+}
+
+// step 2 from registers in one launch (it runs beside fwd_line): the first
+// inner_blocks blocks take the inner-ADMM devices, one warp each, which form
+// their inputs themselves, the others the closed-form devices.  As two
+// kernels in a row, behind the line prox, the phase took 28 us of a 2k
+// iteration's 44.
+template <int C, int VW>
+__global__ void __launch_bounds__(TB, 1) fwd_devs(DP p, St s, St nx, float *DEL, unsigned long long *grec,
+                                                  unsigned char *dmask, int inner_blocks) {
+  if ((int)blockIdx.x >= inner_blocks) {
+    closed_part<VW>(p, s, nx, nullptr, dmask, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
+    return;
+  }
   const int lane = threadIdx.x & 31, w = blockIdx.x * RWARPS + (threadIdx.x >> 5), T = p.T, t0 = lane * C;
   if (w >= p.n_inner) return;
   const RDev dv = rdev(p, w);
   unsigned long long *mask = grec ? grec + (size_t)w * RREC_WORDS : nullptr;
   float *Bo = nx.INS + dv.h, *Lo = nx.INS + p.Mtot + dv.h;
-  float x[C];
+  float x[C], xd[C];
   TriFac<C> tf;
+  lane_x<C>(p, s, dv.dev, t0, xd);
   if (dv.bat < 0) {
     float hU[C], hL[C], hRU[C], hRD[C], bU[C], lU[C], bL[C], lL[C], bRU[C], lRU[C], bRD[C], lRD[C], z[C];
-    ramp_load<C>(p, s, dv, T, lane, x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD, XD);
-    ramp_fwd_r<C>(T, lane, p.rd, p.rd, p.gb[dv.dev], x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
+    ramp_load<C>(p, s, dv, T, lane, x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD, nullptr);
+    ramp_fwd_r<C>(T, lane, p.rd, p.rd, p.gb[dv.dev], xd, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD,
                   lRD, z, mask);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -1235,8 +1281,8 @@ __global__ void __launch_bounds__(TB, 1) fwd_inner_r(DP p, St s, St nx, const fl
     StorK k;
     float cost, Pm, Em, zp[C], zd[C];
     StorRows<C> lam, bet;
-    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, tf, lam, bet, XD);
-    stor_fwd_r<C>(T, lane, k, cost, Pm, Em, x, tf, lam, bet, zp, zd, mask);
+    stor_load<C>(p, s, dv, T, lane, k, cost, Pm, Em, x, tf, lam, bet, nullptr);
+    stor_fwd_r<C>(T, lane, k, cost, Pm, Em, xd, tf, lam, bet, zp, zd, mask);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
@@ -1756,8 +1802,9 @@ size_t bwd_inner_smem(int T, int n, int m, int nnz, int level) {
 struct opf_diff {
   int N = 0, L = 0, T = 0, Kp = 0, G = 0, D = 0, B = 0, H = 0, S = 0, ckpt = 1;
   cudaStream_t stream = nullptr;
-  // the reverse pass runs the node gathers of the line terms here, beside
-  // the inner ADMM on `stream` (created by the first gradient call)
+  // the forward pass runs the line proxes here, beside the devices, and the
+  // reverse pass the node gathers of the line terms, beside the inner ADMM
+  // (created by the first call)
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   DP p{};
@@ -1963,29 +2010,48 @@ St carve_state(const opf_diff *d, float *base) {
 
 // mask (optional): the iteration's record for the reverse pass -- the
 // clipped inner rows, then a byte per line item, then one per device step
-void forward_step(const opf_diff *d, const St &s, const St &nx, float *XD, float *DEL,
-                  unsigned char *mask = nullptr) {
+// The line proxes run on sa beside the devices on sm (both read only the old
+// state); the node averages follow both.
+cudaError_t forward_step(const opf_diff *d, cudaStream_t sm, cudaStream_t sa, const St &s, const St &nx, float *XD,
+                         float *DEL, unsigned char *mask = nullptr) {
   const DP &p = d->p;
   const long long nl = (long long)p.Kp * p.L * p.T, nn = (long long)p.Kp * p.N * p.T, ns = (long long)p.S * p.T;
   unsigned char *lmask = mask ? mask + inner_record_bytes(p) : nullptr;
   unsigned char *dmask = mask ? lmask + nl : nullptr;
   unsigned long long *rrec = reinterpret_cast<unsigned long long *>(mask);
-  const bool v4 = p.T % 4 == 0;   // four steps per thread in the line and node kernels
-  if (v4) fwd_line<4><<<grid_for(nl / 4), TB, 0, d->stream>>>(p, s, nx, lmask);
-  else fwd_line<1><<<grid_for(nl), TB, 0, d->stream>>>(p, s, nx, lmask);
-  fwd_dev<<<grid_for(ns * KL), TB, 0, d->stream>>>(p, s, nx, XD, dmask);
-  if (p.n_inner) {
-    const int g = (p.n_inner + RWARPS - 1) / RWARPS;
+  const bool v4 = p.T % 4 == 0;   // four steps per thread in the element-wise kernels
+  cudaError_t e = cudaEventRecord(d->ev_fork, sm);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(sa, d->ev_fork, 0);
+  if (e != cudaSuccess) return e;
+  if (v4) fwd_line<4><<<grid_for(nl / 4), TB, 0, sa>>>(p, s, nx, lmask);
+  else fwd_line<1><<<grid_for(nl), TB, 0, sa>>>(p, s, nx, lmask);
+  e = cudaEventRecord(d->ev_join, sa);
+  if (e != cudaSuccess) return e;
+  const int dg = grid_for(ns / (v4 ? 4 : 1) * KL);
+  if (p.reg_c) {
+    const int ni = (p.n_inner + RWARPS - 1) / RWARPS, g = ni + dg;
+#define DEVS_LAUNCH(C)                                                                     \
+  case C:                                                                                  \
+    if (v4) fwd_devs<C, 4><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);              \
+    else fwd_devs<C, 1><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);                 \
+    break
     switch (p.reg_c) {
-      case 1: fwd_inner_r<1><<<g, TB, 0, d->stream>>>(p, s, nx, XD, DEL, rrec); break;
-      case 2: fwd_inner_r<2><<<g, TB, 0, d->stream>>>(p, s, nx, XD, DEL, rrec); break;
-      case 3: fwd_inner_r<3><<<g, TB, 0, d->stream>>>(p, s, nx, XD, DEL, rrec); break;
-      case 4: fwd_inner_r<4><<<g, TB, 0, d->stream>>>(p, s, nx, XD, DEL, rrec); break;
-      default: fwd_inner<<<p.n_inner, TBI, d->smem_fwd, d->stream>>>(p, s, nx, XD, DEL, d->stage, mask); break;
+      DEVS_LAUNCH(1);
+      DEVS_LAUNCH(2);
+      DEVS_LAUNCH(3);
+      DEVS_LAUNCH(4);
     }
+#undef DEVS_LAUNCH
+  } else {
+    if (v4) fwd_dev<4><<<dg, TB, 0, sm>>>(p, s, nx, XD, dmask);
+    else fwd_dev<1><<<dg, TB, 0, sm>>>(p, s, nx, XD, dmask);
+    if (p.n_inner) fwd_inner<<<p.n_inner, TBI, d->smem_fwd, sm>>>(p, s, nx, XD, DEL, d->stage, mask);
   }
-  if (v4) fwd_avg<4><<<grid_for(nn / 4), TB, 0, d->stream>>>(p, s, nx);
-  else fwd_avg<1><<<grid_for(nn), TB, 0, d->stream>>>(p, s, nx);
+  e = cudaStreamWaitEvent(sm, d->ev_join, 0);
+  if (e != cudaSuccess) return e;
+  if (v4) fwd_avg<4><<<grid_for(nn / 4), TB, 0, sm>>>(p, s, nx);
+  else fwd_avg<1><<<grid_for(nn), TB, 0, sm>>>(p, s, nx);
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -2409,13 +2475,20 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   float *LPDT = XD + ST, *GL = LPDT + ST, *GP = GL + DT, *HB = GP + GT, *DEL = HB + MT;
   auto ckst = [&](int j) { return carve_state(d, ck + (size_t)j * SF); };
   auto sgst = [&](int j) { return carve_state(d, seg + (size_t)j * SF); };
+  {
+    cudaError_t ce = cudaSuccess;
+    if (!d->aux) ce = cudaStreamCreateWithFlags(&d->aux, cudaStreamNonBlocking);
+    if (ce == cudaSuccess && !d->ev_fork) ce = cudaEventCreateWithFlags(&d->ev_fork, cudaEventDisableTiming);
+    if (ce == cudaSuccess && !d->ev_join) ce = cudaEventCreateWithFlags(&d->ev_join, cudaEventDisableTiming);
+    if (ce != cudaSuccess) return dfail(OPF_ECUDA, cudaGetErrorString(ce));
+  }
   // forward, keeping checkpoints
   e = cudaMemsetAsync(ck, 0, SF * 4, d->stream);
   St cur = ckst(0);
   float *scratch = seg;  // two alternating states in the segment buffer
   for (int i = 1; e == cudaSuccess && i <= K; ++i) {
     St nx = (i % C == 0) ? ckst(i / C) : carve_state(d, scratch + (size_t)(i & 1) * SF);
-    forward_step(d, cur, nx, XD, DEL, mask_of(i));
+    e = forward_step(d, d->stream, d->aux, cur, nx, XD, DEL, mask_of(i));
     cur = nx;
   }
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -2424,7 +2497,12 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   if (e == cudaSuccess && BT) e = cudaMemcpyAsync(del.data(), DEL, BT * 4, cudaMemcpyDeviceToHost, d->stream);
   if (e == cudaSuccess && DT) e = cudaMemcpyAsync(lp.data(), p.load_p, DT * 4, cudaMemcpyDeviceToHost, d->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);
-  if (e != cudaSuccess) return dfail(OPF_ECUDA, cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    // a failed fork or join may leave work queued on the second stream
+    cudaStreamSynchronize(d->stream);
+    cudaStreamSynchronize(d->aux);
+    return dfail(OPF_ECUDA, cudaGetErrorString(e));
+  }
   if (cost) {
     double f = 0.0;
     for (int g = 0; g < d->G; ++g)
@@ -2442,13 +2520,6 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
     *cost = f;
   }
   if (!grads) return OPF_OK;
-  {
-    cudaError_t ce = cudaSuccess;
-    if (!d->aux) ce = cudaStreamCreateWithFlags(&d->aux, cudaStreamNonBlocking);
-    if (ce == cudaSuccess && !d->ev_fork) ce = cudaEventCreateWithFlags(&d->ev_fork, cudaEventDisableTiming);
-    if (ce == cudaSuccess && !d->ev_join) ce = cudaEventCreateWithFlags(&d->ev_join, cudaEventDisableTiming);
-    if (ce != cudaSuccess) return dfail(OPF_ECUDA, cudaGetErrorString(ce));
-  }
   // reverse pass
   Adj a;
   a.LP = adj;
@@ -2477,7 +2548,7 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
     const int lo = ((hi - 1) / C) * C;
     auto state = [&](int j) { return (j == lo || masks) ? ckst(lo / C) : sgst(j - lo); };   // state j, lo <= j < hi
     for (int i = lo + 1; e == cudaSuccess && !masks && i < hi; ++i)
-      forward_step(d, state(i - 1), sgst(i - lo), XD, DEL);
+      e = forward_step(d, d->stream, d->aux, state(i - 1), sgst(i - lo), XD, DEL);
     for (int i = hi; e == cudaSuccess && i > lo; --i) {
       const St s = state(i - 1);
       unsigned char *mi = mask_of(i);
