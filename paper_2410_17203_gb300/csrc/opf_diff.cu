@@ -1799,6 +1799,16 @@ size_t bwd_inner_smem(int T, int n, int m, int nnz, int level) {
 
 }  // namespace
 
+// what the launches of a call depend on, beside the context
+struct PassKey {
+  int K = 0;
+  bool grads = false, rec = false;
+  const void *buf[5] = {};   // checkpoints, segment, adjoint, work, record
+  bool operator==(const PassKey &o) const {
+    return K == o.K && grads == o.grads && rec == o.rec && std::equal(buf, buf + 5, o.buf);
+  }
+};
+
 struct opf_diff {
   int N = 0, L = 0, T = 0, Kp = 0, G = 0, D = 0, B = 0, H = 0, S = 0, ckpt = 1;
   cudaStream_t stream = nullptr;
@@ -1807,6 +1817,18 @@ struct opf_diff {
   // (created by the first call)
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // The launches of a call's forward and reverse pass as CUDA graphs, kept
+  // for the next calls of the same shape (PassKey): a graph starts a small
+  // kernel every 0.7 us, a stream every 2 us, and an iteration has seven.
+  // They are built by the second call of a shape in a row (a first call
+  // launches directly: capture and instantiation take about 2 us a kernel),
+  // up to GRAPH_MAX_K iterations, captured on `cap`.
+  cudaStream_t cap = nullptr;
+  cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
+  PassKey key{};
+  // host staging of the cost's inputs (pinned), read while the reverse pass runs
+  cudaEvent_t ev_cost = nullptr;
+  float *stage_host = nullptr;
   DP p{};
   std::vector<float> ga, gb, voll, load_p, gpmax, lu, scost;  // host copies (cost and defaults)
   std::vector<double> gpmin, ramp, sP, sdur;                 // right-hand sides of the inner rows
@@ -2424,6 +2446,36 @@ cudaError_t ensure(float **buf, size_t *cap, size_t n) {
   return e;
 }
 
+constexpr int GRAPH_MAX_K = 512;
+
+void drop_graphs(opf_diff *d) {
+  if (d->g_fwd) cudaGraphExecDestroy(d->g_fwd);
+  if (d->g_bwd) cudaGraphExecDestroy(d->g_bwd);
+  d->g_fwd = d->g_bwd = nullptr;
+}
+
+// the launches that `pass` makes on a stream as a graph; false (no error left
+// behind) where that fails, and the caller launches directly
+template <class F>
+bool build_graph(opf_diff *d, F pass, cudaGraphExec_t *out) {
+  cudaError_t e = cudaSuccess;
+  if (!d->cap) e = cudaStreamCreateWithFlags(&d->cap, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamBeginCapture(d->cap, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    const cudaError_t pe = pass(d->cap);
+    cudaGraph_t g = nullptr;
+    e = cudaStreamEndCapture(d->cap, &g);
+    if (e == cudaSuccess) e = pe;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+  }
+  if (e != cudaSuccess) {
+    *out = nullptr;
+    cudaGetLastError();
+  }
+  return e == cudaSuccess;
+}
+
 opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p, const float *gen_pmax,
                      const float *line_u, double *cost, float *g_load, float *g_pmax, float *g_u) {
   if (!d) return dfail(OPF_EINVAL, "diff is NULL");
@@ -2440,8 +2492,6 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   else DCK(cudaMemcpyAsync(const_cast<float *>(p.gpmax), d->gpmax.data(), GT * 4, cudaMemcpyHostToDevice, d->stream));
   if (line_u) DCK(cudaMemcpyAsync(const_cast<float *>(p.lu), line_u, L * 4, in_kind, d->stream));
   else DCK(cudaMemcpyAsync(const_cast<float *>(p.lu), d->lu.data(), L * 4, cudaMemcpyHostToDevice, d->stream));
-  // the capacity rows of the ramp-limited generators' inner problems
-  if (p.n_inner) set_ramp_rhs<<<grid_for((long long)p.n_inner * T), TB, 0, d->stream>>>(p, d->RH);
   // states: checkpoints 0, C, 2C, ... and room for a segment's C - 1
   // recomputed states (at least the forward pass's two alternating ones)
   const int C = std::min(d->ckpt, K);
@@ -2478,32 +2528,149 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   {
     cudaError_t ce = cudaSuccess;
     if (!d->aux) ce = cudaStreamCreateWithFlags(&d->aux, cudaStreamNonBlocking);
-    if (ce == cudaSuccess && !d->ev_fork) ce = cudaEventCreateWithFlags(&d->ev_fork, cudaEventDisableTiming);
-    if (ce == cudaSuccess && !d->ev_join) ce = cudaEventCreateWithFlags(&d->ev_join, cudaEventDisableTiming);
-    if (ce != cudaSuccess) return dfail(OPF_ECUDA, cudaGetErrorString(ce));
+    for (cudaEvent_t *ev : {&d->ev_fork, &d->ev_join, &d->ev_cost})
+      if (ce == cudaSuccess && !*ev) ce = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (ce == cudaSuccess && !d->stage_host)
+      ce = cudaMallocHost(reinterpret_cast<void **>(&d->stage_host), std::max<size_t>(ST + BT + DT, 1) * sizeof(float));
+    if (ce != cudaSuccess)
+      return dfail(ce == cudaErrorMemoryAllocation ? OPF_ENOMEM : OPF_ECUDA, cudaGetErrorString(ce));
   }
-  // forward, keeping checkpoints
-  e = cudaMemsetAsync(ck, 0, SF * 4, d->stream);
-  St cur = ckst(0);
-  float *scratch = seg;  // two alternating states in the segment buffer
-  for (int i = 1; e == cudaSuccess && i <= K; ++i) {
-    St nx = (i % C == 0) ? ckst(i / C) : carve_state(d, scratch + (size_t)(i & 1) * SF);
-    e = forward_step(d, d->stream, d->aux, cur, nx, XD, DEL, mask_of(i));
-    cur = nx;
+  // state K (the reverse pass may overwrite it; its cost inputs are copied first)
+  const St last = (K % C == 0) ? ckst(K / C) : carve_state(d, seg + (size_t)(K & 1) * SF);
+  // forward, keeping checkpoints, on sm (and the second stream)
+  auto forward = [&](cudaStream_t sm) {
+    // the capacity rows of the ramp-limited generators' inner problems
+    if (p.n_inner) set_ramp_rhs<<<grid_for((long long)p.n_inner * T), TB, 0, sm>>>(p, d->RH);
+    cudaError_t e = cudaMemsetAsync(ck, 0, SF * 4, sm);
+    St cur = ckst(0);
+    for (int i = 1; e == cudaSuccess && i <= K; ++i) {   // between checkpoints, two alternating states
+      St nx = (i % C == 0) ? ckst(i / C) : carve_state(d, seg + (size_t)(i & 1) * SF);
+      e = forward_step(d, sm, d->aux, cur, nx, XD, DEL, mask_of(i));
+      cur = nx;
+    }
+    return e == cudaSuccess ? cudaGetLastError() : e;
+  };
+  // reverse pass
+  Adj a;
+  a.LP = adj;
+  a.LT1 = a.LP + KLT;
+  a.LT2 = a.LT1 + KLT;
+  a.LV1 = a.LT2 + KLT;
+  a.LV2 = a.LV1 + KLT;
+  a.LPD = a.LV2 + KLT;
+  a.LU = a.LPD + ST;
+  a.LINS = a.LU + KNT;
+  auto reverse = [&](cudaStream_t sm) {
+    cudaError_t e = cudaMemsetAsync(adj, 0, adj_floats * 4, sm);
+    if (e == cudaSuccess) e = cudaMemsetAsync(GU, 0, KLT * 4, sm);
+    if (e == cudaSuccess) e = cudaMemsetAsync(GL, 0, (DT + GT + MT) * 4, sm);
+    if (e == cudaSuccess) bwd_init<<<grid_for((long long)ST), TB, 0, sm>>>(p, last, a, GL);
+    const long long nl = (long long)KLT, nn = (long long)KNT, ns = (long long)ST;
+    // d/d pbar' is u's adjoint itself (u' = u + pbar'), read before bwd_node2 or
+    // bwd_node3 adds the iteration's increment to it
+    const float *A = a.LU;
+    const bool v4 = T % 4 == 0;   // four steps per thread in the line and node kernels
+    bool primed = false;   // iteration i's first half already ran, fused into iteration i+1's second half
+    for (int hi = K; e == cudaSuccess && hi > 0;) {
+      // segment (lo, hi]: states lo + 1 .. hi - 1 recomputed from checkpoint lo
+      // (read in place).  With the record the reverse pass reads no state (the
+      // clips, and the inner rows that clipped, are all it needs), so nothing
+      // is recomputed and every kernel is handed checkpoint lo, unread.
+      const int lo = ((hi - 1) / C) * C;
+      auto state = [&](int j) { return (j == lo || masks) ? ckst(lo / C) : sgst(j - lo); };   // state j, lo <= j < hi
+      for (int i = lo + 1; e == cudaSuccess && !masks && i < hi; ++i)
+        e = forward_step(d, sm, d->aux, state(i - 1), sgst(i - lo), XD, DEL);
+      for (int i = hi; e == cudaSuccess && i > lo; --i) {
+        const St s = state(i - 1);
+        unsigned char *mi = mask_of(i);
+        float *LX = (i & 1) ? LX1 : LX0, *LXn = (i & 1) ? LX0 : LX1;   // d/dX of iterations i and i - 1
+        if (!primed) {
+          const unsigned char *lmask = mi ? mi + inner_record_bytes(p) : nullptr, *dmask = mi ? lmask + KLT : nullptr;
+          if (v4) {
+            bwd_node1<4><<<grid_for(nn / 4), TB, 0, sm>>>(p, a, Bn);
+            bwd_line1<4><<<grid_for(nl / 4), TB, 0, sm>>>(p, s, a, A, Bn, X2, Y1, Y2, GU, lmask);
+          } else {
+            bwd_node1<1><<<grid_for(nn), TB, 0, sm>>>(p, a, Bn);
+            bwd_line1<1><<<grid_for(nl), TB, 0, sm>>>(p, s, a, A, Bn, X2, Y1, Y2, GU, lmask);
+          }
+          if (v4) bwd_dev<4><<<grid_for(ns / 4 * KL), TB, 0, sm>>>(p, s, a, A, LX, GL, GP, XD, LPDT, dmask);
+          else bwd_dev<1><<<grid_for(ns * KL), TB, 0, sm>>>(p, s, a, A, LX, GL, GP, XD, LPDT, dmask);
+        }
+        // iteration i - 1's first half joins this second half when what it
+        // reads is at hand: its record, or its input state i - 2 in this segment
+        unsigned char *mp = i > 1 ? mask_of(i - 1) : nullptr;
+        const int nxt = i > 1 && (mp || i - 2 >= lo) ? 1 : 0;
+        // the node gathers beside the inner ADMM (at the nodes with its devices,
+        // only the line terms; bwd_node3 adds the device terms after it)
+        if (e == cudaSuccess) e = cudaEventRecord(d->ev_fork, sm);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(d->aux, d->ev_fork, 0);
+        if (e != cudaSuccess) break;
+        if (v4) bwd_node2<4><<<grid_for(nn / 4), TB, 0, d->aux>>>(p, a, X2, Y1, Y2, LX, Cn, Dn, Bn, nxt);
+        else bwd_node2<1><<<grid_for(nn), TB, 0, d->aux>>>(p, a, X2, Y1, Y2, LX, Cn, Dn, Bn, nxt);
+        e = cudaEventRecord(d->ev_join, d->aux);
+        if (p.n_inner) {
+          const int g = (p.n_inner + RWARPS - 1) / RWARPS, lst = i == K ? 1 : 0;
+          unsigned long long *m1 = reinterpret_cast<unsigned long long *>(d->mask1);
+          const unsigned long long *rr = reinterpret_cast<const unsigned long long *>(mi);
+          switch (p.reg_c) {
+            case 1: bwd_inner_r<1><<<g, TB, 0, sm>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
+            case 2: bwd_inner_r<2><<<g, TB, 0, sm>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
+            case 3: bwd_inner_r<3><<<g, TB, 0, sm>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
+            case 4: bwd_inner_r<4><<<g, TB, 0, sm>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
+            default:
+              bwd_inner<<<p.n_inner, TBI, d->smem_bwd, sm>>>(p, s, a, XD, LPDT, LX, HB, lst, d->stage, mi);
+              break;
+          }
+        }
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(sm, d->ev_join, 0);
+        if (e != cudaSuccess) break;
+        const St sp = nxt && i - 2 >= lo ? state(i - 2) : s;   // read only without a record
+        const unsigned char *lmp = mp ? mp + inner_record_bytes(p) : nullptr, *dmp = mp ? lmp + KLT : nullptr;
+        const long long ni3 = (long long)p.Kp * p.n_inode * T;   // items of the nodes with inner-ADMM devices
+        if (ni3 && v4) bwd_node3<4><<<grid_for(ni3 / 4), TB, 0, sm>>>(p, a, LX, Cn);
+        else if (ni3) bwd_node3<1><<<grid_for(ni3), TB, 0, sm>>>(p, a, LX, Cn);
+        {
+          const Scatter g{Cn, Dn, A, Bn, LX, X2, Y1, Y2, GU, LXn, GL, GP, XD, LPDT, lmp, dmp};
+          const int db = grid_for(ns / (v4 ? 4 : 1) * KL);
+          if (v4) bwd_scatter<4><<<db + grid_for(nl / 4), TB, 0, sm>>>(p, sp, a, g, nxt, db);
+          else bwd_scatter<1><<<db + grid_for(nl), TB, 0, sm>>>(p, sp, a, g, nxt, db);
+        }
+        primed = nxt != 0;
+      }
+      hi = lo;
+      if (e == cudaSuccess) e = cudaGetLastError();
+    }
+    return e;
+  };
+  // the call's launches: the kept graphs, or directly
+  const PassKey key{K, grads, rec, {ck, seg, adj, work, masks}};
+  const bool same = key == d->key;
+  if (!same) {
+    drop_graphs(d);
+    d->key = key;
+  } else if (!d->g_fwd && K <= GRAPH_MAX_K) {
+    if (!build_graph(d, forward, &d->g_fwd) || (grads && !build_graph(d, reverse, &d->g_bwd))) drop_graphs(d);
   }
-  if (e == cudaSuccess) e = cudaGetLastError();
-  std::vector<float> pd(ST), del(BT), lp(DT);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(pd.data(), cur.PD, ST * 4, cudaMemcpyDeviceToHost, d->stream);
-  if (e == cudaSuccess && BT) e = cudaMemcpyAsync(del.data(), DEL, BT * 4, cudaMemcpyDeviceToHost, d->stream);
-  if (e == cudaSuccess && DT) e = cudaMemcpyAsync(lp.data(), p.load_p, DT * 4, cudaMemcpyDeviceToHost, d->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);
-  if (e != cudaSuccess) {
-    // a failed fork or join may leave work queued on the second stream
-    cudaStreamSynchronize(d->stream);
-    cudaStreamSynchronize(d->aux);
-    return dfail(OPF_ECUDA, cudaGetErrorString(e));
-  }
+  e = d->g_fwd ? cudaGraphLaunch(d->g_fwd, d->stream) : forward(d->stream);
+  // the cost's inputs to the host, where it is summed while the reverse pass runs
+  float *pd = d->stage_host, *del = pd + ST, *lpd = del + BT;
+  const float *lp = load_p ? load_p : d->load_p.data();
   if (cost) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(pd, last.PD, ST * 4, cudaMemcpyDeviceToHost, d->stream);
+    if (e == cudaSuccess && BT) e = cudaMemcpyAsync(del, DEL, BT * 4, cudaMemcpyDeviceToHost, d->stream);
+    if (e == cudaSuccess && DT && on_device && load_p) {
+      e = cudaMemcpyAsync(lpd, p.load_p, DT * 4, cudaMemcpyDeviceToHost, d->stream);
+      lp = lpd;
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(d->ev_cost, d->stream);
+  }
+  if (e == cudaSuccess && grads) e = d->g_bwd ? cudaGraphLaunch(d->g_bwd, d->stream) : reverse(d->stream);
+  if (e == cudaSuccess && g_pmax && p.n_inner)
+    finish_cap_grad<<<grid_for((long long)p.n_inner * T), TB, 0, d->stream>>>(p, HB, GP);
+  if (e == cudaSuccess && g_u) finish_line_grad<<<grid_for(32 * (long long)L), TB, 0, d->stream>>>(p, GU, d->gline);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess && cost) e = cudaEventSynchronize(d->ev_cost);
+  if (e == cudaSuccess && cost) {
     double f = 0.0;
     for (int g = 0; g < d->G; ++g)
       for (int t = 0; t < T; ++t) {
@@ -2519,100 +2686,6 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
       for (int t = 0; t < T; ++t) f += (double)d->scost[bt] * del[(size_t)bt * T + t];
     *cost = f;
   }
-  if (!grads) return OPF_OK;
-  // reverse pass
-  Adj a;
-  a.LP = adj;
-  a.LT1 = a.LP + KLT;
-  a.LT2 = a.LT1 + KLT;
-  a.LV1 = a.LT2 + KLT;
-  a.LV2 = a.LV1 + KLT;
-  a.LPD = a.LV2 + KLT;
-  a.LU = a.LPD + ST;
-  a.LINS = a.LU + KNT;
-  e = cudaMemsetAsync(adj, 0, adj_floats * 4, d->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(GU, 0, KLT * 4, d->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(GL, 0, (DT + GT + MT) * 4, d->stream);
-  if (e == cudaSuccess) bwd_init<<<grid_for((long long)ST), TB, 0, d->stream>>>(p, cur, a, GL);
-  const long long nl = (long long)KLT, nn = (long long)KNT, ns = (long long)ST;
-  // d/d pbar' is u's adjoint itself (u' = u + pbar'), read before bwd_node2 or
-  // bwd_node3 adds the iteration's increment to it
-  const float *A = a.LU;
-  const bool v4 = T % 4 == 0;   // four steps per thread in the line and node kernels
-  bool primed = false;   // iteration i's first half already ran, fused into iteration i+1's second half
-  for (int hi = K; e == cudaSuccess && hi > 0;) {
-    // segment (lo, hi]: states lo + 1 .. hi - 1 recomputed from checkpoint lo
-    // (read in place).  With the record the reverse pass reads no state (the
-    // clips, and the inner rows that clipped, are all it needs), so nothing
-    // is recomputed and every kernel is handed checkpoint lo, unread.
-    const int lo = ((hi - 1) / C) * C;
-    auto state = [&](int j) { return (j == lo || masks) ? ckst(lo / C) : sgst(j - lo); };   // state j, lo <= j < hi
-    for (int i = lo + 1; e == cudaSuccess && !masks && i < hi; ++i)
-      e = forward_step(d, d->stream, d->aux, state(i - 1), sgst(i - lo), XD, DEL);
-    for (int i = hi; e == cudaSuccess && i > lo; --i) {
-      const St s = state(i - 1);
-      unsigned char *mi = mask_of(i);
-      float *LX = (i & 1) ? LX1 : LX0, *LXn = (i & 1) ? LX0 : LX1;   // d/dX of iterations i and i - 1
-      if (!primed) {
-        const unsigned char *lmask = mi ? mi + inner_record_bytes(p) : nullptr, *dmask = mi ? lmask + KLT : nullptr;
-        if (v4) {
-          bwd_node1<4><<<grid_for(nn / 4), TB, 0, d->stream>>>(p, a, Bn);
-          bwd_line1<4><<<grid_for(nl / 4), TB, 0, d->stream>>>(p, s, a, A, Bn, X2, Y1, Y2, GU, lmask);
-        } else {
-          bwd_node1<1><<<grid_for(nn), TB, 0, d->stream>>>(p, a, Bn);
-          bwd_line1<1><<<grid_for(nl), TB, 0, d->stream>>>(p, s, a, A, Bn, X2, Y1, Y2, GU, lmask);
-        }
-        if (v4) bwd_dev<4><<<grid_for(ns / 4 * KL), TB, 0, d->stream>>>(p, s, a, A, LX, GL, GP, XD, LPDT, dmask);
-        else bwd_dev<1><<<grid_for(ns * KL), TB, 0, d->stream>>>(p, s, a, A, LX, GL, GP, XD, LPDT, dmask);
-      }
-      // iteration i - 1's first half joins this second half when what it
-      // reads is at hand: its record, or its input state i - 2 in this segment
-      unsigned char *mp = i > 1 ? mask_of(i - 1) : nullptr;
-      const int nxt = i > 1 && (mp || i - 2 >= lo) ? 1 : 0;
-      // the node gathers beside the inner ADMM (at the nodes with its devices,
-      // only the line terms; bwd_node3 adds the device terms after it)
-      if (e == cudaSuccess) e = cudaEventRecord(d->ev_fork, d->stream);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(d->aux, d->ev_fork, 0);
-      if (e != cudaSuccess) break;
-      if (v4) bwd_node2<4><<<grid_for(nn / 4), TB, 0, d->aux>>>(p, a, X2, Y1, Y2, LX, Cn, Dn, Bn, nxt);
-      else bwd_node2<1><<<grid_for(nn), TB, 0, d->aux>>>(p, a, X2, Y1, Y2, LX, Cn, Dn, Bn, nxt);
-      e = cudaEventRecord(d->ev_join, d->aux);
-      if (p.n_inner) {
-        const int g = (p.n_inner + RWARPS - 1) / RWARPS, lst = i == K ? 1 : 0;
-        unsigned long long *m1 = reinterpret_cast<unsigned long long *>(d->mask1);
-        const unsigned long long *rr = reinterpret_cast<const unsigned long long *>(mi);
-        switch (p.reg_c) {
-          case 1: bwd_inner_r<1><<<g, TB, 0, d->stream>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
-          case 2: bwd_inner_r<2><<<g, TB, 0, d->stream>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
-          case 3: bwd_inner_r<3><<<g, TB, 0, d->stream>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
-          case 4: bwd_inner_r<4><<<g, TB, 0, d->stream>>>(p, s, a, XD, LPDT, LX, HB, lst, rr, m1); break;
-          default:
-            bwd_inner<<<p.n_inner, TBI, d->smem_bwd, d->stream>>>(p, s, a, XD, LPDT, LX, HB, lst, d->stage, mi);
-            break;
-        }
-      }
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(d->stream, d->ev_join, 0);
-      if (e != cudaSuccess) break;
-      const St sp = nxt && i - 2 >= lo ? state(i - 2) : s;   // read only without a record
-      const unsigned char *lmp = mp ? mp + inner_record_bytes(p) : nullptr, *dmp = mp ? lmp + KLT : nullptr;
-      const long long ni3 = (long long)p.Kp * p.n_inode * T;   // items of the nodes with inner-ADMM devices
-      if (ni3 && v4) bwd_node3<4><<<grid_for(ni3 / 4), TB, 0, d->stream>>>(p, a, LX, Cn);
-      else if (ni3) bwd_node3<1><<<grid_for(ni3), TB, 0, d->stream>>>(p, a, LX, Cn);
-      {
-        const Scatter g{Cn, Dn, A, Bn, LX, X2, Y1, Y2, GU, LXn, GL, GP, XD, LPDT, lmp, dmp};
-        const int db = grid_for(ns / (v4 ? 4 : 1) * KL);
-        if (v4) bwd_scatter<4><<<db + grid_for(nl / 4), TB, 0, d->stream>>>(p, sp, a, g, nxt, db);
-        else bwd_scatter<1><<<db + grid_for(nl), TB, 0, d->stream>>>(p, sp, a, g, nxt, db);
-      }
-      primed = nxt != 0;
-    }
-    hi = lo;
-    if (e == cudaSuccess) e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && g_pmax && p.n_inner)
-    finish_cap_grad<<<grid_for((long long)p.n_inner * T), TB, 0, d->stream>>>(p, HB, GP);
-  if (e == cudaSuccess && g_u) finish_line_grad<<<grid_for(32 * (long long)L), TB, 0, d->stream>>>(p, GU, d->gline);
-  if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess && g_load) e = cudaMemcpyAsync(g_load, GL, DT * 4, out_kind, d->stream);
   if (e == cudaSuccess && g_pmax) e = cudaMemcpyAsync(g_pmax, GP, GT * 4, out_kind, d->stream);
   if (e == cudaSuccess && g_u) e = cudaMemcpyAsync(g_u, d->gline, L * 4, out_kind, d->stream);
@@ -2652,9 +2725,12 @@ void opf_diff_destroy(opf_diff *d) {
   if (!d) return;
   cudaStreamSynchronize(d->stream);
   if (d->aux) cudaStreamSynchronize(d->aux);
-  if (d->ev_fork) cudaEventDestroy(d->ev_fork);
-  if (d->ev_join) cudaEventDestroy(d->ev_join);
+  drop_graphs(d);
+  for (cudaEvent_t ev : {d->ev_fork, d->ev_join, d->ev_cost})
+    if (ev) cudaEventDestroy(ev);
   if (d->aux) cudaStreamDestroy(d->aux);
+  if (d->cap) cudaStreamDestroy(d->cap);
+  if (d->stage_host) cudaFreeHost(d->stage_host);
   for (void *q : d->allocs) cudaFree(q);
   for (float *q : {d->ck, d->seg, d->adj, d->work, d->gline, d->masks})
     if (q) cudaFree(q);
