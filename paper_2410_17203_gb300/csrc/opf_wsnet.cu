@@ -3,13 +3,20 @@
 // The paper has no counterpart; the network only proposes a starting point
 // for the message-passing iteration.
 //
-// Layout: activations are row-major [R][64] with rows r = t * N + n.  The
-// layers are small dense contractions (64 x 64) over many rows, so each
-// linear kernel stages the bfloat16 weights of a layer in shared memory as
-// FP32 and a tile of 32 input rows, and every thread accumulates eight
-// outputs in FP32.  Weight gradients are reduced per CTA over fixed row
-// ranges and then across CTAs in a fixed order, so results are
-// deterministic.  The neighbour average and its adjoint are CSR gathers.
+// Layout: activations are row-major [R][64] with rows r = t * N + n.  A layer
+// is one kernel: persistent CTAs hold the layer's bfloat16 weights in shared
+// memory as FP32 and walk tiles of 32 rows; the neighbour average (a CSR
+// gather) is formed tile by tile where it is used, in the forward pass from
+// the layer's input, in the backward pass, transposed, from the previous
+// layer's product.  Every output is summed over k in order in FP32.  Weight
+// gradients are partial sums over fixed row ranges, each over its rows in
+// order, reduced in a fixed order, so results are deterministic.  The relu
+// mask is the sign of the kept output.
+//
+// A training pass over 48,000 rows (2k buses, T = 24) moves about 0.35 GB and
+// does 7.3 GFLOP outside the tensor cores (the FP32 activations keep their
+// precision): bound by the FP32 pipes.  As fifty launches (averages, layers,
+// relu masks and each weight gradient apart) it took 0.97 ms, as sixteen @@.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -26,240 +33,389 @@ namespace {
 constexpr int HID = OPF_WSNET_HIDDEN;
 constexpr int NOUT = OPF_WSNET_OUT;
 constexpr int NMP = 3;         // message-passing layers
-constexpr int TB = 256;        // threads per CTA
-constexpr int ROWS = 32;       // rows per CTA in the linear kernels
-constexpr int GRAD_ROWS = 256; // rows per CTA in the weight-gradient partial sums
+constexpr int TB = 256;        // threads per CTA of the element-wise kernels
+constexpr int LB = 128;        // threads per CTA of the layer kernels
+constexpr int TR = 32;         // rows per tile of the layer kernels
+constexpr int AS = HID + 4;    // row stride of a tile in shared memory (16-byte rows on shifting banks)
+constexpr int GRAD_ROWS = 256; // rows per partial sum of the weight gradients
+constexpr int GB = 64;         // threads per CTA of the weight-gradient kernel
+constexpr int GK = 16;         // weight rows (k) per CTA there
+constexpr int GS = 32;         // activation rows staged together there
 
-// ---------------------------------------------------------------------------
-// out[r][j] = act(sum_k a[r][k] W(k, j) + sum_k a2[r][k] W2(k, j) + bias[j]
-//                 + (accum ? out[r][j] : 0)),  W(k, j) = W[k * J + j], or
-// W[j * K + k] with TRANS (the product with W transposed, for the backward
-// pass).  `pre` (optional) receives the value before the activation.
-// ---------------------------------------------------------------------------
-template <bool TRANS>
-__global__ void __launch_bounds__(TB) linear_kernel(const float *__restrict__ a, const __nv_bfloat16 *__restrict__ W,
-                                                    const float *__restrict__ a2,
-                                                    const __nv_bfloat16 *__restrict__ W2,
-                                                    const float *__restrict__ bias, float *out, float *pre,
-                                                    int R, int K, int J, int relu, int accum) {
-  __shared__ float ws[HID * HID], ws2[HID * HID];
-  __shared__ float at[ROWS * HID], at2[ROWS * HID];
-  const int r0 = blockIdx.x * ROWS;
-  for (int i = threadIdx.x; i < K * J; i += TB) {
-    const int k = i / J, j = i - k * J;
-    const int src = TRANS ? j * K + k : k * J + j;
-    ws[i] = __bfloat162float(W[src]);
-    if (W2) ws2[i] = __bfloat162float(W2[src]);
-  }
-  for (int i = threadIdx.x; i < ROWS * K; i += TB) {
-    const int rr = i / K, k = i - rr * K;
-    const int r = r0 + rr;
-    at[i] = r < R ? a[(size_t)r * K + k] : 0.f;
-    if (a2) at2[i] = r < R ? a2[(size_t)r * K + k] : 0.f;
-  }
-  __syncthreads();
-  for (int o = threadIdx.x; o < ROWS * J; o += TB) {
-    const int rr = o / J, j = o - rr * J;
-    const int r = r0 + rr;
-    if (r >= R) continue;
-    float s = 0.f;
-    for (int k = 0; k < K; ++k) s = fmaf(at[rr * K + k], ws[k * J + j], s);
-    if (a2)
-      for (int k = 0; k < K; ++k) s = fmaf(at2[rr * K + k], ws2[k * J + j], s);
-    if (bias) s += bias[j];
-    const size_t oi = (size_t)r * J + j;
-    if (accum) s += out[oi];
-    if (pre) pre[oi] = s;
-    out[oi] = relu ? fmaxf(s, 0.f) : s;
-  }
+// Neighbours of a node: the first four (-1 = none) and their weights, the
+// rest at ptr[n] + 4 .. ptr[n + 1] of the CSR arrays.
+struct Graph {
+  const int *ptr, *nbr;
+  const float *w;      // A's weights, or A^T's
+  const int4 *nbr4;
+  const float4 *w4;
+  int N;
+};
+
+__device__ __forceinline__ float4 fma4(float a, const float4 &x, const float4 &s) {
+  return make_float4(fmaf(a, x.x, s.x), fmaf(a, x.y, s.y), fmaf(a, x.z, s.z), fmaf(a, x.w, s.w));
 }
 
-// The same for J = 64 outputs, register-tiled: a CTA computes TROWS rows x
-// 64 columns, each thread 8 rows x 4 columns in registers (32 products per
-// 12 shared-memory reads), with the layer's weights staged once per TROWS
-// rows (the kernel above re-stages them for every 32 rows and runs one
-// dependent chain of K products per output).  Shared memory: the weights
-// [K][64] (twice with a2) and the row tiles [TROWS][K + 1] (the padding
-// spreads a column's rows over the banks).
-constexpr int TROWS = 128;
-
-__host__ __device__ inline size_t linear64_smem(int K, bool two) {
-  return ((size_t)(two ? 2 : 1) * (K * HID + TROWS * (K + 1))) * sizeof(float);
+// sum_j w[j] in[t, nbr[j]][4 c4 ..] over row r's neighbours, in CSR order;
+// the first four rows are requested together
+__device__ __forceinline__ float4 gather4(const Graph &g, const float *__restrict__ in, int r, int c4) {
+  const int t = r / g.N, n = r - t * g.N;
+  const int4 nb = g.nbr4[n];
+  const float4 w = g.w4[n];
+  const float *base = in + (size_t)t * g.N * HID + 4 * c4;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto row = [&](int j) { return *reinterpret_cast<const float4 *>(base + (size_t)j * HID); };
+  const float4 x0 = nb.x >= 0 ? row(nb.x) : z, x1 = nb.y >= 0 ? row(nb.y) : z;
+  const float4 x2 = nb.z >= 0 ? row(nb.z) : z, x3 = nb.w >= 0 ? row(nb.w) : z;
+  float4 s = z;
+  if (nb.x >= 0) s = fma4(w.x, x0, s);
+  if (nb.y >= 0) s = fma4(w.y, x1, s);
+  if (nb.z >= 0) s = fma4(w.z, x2, s);
+  if (nb.w >= 0) {
+    s = fma4(w.w, x3, s);
+    for (int j = g.ptr[n] + 4; j < g.ptr[n + 1]; ++j) s = fma4(g.w[j], row(g.nbr[j]), s);
+  }
+  return s;
 }
 
+// a layer's weights [64][64] into shared memory as FP32, ws[k][j] = W[k][j],
+// or W[j][k] with TRANS
 template <bool TRANS>
-__global__ void __launch_bounds__(TB) linear64_kernel(const float *__restrict__ a, const __nv_bfloat16 *__restrict__ W,
-                                                      const float *__restrict__ a2,
-                                                      const __nv_bfloat16 *__restrict__ W2,
-                                                      const float *__restrict__ bias, float *out, float *pre, int R,
-                                                      int K, int relu, int accum) {
-  extern __shared__ float sm64[];
-  const int KP = K + 1;
-  float *ws = sm64, *at = ws + K * HID;
-  float *ws2 = at + TROWS * KP, *at2 = ws2 + K * HID;
-  const int r0 = blockIdx.x * TROWS;
-  for (int i = threadIdx.x; i < K * HID; i += TB) {
+__device__ __forceinline__ void stage_weights(float *ws, const __nv_bfloat16 *__restrict__ W) {
+  for (int i = threadIdx.x; i < HID * HID; i += LB) {
     const int k = i / HID, j = i - k * HID;
-    const int src = TRANS ? j * K + k : k * HID + j;
-    ws[i] = __bfloat162float(W[src]);
-    if (a2) ws2[i] = __bfloat162float(W2[src]);
+    ws[i] = __bfloat162float(W[TRANS ? j * HID + k : i]);
   }
-  for (int i = threadIdx.x; i < TROWS * K; i += TB) {
-    const int rr = i / K, k = i - rr * K;
-    const int r = r0 + rr;
-    at[rr * KP + k] = r < R ? a[(size_t)r * K + k] : 0.f;
-    if (a2) at2[rr * KP + k] = r < R ? a2[(size_t)r * K + k] : 0.f;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // columns 4 tx .. 4 tx + 3, rows 8 ty .. 8 ty + 7
-  float acc[8][4];
+}
+
+// acc[i][c] += sum_k at[4 ty + i][k] ws[k][4 tx + c], k in order; a thread's
+// rows are read four k at a time, so that the products outnumber the
+// shared-memory wavefronts (64 to 48 per four warps)
+__device__ __forceinline__ void tile_mma(float (&acc)[4][4], const float *__restrict__ at,
+                                         const float *__restrict__ ws, int tx, int ty) {
+#pragma unroll 4
+  for (int k = 0; k < HID; k += 4) {
+    float a[4][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 4; ++i) {
+      const float4 v = *reinterpret_cast<const float4 *>(at + (4 * ty + i) * AS + k);
+      a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
+    }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
-  for (int pass = 0; pass < (a2 ? 2 : 1); ++pass) {
-    const float *A = pass ? at2 : at, *Ws = pass ? ws2 : ws;
-    for (int k = 0; k < K; ++k) {
-      const float4 w4 = *reinterpret_cast<const float4 *>(Ws + k * HID + 4 * tx);
+    for (int q = 0; q < 4; ++q) {
+      const float4 w = *reinterpret_cast<const float4 *>(ws + (k + q) * HID + 4 * tx);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float av = A[(8 * ty + i) * KP + k];
-        acc[i][0] = fmaf(av, w4.x, acc[i][0]);
-        acc[i][1] = fmaf(av, w4.y, acc[i][1]);
-        acc[i][2] = fmaf(av, w4.z, acc[i][2]);
-        acc[i][3] = fmaf(av, w4.w, acc[i][3]);
+      for (int i = 0; i < 4; ++i) {
+        acc[i][0] = fmaf(a[i][q], w.x, acc[i][0]);
+        acc[i][1] = fmaf(a[i][q], w.y, acc[i][1]);
+        acc[i][2] = fmaf(a[i][q], w.z, acc[i][2]);
+        acc[i][3] = fmaf(a[i][q], w.w, acc[i][3]);
       }
     }
   }
-  float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (bias) b4 = *reinterpret_cast<const float4 *>(bias + 4 * tx);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = r0 + 8 * ty + i;
-    if (r >= R) break;
-    const size_t oi = (size_t)r * HID + 4 * tx;
-    float4 v = make_float4(acc[i][0] + b4.x, acc[i][1] + b4.y, acc[i][2] + b4.z, acc[i][3] + b4.w);
-    if (accum) {
-      const float4 o = *reinterpret_cast<const float4 *>(out + oi);
-      v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
-    }
-    if (pre) *reinterpret_cast<float4 *>(pre + oi) = v;
-    if (relu) {
-      v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
-    }
-    *reinterpret_cast<float4 *>(out + oi) = v;
-  }
 }
 
-// out[t, n][c] = sum_{j in ptr[n]..ptr[n+1]} w[j] in[t, nbr[j]][c]
-__global__ void __launch_bounds__(TB) agg_kernel(const float *__restrict__ in, float *__restrict__ out,
-                                                 const int *__restrict__ ptr, const int *__restrict__ nbr,
-                                                 const float *__restrict__ w, int N, int R) {
-  const size_t total = (size_t)R * HID;
-  for (size_t i = (size_t)blockIdx.x * TB + threadIdx.x; i < total; i += (size_t)gridDim.x * TB) {
-    const int r = (int)(i / HID), c = (int)(i - (size_t)r * HID);
-    const int t = r / N, n = r - t * N;
-    float s = 0.f;
-    for (int j = ptr[n]; j < ptr[n + 1]; ++j) s = fmaf(w[j], in[((size_t)t * N + nbr[j]) * HID + c], s);
-    out[i] = s;
-  }
-}
-
-// g *= (z > 0)
-__global__ void __launch_bounds__(TB) relu_bwd_kernel(float *g, const float *__restrict__ z, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * TB + threadIdx.x; i < n; i += (size_t)gridDim.x * TB)
-    if (!(z[i] > 0.f)) g[i] = 0.f;
-}
-
-// part[cta][k][j] = sum over the CTA's rows of a[r][k] g[r][j] (a == NULL:
-// a = 1, K = 1, the bias gradient)
-__global__ void __launch_bounds__(TB) wgrad_part_kernel(const float *__restrict__ a, const float *__restrict__ g,
-                                                        float *__restrict__ part, int R, int K, int J) {
-  __shared__ float at[ROWS * HID], gt[ROWS * HID];
-  const int r0 = blockIdx.x * GRAD_ROWS, r1 = min(R, r0 + GRAD_ROWS);
-  float acc[16];
-#pragma unroll
-  for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-  for (int rb = r0; rb < r1; rb += ROWS) {
-    const int nr = min(ROWS, r1 - rb);
-    __syncthreads();
-    for (int i = threadIdx.x; i < ROWS * K; i += TB) {
-      const int rr = i / K, k = i - rr * K;
-      at[i] = rr < nr ? (a ? a[(size_t)(rb + rr) * K + k] : 1.f) : 0.f;
-    }
-    for (int i = threadIdx.x; i < ROWS * J; i += TB) {
-      const int rr = i / J, j = i - rr * J;
-      gt[i] = rr < nr ? g[(size_t)(rb + rr) * J + j] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int o = threadIdx.x + q * TB;
-      if (o < K * J) {
-        const int k = o / J, j = o - k * J;
-        float s = acc[q];
-        for (int rr = 0; rr < nr; ++rr) s = fmaf(at[rr * K + k], gt[rr * J + j], s);
-        acc[q] = s;
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const int o = threadIdx.x + q * TB;
-    if (o < K * J) part[(size_t)blockIdx.x * K * J + o] = acc[q];
-  }
-}
-
-// The same for J = 64 and K <= 64, register-tiled: thread (ty, tx) keeps the
-// 4 x 4 block k = 4 ty .., j = 4 tx .. of the partial sums (16 products per 8
-// shared-memory reads); every output still sums the CTA's rows in order, so
-// the partial sums equal the kernel above's.
-__global__ void __launch_bounds__(TB) wgrad64_part_kernel(const float *__restrict__ a, const float *__restrict__ g,
-                                                          float *__restrict__ part, int R, int K) {
-  __shared__ __align__(16) float at[ROWS * HID], gt[ROWS * HID];
-  const int r0 = blockIdx.x * GRAD_ROWS, r1 = min(R, r0 + GRAD_ROWS);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[4][4];
+__device__ __forceinline__ void zero_acc(float (&acc)[4][4]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
-  for (int rb = r0; rb < r1; rb += ROWS) {
-    const int nr = min(ROWS, r1 - rb);
+}
+
+__device__ __forceinline__ float4 relu4(const float4 &v) {
+  return make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+}
+
+// H0 = relu(X W0 + b0), X [R][K], K <= 64
+__global__ void __launch_bounds__(LB) input_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ W,
+                                                   const float *__restrict__ bias, float *__restrict__ out, int R,
+                                                   int K) {
+  __shared__ __align__(16) float ws[HID * HID], at[TR * AS];
+  for (int i = threadIdx.x; i < K * HID; i += LB) ws[i] = __bfloat162float(W[i]);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const float4 b4 = *reinterpret_cast<const float4 *>(bias + 4 * tx);
+  for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
+    const int nr = min(TR, R - r0);
     __syncthreads();
-    for (int i = threadIdx.x; i < ROWS * HID; i += TB) {
-      const int rr = i / HID, k = i - rr * HID;
-      at[i] = (rr < nr && k < K) ? a[(size_t)(rb + rr) * K + k] : 0.f;
-      gt[i] = rr < nr ? g[(size_t)(rb + rr) * HID + k] : 0.f;
+    for (int i = threadIdx.x; i < TR * K; i += LB) {   // a tile's rows are one run
+      const int rr = i / K;
+      at[rr * AS + i - rr * K] = rr < nr ? x[(size_t)r0 * K + i] : 0.f;
     }
     __syncthreads();
+    float acc[4][4];
+    zero_acc(acc);
+    for (int k = 0; k < K; ++k) {
+      const float4 w = *reinterpret_cast<const float4 *>(ws + k * HID + 4 * tx);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float a = at[(4 * ty + i) * AS + k];
+        acc[i][0] = fmaf(a, w.x, acc[i][0]);
+        acc[i][1] = fmaf(a, w.y, acc[i][1]);
+        acc[i][2] = fmaf(a, w.z, acc[i][2]);
+        acc[i][3] = fmaf(a, w.w, acc[i][3]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int rr = 4 * ty + i;
+      if (rr >= nr) break;
+      *reinterpret_cast<float4 *>(out + (size_t)(r0 + rr) * HID + 4 * tx) =
+          relu4(make_float4(acc[i][0] + b4.x, acc[i][1] + b4.y, acc[i][2] + b4.z, acc[i][3] + b4.w));
+    }
+  }
+}
+
+// One message-passing layer: M = A H (kept where m is not NULL), H' = relu(H
+// Ws + M Wn + b).  LAST: also Y = H' Wo + bo; H' is kept where out is not NULL.
+// Dynamic shared memory: LAYER_SMEM.
+constexpr size_t LAYER_SMEM = (2 * HID * HID + 2 * TR * AS) * sizeof(float);
+template <bool LAST>
+__global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__restrict__ h,
+                                                      const __nv_bfloat16 *__restrict__ Ws,
+                                                      const __nv_bfloat16 *__restrict__ Wn,
+                                                      const float *__restrict__ bias, float *__restrict__ m,
+                                                      float *__restrict__ out, const __nv_bfloat16 *__restrict__ Wo,
+                                                      const float *__restrict__ bo, float *__restrict__ y, int R) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float wo[LAST ? HID * NOUT : 1];
+  float *ws = sm, *wn = ws + HID * HID, *at = wn + HID * HID, *am = at + TR * AS;
+  stage_weights<false>(ws, Ws);
+  stage_weights<false>(wn, Wn);
+  if constexpr (LAST)
+    for (int i = threadIdx.x; i < HID * NOUT; i += LB) wo[i] = __bfloat162float(Wo[i]);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const float4 b4 = *reinterpret_cast<const float4 *>(bias + 4 * tx), z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
+    __syncthreads();
+#pragma unroll 2
+    for (int q = 0; q < TR / 8; ++q) {   // 16 threads a row
+      const int rr = ty + 8 * q, r = r0 + rr;
+      const bool in = r < R;
+      const size_t o = (size_t)r * HID + 4 * tx;
+      const float4 v = in ? *reinterpret_cast<const float4 *>(h + o) : z;
+      const float4 a = in ? gather4(g, h, r, tx) : z;
+      *reinterpret_cast<float4 *>(at + rr * AS + 4 * tx) = v;
+      *reinterpret_cast<float4 *>(am + rr * AS + 4 * tx) = a;
+      if (m && in) *reinterpret_cast<float4 *>(m + o) = a;
+    }
+    __syncthreads();
+    float acc[4][4];
+    zero_acc(acc);
+    tile_mma(acc, at, ws, tx, ty);
+    tile_mma(acc, am, wn, tx, ty);
+    if constexpr (LAST) __syncthreads();   // at takes the output rows
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int rr = 4 * ty + i, r = r0 + rr;
+      const float4 v = relu4(make_float4(acc[i][0] + b4.x, acc[i][1] + b4.y, acc[i][2] + b4.z, acc[i][3] + b4.w));
+      if (out && r < R) *reinterpret_cast<float4 *>(out + (size_t)r * HID + 4 * tx) = v;
+      if constexpr (LAST) *reinterpret_cast<float4 *>(at + rr * AS + 4 * tx) = v;
+    }
+    if constexpr (LAST) {
+      __syncthreads();
+      const int rr = threadIdx.x / NOUT, j = threadIdx.x % NOUT, r = r0 + rr;
+      if (rr < TR && r < R) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < HID; k += 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(at + rr * AS + k);
+          s = fmaf(v.x, wo[k * NOUT + j], s);
+          s = fmaf(v.y, wo[(k + 1) * NOUT + j], s);
+          s = fmaf(v.z, wo[(k + 2) * NOUT + j], s);
+          s = fmaf(v.w, wo[(k + 3) * NOUT + j], s);
+        }
+        y[(size_t)r * NOUT + j] = s + bo[j];
+      }
+    }
+  }
+}
+
+// One layer backwards: the adjoint of its output H' -- dY Wo^T (FIRST), else
+// dS + A^T dM of the layer above -- masked where H' > 0 into dZ, and, unless
+// dm is NULL (the input layer), dM = dZ Wn^T and dS = dZ Ws^T for the layer
+// below.  Dynamic shared memory: BACK_SMEM.
+constexpr size_t BACK_SMEM = (2 * HID * HID + TR * AS) * sizeof(float);
+template <bool FIRST>
+__global__ void __launch_bounds__(LB, 4) back_kernel(Graph g, const float *__restrict__ dy,
+                                                     const __nv_bfloat16 *__restrict__ Wo,
+                                                     const float *__restrict__ ds_up, const float *__restrict__ dm_up,
+                                                     const float *__restrict__ h, const __nv_bfloat16 *__restrict__ Ws,
+                                                     const __nv_bfloat16 *__restrict__ Wn, float *__restrict__ dz,
+                                                     float *__restrict__ dm, float *__restrict__ ds, int R) {
+  extern __shared__ __align__(16) float sm[];
+  float *ws = sm, *wn = ws + HID * HID, *at = wn + HID * HID;
+  if (dm) {
+    stage_weights<true>(ws, Ws);
+    stage_weights<true>(wn, Wn);
+  }
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  float wo[4][NOUT];
+  if constexpr (FIRST) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int j = 0; j < NOUT; ++j) wo[c][j] = __bfloat162float(Wo[(4 * tx + c) * NOUT + j]);
+  }
+  for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
+    __syncthreads();
+#pragma unroll 2
+    for (int q = 0; q < TR / 8; ++q) {
+      const int rr = ty + 8 * q, r = r0 + rr;
+      const size_t o = (size_t)r * HID + 4 * tx;
+      float4 d = z;
+      if (r < R) {
+        const float4 hv = *reinterpret_cast<const float4 *>(h + o);
+        if constexpr (FIRST) {
+          const float2 e = *reinterpret_cast<const float2 *>(dy + (size_t)r * NOUT);
+          d = make_float4(fmaf(e.y, wo[0][1], e.x * wo[0][0]), fmaf(e.y, wo[1][1], e.x * wo[1][0]),
+                          fmaf(e.y, wo[2][1], e.x * wo[2][0]), fmaf(e.y, wo[3][1], e.x * wo[3][0]));
+        } else {
+          const float4 sv = *reinterpret_cast<const float4 *>(ds_up + o), a = gather4(g, dm_up, r, tx);
+          d = make_float4(sv.x + a.x, sv.y + a.y, sv.z + a.z, sv.w + a.w);
+        }
+        if (!(hv.x > 0.f)) d.x = 0.f;
+        if (!(hv.y > 0.f)) d.y = 0.f;
+        if (!(hv.z > 0.f)) d.z = 0.f;
+        if (!(hv.w > 0.f)) d.w = 0.f;
+        *reinterpret_cast<float4 *>(dz + o) = d;
+      }
+      if (dm) *reinterpret_cast<float4 *>(at + rr * AS + 4 * tx) = d;
+    }
+    if (!dm) continue;
+    __syncthreads();
+    float acc[4][4];
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      zero_acc(acc);
+      tile_mma(acc, at, pass ? ws : wn, tx, ty);
+      float *o = pass ? ds : dm;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + 4 * ty + i;
+        if (r < R)
+          *reinterpret_cast<float4 *>(o + (size_t)r * HID + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      }
+    }
+  }
+}
+
+// Partial weight gradients over rows GRAD_ROWS blockIdx.x ..: part[k][j] =
+// sum over the rows in order of a[r][k] g[r][j], a [R][K] and g [R][64].
+// blockIdx.y: up to two such products over the same g (a0 into column p0 of
+// the partial's parameter vector, then a1 into p1), GK values of k each; the
+// first also sums g itself (pb, the bias).  vec: a's rows are 64 floats on
+// 16-byte boundaries (the network's own arrays; the caller's features need
+// not be).  A thread keeps a 4 x 4 block in
+// registers (16 products per two shared-memory reads); splitting k over CTAs
+// gives ten small CTAs per SM at 48,000 rows where one CTA per row range left
+// the second wave nearly empty (32 us a product, now @@ for two).
+__global__ void __launch_bounds__(GB) wgrad_kernel(const float *__restrict__ a0, const float *__restrict__ a1,
+                                                   const float *__restrict__ g, float *__restrict__ part, int R, int K,
+                                                   long long C, long long p0, long long p1, long long pb, int vec) {
+  __shared__ __align__(16) float at[GS * GK], gt[GS * HID];
+  const int nk = (K + GK - 1) / GK, second = blockIdx.y >= nk, k0 = (blockIdx.y - (second ? nk : 0)) * GK;
+  const float *a = second ? a1 : a0;
+  float *out = part + (size_t)blockIdx.x * C;
+  const int r0 = blockIdx.x * GRAD_ROWS, r1 = min(R, r0 + GRAD_ROWS);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // j = 4 tx .., k = k0 + 4 ty ..
+  const bool bias = blockIdx.y == 0 && ty == 0;
+  float acc[4][4], ab[4] = {0.f, 0.f, 0.f, 0.f};
+  zero_acc(acc);
+  for (int rb = r0; rb < r1; rb += GS) {
+    const int nr = min(GS, r1 - rb);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * (HID / 4); i += GB)
+      reinterpret_cast<float4 *>(gt)[i] = reinterpret_cast<const float4 *>(g + (size_t)rb * HID)[i];
+    if (vec) {
+      for (int i = threadIdx.x; i < nr * (GK / 4); i += GB) {
+        const int rr = i / (GK / 4), c = i % (GK / 4);
+        reinterpret_cast<float4 *>(at)[i] = *reinterpret_cast<const float4 *>(a + (size_t)(rb + rr) * HID + k0 + 4 * c);
+      }
+    } else {
+      for (int i = threadIdx.x; i < nr * GK; i += GB) {
+        const int rr = i / GK, k = k0 + i % GK;
+        at[i] = k < K ? a[(size_t)(rb + rr) * K + k] : 0.f;
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
     for (int rr = 0; rr < nr; ++rr) {
-      const float4 a4 = *reinterpret_cast<const float4 *>(at + rr * HID + 4 * ty);
+      const float4 a4 = *reinterpret_cast<const float4 *>(at + rr * GK + 4 * ty);
       const float4 g4 = *reinterpret_cast<const float4 *>(gt + rr * HID + 4 * tx);
       const float av[4] = {a4.x, a4.y, a4.z, a4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[i][c] = fmaf(av[i], gv[c], acc[i][c]);
+      if (bias)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ab[c] += gv[c];
     }
   }
+  float *w = out + (second ? p1 : p0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int k = 4 * ty + i;
-    if (k < K)
-      *reinterpret_cast<float4 *>(part + (size_t)blockIdx.x * K * HID + (size_t)k * HID + 4 * tx) =
-          make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    const int k = k0 + 4 * ty + i;
+    if (k >= K) break;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w[(size_t)k * HID + 4 * tx + c] = acc[i][c];
   }
+  if (bias)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[pb + 4 * tx + c] = ab[c];
 }
 
-// grad[o] = sum over CTAs c (in order) of part[c][o]
-__global__ void __launch_bounds__(TB) wgrad_sum_kernel(const float *__restrict__ part, float *__restrict__ grad,
-                                                       int n_part, int KJ) {
-  const int o = blockIdx.x * TB + threadIdx.x;
-  if (o >= KJ) return;
+// the same for the output layer: dWo = H^T dY [64][2] and dbo
+constexpr int OB = HID * NOUT;
+__global__ void __launch_bounds__(OB) wgrad_out_kernel(const float *__restrict__ h, const float *__restrict__ dy,
+                                                       float *__restrict__ part, int R, long long C, long long pw,
+                                                       long long pb) {
+  __shared__ __align__(16) float ht[2 * GS * HID], gt[2 * GS * NOUT];
+  constexpr int ST = 2 * GS;
+  const int r0 = blockIdx.x * GRAD_ROWS, r1 = min(R, r0 + GRAD_ROWS);
+  const int k = threadIdx.x / NOUT, j = threadIdx.x % NOUT;
+  float s = 0.f, b = 0.f;
+  for (int rb = r0; rb < r1; rb += ST) {
+    const int nr = min(ST, r1 - rb);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * (HID / 4); i += OB)
+      reinterpret_cast<float4 *>(ht)[i] = reinterpret_cast<const float4 *>(h + (size_t)rb * HID)[i];
+    for (int i = threadIdx.x; i < nr * NOUT; i += OB) gt[i] = dy[(size_t)rb * NOUT + i];
+    __syncthreads();
+#pragma unroll 8
+    for (int rr = 0; rr < nr; ++rr) {
+      const float gv = gt[rr * NOUT + j];
+      s = fmaf(ht[rr * HID + k], gv, s);
+      b += gv;
+    }
+  }
+  float *out = part + (size_t)blockIdx.x * C;
+  out[pw + k * NOUT + j] = s;
+  if (k == 0) out[pb + j] = b;
+}
+
+// The partial sums reduced in order, grad[o] = sum over c of part[c][o], and
+// with ADAM the step on the FP32 parameters and their bfloat16 copy
+template <bool ADAM>
+__global__ void __launch_bounds__(TB) grad_kernel(const float *__restrict__ part, float *__restrict__ grad, int n_part,
+                                                  long long n, float *p, float *m, float *v, __nv_bfloat16 *pb,
+                                                  float lr, float bc1, float bc2) {
+  const long long i = (long long)blockIdx.x * TB + threadIdx.x;
+  if (i >= n) return;
   float s = 0.f;
-  for (int c = 0; c < n_part; ++c) s += part[(size_t)c * KJ + o];
-  grad[o] = s;
+#pragma unroll 16
+  for (int c = 0; c < n_part; ++c) s += part[(size_t)c * n + i];
+  grad[i] = s;
+  if constexpr (ADAM) {
+    const float mi = 0.9f * m[i] + 0.1f * s;
+    const float vi = 0.999f * v[i] + 0.001f * s * s;
+    m[i] = mi;
+    v[i] = vi;
+    const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
+    p[i] = pi;
+    pb[i] = __float2bfloat16_rn(pi);
+  }
 }
 
 // dY = 2 scale (Y - Y*) / R; per-CTA partial loss sums (FP64)
@@ -284,21 +440,6 @@ __global__ void __launch_bounds__(TB) loss_kernel(const float *__restrict__ y, c
   if (threadIdx.x == 0) lpart[blockIdx.x] = red[0];
 }
 
-// Adam on the FP32 parameters, then their bfloat16 copy
-__global__ void __launch_bounds__(TB) adam_kernel(float *p, const float *__restrict__ g, float *m, float *v,
-                                                  __nv_bfloat16 *pb, long long n, float lr, float bc1, float bc2) {
-  for (long long i = (long long)blockIdx.x * TB + threadIdx.x; i < n; i += (long long)gridDim.x * TB) {
-    const float gi = g[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi;
-    const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
-    p[i] = pi;
-    pb[i] = __float2bfloat16_rn(pi);
-  }
-}
-
 __global__ void __launch_bounds__(TB) to_bf16_kernel(const float *__restrict__ p, __nv_bfloat16 *pb, long long n) {
   for (long long i = (long long)blockIdx.x * TB + threadIdx.x; i < n; i += (long long)gridDim.x * TB)
     pb[i] = __float2bfloat16_rn(p[i]);
@@ -319,10 +460,14 @@ struct opf_wsnet {
   float *wA = nullptr, *wAT = nullptr;
   float *P = nullptr, *G = nullptr, *Mo = nullptr, *Vo = nullptr;
   __nv_bfloat16 *Pb = nullptr;
-  float *Z0 = nullptr, *H0 = nullptr, *M[NMP] = {}, *Z[NMP] = {}, *H[NMP] = {}, *Y = nullptr;
-  float *dY = nullptr, *dA = nullptr, *dB = nullptr, *dC = nullptr, *part = nullptr;
+  int4 *nbr4 = nullptr;
+  float4 *wA4 = nullptr, *wAT4 = nullptr;
+  float *H0 = nullptr, *M[NMP] = {}, *H[NMP] = {}, *Y = nullptr;
+  // dM and dS of a layer, read at the neighbours by the layer below: two of each
+  float *dY = nullptr, *dZ = nullptr, *dM[2] = {}, *dS[2] = {}, *part = nullptr;
   double *lpart = nullptr;
   int n_lpart = 0, n_gpart = 0;
+  int g_in = 0, g_layer = 0, g_back = 0;   // persistent CTAs of the layer kernels
   std::vector<void *> allocs;
 };
 
@@ -372,71 +517,66 @@ void he_init(std::vector<float> &p, const opf_wsnet *w, uint64_t seed) {
   fill(w->oWo, HID, HID * NOUT);
 }
 
-void launch_linear(const opf_wsnet *w, bool trans, const float *a, long long oW, const float *a2, long long oW2,
-                   const float *bias, float *out, float *pre, int K, int J, bool relu, bool accum) {
-  const __nv_bfloat16 *W = w->Pb + oW, *W2 = a2 ? w->Pb + oW2 : nullptr;
-  if (J == HID) {
-    const int g = (w->R + TROWS - 1) / TROWS;
-    const size_t sm = linear64_smem(K, a2 != nullptr);
-    if (trans)
-      linear64_kernel<true><<<g, TB, sm, w->stream>>>(a, W, a2, W2, bias, out, pre, w->R, K, relu, accum);
-    else
-      linear64_kernel<false><<<g, TB, sm, w->stream>>>(a, W, a2, W2, bias, out, pre, w->R, K, relu, accum);
-    return;
-  }
-  const int grid = (w->R + ROWS - 1) / ROWS;
-  if (trans)
-    linear_kernel<true><<<grid, TB, 0, w->stream>>>(a, W, a2, W2, bias, out, pre, w->R, K, J, relu, accum);
-  else
-    linear_kernel<false><<<grid, TB, 0, w->stream>>>(a, W, a2, W2, bias, out, pre, w->R, K, J, relu, accum);
+Graph graph(const opf_wsnet *w, bool transposed) {
+  return Graph{w->ptr, w->nbr, transposed ? w->wAT : w->wA, w->nbr4, transposed ? w->wAT4 : w->wA4, w->N};
 }
 
-void launch_wgrad(opf_wsnet *w, const float *a, const float *g, int K, int J, long long off) {
-  if (a && J == HID)
-    wgrad64_part_kernel<<<w->n_gpart, TB, 0, w->stream>>>(a, g, w->part, w->R, K);
-  else
-    wgrad_part_kernel<<<w->n_gpart, TB, 0, w->stream>>>(a, g, w->part, w->R, K, J);
-  wgrad_sum_kernel<<<(K * J + TB - 1) / TB, TB, 0, w->stream>>>(w->part, w->G + off, w->n_gpart, K * J);
-}
-
-void forward(opf_wsnet *w, const float *x) {
-  const int R = w->R;
-  launch_linear(w, false, x, w->oW0, nullptr, 0, w->P + w->ob0, w->H0, w->Z0, w->F, HID, true, false);
+// Y (into y); keep: the activations the backward pass reads
+void forward(opf_wsnet *w, const float *x, float *y, bool keep) {
+  const Graph g = graph(w, false);
+  input_kernel<<<w->g_in, LB, 0, w->stream>>>(x, w->Pb + w->oW0, w->P + w->ob0, w->H0, w->R, w->F);
   const float *h = w->H0;
   for (int l = 0; l < NMP; ++l) {
-    agg_kernel<<<grid_for((size_t)R * HID), TB, 0, w->stream>>>(h, w->M[l], w->ptr, w->nbr, w->wA, w->N, R);
-    launch_linear(w, false, h, w->oWs[l], w->M[l], w->oWn[l], w->P + w->ob[l], w->H[l], w->Z[l], HID, HID, true,
-                  false);
+    const bool last = l == NMP - 1;
+    const __nv_bfloat16 *Ws = w->Pb + w->oWs[l], *Wn = w->Pb + w->oWn[l];
+    const float *b = w->P + w->ob[l];
+    float *m = keep ? w->M[l] : nullptr;
+    if (last)
+      layer_kernel<true><<<w->g_layer, LB, LAYER_SMEM, w->stream>>>(g, h, Ws, Wn, b, m, keep ? w->H[l] : nullptr,
+                                                                     w->Pb + w->oWo, w->P + w->obo, y, w->R);
+    else
+      layer_kernel<false><<<w->g_layer, LB, LAYER_SMEM, w->stream>>>(g, h, Ws, Wn, b, m, w->H[l], nullptr, nullptr,
+                                                                      nullptr, w->R);
     h = w->H[l];
   }
-  launch_linear(w, false, h, w->oWo, nullptr, 0, w->P + w->obo, w->Y, nullptr, HID, NOUT, false, false);
 }
 
-// loss partials and the gradient in w->G
+// loss partials and the partial weight gradients (grad_kernel finishes them)
 void backward(opf_wsnet *w, const float *x, const float *yt, const float scale[2]) {
   const int R = w->R;
-  const size_t RH = (size_t)R * HID;
+  const Graph g = graph(w, true);
   loss_kernel<<<w->n_lpart, TB, 0, w->stream>>>(w->Y, yt, w->dY, w->lpart, R, scale[0], scale[1]);
-  launch_wgrad(w, w->H[NMP - 1], w->dY, HID, NOUT, w->oWo);
-  launch_wgrad(w, nullptr, w->dY, 1, NOUT, w->obo);
-  // dH = dY Wo^T
-  float *dH = w->dA, *dM = w->dB, *tmp = w->dC;
-  launch_linear(w, true, w->dY, w->oWo, nullptr, 0, nullptr, dH, nullptr, NOUT, HID, false, false);
+  wgrad_out_kernel<<<w->n_gpart, OB, 0, w->stream>>>(w->H[NMP - 1], w->dY, w->part, R, w->C, w->oWo, w->obo);
   for (int l = NMP - 1; l >= 0; --l) {
-    relu_bwd_kernel<<<grid_for(RH), TB, 0, w->stream>>>(dH, w->Z[l], RH);   // dZ, in place
-    const float *hin = l == 0 ? w->H0 : w->H[l - 1];
-    launch_wgrad(w, hin, dH, HID, HID, w->oWs[l]);
-    launch_wgrad(w, w->M[l], dH, HID, HID, w->oWn[l]);
-    launch_wgrad(w, nullptr, dH, 1, HID, w->ob[l]);
-    // dM = dZ Wn^T; dH_in = A^T dM + dZ Ws^T
-    launch_linear(w, true, dH, w->oWn[l], nullptr, 0, nullptr, dM, nullptr, HID, HID, false, false);
-    agg_kernel<<<grid_for(RH), TB, 0, w->stream>>>(dM, tmp, w->ptr, w->nbr, w->wAT, w->N, R);
-    launch_linear(w, true, dH, w->oWs[l], nullptr, 0, nullptr, tmp, nullptr, HID, HID, false, true);
-    std::swap(dH, tmp);
+    const int i = l & 1, up = i ^ 1;
+    const __nv_bfloat16 *Ws = w->Pb + w->oWs[l], *Wn = w->Pb + w->oWn[l];
+    if (l == NMP - 1)
+      back_kernel<true><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, w->dY, w->Pb + w->oWo, nullptr, nullptr, w->H[l], Ws,
+                                                                  Wn, w->dZ, w->dM[i], w->dS[i], R);
+    else
+      back_kernel<false><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, nullptr, nullptr, w->dS[up], w->dM[up], w->H[l], Ws,
+                                                                   Wn, w->dZ, w->dM[i], w->dS[i], R);
+    const dim3 grid(w->n_gpart, 2 * HID / GK);
+    wgrad_kernel<<<grid, GB, 0, w->stream>>>(l == 0 ? w->H0 : w->H[l - 1], w->M[l], w->dZ, w->part, R, HID, w->C,
+                                             w->oWs[l], w->oWn[l], w->ob[l], 1);
   }
-  relu_bwd_kernel<<<grid_for(RH), TB, 0, w->stream>>>(dH, w->Z0, RH);
-  launch_wgrad(w, x, dH, w->F, HID, w->oW0);
-  launch_wgrad(w, nullptr, dH, 1, HID, w->ob0);
+  back_kernel<false><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, nullptr, nullptr, w->dS[0], w->dM[0], w->H0, nullptr,
+                                                               nullptr, w->dZ, nullptr, nullptr, R);
+  const dim3 grid(w->n_gpart, (w->F + GK - 1) / GK);
+  wgrad_kernel<<<grid, GB, 0, w->stream>>>(x, nullptr, w->dZ, w->part, R, w->F, w->C, w->oW0, 0, w->ob0, 0);
+}
+
+// persistent CTAs of a layer kernel: what is resident, or one per tile
+template <class Fn>
+cudaError_t layer_grid(Fn fn, size_t smem, int R, int *grid) {
+  int dev = 0, sms = 0, nb = 0;
+  cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                   : cudaSuccess;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, LB, smem);
+  *grid = std::max(1, std::min((R + TR - 1) / TR, std::max(nb, 1) * sms));
+  return e;
 }
 
 opf_status read_loss(opf_wsnet *w, double *loss) {
@@ -529,27 +669,48 @@ opf_status opf_wsnet_create(int32_t n_nodes, int32_t n_lines, const int32_t *lin
   A(&w->Mo, w->C);
   A(&w->Vo, w->C);
   A(&w->Pb, w->C);
-  A(&w->Z0, RH);
+  A(&w->nbr4, n_nodes);
+  A(&w->wA4, n_nodes);
+  A(&w->wAT4, n_nodes);
   A(&w->H0, RH);
   for (int l = 0; l < NMP; ++l) {
     A(&w->M[l], RH);
-    A(&w->Z[l], RH);
     A(&w->H[l], RH);
   }
   A(&w->Y, (size_t)w->R * NOUT);
   A(&w->dY, (size_t)w->R * NOUT);
-  A(&w->dA, RH);
-  A(&w->dB, RH);
-  A(&w->dC, RH);
-  A(&w->part, (size_t)w->n_gpart * HID * HID);
+  A(&w->dZ, RH);
+  for (int i = 0; i < 2; ++i) {
+    A(&w->dM[i], RH);
+    A(&w->dS[i], RH);
+  }
+  A(&w->part, (size_t)w->n_gpart * w->C);
   A(&w->lpart, w->n_lpart);
-  // the register-tiled layers use up to 97 KB of shared memory per CTA
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(linear64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)linear64_smem(HID, true));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(linear64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)linear64_smem(HID, true));
+  int g2 = 0;
+  if (e == cudaSuccess) e = layer_grid(input_kernel, 0, w->R, &w->g_in);
+  if (e == cudaSuccess) e = layer_grid(layer_kernel<false>, LAYER_SMEM, w->R, &w->g_layer);
+  if (e == cudaSuccess) e = layer_grid(layer_kernel<true>, LAYER_SMEM, w->R, &g2);
+  w->g_layer = std::min(w->g_layer, g2);
+  if (e == cudaSuccess) e = layer_grid(back_kernel<false>, BACK_SMEM, w->R, &w->g_back);
+  if (e == cudaSuccess) e = layer_grid(back_kernel<true>, BACK_SMEM, w->R, &g2);
+  w->g_back = std::min(w->g_back, g2);
+  std::vector<int4> nbr4(n_nodes);
+  std::vector<float4> wa4(n_nodes), wat4(n_nodes);
+  for (int n = 0; n < n_nodes; ++n) {
+    int nb[4] = {-1, -1, -1, -1};
+    float u[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int j = ptr[n], q = 0; j < ptr[n + 1] && q < 4; ++j, ++q) {
+      nb[q] = nbr[j];
+      u[q] = wa[j];
+      v[q] = wat[j];
+    }
+    nbr4[n] = make_int4(nb[0], nb[1], nb[2], nb[3]);
+    wa4[n] = make_float4(u[0], u[1], u[2], u[3]);
+    wat4[n] = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(w->nbr4, nbr4.data(), n_nodes * sizeof(int4), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(w->wA4, wa4.data(), n_nodes * sizeof(float4), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(w->wAT4, wat4.data(), n_nodes * sizeof(float4), cudaMemcpyHostToDevice);
   std::vector<float> p0(w->C);
   if (params) std::memcpy(p0.data(), params, w->C * sizeof(float));
   else he_init(p0, w, seed);
@@ -595,8 +756,7 @@ opf_status opf_wsnet_set_params(opf_wsnet *w, const float *params) {
 
 opf_status opf_wsnet_forward(opf_wsnet *w, const float *x, float *y) {
   if (!w || !x || !y) return wfail(OPF_EINVAL, "NULL argument");
-  forward(w, x);
-  WCK(cudaMemcpyAsync(y, w->Y, (size_t)w->R * NOUT * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
+  forward(w, x, y, false);
   WCK(cudaGetLastError());
   return OPF_OK;
 }
@@ -604,8 +764,10 @@ opf_status opf_wsnet_forward(opf_wsnet *w, const float *x, float *y) {
 opf_status opf_wsnet_gradient(opf_wsnet *w, const float *x, const float *yt, const float scale[2], double *loss,
                               float *grad) {
   if (!w || !x || !yt || !scale) return wfail(OPF_EINVAL, "NULL argument");
-  forward(w, x);
+  forward(w, x, w->Y, true);
   backward(w, x, yt, scale);
+  grad_kernel<false><<<(int)((w->C + TB - 1) / TB), TB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, nullptr, nullptr,
+                                                                       nullptr, nullptr, 0.f, 1.f, 1.f);
   WCK(cudaGetLastError());
   if (grad) WCK(cudaMemcpyAsync(grad, w->G, w->C * sizeof(float), cudaMemcpyDeviceToHost, w->stream));
   if (loss) return read_loss(w, loss);
@@ -617,11 +779,12 @@ opf_status opf_wsnet_train_step(opf_wsnet *w, const float *x, const float *yt, c
                                 double *loss) {
   if (!w || !x || !yt || !scale) return wfail(OPF_EINVAL, "NULL argument");
   if (!(lr > 0.f) || !std::isfinite(lr)) return wfail(OPF_EINVAL, "wsnet: learning rate must be > 0");
-  forward(w, x);
+  forward(w, x, w->Y, true);
   backward(w, x, yt, scale);
   ++w->step;
   const float bc1 = 1.f - std::pow(0.9f, (float)w->step), bc2 = 1.f - std::pow(0.999f, (float)w->step);
-  adam_kernel<<<grid_for(w->C), TB, 0, w->stream>>>(w->P, w->G, w->Mo, w->Vo, w->Pb, w->C, lr, bc1, bc2);
+  grad_kernel<true><<<(int)((w->C + TB - 1) / TB), TB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, w->P, w->Mo, w->Vo,
+                                                                      w->Pb, lr, bc1, bc2);
   WCK(cudaGetLastError());
   if (loss) return read_loss(w, loss);
   return OPF_OK;
