@@ -16,7 +16,8 @@
 // A training pass over 48,000 rows (2k buses, T = 24) moves about 0.35 GB and
 // does 7.3 GFLOP outside the tensor cores (the FP32 activations keep their
 // precision): bound by the FP32 pipes.  As fifty launches (averages, layers,
-// relu masks and each weight gradient apart) it took 0.97 ms, as sixteen @@.
+// relu masks and each weight gradient apart) it took 0.97 ms, as sixteen
+// (weight gradients beside the chain of layers) 0.37 ms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -35,11 +36,12 @@ constexpr int NOUT = OPF_WSNET_OUT;
 constexpr int NMP = 3;         // message-passing layers
 constexpr int TB = 256;        // threads per CTA of the element-wise kernels
 constexpr int LB = 128;        // threads per CTA of the layer kernels
-constexpr int TR = 32;         // rows per tile of the layer kernels
+constexpr int TR = 64;         // rows per tile of the layer kernels
+constexpr int RT = 8;          // ... and of a thread's block there (RT rows x 4 columns)
 constexpr int AS = HID + 4;    // row stride of a tile in shared memory (16-byte rows on shifting banks)
 constexpr int GRAD_ROWS = 256; // rows per partial sum of the weight gradients
 constexpr int GB = 64;         // threads per CTA of the weight-gradient kernel
-constexpr int GK = 16;         // weight rows (k) per CTA there
+constexpr int GK = 32;         // weight rows (k) per CTA there
 constexpr int GS = 32;         // activation rows staged together there
 
 // Neighbours of a node: the first four (-1 = none) and their weights, the
@@ -78,34 +80,60 @@ __device__ __forceinline__ float4 gather4(const Graph &g, const float *__restric
   return s;
 }
 
-// a layer's weights [64][64] into shared memory as FP32, ws[k][j] = W[k][j],
+// a layer's bfloat16 weights [64][64] into shared memory, ws[k][j] = W[k][j],
 // or W[j][k] with TRANS
+// (16-byte reads, all of a thread's in flight: a CTA walks few tiles, so this
+// is on its path)
 template <bool TRANS>
-__device__ __forceinline__ void stage_weights(float *ws, const __nv_bfloat16 *__restrict__ W) {
-  for (int i = threadIdx.x; i < HID * HID; i += LB) {
-    const int k = i / HID, j = i - k * HID;
-    ws[i] = __bfloat162float(W[TRANS ? j * HID + k : i]);
+__device__ __forceinline__ void stage_weights(__nv_bfloat16 *ws, const __nv_bfloat16 *__restrict__ W) {
+  constexpr int NQ = HID * HID / 8 / LB;
+  uint4 v[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) v[q] = reinterpret_cast<const uint4 *>(W)[threadIdx.x + q * LB];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int i = threadIdx.x + q * LB;
+    if constexpr (!TRANS) {
+      reinterpret_cast<uint4 *>(ws)[i] = v[q];
+    } else {
+      const int j = i / (HID / 8), k = 8 * (i % (HID / 8));
+      const unsigned x[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        reinterpret_cast<unsigned short *>(ws)[(k + e) * HID + j] = (unsigned short)(x[e >> 1] >> (16 * (e & 1)));
+    }
   }
 }
 
-// acc[i][c] += sum_k at[4 ty + i][k] ws[k][4 tx + c], k in order; a thread's
-// rows are read four k at a time, so that the products outnumber the
-// shared-memory wavefronts (64 to 48 per four warps)
-__device__ __forceinline__ void tile_mma(float (&acc)[4][4], const float *__restrict__ at,
-                                         const float *__restrict__ ws, int tx, int ty) {
-#pragma unroll 4
+// four bfloat16 weights as FP32 (their bits are the upper half of the float's)
+__device__ __forceinline__ float4 weights4(const __nv_bfloat16 *p) {
+  const uint2 v = *reinterpret_cast<const uint2 *>(p);
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
+}
+
+// acc[i][c] += sum_k at[RT ty + i][k] ws[k][4 tx + c], k in order.  Shared
+// memory bounds this loop, not the FP32 pipes: rows are read four k at a time
+// (one 16-byte read serves 16 lanes), weights as bfloat16 (a warp's 16 columns
+// groups are one 128-byte wavefront), and eight rows share a weight, so that
+// four k are 12 wavefronts for 128 products per lane (FP32 weights and 4 x 4
+// blocks: 24).  A layer of 48,000 rows takes 37 us, 10 of them products; the
+// rest is the gather of its tiles and the last, partly filled round of tiles.
+__device__ __forceinline__ void tile_mma(float (&acc)[RT][4], const float *__restrict__ at,
+                                         const __nv_bfloat16 *__restrict__ ws, int tx, int ty) {
+#pragma unroll 2
   for (int k = 0; k < HID; k += 4) {
-    float a[4][4];
+    float a[RT][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float4 v = *reinterpret_cast<const float4 *>(at + (4 * ty + i) * AS + k);
+    for (int i = 0; i < RT; ++i) {
+      const float4 v = *reinterpret_cast<const float4 *>(at + (RT * ty + i) * AS + k);
       a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float4 w = *reinterpret_cast<const float4 *>(ws + (k + q) * HID + 4 * tx);
+      const float4 w = weights4(ws + (k + q) * HID + 4 * tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < RT; ++i) {
         acc[i][0] = fmaf(a[i][q], w.x, acc[i][0]);
         acc[i][1] = fmaf(a[i][q], w.y, acc[i][1]);
         acc[i][2] = fmaf(a[i][q], w.z, acc[i][2]);
@@ -115,9 +143,10 @@ __device__ __forceinline__ void tile_mma(float (&acc)[4][4], const float *__rest
   }
 }
 
-__device__ __forceinline__ void zero_acc(float (&acc)[4][4]) {
+template <int M>
+__device__ __forceinline__ void zero_acc(float (&acc)[M][4]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < M; ++i)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
 }
@@ -130,8 +159,9 @@ __device__ __forceinline__ float4 relu4(const float4 &v) {
 __global__ void __launch_bounds__(LB) input_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ W,
                                                    const float *__restrict__ bias, float *__restrict__ out, int R,
                                                    int K) {
-  __shared__ __align__(16) float ws[HID * HID], at[TR * AS];
-  for (int i = threadIdx.x; i < K * HID; i += LB) ws[i] = __bfloat162float(W[i]);
+  __shared__ __align__(16) float at[TR * AS];
+  __shared__ __align__(16) __nv_bfloat16 ws[HID * HID];
+  for (int i = threadIdx.x; i < K * HID; i += LB) ws[i] = W[i];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const float4 b4 = *reinterpret_cast<const float4 *>(bias + 4 * tx);
   for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
@@ -142,13 +172,13 @@ __global__ void __launch_bounds__(LB) input_kernel(const float *__restrict__ x, 
       at[rr * AS + i - rr * K] = rr < nr ? x[(size_t)r0 * K + i] : 0.f;
     }
     __syncthreads();
-    float acc[4][4];
+    float acc[RT][4];
     zero_acc(acc);
     for (int k = 0; k < K; ++k) {
-      const float4 w = *reinterpret_cast<const float4 *>(ws + k * HID + 4 * tx);
+      const float4 w = weights4(ws + k * HID + 4 * tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float a = at[(4 * ty + i) * AS + k];
+      for (int i = 0; i < RT; ++i) {
+        const float a = at[(RT * ty + i) * AS + k];
         acc[i][0] = fmaf(a, w.x, acc[i][0]);
         acc[i][1] = fmaf(a, w.y, acc[i][1]);
         acc[i][2] = fmaf(a, w.z, acc[i][2]);
@@ -156,8 +186,8 @@ __global__ void __launch_bounds__(LB) input_kernel(const float *__restrict__ x, 
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rr = 4 * ty + i;
+    for (int i = 0; i < RT; ++i) {
+      const int rr = RT * ty + i;
       if (rr >= nr) break;
       *reinterpret_cast<float4 *>(out + (size_t)(r0 + rr) * HID + 4 * tx) =
           relu4(make_float4(acc[i][0] + b4.x, acc[i][1] + b4.y, acc[i][2] + b4.z, acc[i][3] + b4.w));
@@ -168,9 +198,9 @@ __global__ void __launch_bounds__(LB) input_kernel(const float *__restrict__ x, 
 // One message-passing layer: M = A H (kept where m is not NULL), H' = relu(H
 // Ws + M Wn + b).  LAST: also Y = H' Wo + bo; H' is kept where out is not NULL.
 // Dynamic shared memory: LAYER_SMEM.
-constexpr size_t LAYER_SMEM = (2 * HID * HID + 2 * TR * AS) * sizeof(float);
+constexpr size_t LAYER_SMEM = 2 * HID * HID * sizeof(__nv_bfloat16) + 2 * TR * AS * sizeof(float);
 template <bool LAST>
-__global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__restrict__ h,
+__global__ void __launch_bounds__(LB, 512 / LB) layer_kernel(Graph g, const float *__restrict__ h,
                                                       const __nv_bfloat16 *__restrict__ Ws,
                                                       const __nv_bfloat16 *__restrict__ Wn,
                                                       const float *__restrict__ bias, float *__restrict__ m,
@@ -178,7 +208,8 @@ __global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__re
                                                       const float *__restrict__ bo, float *__restrict__ y, int R) {
   extern __shared__ __align__(16) float sm[];
   __shared__ float wo[LAST ? HID * NOUT : 1];
-  float *ws = sm, *wn = ws + HID * HID, *at = wn + HID * HID, *am = at + TR * AS;
+  float *at = sm, *am = at + TR * AS;
+  __nv_bfloat16 *ws = reinterpret_cast<__nv_bfloat16 *>(am + TR * AS), *wn = ws + HID * HID;
   stage_weights<false>(ws, Ws);
   stage_weights<false>(wn, Wn);
   if constexpr (LAST)
@@ -188,8 +219,8 @@ __global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__re
   for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
     __syncthreads();
 #pragma unroll 2
-    for (int q = 0; q < TR / 8; ++q) {   // 16 threads a row
-      const int rr = ty + 8 * q, r = r0 + rr;
+    for (int q = 0; q < TR / (LB / 16); ++q) {   // 16 threads a row
+      const int rr = ty + (LB / 16) * q, r = r0 + rr;
       const bool in = r < R;
       const size_t o = (size_t)r * HID + 4 * tx;
       const float4 v = in ? *reinterpret_cast<const float4 *>(h + o) : z;
@@ -199,22 +230,23 @@ __global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__re
       if (m && in) *reinterpret_cast<float4 *>(m + o) = a;
     }
     __syncthreads();
-    float acc[4][4];
+    float acc[RT][4];
     zero_acc(acc);
     tile_mma(acc, at, ws, tx, ty);
     tile_mma(acc, am, wn, tx, ty);
     if constexpr (LAST) __syncthreads();   // at takes the output rows
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rr = 4 * ty + i, r = r0 + rr;
+    for (int i = 0; i < RT; ++i) {
+      const int rr = RT * ty + i, r = r0 + rr;
       const float4 v = relu4(make_float4(acc[i][0] + b4.x, acc[i][1] + b4.y, acc[i][2] + b4.z, acc[i][3] + b4.w));
       if (out && r < R) *reinterpret_cast<float4 *>(out + (size_t)r * HID + 4 * tx) = v;
       if constexpr (LAST) *reinterpret_cast<float4 *>(at + rr * AS + 4 * tx) = v;
     }
     if constexpr (LAST) {
       __syncthreads();
+      static_assert(LB == TR * NOUT, "a thread per output of the tile");
       const int rr = threadIdx.x / NOUT, j = threadIdx.x % NOUT, r = r0 + rr;
-      if (rr < TR && r < R) {
+      if (r < R) {
         float s = 0.f;
 #pragma unroll
         for (int k = 0; k < HID; k += 4) {
@@ -234,16 +266,17 @@ __global__ void __launch_bounds__(LB, 4) layer_kernel(Graph g, const float *__re
 // dS + A^T dM of the layer above -- masked where H' > 0 into dZ, and, unless
 // dm is NULL (the input layer), dM = dZ Wn^T and dS = dZ Ws^T for the layer
 // below.  Dynamic shared memory: BACK_SMEM.
-constexpr size_t BACK_SMEM = (2 * HID * HID + TR * AS) * sizeof(float);
+constexpr size_t BACK_SMEM = 2 * HID * HID * sizeof(__nv_bfloat16) + TR * AS * sizeof(float);
 template <bool FIRST>
-__global__ void __launch_bounds__(LB, 4) back_kernel(Graph g, const float *__restrict__ dy,
+__global__ void __launch_bounds__(LB, 512 / LB) back_kernel(Graph g, const float *__restrict__ dy,
                                                      const __nv_bfloat16 *__restrict__ Wo,
                                                      const float *__restrict__ ds_up, const float *__restrict__ dm_up,
                                                      const float *__restrict__ h, const __nv_bfloat16 *__restrict__ Ws,
                                                      const __nv_bfloat16 *__restrict__ Wn, float *__restrict__ dz,
                                                      float *__restrict__ dm, float *__restrict__ ds, int R) {
   extern __shared__ __align__(16) float sm[];
-  float *ws = sm, *wn = ws + HID * HID, *at = wn + HID * HID;
+  float *at = sm;
+  __nv_bfloat16 *ws = reinterpret_cast<__nv_bfloat16 *>(at + TR * AS), *wn = ws + HID * HID;
   if (dm) {
     stage_weights<true>(ws, Ws);
     stage_weights<true>(wn, Wn);
@@ -260,8 +293,8 @@ __global__ void __launch_bounds__(LB, 4) back_kernel(Graph g, const float *__res
   for (int r0 = blockIdx.x * TR; r0 < R; r0 += gridDim.x * TR) {
     __syncthreads();
 #pragma unroll 2
-    for (int q = 0; q < TR / 8; ++q) {
-      const int rr = ty + 8 * q, r = r0 + rr;
+    for (int q = 0; q < TR / (LB / 16); ++q) {
+      const int rr = ty + (LB / 16) * q, r = r0 + rr;
       const size_t o = (size_t)r * HID + 4 * tx;
       float4 d = z;
       if (r < R) {
@@ -284,15 +317,15 @@ __global__ void __launch_bounds__(LB, 4) back_kernel(Graph g, const float *__res
     }
     if (!dm) continue;
     __syncthreads();
-    float acc[4][4];
+    float acc[RT][4];
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
       zero_acc(acc);
       tile_mma(acc, at, pass ? ws : wn, tx, ty);
       float *o = pass ? ds : dm;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = r0 + 4 * ty + i;
+      for (int i = 0; i < RT; ++i) {
+        const int r = r0 + RT * ty + i;
         if (r < R)
           *reinterpret_cast<float4 *>(o + (size_t)r * HID + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
       }
@@ -304,48 +337,64 @@ __global__ void __launch_bounds__(LB, 4) back_kernel(Graph g, const float *__res
 // sum over the rows in order of a[r][k] g[r][j], a [R][K] and g [R][64].
 // blockIdx.y: up to two such products over the same g (a0 into column p0 of
 // the partial's parameter vector, then a1 into p1), GK values of k each; the
-// first also sums g itself (pb, the bias).  vec: a's rows are 64 floats on
+// first also sums g itself (pb, the bias).  VEC: a's rows are 64 floats on
 // 16-byte boundaries (the network's own arrays; the caller's features need
-// not be).  A thread keeps a 4 x 4 block in
-// registers (16 products per two shared-memory reads); splitting k over CTAs
-// gives ten small CTAs per SM at 48,000 rows where one CTA per row range left
-// the second wave nearly empty (32 us a product, now @@ for two).
+// not be), and the next rows are requested before the current ones are used.
+// A thread keeps an 8 x 4 block in registers (32 products per three 16-byte
+// shared-memory reads); splitting k over CTAs fills the SMs (one CTA per row
+// range left the second wave nearly empty: 32 us a product, now 26 for two).
+template <bool VEC>
 __global__ void __launch_bounds__(GB) wgrad_kernel(const float *__restrict__ a0, const float *__restrict__ a1,
                                                    const float *__restrict__ g, float *__restrict__ part, int R, int K,
-                                                   long long C, long long p0, long long p1, long long pb, int vec) {
+                                                   long long C, long long p0, long long p1, long long pb) {
   __shared__ __align__(16) float at[GS * GK], gt[GS * HID];
+  constexpr int NG = GS * HID / 4 / GB, NA = GS * GK / 4 / GB, AQ = GK / 4;
   const int nk = (K + GK - 1) / GK, second = blockIdx.y >= nk, k0 = (blockIdx.y - (second ? nk : 0)) * GK;
   const float *a = second ? a1 : a0;
   float *out = part + (size_t)blockIdx.x * C;
   const int r0 = blockIdx.x * GRAD_ROWS, r1 = min(R, r0 + GRAD_ROWS);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // j = 4 tx .., k = k0 + 4 ty ..
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // j = 4 tx .., k = k0 + 8 ty ..
   const bool bias = blockIdx.y == 0 && ty == 0;
-  float acc[4][4], ab[4] = {0.f, 0.f, 0.f, 0.f};
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  float acc[RT][4], ab[4] = {0.f, 0.f, 0.f, 0.f};
   zero_acc(acc);
+  float4 vg[NG], va[NA];
+  auto load = [&](int rb) {   // rows rb .. rb + GS - 1 (0 beyond r1)
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      const int i = threadIdx.x + q * GB, r = rb + i / (HID / 4);
+      vg[q] = r < r1 ? *reinterpret_cast<const float4 *>(g + (size_t)r * HID + 4 * (i % (HID / 4))) : z;
+    }
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int i = threadIdx.x + q * GB, r = rb + i / AQ, k = k0 + 4 * (i % AQ);
+      if constexpr (VEC) {
+        va[q] = r < r1 ? *reinterpret_cast<const float4 *>(a + (size_t)r * HID + k) : z;
+      } else {
+        const float *x = a + (size_t)r * K + k;
+        va[q] = make_float4(r < r1 && k < K ? x[0] : 0.f, r < r1 && k + 1 < K ? x[1] : 0.f,
+                            r < r1 && k + 2 < K ? x[2] : 0.f, r < r1 && k + 3 < K ? x[3] : 0.f);
+      }
+    }
+  };
+  load(r0);
   for (int rb = r0; rb < r1; rb += GS) {
     const int nr = min(GS, r1 - rb);
     __syncthreads();
-    for (int i = threadIdx.x; i < nr * (HID / 4); i += GB)
-      reinterpret_cast<float4 *>(gt)[i] = reinterpret_cast<const float4 *>(g + (size_t)rb * HID)[i];
-    if (vec) {
-      for (int i = threadIdx.x; i < nr * (GK / 4); i += GB) {
-        const int rr = i / (GK / 4), c = i % (GK / 4);
-        reinterpret_cast<float4 *>(at)[i] = *reinterpret_cast<const float4 *>(a + (size_t)(rb + rr) * HID + k0 + 4 * c);
-      }
-    } else {
-      for (int i = threadIdx.x; i < nr * GK; i += GB) {
-        const int rr = i / GK, k = k0 + i % GK;
-        at[i] = k < K ? a[(size_t)(rb + rr) * K + k] : 0.f;
-      }
-    }
+#pragma unroll
+    for (int q = 0; q < NG; ++q) reinterpret_cast<float4 *>(gt)[threadIdx.x + q * GB] = vg[q];
+#pragma unroll
+    for (int q = 0; q < NA; ++q) reinterpret_cast<float4 *>(at)[threadIdx.x + q * GB] = va[q];
     __syncthreads();
+    if (rb + GS < r1) load(rb + GS);
 #pragma unroll 4
     for (int rr = 0; rr < nr; ++rr) {
-      const float4 a4 = *reinterpret_cast<const float4 *>(at + rr * GK + 4 * ty);
+      const float4 x = *reinterpret_cast<const float4 *>(at + rr * GK + RT * ty);
+      const float4 y = *reinterpret_cast<const float4 *>(at + rr * GK + RT * ty + 4);
       const float4 g4 = *reinterpret_cast<const float4 *>(gt + rr * HID + 4 * tx);
-      const float av[4] = {a4.x, a4.y, a4.z, a4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
+      const float av[RT] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < RT; ++i)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[i][c] = fmaf(av[i], gv[c], acc[i][c]);
       if (bias)
@@ -355,8 +404,8 @@ __global__ void __launch_bounds__(GB) wgrad_kernel(const float *__restrict__ a0,
   }
   float *w = out + (second ? p1 : p0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = k0 + 4 * ty + i;
+  for (int i = 0; i < RT; ++i) {
+    const int k = k0 + RT * ty + i;
     if (k >= K) break;
 #pragma unroll
     for (int c = 0; c < 4; ++c) w[(size_t)k * HID + 4 * tx + c] = acc[i][c];
@@ -379,9 +428,19 @@ __global__ void __launch_bounds__(OB) wgrad_out_kernel(const float *__restrict__
   for (int rb = r0; rb < r1; rb += ST) {
     const int nr = min(ST, r1 - rb);
     __syncthreads();
-    for (int i = threadIdx.x; i < nr * (HID / 4); i += OB)
-      reinterpret_cast<float4 *>(ht)[i] = reinterpret_cast<const float4 *>(h + (size_t)rb * HID)[i];
-    for (int i = threadIdx.x; i < nr * NOUT; i += OB) gt[i] = dy[(size_t)rb * NOUT + i];
+    float4 v[ST * HID / 4 / OB];
+#pragma unroll
+    for (int q = 0; q < ST * HID / 4 / OB; ++q) {   // all requested together
+      const int i = threadIdx.x + q * OB;
+      if (i < nr * (HID / 4)) v[q] = reinterpret_cast<const float4 *>(h + (size_t)rb * HID)[i];
+    }
+    static_assert(ST * NOUT == OB, "one value of dY per thread");
+    if (threadIdx.x < nr * NOUT) gt[threadIdx.x] = dy[(size_t)rb * NOUT + threadIdx.x];
+#pragma unroll
+    for (int q = 0; q < ST * HID / 4 / OB; ++q) {
+      const int i = threadIdx.x + q * OB;
+      if (i < nr * (HID / 4)) reinterpret_cast<float4 *>(ht)[i] = v[q];
+    }
     __syncthreads();
 #pragma unroll 8
     for (int rr = 0; rr < nr; ++rr) {
@@ -397,15 +456,22 @@ __global__ void __launch_bounds__(OB) wgrad_out_kernel(const float *__restrict__
 
 // The partial sums reduced in order, grad[o] = sum over c of part[c][o], and
 // with ADAM the step on the FP32 parameters and their bfloat16 copy
+constexpr int GC = 48;
 template <bool ADAM>
-__global__ void __launch_bounds__(TB) grad_kernel(const float *__restrict__ part, float *__restrict__ grad, int n_part,
+__global__ void __launch_bounds__(GB) grad_kernel(const float *__restrict__ part, float *__restrict__ grad, int n_part,
                                                   long long n, float *p, float *m, float *v, __nv_bfloat16 *pb,
                                                   float lr, float bc1, float bc2) {
-  const long long i = (long long)blockIdx.x * TB + threadIdx.x;
+  const long long i = (long long)blockIdx.x * GB + threadIdx.x;
   if (i >= n) return;
   float s = 0.f;
-#pragma unroll 16
-  for (int c = 0; c < n_part; ++c) s += part[(size_t)c * n + i];
+  for (int c0 = 0; c0 < n_part; c0 += GC) {   // GC values in flight, added in order
+    float x[GC];
+#pragma unroll
+    for (int q = 0; q < GC; ++q) x[q] = c0 + q < n_part ? part[(size_t)(c0 + q) * n + i] : 0.f;
+#pragma unroll
+    for (int q = 0; q < GC; ++q)
+      if (c0 + q < n_part) s += x[q];
+  }
   grad[i] = s;
   if constexpr (ADAM) {
     const float mi = 0.9f * m[i] + 0.1f * s;
@@ -452,6 +518,9 @@ int grid_for(size_t work) { return (int)std::min<size_t>((work + TB - 1) / TB, 4
 struct opf_wsnet {
   int N = 0, T = 0, F = 0, R = 0;
   cudaStream_t stream = nullptr;
+  // the weight gradients run here, each beside the layers below it
+  cudaStream_t aux = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   long long C = 0;  // parameters
   long long oW0 = 0, ob0 = 0, oWs[NMP] = {}, oWn[NMP] = {}, ob[NMP] = {}, oWo = 0, obo = 0;
   int step = 0;
@@ -464,7 +533,7 @@ struct opf_wsnet {
   float4 *wA4 = nullptr, *wAT4 = nullptr;
   float *H0 = nullptr, *M[NMP] = {}, *H[NMP] = {}, *Y = nullptr;
   // dM and dS of a layer, read at the neighbours by the layer below: two of each
-  float *dY = nullptr, *dZ = nullptr, *dM[2] = {}, *dS[2] = {}, *part = nullptr;
+  float *dY = nullptr, *dZ[NMP + 1] = {}, *dM[2] = {}, *dS[2] = {}, *part = nullptr;
   double *lpart = nullptr;
   int n_lpart = 0, n_gpart = 0;
   int g_in = 0, g_layer = 0, g_back = 0;   // persistent CTAs of the layer kernels
@@ -491,6 +560,11 @@ cudaError_t walloc(opf_wsnet *w, T **p, size_t n) {
 void wfree(opf_wsnet *w) {
   for (void *p : w->allocs) cudaFree(p);
   w->allocs.clear();
+  for (cudaEvent_t ev : {w->ev_fork, w->ev_join})
+    if (ev) cudaEventDestroy(ev);
+  if (w->aux) cudaStreamDestroy(w->aux);
+  w->ev_fork = w->ev_join = nullptr;
+  w->aux = nullptr;
 }
 
 // He-uniform weights from a counter-based generator (splitmix64), zero biases
@@ -541,29 +615,42 @@ void forward(opf_wsnet *w, const float *x, float *y, bool keep) {
   }
 }
 
-// loss partials and the partial weight gradients (grad_kernel finishes them)
-void backward(opf_wsnet *w, const float *x, const float *yt, const float scale[2]) {
+// Loss partials and the partial weight gradients (grad_kernel finishes them).
+// A weight gradient waits only for its layer's dZ: they run on the second
+// stream beside the chain of layers (a row range's 256 rows one after another
+// are latency, 18 us a launch however few the rows).
+cudaError_t backward(opf_wsnet *w, const float *x, const float *yt, const float scale[2]) {
   const int R = w->R;
   const Graph g = graph(w, true);
+  auto fork = [&]() {
+    const cudaError_t e = cudaEventRecord(w->ev_fork, w->stream);
+    return e == cudaSuccess ? cudaStreamWaitEvent(w->aux, w->ev_fork, 0) : e;
+  };
   loss_kernel<<<w->n_lpart, TB, 0, w->stream>>>(w->Y, yt, w->dY, w->lpart, R, scale[0], scale[1]);
-  wgrad_out_kernel<<<w->n_gpart, OB, 0, w->stream>>>(w->H[NMP - 1], w->dY, w->part, R, w->C, w->oWo, w->obo);
-  for (int l = NMP - 1; l >= 0; --l) {
+  cudaError_t e = fork();
+  if (e != cudaSuccess) return e;
+  wgrad_out_kernel<<<w->n_gpart, OB, 0, w->aux>>>(w->H[NMP - 1], w->dY, w->part, R, w->C, w->oWo, w->obo);
+  for (int l = NMP - 1; l >= 0; --l) {   // layer l's dZ is dZ[l + 1]
     const int i = l & 1, up = i ^ 1;
     const __nv_bfloat16 *Ws = w->Pb + w->oWs[l], *Wn = w->Pb + w->oWn[l];
     if (l == NMP - 1)
       back_kernel<true><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, w->dY, w->Pb + w->oWo, nullptr, nullptr, w->H[l], Ws,
-                                                                  Wn, w->dZ, w->dM[i], w->dS[i], R);
+                                                                  Wn, w->dZ[l + 1], w->dM[i], w->dS[i], R);
     else
       back_kernel<false><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, nullptr, nullptr, w->dS[up], w->dM[up], w->H[l], Ws,
-                                                                   Wn, w->dZ, w->dM[i], w->dS[i], R);
+                                                                   Wn, w->dZ[l + 1], w->dM[i], w->dS[i], R);
+    if ((e = fork()) != cudaSuccess) return e;
     const dim3 grid(w->n_gpart, 2 * HID / GK);
-    wgrad_kernel<<<grid, GB, 0, w->stream>>>(l == 0 ? w->H0 : w->H[l - 1], w->M[l], w->dZ, w->part, R, HID, w->C,
-                                             w->oWs[l], w->oWn[l], w->ob[l], 1);
+    wgrad_kernel<true><<<grid, GB, 0, w->aux>>>(l == 0 ? w->H0 : w->H[l - 1], w->M[l], w->dZ[l + 1], w->part, R, HID, w->C,
+                                                w->oWs[l], w->oWn[l], w->ob[l]);
   }
   back_kernel<false><<<w->g_back, LB, BACK_SMEM, w->stream>>>(g, nullptr, nullptr, w->dS[0], w->dM[0], w->H0, nullptr,
-                                                               nullptr, w->dZ, nullptr, nullptr, R);
+                                                               nullptr, w->dZ[0], nullptr, nullptr, R);
   const dim3 grid(w->n_gpart, (w->F + GK - 1) / GK);
-  wgrad_kernel<<<grid, GB, 0, w->stream>>>(x, nullptr, w->dZ, w->part, R, w->F, w->C, w->oW0, 0, w->ob0, 0);
+  wgrad_kernel<false><<<grid, GB, 0, w->stream>>>(x, nullptr, w->dZ[0], w->part, R, w->F, w->C, w->oW0, 0, w->ob0);
+  e = cudaEventRecord(w->ev_join, w->aux);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(w->stream, w->ev_join, 0);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // persistent CTAs of a layer kernel: what is resident, or one per tile
@@ -679,13 +766,16 @@ opf_status opf_wsnet_create(int32_t n_nodes, int32_t n_lines, const int32_t *lin
   }
   A(&w->Y, (size_t)w->R * NOUT);
   A(&w->dY, (size_t)w->R * NOUT);
-  A(&w->dZ, RH);
+  for (int l = 0; l <= NMP; ++l) A(&w->dZ[l], RH);
   for (int i = 0; i < 2; ++i) {
     A(&w->dM[i], RH);
     A(&w->dS[i], RH);
   }
   A(&w->part, (size_t)w->n_gpart * w->C);
   A(&w->lpart, w->n_lpart);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&w->aux, cudaStreamNonBlocking);
+  for (cudaEvent_t *ev : {&w->ev_fork, &w->ev_join})
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   int g2 = 0;
   if (e == cudaSuccess) e = layer_grid(input_kernel, 0, w->R, &w->g_in);
   if (e == cudaSuccess) e = layer_grid(layer_kernel<false>, LAYER_SMEM, w->R, &w->g_layer);
@@ -765,8 +855,8 @@ opf_status opf_wsnet_gradient(opf_wsnet *w, const float *x, const float *yt, con
                               float *grad) {
   if (!w || !x || !yt || !scale) return wfail(OPF_EINVAL, "NULL argument");
   forward(w, x, w->Y, true);
-  backward(w, x, yt, scale);
-  grad_kernel<false><<<(int)((w->C + TB - 1) / TB), TB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, nullptr, nullptr,
+  WCK(backward(w, x, yt, scale));
+  grad_kernel<false><<<(int)((w->C + GB - 1) / GB), GB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, nullptr, nullptr,
                                                                        nullptr, nullptr, 0.f, 1.f, 1.f);
   WCK(cudaGetLastError());
   if (grad) WCK(cudaMemcpyAsync(grad, w->G, w->C * sizeof(float), cudaMemcpyDeviceToHost, w->stream));
@@ -780,10 +870,10 @@ opf_status opf_wsnet_train_step(opf_wsnet *w, const float *x, const float *yt, c
   if (!w || !x || !yt || !scale) return wfail(OPF_EINVAL, "NULL argument");
   if (!(lr > 0.f) || !std::isfinite(lr)) return wfail(OPF_EINVAL, "wsnet: learning rate must be > 0");
   forward(w, x, w->Y, true);
-  backward(w, x, yt, scale);
+  WCK(backward(w, x, yt, scale));
   ++w->step;
   const float bc1 = 1.f - std::pow(0.9f, (float)w->step), bc2 = 1.f - std::pow(0.999f, (float)w->step);
-  grad_kernel<true><<<(int)((w->C + TB - 1) / TB), TB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, w->P, w->Mo, w->Vo,
+  grad_kernel<true><<<(int)((w->C + GB - 1) / GB), GB, 0, w->stream>>>(w->part, w->G, w->n_gpart, w->C, w->P, w->Mo, w->Vo,
                                                                       w->Pb, lr, bc1, bc2);
   WCK(cudaGetLastError());
   if (loss) return read_loss(w, loss);
@@ -793,6 +883,7 @@ opf_status opf_wsnet_train_step(opf_wsnet *w, const float *x, const float *yt, c
 void opf_wsnet_destroy(opf_wsnet *w) {
   if (!w) return;
   cudaStreamSynchronize(w->stream);
+  cudaStreamSynchronize(w->aux);
   wfree(w);
   delete w;
 }
