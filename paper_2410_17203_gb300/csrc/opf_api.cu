@@ -1188,7 +1188,7 @@ opf_status build_batch_graph(opf_batch *b, int iters, cudaGraphExec_t *out) {
 // Build the schedule of the n_sched instances that `lay` lists (lay.order;
 // NULL: every instance as given) into d_sched and drop the graphs of the
 // previous one (rebuilt on the next iteration).  Waits for the batch stream.
-opf_status schedule_batch(opf_batch *b, int n_sched, const opfk::BatchLayout &lay) {
+opf_status schedule_batch(opf_batch *b, int n_sched, opfk::BatchLayout lay) {
   const int n = (int)b->ctx.size();
   std::vector<Params> hp(n);
   std::vector<opfk::IterPlan> plans(n);
@@ -1198,6 +1198,7 @@ opf_status schedule_batch(opf_batch *b, int n_sched, const opfk::BatchLayout &la
   }
   long long len = 0;
   opfk::BatchPlan bp{};
+  lay.node_items = opfk_batch_node_items(hp.data(), n);
   if (opfk_batch_plan(hp.data(), plans.data(), n_sched, lay, nullptr, 0, &len, &bp) != 0 || len > b->sched_cap)
     return fail(OPF_ECUDA, "batch schedule");
   std::vector<int> sched(4 * (size_t)std::max(len, 1LL));
@@ -1208,8 +1209,6 @@ opf_status schedule_batch(opf_batch *b, int n_sched, const opfk::BatchLayout &la
   if (b->g_many) cudaGraphExecDestroy(b->g_many);
   b->g_one = b->g_many = nullptr;
   CK(cudaMemcpy(b->d_sched, sched.data(), sched.size() * sizeof(int), cudaMemcpyHostToDevice));
-  // the node phase's CTA count sizes each instance's partial sums
-  for (int i = 0; i < n; ++i) hp[i].node_grid = opfk_batch_node_blocks(plans[i], lay.div);
   CK(cudaMemcpy(b->d_params, hp.data(), n * sizeof(Params), cudaMemcpyHostToDevice));
   b->plan = bp;
   b->n_sched = n_sched;
@@ -1273,7 +1272,8 @@ opf_status opf_batch_create(opf_ctx *const *ctxs, int32_t n, opf_batch **out) {
   }
   long long len = 0;
   opf_status st = OPF_OK;
-  const opfk::BatchLayout lay{nullptr, 0, 1};   // as given, contiguous: the longest schedule
+  // as given, contiguous: the longest schedule
+  const opfk::BatchLayout lay{nullptr, 0, 1, opfk_batch_node_items(hp.data(), n)};
   const int pr = opfk_batch_plan(hp.data(), plans.data(), n, lay, nullptr, 0, &len, &b->plan);
   if (pr == -2) st = fail(OPF_EINVAL, "a batch cannot mix over-relaxed (alpha != 1) and plain instances");
   else if (pr != 0) st = fail(OPF_ECUDA, "batch schedule");
@@ -1341,8 +1341,8 @@ opf_status opf_batch_autotune(opf_batch *b, int32_t steps, int32_t *choice, doub
   };
   std::stable_sort(lpt.begin(), lpt.end(), [&](int x, int y) { return work(x) > work(y); });
   const opfk::BatchLayout cands[OPF_BATCH_LAYOUTS] = {
-      {nullptr, 0, 1}, {lpt.data(), 0, 1}, {lpt.data(), 1, 1},
-      {nullptr, 0, 4}, {lpt.data(), 0, 4}, {lpt.data(), 1, 4}};
+      {nullptr, 0, 1, 0.0}, {lpt.data(), 0, 1, 0.0}, {lpt.data(), 1, 1, 0.0},
+      {nullptr, 0, 4, 0.0}, {lpt.data(), 0, 4, 0.0}, {lpt.data(), 1, 4, 0.0}};   // node_items: schedule_batch
   // save every instance's mutable state after its queued work
   std::vector<size_t> off(n + 1, 0);
   for (int i = 0; i < n; ++i) off[i + 1] = off[i] + mutable_bytes(b->ctx[i]);
@@ -1372,6 +1372,9 @@ opf_status opf_batch_autotune(opf_batch *b, int32_t steps, int32_t *choice, doub
     if (st == OPF_OK) st = ensure_batch_graphs(b);
     if (st != OPF_OK) break;
     copy_all(false);
+    // as in a call: residuals where a stopping test or an adaptation reads
+    // them (past a call's last iteration every iteration would form them)
+    if (e == cudaSuccess && opfk_begin_batch_launch(b->d_params, n, steps + 2, b->stream) != 0) e = cudaErrorUnknown;
     launch_batch_steps(b, 1, &e);                    // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(t0, b->stream);
     launch_batch_steps(b, steps, &e);
@@ -1457,7 +1460,7 @@ opf_status opf_batch_compact(opf_batch *b, int32_t *n_scheduled) {
     if (run[i]) order.push_back(i);
   }
   if ((int)order.size() != b->n_sched) {
-    const opfk::BatchLayout lay{order.data(), b->lay_interleave, b->lay_div};
+    const opfk::BatchLayout lay{order.data(), b->lay_interleave, b->lay_div, 0.0};
     const opf_status st = schedule_batch(b, (int)order.size(), lay);
     if (st != OPF_OK) return st;
   }

@@ -47,6 +47,11 @@ constexpr int WARPS = BLOCK / 32;
 constexpr int ST_NONFINITE = 5;  // opf_status value set on the device
 constexpr int NODE_VW = 4;       // time steps per node item
 constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is compiled for (64 registers)
+// Waves of node CTAs of a batch (its instances share the resident CTAs out by
+// items): 16 mixed instances of up to 3,000 buses, us per iteration: one wave
+// 81, two 84; every instance with a grid of its own, the two step widths in a
+// launch each, 101.
+constexpr double NODE_WAVES = 1.0;
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
@@ -1807,20 +1812,23 @@ __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int
   else closed_body<1>(p, bid, nblk);
 }
 
-template <int VW>
-__global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, const int4 *sched) {
+// the lines of every instance: the first n4 CTAs of the schedule take those
+// whose horizon is whole 4-step blocks, the others the rest; the nodes alike
+__global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, const int4 *sched, int n4) {
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  line_body<VW>(p, bid);
+  if ((int)blockIdx.x < n4) line_body<4>(p, bid);
+  else line_body<1>(p, bid);
 }
 
-template <int VW, bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched) {
+template <bool RELAX>
+__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched, int n4) {
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  node_body<VW, RELAX, true>(p, bid, nblk);
+  if ((int)blockIdx.x < n4) node_body<4, RELAX, true>(p, bid, nblk);
+  else node_body<1, RELAX, true>(p, bid, nblk);
 }
 
 // A line's terminal values from its stored (p, mid) at contingency k:
@@ -2265,6 +2273,15 @@ int opfk_slice_prime_launch(const Params &p, void *stream) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// node items (of four steps or one) of an instance
+static double node_items(const Params &p) { return (double)p.Kp * p.N * (p.T % NODE_VW == 0 ? p.T / NODE_VW : p.T); }
+
+double opfk_batch_node_items(const Params *hp, int n) {
+  double s = 0.0;
+  for (int i = 0; i < n; ++i) s += node_items(hp[i]);
+  return s;
+}
+
 int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchLayout &lay, int *sched_out,
                     long long sched_cap, long long *sched_len, BatchPlan *bp) {
   long long len = 0;
@@ -2283,6 +2300,8 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     return true;
   };
   const int div = std::max(1, lay.div);
+  const int slots = resident_grid(node_kernel_b<false>, 0);
+  if (slots < 1) return -1;
   std::vector<long long> nb(n);
   for (int kind = 0; kind < BK_COUNT; ++kind) {
     bp->offset[kind] = (int)len;
@@ -2311,12 +2330,15 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
             blocks = plans[i].line_grid;
           break;
         case BK_NODE4: case BK_NODE1:
-          if ((kind == BK_NODE4) == vn) blocks = plans[i].node_grid;
+          // the resident CTAs shared out by items, so that one wave of CTAs, each
+          // walking as many items as the others, serves the batch
+          if ((kind == BK_NODE4) == vn)
+            blocks = std::min<long long>(plans[i].node_grid,
+                                         std::max<long long>(1, (long long)(node_items(p) * NODE_WAVES * slots / lay.node_items)));
           break;
       }
       // the grid-stride phases take any block count: `div` puts more work in
-      // each CTA (for the node phase the caller sets the instance's partial-sum
-      // count to the same number, batch_node_blocks)
+      // each CTA
       if (blocks > 0 && (kind == BK_INNER || kind == BK_CLOSED || kind == BK_NODE4 || kind == BK_NODE1))
         blocks = (blocks + div - 1) / div;
       nb[j] = blocks;
@@ -2347,11 +2369,6 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
   return 0;
 }
 
-int opfk_batch_node_blocks(const IterPlan &plan, int div) {
-  const int d = div > 1 ? div : 1;
-  return (plan.node_grid + d - 1) / d;
-}
-
 int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPlan &bp, void *main_stream,
                        void *aux_stream, void *ev_fork, void *ev_join) {
   cudaStream_t sm = (cudaStream_t)main_stream, sa = (cudaStream_t)aux_stream;
@@ -2359,8 +2376,9 @@ int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPl
   auto at = [&](int kind) { return sched + bp.offset[kind]; };
   if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
-  if (bp.count[BK_LINE4]) line_kernel_b<4><<<bp.count[BK_LINE4], BLOCK, 0, sa>>>(d_params, at(BK_LINE4));
-  if (bp.count[BK_LINE1]) line_kernel_b<1><<<bp.count[BK_LINE1], BLOCK, 0, sa>>>(d_params, at(BK_LINE1));
+  static_assert(BK_LINE1 == BK_LINE4 + 1 && BK_NODE1 == BK_NODE4 + 1, "one launch over both widths' schedules");
+  const int l4 = bp.count[BK_LINE4], nl = l4 + bp.count[BK_LINE1];
+  if (nl) line_kernel_b<<<nl, BLOCK, 0, sa>>>(d_params, at(BK_LINE4), l4);
   if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
   static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
   const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED];
@@ -2375,13 +2393,9 @@ int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPl
     }
   }
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
-  if (!bp.relax) {
-    if (bp.count[BK_NODE4]) node_kernel_b<4, false><<<bp.count[BK_NODE4], BLOCK, 0, sm>>>(d_params, at(BK_NODE4));
-    if (bp.count[BK_NODE1]) node_kernel_b<1, false><<<bp.count[BK_NODE1], BLOCK, 0, sm>>>(d_params, at(BK_NODE1));
-  } else {
-    if (bp.count[BK_NODE4]) node_kernel_b<4, true><<<bp.count[BK_NODE4], BLOCK, 0, sm>>>(d_params, at(BK_NODE4));
-    if (bp.count[BK_NODE1]) node_kernel_b<1, true><<<bp.count[BK_NODE1], BLOCK, 0, sm>>>(d_params, at(BK_NODE1));
-  }
+  const int n4 = bp.count[BK_NODE4], nn = n4 + bp.count[BK_NODE1];
+  if (nn && bp.relax) node_kernel_b<true><<<nn, BLOCK, 0, sm>>>(d_params, at(BK_NODE4), n4);
+  else if (nn) node_kernel_b<false><<<nn, BLOCK, 0, sm>>>(d_params, at(BK_NODE4), n4);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
