@@ -375,8 +375,7 @@ opf_status init_scalars(opf_ctx *c) {
   sc.v_fresh = 1;
   sc.stall_ref = HUGE_VAL;
   opfk::set_iter(c->P, sc);
-  CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  if (opfk_set_scalars_launch(c->P, sc, c->stream) != 0) return fail(OPF_ECUDA, "set_scalars launch failed");
   return OPF_OK;
 }
 
@@ -734,7 +733,6 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   p.n_hvdc = c->H;
   p.hvdc0 = G + D + c->B;
   p.node_grid = c->plan.node_grid;
-  p.line_ipt = c->plan.line_ipt;
   p.n_cnode = (int)crec.size();
   p.eps = opt.eps;
   p.mu = opt.mu;
@@ -838,6 +836,7 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
   up(p.node_perm, node_perm);
   up(p.line_perm, line_perm);
   if (s == OPF_OK) s = init_scalars(c);
+  if (s == OPF_OK && (e = cudaStreamSynchronize(c->stream)) != cudaSuccess) s = cuda_fail(e, "context set-up");
   if (s != OPF_OK) {
     release_cuda(c);
     delete c;
@@ -1608,7 +1607,7 @@ opf_status opf_set_state(opf_ctx *c, int32_t on_device, const opf_state *src) {
   sc.stall_ref = HUGE_VAL;
   sc.stall_it = sc.it;
   opfk::set_iter(c->P, sc);
-  CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
+  if (opfk_set_scalars_launch(c->P, sc, c->stream) != 0) return fail(OPF_ECUDA, "set_scalars launch failed");
   CK(cudaStreamSynchronize(c->stream));
   c->host_status = 0;
   return OPF_OK;
@@ -1650,7 +1649,7 @@ opf_status opf_set_state_from_nodes(opf_ctx *c, int32_t on_device, const float *
   sc.stall_ref = HUGE_VAL;
   sc.stall_it = sc.it;
   opfk::set_iter(c->P, sc);
-  CK(cudaMemcpyAsync(c->P.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
+  if (opfk_set_scalars_launch(c->P, sc, c->stream) != 0) return fail(OPF_ECUDA, "set_scalars launch failed");
   CK(cudaStreamSynchronize(c->stream));
   c->host_status = 0;
   return OPF_OK;

@@ -91,7 +91,6 @@ struct Params {
   int n_dnode, n_ramp, n_stor;
   int n_hvdc, hvdc0;                     // HVDC links; device id of the first link's terminal 1
   // lines (internal numbering)
-  int line_ipt;                  // IterPlan::line_ipt
   const int *line_n1, *line_n2;  // internal node of terminal 1 (from) and terminal 2 (to)
   const float *line_b, *line_u;
   const int *out_line;  // [Kp], internal index of the outaged line, -1 = none
@@ -307,6 +306,8 @@ int opfk_export_lines_launch(const opfk::Params &p, int cur, float *p_line, floa
 int opfk_export_pdev_launch(const opfk::Params &p, float *out, void *stream);
 int opfk_export_nodes_launch(const opfk::Params &p, int cur, float *u, float *theta_node,
                              float *price, void *stream);
+// Write the scalars in stream order, from the launch's own copy (nothing to wait for).
+int opfk_set_scalars_launch(const opfk::Params &p, const opfk::DevScalars &sc, void *stream);
 int opfk_set_rho_launch(const opfk::Params &p, double rho, void *stream);
 // Contingency slices: the local half of one iteration (devices from the
 // exchanged sums, line proxes, node sums, then this slice's sums into the

@@ -55,7 +55,7 @@ constexpr double NODE_WAVES = 1.0;
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
-constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items)
+constexpr int LINE_IPT = 4;      // line items per thread (CTA-sized blocks of items; all of a batch's instances)
 constexpr long long LINE_SHORT = 1 << 20;   // ... one, up to this many items
 constexpr int DEVB = 128;        // threads per CTA of the device kernel (its inner-ADMM warps spread over more SMs)
 constexpr int DEV_WARPS = DEVB / 32;
@@ -1444,10 +1444,10 @@ __device__ __forceinline__ void dsum_body(const Params &p, unsigned bid, unsigne
 // line: step 1 for every (contingency, line, VW time steps)
 // ---------------------------------------------------------------------------
 template <int VW>
-__device__ __forceinline__ void line_body(const Params &p, unsigned bid) {
-  const int L = p.L, TV = p.T / VW, ipt = p.line_ipt;
+__device__ __forceinline__ void line_body(const Params &p, unsigned bid, int ipt) {
+  const int L = p.L, TV = p.T / VW;
   const unsigned n = (unsigned)p.Kp * (unsigned)L * (unsigned)TV;
-  // each CTA takes line_ipt consecutive blocks of BLOCK items, so CTAs are
+  // each CTA takes ipt consecutive blocks of BLOCK items, so CTAs are
   // short-lived and the device kernels' CTAs find room beside them
   const unsigned base = bid * (unsigned)(BLOCK * ipt) + threadIdx.x;
   // items (line, contingency, step block): a line's K+1 rows are contiguous
@@ -1715,8 +1715,8 @@ template <int VW>
 __global__ void __launch_bounds__(BLOCK) dsum_kernel(Params p) { dsum_body<VW>(p, blockIdx.x, gridDim.x); }
 
 template <int VW>
-__global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p) {
-  line_body<VW>(p, blockIdx.x);
+__global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p, int ipt) {
+  line_body<VW>(p, blockIdx.x, ipt);
 }
 
 // The over-relaxed variant reads one more row per terminal and carries the mean
@@ -1818,8 +1818,8 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, cons
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  if ((int)blockIdx.x < n4) line_body<4>(p, bid);
-  else line_body<1>(p, bid);
+  if ((int)blockIdx.x < n4) line_body<4>(p, bid, LINE_IPT);
+  else line_body<1>(p, bid, LINE_IPT);
 }
 
 template <bool RELAX>
@@ -2118,6 +2118,8 @@ __global__ void begin_batch_kernel(const Params *ps, int n_inst, long long n) {
   *ps[i].sc = sc;
 }
 
+__global__ void set_scalars_kernel(DevScalars *d, DevScalars sc) { *d = sc; }
+
 __global__ void set_rho_kernel(Params p, double rho) {
   DevScalars s = *p.sc;
   s.su *= s.rho_p / rho;
@@ -2234,8 +2236,8 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
     else dsum_kernel<1><<<plan.dsum_grid, BLOCK, 0, sm>>>(p);
   }
   if (plan.line_grid > 0) {
-    if (v4) line_kernel<4><<<plan.line_grid, BLOCK, 0, sa>>>(p);
-    else line_kernel<1><<<plan.line_grid, BLOCK, 0, sa>>>(p);
+    if (v4) line_kernel<4><<<plan.line_grid, BLOCK, 0, sa>>>(p, plan.line_ipt);
+    else line_kernel<1><<<plan.line_grid, BLOCK, 0, sa>>>(p, plan.line_ipt);
   }
   if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
@@ -2327,7 +2329,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           break;
         case BK_LINE4: case BK_LINE1:
           if ((kind == BK_LINE4) == v4 && p.L > 0)
-            blocks = plans[i].line_grid;
+            blocks = ((long long)p.Kp * p.L * tv4 + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT);
           break;
         case BK_NODE4: case BK_NODE1:
           // the resident CTAs shared out by items, so that one wave of CTAs, each
@@ -2466,6 +2468,11 @@ int opfk_export_nodes_launch(const Params &p, int cur, float *u, float *theta, f
                              void *stream) {
   export_nodes_kernel<<<aux_grid((long long)p.N * p.T), 256, 0, (cudaStream_t)stream>>>(p, cur, u, theta,
                                                                                          price);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int opfk_set_scalars_launch(const Params &p, const DevScalars &sc, void *stream) {
+  set_scalars_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(p.sc, sc);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
