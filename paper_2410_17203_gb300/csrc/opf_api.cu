@@ -332,6 +332,7 @@ void carve(opf_ctx *c, Arena &a) {
   p.rcnt_p = a.take<float>(c->N);
   p.rcnt_th = a.take<float>(c->N);
   p.nrec = a.take<int4>(3 * (size_t)c->N);
+  p.ndev4 = a.take<int4>(c->N);
   p.tcode = a.take<int>(c->n_tcode);
   p.dev_node = a.take<int>(c->S);
   p.dev_type = a.take<int>(c->S);
@@ -798,6 +799,13 @@ opf_status create_impl(const opf_network *net, int32_t T, const opf_contingencie
       rec[3 * n + 2] = make_int4(tptr[n], tptr[n + 1], dptr[n + 1] - dptr[n], dptr[n]);
     }
     up(p.nrec, rec);
+    std::vector<int4> nd(N);
+    for (int n = 0; n < N; ++n) {
+      int v[4] = {0, 0, 0, 0};
+      for (int j = dptr[n], q = 0; j < dptr[n + 1] && q < 4; ++j, ++q) v[q] = didx[j];
+      nd[n] = make_int4(v[0], v[1], v[2], v[3]);
+    }
+    up(p.ndev4, nd);
   }
   up(p.tcode, tcode);
   up(p.dev_node, dev_node_int);

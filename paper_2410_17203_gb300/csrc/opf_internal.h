@@ -111,6 +111,7 @@ struct Params {
   // four line-terminal codes 2*l + end (-1 = none), (tcode begin, end of the
   // rest, device count, first of the node's entries in dcsr_idx)
   const int4 *nrec;
+  const int4 *ndev4;               // each node's first four devices
   const int *tcode;                // line-terminal codes beyond the first four per node,
                                    // each node's list padded to a multiple of 4 with -1
   // per node and time step, over the node's devices (the same in every
@@ -226,6 +227,7 @@ __host__ __device__ __forceinline__ void set_iter(const Params &p, DevScalars &s
 struct IterPlan {
   int line_grid, node_grid;            // 0: the kernel has no work
   int line_ipt;                        // line items per thread
+  int node_lat;                        // few node items: all loads of an item requested together
   int fused;                           // 1: one device kernel; 0: averages, inner ADMM and device sums apart
   int dev_inner, dev_closed;           // CTAs of the device kernel for inner-ADMM and (fused) closed-form devices
   int xs_grid, dsum_grid;              // not fused: averages with closed-form devices, device sums

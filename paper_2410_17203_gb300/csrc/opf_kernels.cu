@@ -52,6 +52,13 @@ constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is comp
 // 81, two 84; every instance with a grid of its own, the two step widths in a
 // launch each, 101.
 constexpr double NODE_WAVES = 1.0;
+// Up to this many node items (four steps / one step each; about what two CTAs
+// per SM hold at once) the pass is latency alone, and a variant with the
+// registers to request all loads of an item together is faster: us per
+// iteration, 30 buses 9.0 -> 8.6, 301 buses T = 31 14.4 -> 13.8, 5k buses T = 1
+// (105k items) 15.5 -> 14.9, 900 buses T = 24 (76k) 16.9 -> 16.4; beyond it
+// the second wave costs more: 500 buses T = 168 (105k items of four) 35.1 -> 36.5.
+constexpr long long NODE_LAT_ITEMS4 = 2 * 152 * BLOCK, NODE_LAT_ITEMS1 = 1 << 17;
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
@@ -1069,10 +1076,11 @@ __device__ __forceinline__ void line_item(const Params &p, int old, int nw, int 
 // inputs only they need (old p and theta_bar rows, the device Welford state)
 // and their accumulation; the relaxed variant still needs the mean change of p
 // (its u update), so it reads the old p rows and keeps that mean alone.
-// NB: line terminals gathered together.
+// NB: line terminals gathered together.  LAT (with ILD): the first two
+// devices' powers are requested with the first line rows.
 // ILD: the pass sums the node's device powers (and the Welford state of their
 // changes) itself; else dsum_kernel has left them in DSP, DSM and DSQ.
-template <int VW, bool RELAX, bool RES, int NB, bool ILD>
+template <int VW, bool RELAX, bool RES, int NB, bool ILD, bool LAT>
 __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int k, int n, int toff, float fsu,
                                           float *acc) {
   const int T = p.T;
@@ -1107,20 +1115,35 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
       for (int e = 0; e < VW; ++e) { wdp.mean[e] = m.v[e]; wdp.m2[e] = q.v[e]; }
     }
   }
+  FV<VW> pd0, pd1, dd0, dd1;
+  int4 dv = make_int4(0, 0, 0, 0);
   if constexpr (ILD) {
 #pragma unroll
     for (int e = 0; e < VW; ++e) sp.v[e] = 0.f;
     if constexpr (RES) wdp.reset();
     if constexpr (RELAX && !RES) wm.reset();
-    for (int j = r2.w; j < r2.w + r2.z; ++j) {
-      const size_t od = (size_t)p.dcsr_idx[j] * T + toff;
-      const FV<VW> pd = ldv<VW>(p.PD + od);
+    if constexpr (LAT) {
+      dv = p.ndev4[n];
+      if (r2.z > 0) {
+        pd0 = ldv<VW>(p.PD + (size_t)dv.x * T + toff);
+        if constexpr (dp) dd0 = ldv<VW>(p.DPD + (size_t)dv.x * T + toff);
+      }
+      if (r2.z > 1) {
+        pd1 = ldv<VW>(p.PD + (size_t)dv.y * T + toff);
+        if constexpr (dp) dd1 = ldv<VW>(p.DPD + (size_t)dv.y * T + toff);
+      }
+    } else {
+      for (int j = r2.w; j < r2.w + r2.z; ++j) {
+        const size_t od = (size_t)p.dcsr_idx[j] * T + toff;
+        const FV<VW> pd = ldv<VW>(p.PD + od);
 #pragma unroll
-      for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
-      if constexpr (RES) wdp.add(ldv<VW>(p.DPD + od).v);
-      else if constexpr (RELAX) wm.add(ldv<VW>(p.DPD + od).v);
+        for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
+        if constexpr (RES) wdp.add(ldv<VW>(p.DPD + od).v);
+        else if constexpr (RELAX) wm.add(ldv<VW>(p.DPD + od).v);
+      }
     }
   }
+  bool first = ILD && LAT;
   wth.reset();
 #pragma unroll
   for (int e = 0; e < VW; ++e) st.v[e] = 0.f;
@@ -1149,6 +1172,21 @@ __device__ __forceinline__ void node_item(const Params &p, int old, int nw, int 
         mq[q] = ldv<VW>(p.MID[nw] + ol);
         if constexpr (RELAX && RES) mo[q] = ldv<VW>(p.MID[old] + ol);
         bq[q] = p.line_b[l];
+      }
+    }
+    if (first) {   // the device terminals, with the line rows in flight
+      first = false;
+      for (int i = 0; i < r2.z; ++i) {
+        const int d = i == 2 ? dv.z : i == 3 ? dv.w : i < 2 ? 0 : p.dcsr_idx[r2.w + i];
+        const size_t od = (size_t)d * T + toff;
+        const FV<VW> pd = i == 0 ? pd0 : i == 1 ? pd1 : ldv<VW>(p.PD + od);
+#pragma unroll
+        for (int e = 0; e < VW; ++e) sp.v[e] += pd.v[e];
+        if constexpr (dp) {
+          const FV<VW> dd = i == 0 ? dd0 : i == 1 ? dd1 : ldv<VW>(p.DPD + od);
+          if constexpr (RES) wdp.add(dd.v);
+          else wm.add(dd.v);
+        }
       }
     }
 #pragma unroll
@@ -1626,7 +1664,7 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part, double 
 // its 36 us on their launches.  At 64 registers (four CTAs per SM, what the
 // residual-free pass wants) the general pass gathers one terminal at a time.
 // ---------------------------------------------------------------------------
-template <int VW, bool RELAX, bool ILD>
+template <int VW, bool RELAX, bool ILD, bool LAT = false>
 __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk) {
   __shared__ double red[WARPS][NSLOT];
   __shared__ int s_last;
@@ -1647,10 +1685,10 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if (res) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
-      node_item<VW, RELAX, true, NODE_RES_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+      node_item<VW, RELAX, true, LAT ? 4 : NODE_RES_NB, ILD, LAT>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
   } else {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
-      node_item<VW, RELAX, false, NODE_LEAN_NB, ILD>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+      node_item<VW, RELAX, false, LAT ? 4 : NODE_LEAN_NB, ILD, LAT>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
   }
   if (res) {
 #pragma unroll
@@ -1723,9 +1761,9 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p, int ipt) {
 // change of p: three CTAs per SM at 80 registers (1k buses, T = 48, K = 20,
 // alpha = 1.5, us per iteration: two 28.6, three 26.9, four 28.3; 39.8 when
 // every iteration carried the residual sums).  ILD: device sums in the pass.
-template <int VW, bool RELAX, bool ILD>
-__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel(Params p) {
-  node_body<VW, RELAX, ILD>(p, blockIdx.x, gridDim.x);
+template <int VW, bool RELAX, bool ILD, bool LAT>
+__global__ void __launch_bounds__(BLOCK, LAT ? 2 : RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel(Params p) {
+  node_body<VW, RELAX, ILD, LAT>(p, blockIdx.x, gridDim.x);
 }
 
 // a slice's decisions, from the exchanged sums
@@ -2158,7 +2196,7 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // the inner ADMM in registers up to REG_T steps, else in shared memory
   const int ic = inner_chunk(p.T);
   const bool vn = (p.T % NODE_VW == 0);
-  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false, false>, 0) : resident_grid(node_kernel<1, false, false>, 0);
+  const int gn = vn ? resident_grid(node_kernel<NODE_VW, false, false, false>, 0) : resident_grid(node_kernel<1, false, false, false>, 0);
   const int gx = v4 ? resident_grid(xs_kernel<4>, 0) : resident_grid(xs_kernel<1>, 0);
   const int gd = v2 ? resident_grid(dsum_kernel<2>, 0) : resident_grid(dsum_kernel<1>, 0);
   if (gn < 1 || gx < 1 || gd < 1) return -1;
@@ -2192,6 +2230,7 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   if (!allow_smem(dev_kernel<0>, ism)) return -1;
   plan->inner_smem = ism;
   plan->fused = !p.slice && max_rounds < 2;
+  plan->node_lat = plan->fused && nn <= (vn ? NODE_LAT_ITEMS4 : NODE_LAT_ITEMS1);
   plan->xs_grid = plan->dsum_grid = plan->dev_closed = 0;
   plan->dev_inner = one_round;
   if (plan->fused) {
@@ -2243,13 +2282,16 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
   const bool vn = p.T % NODE_VW == 0, rx = p.alpha != 1.f;
   const int g = plan.node_grid;
-#define NODE_LAUNCH(RX, ILD)                                           \
-  if (vn) node_kernel<NODE_VW, RX, ILD><<<g, BLOCK, 0, sm>>>(p);       \
-  else node_kernel<1, RX, ILD><<<g, BLOCK, 0, sm>>>(p)
-  if (rx && plan.fused) { NODE_LAUNCH(true, true); }
-  else if (rx) { NODE_LAUNCH(true, false); }
-  else if (plan.fused) { NODE_LAUNCH(false, true); }
-  else { NODE_LAUNCH(false, false); }
+#define NODE_LAUNCH(RX, ILD, LAT)                                          \
+  if (vn) node_kernel<NODE_VW, RX, ILD, LAT><<<g, BLOCK, 0, sm>>>(p);      \
+  else node_kernel<1, RX, ILD, LAT><<<g, BLOCK, 0, sm>>>(p)
+  if (plan.node_lat) {
+    if (rx) { NODE_LAUNCH(true, true, true); }
+    else { NODE_LAUNCH(false, true, true); }
+  } else if (rx && plan.fused) { NODE_LAUNCH(true, true, false); }
+  else if (rx) { NODE_LAUNCH(true, false, false); }
+  else if (plan.fused) { NODE_LAUNCH(false, true, false); }
+  else { NODE_LAUNCH(false, false, false); }
 #undef NODE_LAUNCH
   if (slice) slice_sums_kernel<<<aux_grid((long long)p.n_dnode * p.T), BLOCK, 0, sm>>>(p, 0);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
