@@ -53,6 +53,7 @@ opf_status cuda_fail(cudaError_t e, const char *what) {
 
 constexpr int kMaxT = 2048;
 constexpr int kMaxHistory = 1 << 20;  // rows of residual history a context may keep
+constexpr int kSmallIters = 1000;  // iterations of a small instance in one launch (a few milliseconds)
 constexpr int kGraphIters = 16;  // iterations in the larger of the two iteration graphs
 
 // bump allocator over one cudaMalloc
@@ -885,7 +886,8 @@ opf_status opf_iterate(opf_ctx *c, int32_t n_iters, double rho) {
   if (c->slice) return fail(OPF_ESTATE, "a contingency slice iterates through opf_slice_local / opf_slice_finish");
   if (n_iters < 0) return fail(OPF_EINVAL, "n_iters must be >= 0");
   if (rho > 0 && !std::isfinite(rho)) return fail(OPF_EINVAL, "rho must be finite");
-  if (n_iters > 0 && !c->g_one) {
+  const bool small = c->plan.small != 0;
+  if (n_iters > 0 && !small && !c->g_one) {
     opf_status gs = build_graph(c, 1, &c->g_one);
     if (gs == OPF_OK) gs = build_graph(c, kGraphIters, &c->g_many);
     if (gs != OPF_OK) return gs;
@@ -896,8 +898,14 @@ opf_status opf_iterate(opf_ctx *c, int32_t n_iters, double rho) {
   if (rho > 0 && opfk_set_rho_launch(c->P, rho, c->s_main) != 0) return fail(OPF_ECUDA, "set_rho launch failed");
   if (n_iters > 0) {
     if (opfk_begin_launch(c->P, n_iters, 1, c->s_main) != 0) return fail(OPF_ECUDA, "begin launch failed");
-    for (int i = 0; i < n_iters / kGraphIters; ++i) CK(cudaGraphLaunch(c->g_many, c->s_main));
-    for (int i = 0; i < n_iters % kGraphIters; ++i) CK(cudaGraphLaunch(c->g_one, c->s_main));
+    if (small) {
+      for (int64_t i = 0; i < n_iters; i += kSmallIters)
+        if (opfk_small_launch(c->P, (int)std::min<int64_t>(kSmallIters, n_iters - i), c->s_main) != 0)
+          return fail(OPF_ECUDA, "iteration launch failed");
+    } else {
+      for (int i = 0; i < n_iters / kGraphIters; ++i) CK(cudaGraphLaunch(c->g_many, c->s_main));
+      for (int i = 0; i < n_iters % kGraphIters; ++i) CK(cudaGraphLaunch(c->g_one, c->s_main));
+    }
   }
   // ... and before its later work
   CK(cudaEventRecord(c->ev_out, c->s_main));
@@ -996,7 +1004,7 @@ opf_status opf_get_info(opf_ctx *c, opf_info *info) {
     // devices (one launch, or averages, inner ADMM and sums), lines, nodes; a
     // slice's decisions are a launch of their own (opf_slice_finish)
     const int dev = (pl.dev_inner + pl.dev_closed > 0) + (pl.fused ? 0 : (pl.xs_grid > 0) + 1);
-    info->kernels_per_iteration = dev + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
+    info->kernels_per_iteration = pl.small ? 1 : dev + (pl.line_grid > 0) + 1 + (c->slice ? 1 : 0);
   }
   info->N = c->N;
   info->L = c->L;

@@ -227,6 +227,7 @@ __host__ __device__ __forceinline__ void set_iter(const Params &p, DevScalars &s
 struct IterPlan {
   int line_grid, node_grid;            // 0: the kernel has no work
   int line_ipt;                        // line items per thread
+  int small;                           // 1: whole iterations on one CTA (opfk_small_launch)
   int node_lat;                        // few node items: all loads of an item requested together
   int fused;                           // 1: one device kernel; 0: averages, inner ADMM and device sums apart
   int dev_inner, dev_closed;           // CTAs of the device kernel for inner-ADMM and (fused) closed-form devices
@@ -276,6 +277,8 @@ int opfk_begin_batch_launch(const opfk::Params *d_params, int n_inst, long long 
 // stream capture.
 int opfk_iteration_enqueue(const opfk::Params &p, const opfk::IterPlan &plan, void *main_stream,
                            void *aux_stream, void *ev_fork, void *ev_join);
+// n iterations of a small instance (IterPlan::small) in one launch.
+int opfk_small_launch(const opfk::Params &p, int n, void *stream);
 // Schedules of the batch kernels for n instances (host parameter copies and
 // their plans): fills sched (4 ints per CTA, BatchPlan order) and the plan.
 int opfk_batch_plan(const opfk::Params *hp, const opfk::IterPlan *plans, int n, const opfk::BatchLayout &lay,

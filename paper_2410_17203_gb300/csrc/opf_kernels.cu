@@ -67,6 +67,9 @@ constexpr long long LINE_SHORT = 1 << 20;   // ... one, up to this many items
 constexpr int DEVB = 128;        // threads per CTA of the device kernel (its inner-ADMM warps spread over more SMs)
 constexpr int DEV_WARPS = DEVB / 32;
 constexpr int CLOSED_LANES4 = 2, CLOSED_LANES1 = 8;   // lanes per closed-form item: the classes of ksum2 / ksum8
+// microseconds of a small instance's iteration on one CTA: base, per round of
+// items, and the limit (opfk_plan)
+constexpr double SMALL_BASE = 2.7, SMALL_LINE = 0.8, SMALL_CLOSED = 0.45, SMALL_NODE = 1.2, SMALL_LIMIT = 8.0;
 constexpr int REG_C = 8;           // largest chunk of the register-resident inner ADMM ...
 constexpr int REG_T = 32 * REG_C - 1;   // ... its longest horizon (T + 1 <= 32 C)
 constexpr int BATCH_C = 4;         // the same in batches, whose kernels hold every chunk up to theirs
@@ -1349,9 +1352,8 @@ __device__ __forceinline__ FV<VW> group_ksum(const float *r, int T, int Kp, int 
 }
 
 template <int VW>
-__device__ __forceinline__ void closed_body(const Params &p, unsigned bid, unsigned nblk) {
+__device__ __forceinline__ void closed_body(const Params &p, const Iter &q, unsigned bid, unsigned nblk) {
   constexpr int G = VW == 4 ? CLOSED_LANES4 : CLOSED_LANES1;
-  const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
   const int T = p.T, TV = T / VW, Kp = p.Kp, c = threadIdx.x & (G - 1);
   const unsigned gmask = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
@@ -1543,6 +1545,15 @@ __device__ __forceinline__ bool reduce_partials(const Params &p, int n_part, dou
   return true;
 }
 
+// the scalars of the iteration after q, which formed no residuals
+__device__ __forceinline__ Iter next_iter(Iter q) {
+  q.fsu = q.fsv = 1.f;
+  q.old ^= 1;
+  q.left -= 1;
+  q.flags = q.left == 0 ? ITF_RES : 0;
+  return q;
+}
+
 // An iteration whose residuals nobody reads (a non-finite value is caught at
 // the next one that forms them): one thread advances the counter with stores
 // alone.  Reading the scalars back and forming the next iteration's from them
@@ -1553,12 +1564,7 @@ __device__ __forceinline__ void advance(const Params &p) {
     Iter r;
     int4 v[2];
   } x;
-  const Iter q = load_iter(p);
-  x.r = q;
-  x.r.fsu = x.r.fsv = 1.f;
-  x.r.old = q.old ^ 1;
-  x.r.left = q.left - 1;
-  x.r.flags = x.r.left == 0 ? ITF_RES : 0;
+  x.r = next_iter(load_iter(p));
   int4 *d = reinterpret_cast<int4 *>(&p.sc->cur);
   d[0] = x.v[0];
   d[1] = x.v[1];
@@ -1653,6 +1659,26 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part, double 
   *p.sc = sc;
 }
 
+// the CTA's residual partial sums, FP32 per thread and FP64 across warps, as
+// partial number `part`
+__device__ __forceinline__ void write_partials(const Params &p, unsigned part, const float (&acc)[NSLOT],
+                                               double (*red)[NSLOT]) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) {
+    float v = acc[s];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[wib][s] = (double)v;
+  }
+  __syncthreads();
+  if (threadIdx.x < NSLOT) {
+    double v = 0.0;
+    for (int w = 0; w < WARPS; ++w) v += red[w][threadIdx.x];
+    p.partials[(size_t)part * NSLOT + threadIdx.x] = v;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // node: step 3 for every (contingency, node, VW time steps); where the
 // residuals are read, the CTA's partial sums (FP32 per thread, FP64 across
@@ -1669,7 +1695,6 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   __shared__ double red[WARPS][NSLOT];
   __shared__ int s_last;
   const int N = p.N, TV = p.T / VW, Kp = p.Kp;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const unsigned n = (unsigned)Kp * (unsigned)N * (unsigned)TV;
   const unsigned stride = nblk * BLOCK;
   unsigned item = bid * BLOCK + threadIdx.x;
@@ -1690,21 +1715,7 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
       node_item<VW, RELAX, false, LAT ? 4 : NODE_LEAN_NB, ILD, LAT>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
   }
-  if (res) {
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-      float v = acc[s];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) red[wib][s] = (double)v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NSLOT) {
-      double v = 0.0;
-      for (int w = 0; w < WARPS; ++w) v += red[w][threadIdx.x];
-      p.partials[(size_t)bid * NSLOT + threadIdx.x] = v;
-    }
-  }
+  if (res) write_partials(p, bid, acc, red);
   if (p.slice) return;
   // the count is taken after every thread of the CTA has read the scalars and
   // (res) its partial sums are written; the last CTA alone goes on
@@ -1745,8 +1756,8 @@ template <int C>
 __global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks, bool avg) {
   extern __shared__ float smem[];
   if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, blockIdx.x, inner_blocks, smem, avg);
-  else if (p.T % 4 == 0) closed_body<4>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
-  else closed_body<1>(p, blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
+  else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
+  else closed_body<1>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
 }
 
 template <int VW>
@@ -1764,6 +1775,77 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p, int ipt) {
 template <int VW, bool RELAX, bool ILD, bool LAT>
 __global__ void __launch_bounds__(BLOCK, LAT ? 2 : RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel(Params p) {
   node_body<VW, RELAX, ILD, LAT>(p, blockIdx.x, gridDim.x);
+}
+
+// ---------------------------------------------------------------------------
+// A small instance on one CTA: n iterations in one launch, their phases apart
+// by CTA barriers instead of kernel boundaries (a microsecond each, and the
+// scalars and static rows come back through L2 every time).  The items, their
+// arithmetic and the residuals' partial sums (one per 256 node items) are
+// those of the kernels above.  30 buses, T = 1, K = 5: 8.35 -> 5.1 us per
+// iteration; what is left are rows that other threads wrote, read through L2.
+// Which instances: opfk_plan.
+// ---------------------------------------------------------------------------
+template <int VW, bool RELAX>
+__device__ __forceinline__ int small_iteration(const Params &p, const Iter &q, double (*red)[NSLOT]) {
+  const int T = p.T, TV = T / VW, Kp = p.Kp;
+  closed_body<VW>(p, q, 0, 1);
+  const unsigned nl = (unsigned)Kp * (unsigned)p.L * (unsigned)TV, nn = (unsigned)Kp * (unsigned)p.N * (unsigned)TV;
+  Idx3 ix;
+  for (unsigned i = threadIdx.x; i < nl; i += BLOCK) {
+    ix.set(i, Kp, TV);
+    line_item<VW>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.frp, q.frt, q.fsu, q.fsv, q.flags & ITF_VFRESH);
+  }
+  __syncthreads();
+  const bool res = q.flags & ITF_RES;
+  unsigned part = 0;
+  for (unsigned base = 0; base < nn; base += BLOCK, ++part) {
+    const unsigned i = base + threadIdx.x;
+    float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    if (i < nn) {
+      ix.set(i, Kp, TV);
+      if (res) node_item<VW, RELAX, true, 4, true, true>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+      else node_item<VW, RELAX, false, 4, true, true>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+    }
+    if (res) {
+      write_partials(p, part, acc, red);
+      __syncthreads();   // red is used again
+    }
+  }
+  return (int)part;
+}
+
+template <bool RELAX>
+__global__ void __launch_bounds__(BLOCK) small_kernel(Params p, int n) {
+  __shared__ double red[WARPS][NSLOT];
+  Iter q = load_iter(p);   // every thread's own copy, stored where residuals are formed and at the end
+  int ahead = 0;           // iterations run since it was last stored
+  auto store = [&]() {
+    if (threadIdx.x == 0 && ahead) {
+      DevScalars sc = *p.sc;
+      sc.it += ahead;
+      sc.su = sc.sv = 1.0;
+      sc.v_fresh = 0;
+      sc.cur = q;
+      *p.sc = sc;
+    }
+    ahead = 0;
+  };
+  for (int i = 0; i < n && !(q.flags & ITF_SKIP); ++i) {
+    const bool res = q.flags & ITF_RES;
+    const int parts = p.T % 4 == 0 ? small_iteration<4, RELAX>(p, q, red) : small_iteration<1, RELAX>(p, q, red);
+    if (res) {
+      store();
+      decide_body(p, parts, red);
+      __syncthreads();
+      q = load_iter(p);
+    } else {
+      q = next_iter(q);
+      ++ahead;
+      __syncthreads();
+    }
+  }
+  store();
 }
 
 // a slice's decisions, from the exchanged sums
@@ -1846,8 +1928,8 @@ __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
   if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true);
-  else if (p.T % 4 == 0) closed_body<4>(p, bid, nblk);
-  else closed_body<1>(p, bid, nblk);
+  else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), bid, nblk);
+  else closed_body<1>(p, load_iter(p), bid, nblk);
 }
 
 // the lines of every instance: the first n4 CTAs of the schedule take those
@@ -2231,6 +2313,15 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   plan->inner_smem = ism;
   plan->fused = !p.slice && max_rounds < 2;
   plan->node_lat = plan->fused && nn <= (vn ? NODE_LAT_ITEMS4 : NODE_LAT_ITEMS1);
+  // A small instance without inner-ADMM devices runs on one CTA (small_kernel)
+  // where its rounds of 256 line, closed-form and node items are estimated to
+  // take less than the kernels' 8.3 us: 30 buses, T = 1, K = 5 8.35 -> 5.1 us,
+  // 100 buses, K = 0 8.2 -> 5.9, 20 buses, T = 24, K = 2 8.5 -> 6.6; beyond
+  // the limit 60 buses, K = 5 8.3 against 8.0, 100 buses, K = 10 8.6 against 14.6.
+  const long long nc = (long long)p.n_cnode * tvl * (v4 ? CLOSED_LANES4 : CLOSED_LANES1);
+  auto rounds = [](long long items) { return (double)((items + BLOCK - 1) / BLOCK); };
+  plan->small = plan->fused && n_inner == 0 &&
+                SMALL_BASE + SMALL_LINE * rounds(nl) + SMALL_CLOSED * rounds(nc) + SMALL_NODE * rounds(nn) <= SMALL_LIMIT;
   plan->xs_grid = plan->dsum_grid = plan->dev_closed = 0;
   plan->dev_inner = one_round;
   if (plan->fused) {
@@ -2305,6 +2396,14 @@ int opfk_iteration_enqueue(const Params &p, const IterPlan &plan, void *main_str
 int opfk_slice_local_enqueue(const Params &p, const IterPlan &plan, void *main_stream, void *aux_stream,
                              void *ev_fork, void *ev_join) {
   return iteration_enqueue(p, plan, main_stream, aux_stream, ev_fork, ev_join, true);
+}
+
+int opfk_small_launch(const Params &p, int n, void *stream) {
+  cudaStream_t s = (cudaStream_t)stream;
+  const bool rx = p.alpha != 1.f;
+  if (rx) small_kernel<true><<<1, BLOCK, 0, s>>>(p, n);
+  else small_kernel<false><<<1, BLOCK, 0, s>>>(p, n);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int opfk_slice_finish_enqueue(const Params &p, void *stream) {

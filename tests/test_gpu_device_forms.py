@@ -110,3 +110,39 @@ def test_inner_state_round_trip(T):
         compare_states(s.state(), o)
         s.close()
     a.close()
+
+
+@pytest.mark.parametrize("n, T, K, alpha", [(30, 1, 5, 1.0), (20, 24, 2, 1.0), (12, 7, 1, 1.5), (2, 1, 0, 1.0), (20, 8, 2, 1.5)])
+def test_small_instance_on_one_cta(n, T, K, alpha):
+    """An instance without inner-ADMM devices that fits one CTA's rounds runs
+    whole calls in one launch: iterates, residuals, penalties and the residual
+    history equal those of the batch kernels bit for bit, over calls that end
+    on and between residual iterations."""
+    from paper_2410_17203_gb300 import Solver, opf_batch_create, opf_batch_destroy, opf_batch_iterate
+    case = make_case(scale_case(n, T, K, seed=n + T, stor_per_node=0.0, ramp=False, fixed_frac=0.3,
+                                n_hvdc=0, lines_per_node=1.3 if n > 2 else 0.5))
+    opts = dict(adapt_every=10, eps=1e-9, check_every=7, alpha=alpha)
+    a, b = Solver(case, opts), Solver(case, opts)
+    assert a.info["kernels_per_iteration"] == 1
+    h = opf_batch_create([b.h])
+    try:
+        for m in (1, 6, 13, 20, 1, 1060):
+            a.iterate(m)
+            opf_batch_iterate(h, m)
+            x, y = a.state(), b.state()
+            for k in x:
+                np.testing.assert_array_equal(x[k], y[k], err_msg=k)
+            np.testing.assert_array_equal(a.residuals(), b.residuals())
+        np.testing.assert_array_equal(a.history(), b.history())
+        i, j = a.get_info(), b.get_info()
+        assert (i["iterations"], i["rho_p"], i["rho_theta"]) == (j["iterations"], j["rho_p"], j["rho_theta"])
+        o = Oracle(case, OracleOptions(adapt_every=10, eps=0.0, alpha=alpha))
+        o.iterate(30, stop=False)
+        c = Solver(case, dict(adapt_every=10, eps=0.0, alpha=alpha))
+        c.iterate(30)
+        compare_states(c.state(), o)
+        c.close()
+    finally:
+        opf_batch_destroy(h)
+        a.close()
+        b.close()
