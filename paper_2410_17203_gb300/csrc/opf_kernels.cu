@@ -635,6 +635,9 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
 // instance, a batch) computes the same bits.
 // ---------------------------------------------------------------------------
 
+// Lanes beyond the horizon run along (right-hand side 0, nothing of theirs is
+// stored or read by others), which spares the inner iterations a branch per
+// element.
 // The state that does not depend on the iteration's scalars is requested
 // first, with them; the contingency rows of the node and the box follow when
 // the device's record arrives, so the ten inner iterations wait for two rounds
@@ -705,28 +708,23 @@ __device__ void ramp_prox_r(const Params &p, int r, int lane, bool avg) {
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int t = t0 + j;
-      if (t < T) {
-        float atr = rsub(rsub(radd(hi[j], bet[RG_UP][j]), lam[RG_UP][j]),
-                         rsub(radd(-lo[j], bet[RG_LO][j]), lam[RG_LO][j]));
-        if (t >= 1) atr = radd(atr, (j == 0) ? wprev : W[j - 1]);
-        if (t <= T - 2) atr = rsub(atr, W[j]);
-        Z[j] = rfma(om, atr, rfma(rho, X[j], -b));
-      }
+      float atr = rsub(rsub(radd(hi[j], bet[RG_UP][j]), lam[RG_UP][j]),
+                       rsub(radd(-lo[j], bet[RG_LO][j]), lam[RG_LO][j]));
+      if (t >= 1) atr = radd(atr, (j == 0) ? wprev : W[j - 1]);
+      if (t <= T - 2) atr = rsub(atr, W[j]);
+      Z[j] = t < T ? rfma(om, atr, rfma(rho, X[j], -b)) : 0.f;
     }
     warp_tri_solve_r<C>(tf, Z, T, lane);
     const float znext = __shfl_down_sync(FULL, Z[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-      const int t = t0 + j;
-      if (t < T) {
-        const float pt = Z[j];
-        ineq_step(rsub(pt, hi[j]), lam[RG_UP][j], bet[RG_UP][j]);
-        ineq_step(rsub(lo[j], pt), lam[RG_LO][j], bet[RG_LO][j]);
-        if (t < T - 1) {
-          const float pn = (j == C - 1) ? znext : Z[j + 1];
-          ineq_step(rsub(rsub(pn, pt), R), lam[RG_RU][j], bet[RG_RU][j]);
-          ineq_step(rsub(rsub(pt, pn), R), lam[RG_RD][j], bet[RG_RD][j]);
-        }
+      const float pt = Z[j];
+      ineq_step(rsub(pt, hi[j]), lam[RG_UP][j], bet[RG_UP][j]);
+      ineq_step(rsub(lo[j], pt), lam[RG_LO][j], bet[RG_LO][j]);
+      if (t0 + j < T - 1) {
+        const float pn = (j == C - 1) ? znext : Z[j + 1];
+        ineq_step(rsub(rsub(pn, pt), R), lam[RG_RU][j], bet[RG_RU][j]);
+        ineq_step(rsub(rsub(pt, pn), R), lam[RG_RD][j], bet[RG_RD][j]);
       }
     }
   }
@@ -824,64 +822,55 @@ __device__ void stor_prox_r(const Params &p, int sidx, int lane, bool avg) {
     float f0c[C], f0d[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-      f0c[j] = f0d[j] = 0.f;
-      if (t0 + j < T) {
-        const float r1 = -lE1[j], r2 = -lE2[j];
-        const float mc = rmul(0.5f, rsub(rsub(radd(Pm, bCU[j]), lCU[j]), rsub(bCL[j], lCL[j])));
-        const float md = rmul(0.5f, rsub(rsub(radd(Pm, bDU[j]), lDU[j]), rsub(bDL[j], lDL[j])));
-        const float e1 = rsub(r1, X[j]);
-        f0c[j] = rfma(kap, e1, rmul(om2, mc));
-        f0d[j] = rfma(om2, md, rsub(rmul(-kap, e1), q));
-        TAU[j] = radd(r2, qdiv(rfma(w0, f0c[j], rmul(w1, f0d[j])), gam, rgam));
-      }
+      const float r1 = -lE1[j], r2 = -lE2[j];
+      const float mc = rmul(0.5f, rsub(rsub(radd(Pm, bCU[j]), lCU[j]), rsub(bCL[j], lCL[j])));
+      const float md = rmul(0.5f, rsub(rsub(radd(Pm, bDU[j]), lDU[j]), rsub(bDL[j], lDL[j])));
+      const float e1 = rsub(r1, X[j]);
+      f0c[j] = rfma(kap, e1, rmul(om2, mc));
+      f0d[j] = rfma(om2, md, rsub(rmul(-kap, e1), q));
+      TAU[j] = radd(r2, qdiv(rfma(w0, f0c[j], rmul(w1, f0d[j])), gam, rgam));
     }
     const float tprev = __shfl_up_sync(FULL, TAU[C - 1], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
-      if (e < Tp) {
-        const float ms = rmul(0.5f, rsub(rsub(radd(Em, bSU[j]), lSU[j]), rsub(bSL[j], lSL[j])));
-        float rhs = rmul(om2, ms);
-        if (e >= 1) rhs = rfma(gam, (j == 0) ? tprev : TAU[j - 1], rhs);
-        if (e <= T - 1) rhs = rfma(-gam, TAU[j], rhs);
-        if (e == 0) rhs = rfma(-om, e3a, rhs);
-        if (e == T) rhs = rfma(-om, e3b, rhs);
-        S[j] = rhs;
-      }
+      const float ms = rmul(0.5f, rsub(rsub(radd(Em, bSU[j]), lSU[j]), rsub(bSL[j], lSL[j])));
+      float rhs = rmul(om2, ms);
+      if (e >= 1) rhs = rfma(gam, (j == 0) ? tprev : TAU[j - 1], rhs);
+      if (e <= T - 1) rhs = rfma(-gam, TAU[j], rhs);
+      if (e == 0) rhs = rfma(-om, e3a, rhs);
+      if (e == T) rhs = rfma(-om, e3b, rhs);
+      S[j] = e < Tp ? rhs : 0.f;
     }
     warp_tri_solve_r<C>(tf, S, Tp, lane);
     const float snext = __shfl_down_sync(FULL, S[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-      if (t0 + j < T) {
-        const float r1 = -lE1[j], r2 = -lE2[j];
-        const float s0 = S[j], s1 = (j == C - 1) ? snext : S[j + 1];
-        const float ds = rsub(s1, s0);
-        const float g = rsub(ds, r2);
-        const float fc = rfma(g, f1c, f0c[j]), fd = rfma(g, f1d, f0d[j]);
-        const float c = rfma(i00, fc, rmul(i01, fd));
-        const float dl = rfma(i01, fc, rmul(i11, fd));
-        const float pt = qdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[j])), rpo, rrpo);
-        TAU[j] = pt;   // TAU is consumed; keep p_t for the end
-        DL[j] = dl;
-        lE1[j] = radd(lE1[j], rsub(radd(pt, c), dl));   // equality rows: beta = 0
-        lE2[j] = radd(lE2[j], radd(rfma(-eta, c, ds), dl));
-        ineq_step(rsub(c, Pm), lCU[j], bCU[j]);
-        ineq_step(-c, lCL[j], bCL[j]);
-        ineq_step(rsub(dl, Pm), lDU[j], bDU[j]);
-        ineq_step(-dl, lDL[j], bDL[j]);
-      }
+      const float r1 = -lE1[j], r2 = -lE2[j];
+      const float s0 = S[j], s1 = (j == C - 1) ? snext : S[j + 1];
+      const float ds = rsub(s1, s0);
+      const float g = rsub(ds, r2);
+      const float fc = rfma(g, f1c, f0c[j]), fd = rfma(g, f1d, f0d[j]);
+      const float c = rfma(i00, fc, rmul(i01, fd));
+      const float dl = rfma(i01, fc, rmul(i11, fd));
+      const float pt = qdiv(rfma(om, radd(rsub(r1, c), dl), rmul(rho, X[j])), rpo, rrpo);
+      TAU[j] = pt;   // TAU is consumed; keep p_t for the end
+      DL[j] = dl;
+      lE1[j] = radd(lE1[j], rsub(radd(pt, c), dl));   // equality rows: beta = 0
+      lE2[j] = radd(lE2[j], radd(rfma(-eta, c, ds), dl));
+      ineq_step(rsub(c, Pm), lCU[j], bCU[j]);
+      ineq_step(-c, lCL[j], bCL[j]);
+      ineq_step(rsub(dl, Pm), lDU[j], bDU[j]);
+      ineq_step(-dl, lDL[j], bDL[j]);
     }
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
-      if (e < Tp) {
-        const float sj = S[j];
-        if (e == 0) e3a = radd(e3a, sj);
-        if (e == T) e3b = radd(e3b, sj);
-        ineq_step(rsub(sj, Em), lSU[j], bSU[j]);
-        ineq_step(-sj, lSL[j], bSL[j]);
-      }
+      const float sj = S[j];
+      if (e == 0) e3a = radd(e3a, sj);
+      if (e == T) e3b = radd(e3b, sj);
+      ineq_step(rsub(sj, Em), lSU[j], bSU[j]);
+      ineq_step(-sj, lSL[j], bSL[j]);
     }
   }
 #define ST_L(arr, g) lam_g[(g) * Tp + e] = arr[j]

@@ -37,16 +37,16 @@ __device__ __forceinline__ float qdiv(float x, float q, float rq) {
 template <int C>
 struct TriFac {
   float q[C], rq[C], a[C], f[5], b[5];
-  // q set; off_neg = -off
+  // q set (1 from element n on); off_neg = -off
   __device__ __forceinline__ void init(float off_neg, int n, int lane) {
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       rq[j] = __frcp_rn(q[j]);
-      a[j] = qdiv(off_neg, q[j], rq[j]);
+      a[j] = lane * C + j < n ? qdiv(off_neg, q[j], rq[j]) : 0.f;
     }
     init_scans(n, lane);
   }
-  // q and a set
+  // q and a set (1 and 0 from element n on)
   __device__ __forceinline__ void init(int n, int lane) {
 #pragma unroll
     for (int j = 0; j < C; ++j) rq[j] = __frcp_rn(q[j]);
@@ -56,11 +56,9 @@ struct TriFac {
     const int i0 = lane * C;
     float Af = 1.f, Ab = 1.f;
 #pragma unroll
-    for (int j = 0; j < C; ++j)
-      if (i0 + j < n) Af = rmul((i0 + j == 0) ? 0.f : a[j], Af);
+    for (int j = 0; j < C; ++j) Af = rmul((i0 + j == 0) ? 0.f : a[j], Af);
 #pragma unroll
-    for (int j = C - 1; j >= 0; --j)
-      if (i0 + j < n) Ab = rmul((i0 + j == n - 1) ? 0.f : a[j], Ab);
+    for (int j = C - 1; j >= 0; --j) Ab = rmul((i0 + j == n - 1) ? 0.f : a[j], Ab);
 #pragma unroll
     for (int l = 0; l < 5; ++l) {
       const int d = 1 << l;
@@ -75,7 +73,8 @@ struct TriFac {
 
 // x := M^-1 x on a chunk held in registers: first-order recurrences (forward
 // y_i = a_i y_{i-1} + r_i / q_i, then backward) composed over each lane's
-// chunk, then across the warp by shuffle scans
+// chunk, then across the warp by shuffle scans.  Elements from n on take part
+// with x = 0, pivot 1 and a = 0 (and stay 0), so no lane branches.
 template <int C>
 __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[C], int n, int lane) {
   const int i0 = lane * C;
@@ -83,11 +82,8 @@ __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[
   float Bc = 0.f;
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    r[j] = 0.f;
-    if (i0 + j < n) {
-      r[j] = qdiv(x[j], m.q[j], m.rq[j]);
-      Bc = rfma((i0 + j == 0) ? 0.f : m.a[j], Bc, r[j]);
-    }
+    r[j] = qdiv(x[j], m.q[j], m.rq[j]);
+    Bc = rfma((i0 + j == 0) ? 0.f : m.a[j], Bc, r[j]);
   }
 #pragma unroll
   for (int l = 0; l < 5; ++l) {
@@ -98,15 +94,12 @@ __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[
   if (lane == 0) prev = 0.f;
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    if (i0 + j < n) {
-      prev = rfma((i0 + j == 0) ? 0.f : m.a[j], prev, r[j]);
-      x[j] = prev;
-    }
+    prev = rfma((i0 + j == 0) ? 0.f : m.a[j], prev, r[j]);
+    x[j] = prev;
   }
   Bc = 0.f;
 #pragma unroll
-  for (int j = C - 1; j >= 0; --j)
-    if (i0 + j < n) Bc = rfma((i0 + j == n - 1) ? 0.f : m.a[j], Bc, x[j]);
+  for (int j = C - 1; j >= 0; --j) Bc = rfma((i0 + j == n - 1) ? 0.f : m.a[j], Bc, x[j]);
 #pragma unroll
   for (int l = 0; l < 5; ++l) {
     const float Bp = __shfl_down_sync(FULL, Bc, 1 << l);
@@ -116,10 +109,8 @@ __device__ __forceinline__ void warp_tri_solve_r(const TriFac<C> &m, float (&x)[
   if (lane == 31) nxt = 0.f;
 #pragma unroll
   for (int j = C - 1; j >= 0; --j) {
-    if (i0 + j < n) {
-      nxt = rfma((i0 + j == n - 1) ? 0.f : m.a[j], nxt, x[j]);
-      x[j] = nxt;
-    }
+    nxt = rfma((i0 + j == n - 1) ? 0.f : m.a[j], nxt, x[j]);
+    x[j] = nxt;
   }
 }
 
