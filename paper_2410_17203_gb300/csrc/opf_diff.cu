@@ -1043,7 +1043,9 @@ struct StorK {
 };
 
 // z := M^-1 z for a battery, z = (p, c, delta) at steps t < T, s at j <= T
-// (element e = lane C + j holds step e and state of charge e)
+// (element e = lane C + j holds step e and state of charge e).  Steps from T
+// and charges from T + 1 on come in as 0 and take part without a branch: the
+// latter stay 0, the former leave with values that nobody reads.
 template <int C>
 __device__ __forceinline__ void stor_solve_r(const StorK &k, const TriFac<C> &tf,
                                              float (&zp)[C], float (&zc)[C], float (&zd)[C], float (&zs)[C], int T,
@@ -1053,37 +1055,30 @@ __device__ __forceinline__ void stor_solve_r(const StorK &k, const TriFac<C> &tf
   float u[C], yc[C], yd[C], fy[C];
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    u[j] = yc[j] = yd[j] = fy[j] = 0.f;
-    if (t0 + j < T) {
-      u[j] = qdiv(zp[j], k.rpo, k.rrpo);                          // p = u - omega (c - delta) / (rho + omega)
-      const float rc = rsub(zc[j], rmul(k.om, u[j])), rd = radd(zd[j], rmul(k.om, u[j]));
-      yc[j] = rfma(k.i00, rc, rmul(k.i01, rd));             // y = H^-1 r'
-      yd[j] = rfma(k.i01, rc, rmul(k.i11, rd));
-      fy[j] = rfma(fc, yc[j], rmul(fd, yd[j]));
-    }
+    u[j] = qdiv(zp[j], k.rpo, k.rrpo);                      // p = u - omega (c - delta) / (rho + omega)
+    const float rc = rsub(zc[j], rmul(k.om, u[j])), rd = radd(zd[j], rmul(k.om, u[j]));
+    yc[j] = rfma(k.i00, rc, rmul(k.i01, rd));               // y = H^-1 r'
+    yd[j] = rfma(k.i01, rc, rmul(k.i11, rd));
+    fy[j] = rfma(fc, yc[j], rmul(fd, yd[j]));
   }
   const float fyp = __shfl_up_sync(FULLM, fy[C - 1], 1);
 #pragma unroll
   for (int j = 0; j < C; ++j) {
     const int e = t0 + j;
-    if (e <= T) {
-      float r = zs[j];
-      if (e <= T - 1) r = radd(r, fy[j]);
-      if (e >= 1) r = rsub(r, (j == 0) ? fyp : fy[j - 1]);
-      zs[j] = r;
-    }
+    float r = zs[j];
+    if (e <= T - 1) r = radd(r, fy[j]);
+    if (e >= 1) r = rsub(r, (j == 0) ? fyp : fy[j - 1]);
+    zs[j] = r;
   }
   warp_tri_solve_r<C>(tf, zs, T + 1, lane);
   const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
   for (int j = 0; j < C; ++j) {
-    if (t0 + j < T) {
-      const float dsv = rsub((j == C - 1) ? sn : zs[j + 1], zs[j]);
-      const float c = rsub(yc[j], rmul(k.gc, dsv)), dl = rsub(yd[j], rmul(k.gd, dsv));
-      zc[j] = c;
-      zd[j] = dl;
-      zp[j] = rsub(u[j], qdiv(rmul(k.om, rsub(c, dl)), k.rpo, k.rrpo));
-    }
+    const float dsv = rsub((j == C - 1) ? sn : zs[j + 1], zs[j]);
+    const float c = rsub(yc[j], rmul(k.gc, dsv)), dl = rsub(yd[j], rmul(k.gd, dsv));
+    zc[j] = c;
+    zd[j] = dl;
+    zp[j] = rsub(u[j], qdiv(rmul(k.om, rsub(c, dl)), k.rpo, k.rrpo));
   }
 }
 
@@ -1110,27 +1105,21 @@ __device__ void ramp_fwd_r(int T, int lane, float rho, float om, float qlin, con
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int t = t0 + j;
-      z[j] = 0.f;
-      if (t < T) {
-        float acc = rsub(rsub(radd(hU[j], bU[j]), lU[j]), rsub(radd(hL[j], bL[j]), lL[j]));   // A'w, w = h + beta - lambda
-        if (t >= 1) acc = radd(acc, rsub(j ? wRU[j - 1] : pRU, j ? wRD[j - 1] : pRD));
-        if (t <= T - 2) acc = rsub(acc, rsub(wRU[j], wRD[j]));
-        z[j] = rfma(rho, x[j], rfma(om, acc, -qlin));                                           // r
-      }
+      float acc = rsub(rsub(radd(hU[j], bU[j]), lU[j]), rsub(radd(hL[j], bL[j]), lL[j]));   // A'w, w = h + beta - lambda
+      if (t >= 1) acc = radd(acc, rsub(j ? wRU[j - 1] : pRU, j ? wRD[j - 1] : pRD));
+      if (t <= T - 2) acc = rsub(acc, rsub(wRU[j], wRD[j]));
+      z[j] = t < T ? rfma(rho, x[j], rfma(om, acc, -qlin)) : 0.f;                           // r
     }
     warp_tri_solve_r<C>(tf, z, T, lane);
     const float zn = __shfl_down_sync(FULLM, z[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-      const int t = t0 + j;
-      if (t < T) {
-        ineq_r(rsub(z[j], hU[j]), lU[j], bU[j], bits, j);
-        ineq_r(rsub(-z[j], hL[j]), lL[j], bL[j], bits, C + j);
-        if (t < T - 1) {
-          const float znx = (j == C - 1) ? zn : z[j + 1];
-          ineq_r(rsub(rsub(znx, z[j]), hRU[j]), lRU[j], bRU[j], bits, 2 * C + j);
-          ineq_r(rsub(rsub(z[j], znx), hRD[j]), lRD[j], bRD[j], bits, 3 * C + j);
-        }
+      ineq_r(rsub(z[j], hU[j]), lU[j], bU[j], bits, j);
+      ineq_r(rsub(-z[j], hL[j]), lL[j], bL[j], bits, C + j);
+      if (t0 + j < T - 1) {
+        const float znx = (j == C - 1) ? zn : z[j + 1];
+        ineq_r(rsub(rsub(znx, z[j]), hRU[j]), lRU[j], bRU[j], bits, 2 * C + j);
+        ineq_r(rsub(rsub(z[j], znx), hRD[j]), lRD[j], bRD[j], bits, 3 * C + j);
       }
     }
     if (rec) rec[(size_t)it * 32 + lane] = bits;
@@ -1170,44 +1159,36 @@ __device__ void stor_fwd_r(int T, int lane, const StorK &k, float cost, float Pm
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
-      zp[j] = zc[j] = zd[j] = zs[j] = 0.f;
-      if (e < T) {
-        const float wE1 = -lam.v[SE1][j];
-        const float wCU = rsub(radd(Pm, bet.v[SCU][j]), lam.v[SCU][j]), wCL = rsub(bet.v[SCL][j], lam.v[SCL][j]);
-        const float wDU = rsub(radd(Pm, bet.v[SDU][j]), lam.v[SDU][j]), wDL = rsub(bet.v[SDL][j], lam.v[SDL][j]);
-        zp[j] = rfma(k.rho, x[j], rmul(k.om, wE1));
-        zc[j] = rmul(k.om, rsub(radd(rfma(-k.eta, wE2[j], wE1), wCU), wCL));
-        zd[j] = rsub(rmul(k.om, rsub(radd(radd(-wE1, wE2[j]), wDU), wDL)), cost);
-      }
-      if (e <= T) {
-        float as = rsub(rsub(radd(Em, bet.v[SSU][j]), lam.v[SSU][j]), rsub(bet.v[SSL][j], lam.v[SSL][j]));
-        if (e >= 1) as = radd(as, (j == 0) ? pE2 : wE2[j - 1]);
-        if (e <= T - 1) as = rsub(as, wE2[j]);
-        if (e == 0) as = rsub(as, lam.E3a);
-        if (e == T) as = rsub(as, lam.E3b);
-        zs[j] = rmul(k.om, as);
-      }
+      const bool st = e < T;
+      const float wE1 = -lam.v[SE1][j];
+      const float wCU = rsub(radd(Pm, bet.v[SCU][j]), lam.v[SCU][j]), wCL = rsub(bet.v[SCL][j], lam.v[SCL][j]);
+      const float wDU = rsub(radd(Pm, bet.v[SDU][j]), lam.v[SDU][j]), wDL = rsub(bet.v[SDL][j], lam.v[SDL][j]);
+      zp[j] = st ? rfma(k.rho, x[j], rmul(k.om, wE1)) : 0.f;
+      zc[j] = st ? rmul(k.om, rsub(radd(rfma(-k.eta, wE2[j], wE1), wCU), wCL)) : 0.f;
+      zd[j] = st ? rsub(rmul(k.om, rsub(radd(radd(-wE1, wE2[j]), wDU), wDL)), cost) : 0.f;
+      float as = rsub(rsub(radd(Em, bet.v[SSU][j]), lam.v[SSU][j]), rsub(bet.v[SSL][j], lam.v[SSL][j]));
+      if (e >= 1) as = radd(as, (j == 0) ? pE2 : wE2[j - 1]);
+      if (e <= T - 1) as = rsub(as, wE2[j]);
+      if (e == 0) as = rsub(as, lam.E3a);
+      if (e == T) as = rsub(as, lam.E3b);
+      zs[j] = e <= T ? rmul(k.om, as) : 0.f;
     }
     stor_solve_r<C>(k, tf, zp, zc, zd, zs, T, lane);
     const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int e = t0 + j;
-      if (e < T) {
-        const float snx = (j == C - 1) ? sn : zs[j + 1];
-        lam.v[SE1][j] = radd(rsub(radd(zp[j], zc[j]), zd[j]), lam.v[SE1][j]);                          // equality rows
-        lam.v[SE2][j] = radd(radd(rfma(-k.eta, zc[j], rsub(snx, zs[j])), zd[j]), lam.v[SE2][j]);
-        ineq_r(rsub(zc[j], Pm), lam.v[SCU][j], bet.v[SCU][j], bits, SCU * C + j);
-        ineq_r(-zc[j], lam.v[SCL][j], bet.v[SCL][j], bits, SCL * C + j);
-        ineq_r(rsub(zd[j], Pm), lam.v[SDU][j], bet.v[SDU][j], bits, SDU * C + j);
-        ineq_r(-zd[j], lam.v[SDL][j], bet.v[SDL][j], bits, SDL * C + j);
-      }
-      if (e <= T) {
-        if (e == 0) lam.E3a = radd(zs[j], lam.E3a);
-        if (e == T) lam.E3b = radd(zs[j], lam.E3b);
-        ineq_r(rsub(zs[j], Em), lam.v[SSU][j], bet.v[SSU][j], bits, SSU * C + j);
-        ineq_r(-zs[j], lam.v[SSL][j], bet.v[SSL][j], bits, SSL * C + j);
-      }
+      const float snx = (j == C - 1) ? sn : zs[j + 1];
+      lam.v[SE1][j] = radd(rsub(radd(zp[j], zc[j]), zd[j]), lam.v[SE1][j]);                          // equality rows
+      lam.v[SE2][j] = radd(radd(rfma(-k.eta, zc[j], rsub(snx, zs[j])), zd[j]), lam.v[SE2][j]);
+      ineq_r(rsub(zc[j], Pm), lam.v[SCU][j], bet.v[SCU][j], bits, SCU * C + j);
+      ineq_r(-zc[j], lam.v[SCL][j], bet.v[SCL][j], bits, SCL * C + j);
+      ineq_r(rsub(zd[j], Pm), lam.v[SDU][j], bet.v[SDU][j], bits, SDU * C + j);
+      ineq_r(-zd[j], lam.v[SDL][j], bet.v[SDL][j], bits, SDL * C + j);
+      if (e == 0) lam.E3a = radd(zs[j], lam.E3a);
+      if (e == T) lam.E3b = radd(zs[j], lam.E3b);
+      ineq_r(rsub(zs[j], Em), lam.v[SSU][j], bet.v[SSU][j], bits, SSU * C + j);
+      ineq_r(-zs[j], lam.v[SSL][j], bet.v[SSL][j], bits, SSL * C + j);
     }
     if (rec) rec[(size_t)it * 32 + lane] = bits;   // equality rows never clip: their bits stay 0
   }
@@ -1477,34 +1458,26 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
 #pragma unroll
       for (int j = 0; j < C; ++j) {
         const int t = t0 + j;
-        rb[j] = 0.f;
-        if (t < T) {
-          float acc = rsub(sv[0][j], sv[1][j]);   // A' d s
-          if (t >= 1) acc = radd(acc, rsub(j ? sv[2][j - 1] : pRU, j ? sv[3][j - 1] : pRD));
-          if (t <= T - 2) acc = rsub(acc, rsub(sv[2][j], sv[3][j]));
-          if (it == N_INNER - 1) acc = radd(acc, LPDT[(size_t)dv.dev * T + t]);   // the output p = z_p
-          rb[j] = acc;
-        }
+        float acc = rsub(sv[0][j], sv[1][j]);   // A' d s
+        if (t >= 1) acc = radd(acc, rsub(j ? sv[2][j - 1] : pRU, j ? sv[3][j - 1] : pRD));
+        if (t <= T - 2) acc = rsub(acc, rsub(sv[2][j], sv[3][j]));
+        if (it == N_INNER - 1 && t < T) acc = radd(acc, LPDT[(size_t)dv.dev * T + t]);   // the output p = z_p
+        rb[j] = t < T ? acc : 0.f;
       }
       warp_tri_solve_r<C>(tf, rb, T, lane);
       const float rn = __shfl_down_sync(FULLM, rb[0], 1);
 #pragma unroll
       for (int j = 0; j < C; ++j) {
-        const int t = t0 + j;
-        if (t < T) {
-          xb[j] = rfma(rho, rb[j], xb[j]);
-          const float rnx = (j == C - 1) ? rn : rb[j + 1];
-          float wv[4] = {rmul(om, rb[j]), -rmul(om, rb[j]), 0.f, 0.f};
-          if (t < T - 1) {
-            wv[2] = rmul(om, rsub(rnx, rb[j]));
-            wv[3] = rmul(om, rsub(rb[j], rnx));
-          }
+        const bool rr = t0 + j < T - 1;
+        xb[j] = rfma(rho, rb[j], xb[j]);
+        const float rnx = (j == C - 1) ? rn : rb[j + 1];
+        const float wv[4] = {rmul(om, rb[j]), -rmul(om, rb[j]), rr ? rmul(om, rsub(rnx, rb[j])) : 0.f,
+                             rr ? rmul(om, rsub(rb[j], rnx)) : 0.f};
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            ah[g][j] = radd(ah[g][j], wv[g]);
-            ab[g][j] = wv[g];
-            al[g][j] = rsub(sv[g][j], wv[g]);
-          }
+        for (int g = 0; g < 4; ++g) {
+          ah[g][j] = radd(ah[g][j], wv[g]);
+          ab[g][j] = wv[g];
+          al[g][j] = rsub(sv[g][j], wv[g]);
         }
       }
     }
@@ -1574,54 +1547,39 @@ __global__ void __launch_bounds__(TB, 1) bwd_inner_r(DP p, St s, Adj a, const fl
 #pragma unroll
       for (int j = 0; j < C; ++j) {
         const int e = t0 + j;
-        zp[j] = zc[j] = zd[j] = zs[j] = 0.f;
-        if (e < T) {   // A' d s, and the outputs' adjoints on the last inner iterate
-          zp[j] = sv.v[SE1][j];
-          zc[j] = rsub(radd(rfma(-k.eta, sv.v[SE2][j], sv.v[SE1][j]), sv.v[SCU][j]), sv.v[SCL][j]);
-          zd[j] = rsub(radd(radd(-sv.v[SE1][j], sv.v[SE2][j]), sv.v[SDU][j]), sv.v[SDL][j]);
-          if (it == N_INNER - 1) {
-            zp[j] = radd(zp[j], LPDT[(size_t)dv.dev * T + e]);
-            zd[j] = radd(zd[j], dcost);
-          }
+        // A' d s (0 beyond the horizon, as its rows are), and the outputs'
+        // adjoints on the last inner iterate
+        zp[j] = sv.v[SE1][j];
+        zc[j] = rsub(radd(rfma(-k.eta, sv.v[SE2][j], sv.v[SE1][j]), sv.v[SCU][j]), sv.v[SCL][j]);
+        zd[j] = rsub(radd(radd(-sv.v[SE1][j], sv.v[SE2][j]), sv.v[SDU][j]), sv.v[SDL][j]);
+        if (it == N_INNER - 1 && e < T) {
+          zp[j] = radd(zp[j], LPDT[(size_t)dv.dev * T + e]);
+          zd[j] = radd(zd[j], dcost);
         }
-        if (e <= T) {
-          float as = rsub(sv.v[SSU][j], sv.v[SSL][j]);
-          if (e >= 1) as = radd(as, (j == 0) ? pE2 : sv.v[SE2][j - 1]);
-          if (e <= T - 1) as = rsub(as, sv.v[SE2][j]);
-          if (e == 0) as = radd(as, sv.E3a);
-          if (e == T) as = radd(as, sv.E3b);
-          zs[j] = as;
-        }
+        float as = rsub(sv.v[SSU][j], sv.v[SSL][j]);
+        if (e >= 1) as = radd(as, (j == 0) ? pE2 : sv.v[SE2][j - 1]);
+        if (e <= T - 1) as = rsub(as, sv.v[SE2][j]);
+        if (e == 0) as = radd(as, sv.E3a);
+        if (e == T) as = radd(as, sv.E3b);
+        zs[j] = as;
       }
       stor_solve_r<C>(k, tf, zp, zc, zd, zs, T, lane);
       const float sn = __shfl_down_sync(FULLM, zs[0], 1);
 #pragma unroll
       for (int j = 0; j < C; ++j) {
         const int e = t0 + j;
-        float wv[SGROUPS];
-#pragma unroll
-        for (int g = 0; g < SGROUPS; ++g) wv[g] = 0.f;
-        if (e < T) {
-          xb[j] = rfma(rho, zp[j], xb[j]);
-          const float snx = (j == C - 1) ? sn : zs[j + 1];
-          wv[0] = rmul(om, rsub(radd(zp[j], zc[j]), zd[j]));
-          wv[1] = rmul(om, radd(rfma(-k.eta, zc[j], rsub(snx, zs[j])), zd[j]));
-          wv[2] = rmul(om, zc[j]);
-          wv[3] = -rmul(om, zc[j]);
-          wv[4] = rmul(om, zd[j]);
-          wv[5] = -rmul(om, zd[j]);
-        }
-        if (e <= T) {
-          wv[6] = rmul(om, zs[j]);
-          wv[7] = -rmul(om, zs[j]);
-        }
+        const bool st = e < T;
+        xb[j] = rfma(rho, zp[j], xb[j]);
+        const float snx = (j == C - 1) ? sn : zs[j + 1];
+        const float wc = rmul(om, zc[j]), wd = rmul(om, zd[j]), ws = rmul(om, zs[j]);
+        const float wv[SGROUPS] = {st ? rmul(om, rsub(radd(zp[j], zc[j]), zd[j])) : 0.f,
+                                   st ? rmul(om, radd(rfma(-k.eta, zc[j], rsub(snx, zs[j])), zd[j])) : 0.f,
+                                   st ? wc : 0.f, st ? -wc : 0.f, st ? wd : 0.f, st ? -wd : 0.f, ws, -ws};
 #pragma unroll
         for (int g = 0; g < SGROUPS; ++g) {
-          if (shas(g, e, T)) {
-            ah.v[g][j] = radd(ah.v[g][j], wv[g]);
-            ab.v[g][j] = wv[g];
-            al.v[g][j] = rsub(sv.v[g][j], wv[g]);
-          }
+          ah.v[g][j] = radd(ah.v[g][j], wv[g]);
+          ab.v[g][j] = wv[g];
+          al.v[g][j] = rsub(sv.v[g][j], wv[g]);
         }
         if (e == 0) {
           const float w3 = rmul(om, zs[j]);
