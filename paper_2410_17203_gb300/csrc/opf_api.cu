@@ -306,11 +306,11 @@ void carve(opf_ctx *c, Arena &a) {
   p.DPD = a.take<float>(ST);
   p.ramp_lam = a.take<float>((size_t)c->n_ramp * opfk::RG_N * T);
   p.ramp_beta = a.take<float>((size_t)c->n_ramp * opfk::RG_N * T);
-  p.ramp_q = a.take<float>((size_t)c->n_ramp * T);
+  p.ramp_q = a.take<float>((size_t)c->n_ramp * 3 * T);
   p.ramp_rho = a.take<float>(c->n_ramp);
   p.stor_lam = a.take<float>((size_t)c->n_stor * opfk::SG_N * Tp);
   p.stor_beta = a.take<float>((size_t)c->n_stor * opfk::SG_N * Tp);
-  p.stor_q = a.take<float>((size_t)c->n_stor * Tp);
+  p.stor_q = a.take<float>((size_t)c->n_stor * 3 * Tp);
   p.stor_rho = a.take<float>(c->n_stor);
   p.stor_delta = a.take<float>((size_t)c->n_stor * T);
   // residual history: part of the mutable state that a batch autotune saves

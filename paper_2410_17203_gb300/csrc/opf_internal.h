@@ -14,8 +14,9 @@
 // (line- and node-major: the K+1 contingency rows of one line or node are
 // one contiguous run, so the node sums gather long runs per terminal)
 //   devices PD, DPD                         [S][T]         float
-//   inner ADMM state of ramp generators     lam, beta [n_ramp][4][T],  q [n_ramp][T]
-//   inner ADMM state of batteries           lam, beta [n_stor][9][T+1], q [n_stor][T+1]
+//   inner ADMM state of ramp generators     lam, beta [n_ramp][4][T],  q [n_ramp][3][T]
+//   inner ADMM state of batteries           lam, beta [n_stor][9][T+1], q [n_stor][3][T+1]
+// (q: pivots; 1 / q and -off / q beside them where the shared-memory path solves)
 // Buffer (it & 1) holds the state after `it` iterations; an iteration reads
 // the old buffers and writes the other ones, because both ends of a line
 // evaluate its prox from the old line and node values.
@@ -233,6 +234,7 @@ struct IterPlan {
   int dev_inner, dev_closed;           // CTAs of the device kernel for inner-ADMM and (fused) closed-form devices
   int xs_grid, dsum_grid;              // not fused: averages with closed-form devices, device sums
   size_t inner_smem;
+  int inner_warps; // warps of a CTA that take inner-ADMM devices
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
 };
 

@@ -76,12 +76,8 @@ constexpr int BATCH_C = 4;         // the same in batches, whose kernels hold ev
 constexpr int BATCH_REG_T = 32 * BATCH_C - 1;
 
 // shared floats per warp of the shared-memory inner ADMM: 3 (T+1) for the
-// work arrays, plus room for one device's (lam, beta) while the horizon is
-// short enough
-__host__ __device__ inline int warp_smem_floats(int T) {
-  const int work = 3 * (T + 1), state = 2 * SG_N * (T + 1);
-  return T <= 128 ? work + state : work;
-}
+// work arrays and, staged, one device's (lam, beta)
+__host__ __device__ inline int warp_smem_floats(int T, bool staged) { return (T + 1) * (staged ? 3 + 2 * SG_N : 3); }
 
 // register chunk of the inner ADMM at horizon T: a battery's T + 1 elements
 // over 32 lanes (1 .. REG_C); 0 beyond longest (the shared-memory path)
@@ -118,22 +114,36 @@ __device__ void tri_factor(float *q, int n, float d_end, float d_mid, float off)
   }
 }
 
-// Solve in place (buf: right-hand side in, solution out; shared memory).
-// Forward  y_i = A_i y_{i-1} + r_i / q_i  and backward  x_i = A_i x_{i+1} + y_i
-// with A_i = -off / q_i are first-order linear recurrences; each lane composes
-// the affine maps of a contiguous chunk, a 5-step shuffle scan composes the
-// chunks across the warp, then each lane applies the prefix to its chunk.
-__device__ void warp_tri_solve(const float *__restrict__ q, float off, float *buf, int n,
-                               int lane) {
+// What the solves read of a factored system, [3][n]: the pivots q, then (by
+// the whole warp) their reciprocals and a_i = -off / q_i.
+__device__ __forceinline__ void tri_tables(float *m, int n, float off, int lane) {
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) {
+    const float q = m[i], rq = __frcp_rn(q);
+    m[n + i] = rq;
+    m[2 * n + i] = qdiv(-off, q, rq);
+  }
+  __syncwarp();
+}
+
+// Solve in place (buf: right-hand side in, solution out; shared memory), with
+// m the tables above.  Forward  y_i = a_i y_{i-1} + r_i / q_i  and backward
+// x_i = a_i x_{i+1} + y_i are first-order linear recurrences; each lane
+// composes the affine maps of a contiguous chunk, a 5-step shuffle scan
+// composes the chunks across the warp, then each lane applies the prefix to
+// its chunk.  The chunks are serial chains (32 elements at T = 1000), so what
+// they read comes from the tables, without a division on the way: 30 buses,
+// T = 1000, 1060 -> 1005 us per iteration.
+__device__ void warp_tri_solve(const float *__restrict__ m, float *buf, int n, int lane) {
+  const float *q = m, *rq = m + n, *a = m + 2 * n;
   const int cs = (n + 31) >> 5;
   const int i0 = min(lane * cs, n), i1 = min(i0 + cs, n);
-  const float noff = -off;
   // forward (r_i = buf_i / q_i is kept in buf for the second pass)
   float Ac = 1.f, Bc = 0.f;
+#pragma unroll 4
   for (int i = i0; i < i1; ++i) {
-    const float rq = __frcp_rn(q[i]);
-    const float ri = qdiv(buf[i], q[i], rq);
-    const float Ai = (i == 0) ? 0.f : qdiv(noff, q[i], rq);
+    const float ri = qdiv(buf[i], q[i], rq[i]);
+    const float Ai = (i == 0) ? 0.f : a[i];
     buf[i] = ri;
     Bc = rfma(Ai, Bc, ri);
     Ac = rmul(Ai, Ac);
@@ -149,17 +159,18 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   }
   float prev = __shfl_up_sync(FULL, Bc, 1);
   if (lane == 0) prev = 0.f;
+#pragma unroll 4
   for (int i = i0; i < i1; ++i) {
-    const float Ai = (i == 0) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
-    prev = rfma(Ai, prev, buf[i]);
+    prev = rfma((i == 0) ? 0.f : a[i], prev, buf[i]);
     buf[i] = prev;
   }
   __syncwarp();
   // backward
   Ac = 1.f;
   Bc = 0.f;
+#pragma unroll 4
   for (int i = i1 - 1; i >= i0; --i) {
-    const float Ci = (i == n - 1) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
+    const float Ci = (i == n - 1) ? 0.f : a[i];
     Bc = rfma(Ci, Bc, buf[i]);
     Ac = rmul(Ci, Ac);
   }
@@ -174,9 +185,9 @@ __device__ void warp_tri_solve(const float *__restrict__ q, float off, float *bu
   }
   float nxt = __shfl_down_sync(FULL, Bc, 1);
   if (lane == 31) nxt = 0.f;
+#pragma unroll 4
   for (int i = i1 - 1; i >= i0; --i) {
-    const float Ci = (i == n - 1) ? 0.f : qdiv(noff, q[i], __frcp_rn(q[i]));
-    nxt = rfma(Ci, nxt, buf[i]);
+    nxt = rfma((i == n - 1) ? 0.f : a[i], nxt, buf[i]);
     buf[i] = nxt;
   }
   __syncwarp();
@@ -393,7 +404,21 @@ __device__ __forceinline__ void lane_avg(const Params &p, const Iter &q, int n, 
 __device__ __forceinline__ void stage_in(float *&lam, float *&bet, float *lam_sh, int n, int lane) {
   if (!lam_sh) return;
   float *bsh = lam_sh + n;
-  for (int i = lane; i < n; i += 32) {
+  int i = lane;
+  for (; i + 7 * 32 < n; i += 8 * 32) {   // 16 values in flight
+    float x[8], y[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      x[q] = lam[i + 32 * q];
+      y[q] = bet[i + 32 * q];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      lam_sh[i + 32 * q] = x[q];
+      bsh[i + 32 * q] = y[q];
+    }
+  }
+  for (; i < n; i += 32) {
     lam_sh[i] = lam[i];
     bsh[i] = bet[i];
   }
@@ -429,7 +454,7 @@ __device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, in
   float *const bet_g = p.ramp_beta + (size_t)r * RG_N * T;
   float *lam = lam_g, *bet = bet_g;
   stage_in(lam, bet, state_sh, RG_N * T, lane);
-  float *mf = p.ramp_q + (size_t)r * T;
+  float *mf = p.ramp_q + (size_t)r * 3 * T;
   const float *lo = p.dev_lo + (size_t)d * T;
   const float *hi = p.dev_hi + (size_t)d * T;
   float *pd = p.PD + (size_t)d * T;
@@ -446,7 +471,7 @@ __device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, in
       tri_factor(mf, T, radd(base, rmul(4.f, om)), radd(base, rmul(6.f, om)), -om2);
       p.ramp_rho[r] = rho;
     }
-    __syncwarp();
+    tri_tables(mf, T, -om2, lane);
   }
   device_x(p, q, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
   for (int itn = 0; itn < p.inner_iters; ++itn) {
@@ -461,7 +486,7 @@ __device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, in
       Z[t] = rfma(om, atr, rfma(rho, X[t], -b));
     }
     __syncwarp();
-    warp_tri_solve(mf, -om2, Z, T, lane);
+    warp_tri_solve(mf, Z, T, lane);
     for (int t = lane; t < T; t += 32) {
       const float pt = Z[t];
       ineq_step(rsub(pt, hi[t]), lam[RG_UP * T + t], bet[RG_UP * T + t]);
@@ -530,7 +555,7 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
   float *const bet_g = p.stor_beta + (size_t)sidx * SG_N * Tp;
   float *lam = lam_g, *bet = bet_g;
   stage_in(lam, bet, state_sh, SG_N * Tp, lane);
-  float *mf = p.stor_q + (size_t)sidx * Tp;
+  float *mf = p.stor_q + (size_t)sidx * 3 * Tp;
   float *pd = p.PD + (size_t)d * T;
   float *dl_out = p.stor_delta + (size_t)sidx * T;
   float *X = sm, *TAU = sm + Tp, *S = sm + 2 * Tp;
@@ -554,7 +579,7 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
       tri_factor(mf, Tp, radd(gam, rmul(3.f, om)), radd(rmul(2.f, gam), om2), -gam);
       p.stor_rho[sidx] = rho;
     }
-    __syncwarp();
+    tri_tables(mf, Tp, -gam, lane);
   }
   device_x(p, it, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
 #define LAM(g, t) lam[(g) * Tp + (t)]
@@ -580,7 +605,7 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
       S[j] = rhs;
     }
     __syncwarp();
-    warp_tri_solve(mf, -gam, S, Tp, lane);
+    warp_tri_solve(mf, S, Tp, lane);
     for (int t = lane; t < T; t += 32) {
       const float r1 = -LAM(SG_E1, t), r2 = -LAM(SG_E2, t);
       const float mc = rmul(0.5f, rsub(rsub(radd(Pm, BET(SG_CU, t)), LAM(SG_CU, t)), rsub(BET(SG_CL, t), LAM(SG_CL, t))));
@@ -649,7 +674,7 @@ __device__ void ramp_prox_r(const Params &p, int r, int lane, bool avg) {
   const float4 par = p.ipar[p.n_stor + r];         // a, b, ramp limit
   float *const lam_g = p.ramp_lam + (size_t)r * RG_N * T;
   float *const bet_g = p.ramp_beta + (size_t)r * RG_N * T;
-  float *mf = p.ramp_q + (size_t)r * T;
+  float *mf = p.ramp_q + (size_t)r * 3 * T;
   const float rho_old = p.ramp_rho[r];
   float lam[RG_N][C], bet[RG_N][C], hi[C], lo[C], X[C], pd[C], Z[C];
   TriFac<C> tf;
@@ -751,7 +776,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, int lane, bool avg) {
   const float4 par = p.ipar[sidx];                 // efficiency, power, duration, cost
   float *const lam_g = p.stor_lam + (size_t)sidx * SG_N * Tp;
   float *const bet_g = p.stor_beta + (size_t)sidx * SG_N * Tp;
-  float *mf = p.stor_q + (size_t)sidx * Tp;
+  float *mf = p.stor_q + (size_t)sidx * 3 * Tp;
   const float rho_old = p.stor_rho[sidx];
   // element e = t0 + j: step t = e of (p, c, delta) while e < T, state of
   // charge s_e while e < T + 1
@@ -1395,20 +1420,25 @@ __device__ __forceinline__ void ramp_r(const Params &p, int r, int lane, int cr,
 // REG_T steps (chunks of at most C); C = 0: the shared-memory path.  MIXED
 // (batches): the instance's horizon chooses, beyond BATCH_REG_T the
 // shared-memory path.  avg: each warp forms its node's average over
-// contingencies (else it is in XS).
+// contingencies (else it is in XS).  nw: the CTA's warps that take devices.  staged: the
+// shared-memory path holds the device's state there through the ten inner
+// iterations; in global memory each row's read, step and write is a round trip
+// to L2 (30 buses, T = 1000: 1005 -> 352 us per iteration; 40 buses, T = 300,
+// where L1 holds it: 103 -> 108).  Batches, whose instances share one launch's shared memory, do not stage.
 // ---------------------------------------------------------------------------
 template <int C, bool MIXED>
-__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem, bool avg) {
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem, bool avg, int nw,
+                                           bool staged) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  if (wib >= nw) return;
   const int T = p.T;
   const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
   constexpr bool HAS_SMEM = C == 0 || MIXED, HAS_REG = C > 0;
   const bool reg = HAS_REG && (!HAS_SMEM || T <= BATCH_REG_T);
   float *wsm = nullptr, *state_sh = nullptr;
   if (HAS_SMEM && !reg) {
-    const int wfl = warp_smem_floats(T);
-    wsm = smem + (size_t)wib * wfl;
-    state_sh = (wfl > 3 * (T + 1)) ? wsm + 3 * (T + 1) : nullptr;
+    wsm = smem + (size_t)wib * warp_smem_floats(T, staged);
+    state_sh = staged ? wsm + 3 * (T + 1) : nullptr;
   }
   const int cs = (T + 32) >> 5, cr = (T + 31) >> 5;   // chunks of T + 1 and T elements
   for (int w = bid * nw + wib; w < n_inner; w += nblk * nw) {
@@ -1742,9 +1772,9 @@ __global__ void __launch_bounds__(BLOCK) xs_kernel(Params p) { xs_body<VW>(p, bl
 // closed-form devices are a kernel of their own (avg false), only the first
 // part is launched.
 template <int C>
-__global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks, bool avg) {
+__global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks, bool avg, int nw) {
   extern __shared__ float smem[];
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, blockIdx.x, inner_blocks, smem, avg);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, blockIdx.x, inner_blocks, smem, avg, nw, true);
   else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
   else closed_body<1>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
 }
@@ -1916,7 +1946,7 @@ __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int
   __shared__ Params sp;
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true, DEV_WARPS, false);
   else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), bid, nblk);
   else closed_body<1>(p, load_iter(p), bid, nblk);
 }
@@ -2239,7 +2269,9 @@ __global__ void set_rho_kernel(Params p, double rho) {
   *p.sc = s;
 }
 
-static size_t inner_smem(int T, int warps) { return (size_t)warps * warp_smem_floats(T) * sizeof(float); }
+static size_t inner_smem(int T, int warps, bool staged) {
+  return (size_t)warps * warp_smem_floats(T, staged) * sizeof(float);
+}
 
 }  // namespace opfk
 
@@ -2255,11 +2287,25 @@ static int resident_grid(F fn, size_t smem) {
   return nb * sms;
 }
 
-// dynamic shared memory of the device kernels, set on each of them
+// shared memory a CTA may take on this device
+static size_t max_smem() {
+  int dev = 0, m = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return 0;
+  return (size_t)m;
+}
+
+// let a device kernel take it (the limit is the function's, not a context's:
+// always the same value, so that no context lowers another's)
 template <class F>
 static bool allow_smem(F fn, size_t smem) {
-  return smem <= 48 * 1024 ||
-         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+  if (smem <= 48 * 1024) return true;
+  cudaFuncAttributes a;
+  const size_t m = max_smem();
+  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess || a.sharedSizeBytes + smem > m) return false;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(m - a.sharedSizeBytes)) ==
+         cudaSuccess;
 }
 
 int opfk_plan(const Params &p, IterPlan *plan) {
@@ -2294,10 +2340,15 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // line pass; device sums in the node pass 0.701 against 0.697.  At 2k buses,
   // T = 24, K = 20: three device kernels 31.7 us per iteration, one 25.2.
   const double line_us = (double)p.Kp * p.L * p.T * 32.0 / 6.5e6;
-  const int one_round = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
+  // warps per CTA: the shared-memory path as many as its staged states leave room for
+  int nw = DEV_WARPS;
+  if (!ic)
+    for (const size_t m = max_smem(); nw > 1 && inner_smem(p.T, nw, true) > m;) nw /= 2;
+  plan->inner_warps = nw;
+  const int one_round = (n_inner + nw - 1) / nw;
   const double round_us = ic ? 5.0 + 0.08 * p.T : 0.45 * p.T;
   const int max_rounds = (int)std::floor((ic ? 0.5 : 0.7) * line_us / round_us);
-  const size_t ism = ic ? 0 : inner_smem(p.T, DEV_WARPS);
+  const size_t ism = ic ? 0 : inner_smem(p.T, nw, true);
   if (!allow_smem(dev_kernel<0>, ism)) return -1;
   plan->inner_smem = ism;
   plan->fused = !p.slice && max_rounds < 2;
@@ -2342,7 +2393,7 @@ static int iteration_enqueue(const Params &p, const IterPlan &plan, void *main_s
   const int ni = plan.dev_inner, nd = ni + plan.dev_closed;
   const bool avg = plan.fused;
   if (nd > 0) {
-#define DEV_LAUNCH(C) case C: dev_kernel<C><<<nd, DEVB, plan.inner_smem, sm>>>(p, ni, avg); break
+#define DEV_LAUNCH(C) case C: dev_kernel<C><<<nd, DEVB, plan.inner_smem, sm>>>(p, ni, avg, plan.inner_warps); break
     static_assert(REG_C == 8, "the chunks launched below");
     switch (plan.inner_c) {
       DEV_LAUNCH(0); DEV_LAUNCH(1); DEV_LAUNCH(2); DEV_LAUNCH(3); DEV_LAUNCH(4);
@@ -2451,7 +2502,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           if (blocks) {
             const int ic = inner_chunk(p.T, BATCH_REG_T);
             if (ic) ic_max = std::max(ic_max, ic);
-            else ism = std::max(ism, inner_smem(p.T, DEV_WARPS));   // the shared-memory path
+            else ism = std::max(ism, inner_smem(p.T, DEV_WARPS, false));   // the shared-memory path
           }
           break;
         case BK_CLOSED:
