@@ -204,12 +204,13 @@ opf_status opf_create(const opf_network *net, int32_t horizon_T,
                       opf_ctx **out);
 
 /* Enqueue n_iters message-passing iterations (Section 3.2).  Each iteration
- * is seven kernels (device averages and closed-form devices, inner-ADMM
- * devices, device sums, line proxes on a second stream, the node sums -- a
- * general pass on iterations that form residuals and a lean pass on the
- * others, each returning at once on the other's iterations -- and the
- * decisions), replayed from CUDA graphs of 1 and 16 iterations after a
- * one-thread kernel that records the call's last iteration.  Residuals
+ * is three phases: the devices (one kernel, or, where the line pass hides
+ * them, three: device averages and closed forms, inner-ADMM devices, device
+ * sums), the line proxes on a second stream beside them, and the node sums,
+ * whose last CTA takes the decisions; they are replayed from CUDA graphs of 1
+ * and 16 iterations.  Small instances without inner-ADMM devices run many
+ * iterations per launch on one CTA instead (the same results).  A one-thread
+ * kernel first records the call's last iteration.  Residuals
  * (Section 3.3) are formed on stopping-test iterations (every check_every),
  * adaptation iterations (every adapt_every) and the call's last iteration;
  * a non-finite value is reported (OPF_ENONFINITE) at the first of these
@@ -352,16 +353,17 @@ void opf_batch_destroy(opf_batch *batch);
  *   2 longest first, round-robin, 1x   3 as given, contiguous, 1/4
  *   4 longest first, contiguous, 1/4   5 longest first, round-robin, 1/4
  * ("longest first" orders instances by (K+1) T (L + N); "round-robin" deals
- * one CTA per instance in turn; "1/4" gives the device-sum, inner-ADMM,
- * device-average and node-sum phases a quarter of the CTAs, each doing four
- * times the work; deeper divisors tuned on the first iterations lose on the
+ * one CTA per instance in turn; "1/4" gives the inner-ADMM, closed-form device
+ * and node-sum work a quarter of the CTAs, each doing four times the work;
+ * the node CTAs of 1x are shared out in proportion to the instances' items; deeper divisors tuned on the first iterations lose on the
  * tail, when the largest instances run alone).  Every candidate runs
  * `steps` >= 1 batch iterations (after one warm-up) from the instances'
  * current state, which is saved before and restored after, so the call
  * leaves every iterate unchanged; the fastest layout is kept for later
  * opf_batch_iterate calls.  The layout changes which CTA computes what, not
  * the arithmetic of an iterate; only the split of the residual norms'
- * partial sums over CTAs moves (their last bits).  choice and
+ * partial sums over CTAs moves (their last bits, which also may differ from
+ * those of the instance iterated alone).  choice and
  * ms_each [OPF_BATCH_LAYOUTS] (each may be NULL) receive the chosen index
  * and every layout's milliseconds per batch iteration.  Synchronizes;
  * allocates a temporary copy of the instances' states. */

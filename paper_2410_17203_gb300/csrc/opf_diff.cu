@@ -6,7 +6,8 @@
 // duals beta, lambda of ramp-limited generators and batteries) is kept in
 // plain arrays, and every step of the iteration has a forward kernel and an
 // adjoint kernel.  Forward states are stored every `checkpoint_every`
-// iterations and recomputed segment by segment during the reverse pass.
+// iterations and recomputed segment by segment during the reverse pass where
+// the forward pass kept no record of its clipping decisions.
 // Every adjoint item writes only its own entries (sums over a node's
 // terminals are CSR gathers, an inner device is one CTA), so the gradients
 // are deterministic.

@@ -1,26 +1,30 @@
 // Proximal message passing for contingency-constrained DC OPF -- sm_103a kernels.
 //
-// One iteration of the message-passing form of ADMM (Section 3.2) is seven
-// kernels replayed from CUDA graphs; each reads the iteration's scalars
-// (penalties, pending rescales, buffer parity, whether residuals are read)
-// from the device, so the same graph serves every iteration:
-//   xs     step 2 input: avg_k(pbar + u) from the stored pbar + u at every
-//          node with devices (a node's K+1 rows are one run), and the
-//          closed-form prox with weight (K+1) rho_p of its generators/loads;
-//   inner  step 2, one warp per ramp-limited generator, battery or HVDC link:
-//          the inner ADMM of Appendix D (lanes over time steps, tridiagonal
-//          x-updates by warp-wide scans) or the link's closed form;
-//   dsum   the node sums of device powers and their Welford change state;
+// One iteration of the message-passing form of ADMM (Section 3.2) is three
+// phases replayed from CUDA graphs; each kernel reads the iteration's scalars
+// (penalty factors, buffer parity, whether residuals are read) from the
+// device, so the same graph serves every iteration:
+//   dev    step 2: avg_k(pbar + u) from the stored pbar + u at every node with
+//          devices (a node's K+1 rows are one run), the closed-form prox with
+//          weight (K+1) rho_p of its generators/loads, and one warp per
+//          ramp-limited generator, battery or HVDC link: the inner ADMM of
+//          Appendix D (lanes over time steps, tridiagonal x-updates by
+//          warp-wide scans) or the link's closed form.  Where the line pass is
+//          long enough to hide the devices this is three kernels: xs (averages
+//          and closed forms), dev (the inner ADMM alone), dsum (the node sums
+//          of device powers and their Welford change state);
 //   line   step 1, one thread per (line, contingency, 4 time steps): the line
 //          prox from the previous iterate at both ends (second stream, beside
-//          xs, inner and dsum), the deferred v update, over-relaxed blends;
-//   node   step 3 where the residuals are read (stopping test, adaptation,
-//          end of a call): pbar, theta_bar, u += pbar as register sums over
-//          the node's terminals in CSR order (no atomics), the residual
-//          partial sums (one-pass Welford sums); node_lean does step 3 alone
-//          on the other iterations (each returns at once on the other's);
-//   decide FP64 reduction of the partial sums in a fixed order, stopping
-//          test and adaptive penalty (Section 3.5); advances the counter.
+//          the devices), the deferred v update, over-relaxed blends;
+//   node   step 3: pbar, theta_bar, u += pbar as register sums over the node's
+//          terminals in CSR order (no atomics).  One kernel holds two passes:
+//          the one without residuals, and, where they are read (stopping test,
+//          adaptation, end of a call), one that also forms their partial sums
+//          (one-pass Welford sums).  The CTA that ends last reduces them in
+//          FP64 in a fixed order, decides the stopping test and the adaptive
+//          penalty (Section 3.5) and advances the counter.
+// Small instances without inner-ADMM devices run the three phases on one CTA,
+// many iterations per launch (small_kernel).
 //
 // Splitting the phases lets each kernel run at its own register budget.
 // There is no spin-wait on the device: ordering comes from kernel boundaries
