@@ -5,7 +5,7 @@
 //
 // Layout: activations are row-major [R][64] with rows r = t * N + n.  A layer
 // is one kernel: persistent CTAs hold the layer's bfloat16 weights in shared
-// memory as FP32 and walk tiles of 32 rows; the neighbour average (a CSR
+// memory and walk tiles of 64 rows; the neighbour average (a CSR
 // gather) is formed tile by tile where it is used, in the forward pass from
 // the layer's input, in the backward pass, transposed, from the previous
 // layer's product.  Every output is summed over k in order in FP32.  Weight
