@@ -50,7 +50,7 @@ def workload_name(config, d):
     """Name of the timed workload: the network size, horizon and contingencies."""
     return f"dcopf-{config}-bus-T{d['T']}-K{d['K']}"
 KERNEL_SRC = [os.path.join(ROOT, "paper_2410_17203_gb300", "csrc", f)
-              for f in ("opf_kernels.cu", "opf_internal.h")]
+              for f in ("opf_kernels.cu", "opf_internal.h", "opf_tri.h")]
 PROFILE = os.path.join(ROOT, "profiles", "iteration_10k.txt")
 FALLBACK_HBM_GBS = 6800.0
 
@@ -855,7 +855,7 @@ def ours_arm(args):
                          "frac": achieved / peak, "peak_source": src,
                          "traffic": traffic,
                          "algorithmic_bytes_per_iteration": B,
-                         "kernel": "one iteration: xs, inner, dsum, line, node and decide kernels "
+                         "kernel": "one iteration: xs, dev, dsum, line and node kernels "
                                    "replayed from CUDA graphs (unit = iteration; per-kernel shares in "
                                    "profiles/iteration_10k.txt)"},
             "variable_updates_per_s": value * variables_per_iter(d),
