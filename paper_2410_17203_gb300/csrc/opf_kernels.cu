@@ -664,6 +664,15 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
 // instance, a batch) computes the same bits.
 // ---------------------------------------------------------------------------
 
+// Whether a batch solves a device of this horizon from shared memory: it then
+// reads the tables of tri_tables, which are written with the pivots, under the
+// same record of the penalty they belong to (ramp_rho, stor_rho), whichever
+// form factors.
+template <int C>
+__device__ __forceinline__ bool tables_too(int T) {
+  return 32 * C > BATCH_REG_T && T > BATCH_REG_T;   // a chunk of C holds up to 32 C elements
+}
+
 // Lanes beyond the horizon run along (right-hand side 0, nothing of theirs is
 // stored or read by others), which spares the inner iterations a branch per
 // element.
@@ -718,6 +727,7 @@ __device__ void ramp_prox_r(const Params &p, int r, int lane, bool avg) {
       p.ramp_rho[r] = rho;
     }
     __syncwarp();
+    if (tables_too<C>(T)) tri_tables(mf, T, -om2, lane);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
 #pragma unroll
@@ -833,6 +843,7 @@ __device__ void stor_prox_r(const Params &p, int sidx, int lane, bool avg) {
       p.stor_rho[sidx] = rho;
     }
     __syncwarp();
+    if (tables_too<C>(T)) tri_tables(mf, Tp, -gam, lane);
     e3a = rmul(e3a, ls);
     e3b = rmul(e3b, ls);
 #pragma unroll
