@@ -74,6 +74,10 @@ constexpr int CLOSED_LANES4 = 2, CLOSED_LANES1 = 8;   // lanes per closed-form i
 // microseconds of a small instance's iteration on one CTA: base, per round of
 // items, and the limit (opfk_plan)
 constexpr double SMALL_BASE = 2.7, SMALL_LINE = 0.8, SMALL_CLOSED = 0.45, SMALL_NODE = 1.2, SMALL_LIMIT = 8.0;
+// Without inner-ADMM devices: the line pass (microseconds, estimated) from
+// which averages and device sums as kernels of their own are hidden beside it
+// (opfk_plan).
+constexpr double HIDE_US = 16.0;
 constexpr int REG_C = 8;           // largest chunk of the register-resident inner ADMM ...
 constexpr int REG_T = 32 * REG_C - 1;   // ... its longest horizon (T + 1 <= 32 C)
 constexpr int BATCH_C = 4;         // the same in batches, whose kernels hold every chunk up to theirs
@@ -2355,18 +2359,29 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // line pass; device sums in the node pass 0.701 against 0.697.  At 2k buses,
   // T = 24, K = 20: three device kernels 31.7 us per iteration, one 25.2.
   const double line_us = (double)p.Kp * p.L * p.T * 32.0 / 6.5e6;
-  // warps per CTA: the shared-memory path as many as its staged states leave room for
+  // warps per CTA: the shared-memory path as many as its staged states leave
+  // room for (no shared memory where no device needs it: every CTA of the
+  // device kernel would take it, the closed-form ones too, and run one or two
+  // to an SM)
+  const bool admm = p.n_stor + p.n_ramp > 0;
   int nw = DEV_WARPS;
-  if (!ic)
+  if (!ic && admm)
     for (const size_t m = max_smem(); nw > 1 && inner_smem(p.T, nw, true) > m;) nw /= 2;
   plan->inner_warps = nw;
   const int one_round = (n_inner + nw - 1) / nw;
   const double round_us = ic ? 5.0 + 0.08 * p.T : 0.45 * p.T;
   const int max_rounds = (int)std::floor((ic ? 0.5 : 0.7) * line_us / round_us);
-  const size_t ism = ic ? 0 : inner_smem(p.T, nw, true);
+  const size_t ism = ic || !admm ? 0 : inner_smem(p.T, nw, true);
   if (!allow_smem(dev_kernel<0>, ism)) return -1;
   plan->inner_smem = ism;
-  plan->fused = !p.slice && max_rounds < 2;
+  // Without inner-ADMM devices the chain is averages and closed forms alone,
+  // which a line pass of HIDE_US hides (us per iteration with one device
+  // kernel / with averages and sums apart, by the line pass's estimate: 2k
+  // buses T = 24 K = 20 7.9 us 21.1 / 24.5, 5k T = 24 K = 10 10.4 us 27.7 /
+  // 27.7, 3k T = 25 K = 20 12.4 us 64.3 / 56.8, 1k T = 96 K = 20 with three
+  // links 15.9 us 39.3 / 42.0, 2k T = 96 K = 10 16.6 us 43.1 / 39.3, 2k T = 252
+  // K = 4 19.8 us 59.1 / 49.5).
+  plan->fused = !p.slice && (admm ? max_rounds < 2 : line_us < HIDE_US);
   plan->node_lat = plan->fused && nn <= (vn ? NODE_LAT_ITEMS4 : NODE_LAT_ITEMS1);
   // A small instance without inner-ADMM devices runs on one CTA (small_kernel)
   // where its rounds of 256 line, closed-form and node items are estimated to

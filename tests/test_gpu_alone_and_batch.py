@@ -46,3 +46,31 @@ def test_alone_then_batch_by_turns(T, adapt_every):
         opf_batch_destroy(b)
         ref.close()
         ctx.close()
+
+
+@pytest.mark.parametrize("n, T, K, n_hvdc", [
+    (40, 300, 4, 0), (40, 300, 4, 2), (30, 2048, 1, 1),   # one device kernel, no shared memory
+    (2000, 100, 12, 2), (3000, 33, 22, 0),                # averages and device sums apart, beside the line pass
+])
+def test_instances_without_inner_admm_devices(n, T, K, n_hvdc):
+    """Closed-form devices and links alone: every plan gives the batch's bits
+    (one device kernel whatever the size), short ones also the oracle's."""
+    from helpers import compare_states
+    from oracle import Oracle, OracleOptions
+    from paper_2410_17203_gb300 import Solver, opf_batch_create, opf_batch_destroy, opf_batch_iterate
+    case = make_case(scale_case(n, T, K, seed=31 + T, stor_per_node=0.0, ramp=False, n_hvdc=n_hvdc))
+    opts = dict(adapt_every=5, eps=0.0)
+    single, member = Solver(case, opts), Solver(case, opts)
+    single.iterate(12)
+    b = opf_batch_create([member.h])
+    try:
+        opf_batch_iterate(b, 12)
+        _assert_same_state(member, single)
+        if n <= 40:
+            o = Oracle(case, OracleOptions(**opts))
+            o.iterate(12, stop=False)
+            compare_states(single.state(), o)
+    finally:
+        opf_batch_destroy(b)
+        single.close()
+        member.close()
