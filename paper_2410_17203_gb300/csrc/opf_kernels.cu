@@ -87,6 +87,9 @@ constexpr int BATCH_REG_T = 32 * BATCH_C - 1;
 // work arrays and, staged, one device's (lam, beta)
 __host__ __device__ inline int warp_smem_floats(int T, bool staged) { return (T + 1) * (staged ? 3 + 2 * SG_N : 3); }
 
+// warps' worth of work of the inner kernels: a device each, a link one per 32 steps
+__host__ __device__ inline int inner_units(const Params &p) { return p.n_stor + p.n_ramp + p.n_hvdc * ((p.T + 31) >> 5); }
+
 // register chunk of the inner ADMM at horizon T: a battery's T + 1 elements
 // over 32 lanes (1 .. REG_C); 0 beyond longest (the shared-memory path)
 __host__ __device__ inline int inner_chunk(int T, int longest = REG_T) { return T <= longest ? (T + 32) >> 5 : 0; }
@@ -517,20 +520,23 @@ __device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, in
 }
 
 // ---------------------------------------------------------------------------
-// HVDC link (one warp, lanes over t): with x_i = p_i - avg_k(pbar + u) at
+// HVDC link (a warp per link and 32 time steps, lanes over t: each step's
+// averages are a chain of loads, and one warp walking a long horizon was the
+// whole phase: 100 buses, K = 4, us per iteration, T = 1000 51.7 -> 15.7,
+// T = 2048 118 -> 24.7, T = 300 28.3 -> 14.5, T = 168 18.5 -> 12.6): with x_i = p_i - avg_k(pbar + u) at
 // terminal i, p2 = clip((x2 - x1) / 2, -u, u) and p1 = -p2 (the minimiser
 // of the two squared distances over p1 + p2 = 0, clipped to the limit)
 // ---------------------------------------------------------------------------
-__device__ void hvdc_prox(const Params &p, int h, int lane, bool avg) {
+__device__ void hvdc_prox(const Params &p, int unit, int lane, bool avg) {
   const Iter q = load_iter(p);
   if (q.flags & ITF_SKIP) return;
-  const int T = p.T;
+  const int T = p.T, nt = (T + 31) >> 5, h = unit / nt, t = (unit - h * nt) * 32 + lane;
   const int d1 = p.hvdc0 + 2 * h, d2 = d1 + 1;
   const float u = p.hvdc_u[h];
   const int m1 = p.dev_node[d1], m2 = p.dev_node[d2];
   const float *xs1 = p.XS + (size_t)m1 * T, *xs2 = p.XS + (size_t)m2 * T;
   float *pd1 = p.PD + (size_t)d1 * T, *pd2 = p.PD + (size_t)d2 * T;
-  for (int t = lane; t < T; t += 32) {
+  if (t < T) {
     const float q1 = pd1[t], q2 = pd2[t];
     const float x1 = q1 - (avg ? node_avg<1>(p, q, m1, t).v[0] : __ldcg(xs1 + t));
     const float x2 = q2 - (avg ? node_avg<1>(p, q, m2, t).v[0] : __ldcg(xs2 + t));
@@ -1435,7 +1441,7 @@ __device__ __forceinline__ void ramp_r(const Params &p, int r, int lane, int cr,
 
 // ---------------------------------------------------------------------------
 // inner: one warp per battery, then per ramp-limited generator (Appendix D),
-// then per HVDC link.  C > 0: the register path, for horizons of at most
+// then per HVDC link and 32 steps.  C > 0: the register path, for horizons of at most
 // REG_T steps (chunks of at most C); C = 0: the shared-memory path.  MIXED
 // (batches): the instance's horizon chooses, beyond BATCH_REG_T the
 // shared-memory path.  avg: each warp forms its node's average over
@@ -1451,7 +1457,7 @@ __device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsign
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (wib >= nw) return;
   const int T = p.T;
-  const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
+  const int n_inner = inner_units(p);
   constexpr bool HAS_SMEM = C == 0 || MIXED, HAS_REG = C > 0;
   const bool reg = HAS_REG && (!HAS_SMEM || T <= BATCH_REG_T);
   float *wsm = nullptr, *state_sh = nullptr;
@@ -2339,7 +2345,7 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   const long long tvl = p.T / (v4 ? 4 : 1), tvn = p.T / (vn ? NODE_VW : 1);
   const long long nl = (long long)p.Kp * p.L * tvl, nn = (long long)p.Kp * p.N * tvn;
   const long long nx = (long long)p.n_dnode * tvl;
-  const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
+  const int n_inner = inner_units(p);
   plan->line_ipt = nl <= LINE_SHORT ? 1 : LINE_IPT;
   plan->line_grid = (int)((nl + (long long)BLOCK * plan->line_ipt - 1) / ((long long)BLOCK * plan->line_ipt));
   plan->node_grid = (int)std::min<long long>(gn, (nn + BLOCK - 1) / BLOCK);
@@ -2524,7 +2530,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
       const Params &p = hp[i];
       const bool v4 = (p.T % 4 == 0), vn = (p.T % NODE_VW == 0);
       const long long tv4 = p.T / (v4 ? 4 : 1);
-      const int n_inner = p.n_stor + p.n_ramp + p.n_hvdc;
+      const int n_inner = inner_units(p);
       long long blocks = 0;
       switch (kind) {
         case BK_INNER:
