@@ -2325,10 +2325,11 @@ static size_t max_smem() {
 // always the same value, so that no context lowers another's)
 template <class F>
 static bool allow_smem(F fn, size_t smem) {
-  if (smem <= 48 * 1024) return true;
   cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess) return false;
+  if (a.sharedSizeBytes + smem <= 48 * 1024) return true;   // static and dynamic together
   const size_t m = max_smem();
-  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess || a.sharedSizeBytes + smem > m) return false;
+  if (a.sharedSizeBytes + smem > m) return false;
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(m - a.sharedSizeBytes)) ==
          cudaSuccess;
 }

@@ -74,3 +74,23 @@ def test_instances_without_inner_admm_devices(n, T, K, n_hvdc):
         opf_batch_destroy(b)
         single.close()
         member.close()
+
+
+@pytest.mark.parametrize("T", [1000, 1015, 1023, 1024])
+def test_batch_at_the_edge_of_48_kb(T):
+    """A batch's device kernel takes 48 (T + 1) bytes of shared memory beside
+    its own: the sum, not the former alone, decides whether it must ask for
+    more than the default 48 KB.  The bits are those of the context alone."""
+    from paper_2410_17203_gb300 import Solver, opf_batch_create, opf_batch_destroy, opf_batch_iterate
+    case = make_case(scale_case(5, T, 0, seed=T, stor_per_node=0.2))
+    opts = dict(adapt_every=0, eps=0.0)
+    single, member = Solver(case, opts), Solver(case, opts)
+    single.iterate(2)
+    b = opf_batch_create([member.h])
+    try:
+        opf_batch_iterate(b, 2)
+        _assert_same_state(member, single)
+    finally:
+        opf_batch_destroy(b)
+        single.close()
+        member.close()
