@@ -348,22 +348,21 @@ opf_status opf_batch_stopped(opf_batch *batch, int32_t *n_converged, int32_t *n_
 void opf_batch_destroy(opf_batch *batch);
 
 /* Pick the batch's CTA-to-instance schedule by timing.  Candidate layouts
- * (index: instance order, CTAs per phase, CTAs of the grid-stride phases):
+ * (index: instance order, CTAs per phase, CTAs of the device phase):
  *   0 as given, contiguous, 1x   1 longest first, contiguous, 1x
  *   2 longest first, round-robin, 1x   3 as given, contiguous, 1/4
  *   4 longest first, contiguous, 1/4   5 longest first, round-robin, 1/4
  * ("longest first" orders instances by (K+1) T (L + N); "round-robin" deals
- * one CTA per instance in turn; "1/4" gives the inner-ADMM, closed-form device
- * and node-sum work a quarter of the CTAs, each doing four times the work;
- * the node CTAs of 1x are shared out in proportion to the instances' items; deeper divisors tuned on the first iterations lose on the
- * tail, when the largest instances run alone).  Every candidate runs
+ * one CTA per instance in turn; "1/4" gives the inner-ADMM and closed-form
+ * device work a quarter of the CTAs, each doing four times the work; the node
+ * sums' CTAs are dealt out on the device, over the instances that run, in every
+ * layout).  Every candidate runs
  * `steps` >= 1 batch iterations (after one warm-up) from the instances'
  * current state, which is saved before and restored after, so the call
  * leaves every iterate unchanged; the fastest layout is kept for later
  * opf_batch_iterate calls.  The layout changes which CTA computes what, not
- * the arithmetic of an iterate; only the split of the residual norms'
- * partial sums over CTAs moves (their last bits, which also may differ from
- * those of the instance iterated alone).  choice and
+ * the arithmetic: iterates and residuals are those of each instance iterated
+ * alone, bit for bit.  choice and
  * ms_each [OPF_BATCH_LAYOUTS] (each may be NULL) receive the chosen index
  * and every layout's milliseconds per batch iteration.  Synchronizes;
  * allocates a temporary copy of the instances' states. */
@@ -373,9 +372,9 @@ opf_status opf_batch_autotune(opf_batch *batch, int32_t steps, int32_t *choice, 
 /* Drop the batch's stopped instances (converged, stalled, error) from its
  * schedule, so that later steps launch CTAs for the running ones only (a
  * batch's last steps often run one or two instances while the stopped ones'
- * CTAs would still be scheduled).  The layout in force keeps its order and
- * CTA split, restricted to the running instances, so iterates do not change,
- * not even the residuals' last bits; counts and queries still cover every
+ * CTAs would still be scheduled).  The layout in force keeps its order,
+ * restricted to the running instances; iterates and residuals do not change,
+ * bit for bit; counts and queries still cover every
  * instance, and an instance once dropped is not iterated again by this batch.
  * n_scheduled (may be NULL) receives the number of instances still
  * scheduled; with none, opf_batch_iterate does nothing.  Synchronizes; a

@@ -1158,8 +1158,13 @@ struct opf_batch {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_done = nullptr;
   opfk::Params *d_params = nullptr;
   int *d_sched = nullptr;
+  // the deal of the node kernel's CTAs (opfk::NodeDeal)
+  opfk::NodeShare *d_share = nullptr;
+  int4 *d_slot = nullptr;
+  int *d_dirty = nullptr;
   opfk::BatchPlan plan{};
   long long sched_cap = 0;    // schedule entries d_sched holds (the longest layout)
+  int slot_cap = 0;           // entries d_slot holds (every instance scheduled)
   cudaGraphExec_t g_one = nullptr, g_many = nullptr;
   // the layout in force (opf_batch_autotune) and how many instances it
   // schedules (all, or those still running after opf_batch_compact)
@@ -1179,6 +1184,9 @@ void release_batch(opf_batch *b) {
   if (b->s_aux) cudaStreamDestroy(b->s_aux);
   if (b->d_params) cudaFree(b->d_params);
   if (b->d_sched) cudaFree(b->d_sched);
+  if (b->d_share) cudaFree(b->d_share);
+  if (b->d_slot) cudaFree(b->d_slot);
+  if (b->d_dirty) cudaFree(b->d_dirty);
 }
 
 // `iters` iterations of every instance as one graph: per iteration one
@@ -1200,10 +1208,16 @@ opf_status build_batch_graph(opf_batch *b, int iters, cudaGraphExec_t *out) {
   return OPF_OK;
 }
 
+void set_deal(const opf_batch *b, opfk::BatchPlan &bp) {
+  bp.deal.share = b->d_share;
+  bp.deal.slot = b->d_slot;
+  bp.deal.dirty = b->d_dirty;
+}
+
 // Build the schedule of the n_sched instances that `lay` lists (lay.order;
 // NULL: every instance as given) into d_sched and drop the graphs of the
 // previous one (rebuilt on the next iteration).  Waits for the batch stream.
-opf_status schedule_batch(opf_batch *b, int n_sched, opfk::BatchLayout lay) {
+opf_status schedule_batch(opf_batch *b, int n_sched, const opfk::BatchLayout &lay) {
   const int n = (int)b->ctx.size();
   std::vector<Params> hp(n);
   std::vector<opfk::IterPlan> plans(n);
@@ -1213,18 +1227,23 @@ opf_status schedule_batch(opf_batch *b, int n_sched, opfk::BatchLayout lay) {
   }
   long long len = 0;
   opfk::BatchPlan bp{};
-  lay.node_items = opfk_batch_node_items(hp.data(), n);
-  if (opfk_batch_plan(hp.data(), plans.data(), n_sched, lay, nullptr, 0, &len, &bp) != 0 || len > b->sched_cap)
+  std::vector<opfk::NodeShare> share(std::max(n_sched, 1));
+  if (opfk_batch_plan(hp.data(), plans.data(), n_sched, lay, nullptr, 0, &len, nullptr, &bp) != 0 ||
+      len > b->sched_cap || bp.deal.cap > b->slot_cap)
     return fail(OPF_ECUDA, "batch schedule");
   std::vector<int> sched(4 * (size_t)std::max(len, 1LL));
-  if (opfk_batch_plan(hp.data(), plans.data(), n_sched, lay, sched.data(), len, &len, &bp) != 0)
+  if (opfk_batch_plan(hp.data(), plans.data(), n_sched, lay, sched.data(), len, &len, share.data(), &bp) != 0)
     return fail(OPF_ECUDA, "batch schedule");
   CK(cudaStreamSynchronize(b->stream));
   if (b->g_one) cudaGraphExecDestroy(b->g_one);
   if (b->g_many) cudaGraphExecDestroy(b->g_many);
   b->g_one = b->g_many = nullptr;
-  CK(cudaMemcpy(b->d_sched, sched.data(), sched.size() * sizeof(int), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(b->d_params, hp.data(), n * sizeof(Params), cudaMemcpyHostToDevice));
+  // in the order of the batch's own stream, which does not wait for the default one
+  CK(cudaMemcpyAsync(b->d_sched, sched.data(), sched.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
+  CK(cudaMemcpyAsync(b->d_params, hp.data(), n * sizeof(Params), cudaMemcpyHostToDevice, b->stream));
+  CK(cudaMemcpyAsync(b->d_share, share.data(), n_sched * sizeof(opfk::NodeShare), cudaMemcpyHostToDevice, b->stream));
+  CK(cudaStreamSynchronize(b->stream));
+  set_deal(b, bp);
   b->plan = bp;
   b->n_sched = n_sched;
   return OPF_OK;
@@ -1288,14 +1307,17 @@ opf_status opf_batch_create(opf_ctx *const *ctxs, int32_t n, opf_batch **out) {
   long long len = 0;
   opf_status st = OPF_OK;
   // as given, contiguous: the longest schedule
-  const opfk::BatchLayout lay{nullptr, 0, 1, opfk_batch_node_items(hp.data(), n)};
-  const int pr = opfk_batch_plan(hp.data(), plans.data(), n, lay, nullptr, 0, &len, &b->plan);
+  const opfk::BatchLayout lay{nullptr, 0, 1};
+  std::vector<opfk::NodeShare> share(n);
+  const int pr = opfk_batch_plan(hp.data(), plans.data(), n, lay, nullptr, 0, &len, nullptr, &b->plan);
   if (pr == -2) st = fail(OPF_EINVAL, "a batch cannot mix over-relaxed (alpha != 1) and plain instances");
   else if (pr != 0) st = fail(OPF_ECUDA, "batch schedule");
   std::vector<int> sched(4 * (size_t)std::max(len, 1LL));
-  if (st == OPF_OK && opfk_batch_plan(hp.data(), plans.data(), n, lay, sched.data(), len, &len, &b->plan) != 0)
+  if (st == OPF_OK &&
+      opfk_batch_plan(hp.data(), plans.data(), n, lay, sched.data(), len, &len, share.data(), &b->plan) != 0)
     st = fail(OPF_ECUDA, "batch schedule");
   b->sched_cap = len;
+  b->slot_cap = b->plan.deal.cap;
   b->n_sched = n;
   int lo = 0, hi = 0;
   cudaError_t e = st == OPF_OK ? cudaDeviceGetStreamPriorityRange(&lo, &hi) : cudaSuccess;
@@ -1306,8 +1328,17 @@ opf_status opf_batch_create(opf_ctx *const *ctxs, int32_t n, opf_batch **out) {
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_params, n * sizeof(Params));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_sched, sched.size() * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_params, hp.data(), n * sizeof(Params), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_sched, sched.data(), sched.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_share, n * sizeof(opfk::NodeShare));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_slot, b->slot_cap * sizeof(int4));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_dirty, sizeof(int));
+    auto put = [&](void *dst, const void *src, size_t bytes) {
+      if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream);
+    };
+    put(b->d_params, hp.data(), n * sizeof(Params));
+    put(b->d_sched, sched.data(), sched.size() * sizeof(int));
+    put(b->d_share, share.data(), n * sizeof(opfk::NodeShare));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    set_deal(b, b->plan);
     if (e != cudaSuccess) st = cuda_fail(e, "batch set-up");
   }
   if (st != OPF_OK) {
@@ -1332,7 +1363,7 @@ opf_status opf_batch_iterate(opf_batch *b, int32_t n_iters) {
     CK(cudaEventRecord(c->ev_in, c->stream));
     CK(cudaStreamWaitEvent(b->stream, c->ev_in, 0));
   }
-  if (opfk_begin_batch_launch(b->d_params, (int)b->ctx.size(), n_iters, b->stream) != 0)
+  if (opfk_begin_batch_launch(b->d_params, b->plan, (int)b->ctx.size(), n_iters, b->stream) != 0)
     return fail(OPF_ECUDA, "begin launch failed");
   cudaError_t le = cudaSuccess;
   launch_batch_steps(b, n_iters, &le);
@@ -1356,8 +1387,8 @@ opf_status opf_batch_autotune(opf_batch *b, int32_t steps, int32_t *choice, doub
   };
   std::stable_sort(lpt.begin(), lpt.end(), [&](int x, int y) { return work(x) > work(y); });
   const opfk::BatchLayout cands[OPF_BATCH_LAYOUTS] = {
-      {nullptr, 0, 1, 0.0}, {lpt.data(), 0, 1, 0.0}, {lpt.data(), 1, 1, 0.0},
-      {nullptr, 0, 4, 0.0}, {lpt.data(), 0, 4, 0.0}, {lpt.data(), 1, 4, 0.0}};   // node_items: schedule_batch
+      {nullptr, 0, 1}, {lpt.data(), 0, 1}, {lpt.data(), 1, 1},
+      {nullptr, 0, 4}, {lpt.data(), 0, 4}, {lpt.data(), 1, 4}};
   // save every instance's mutable state after its queued work
   std::vector<size_t> off(n + 1, 0);
   for (int i = 0; i < n; ++i) off[i + 1] = off[i] + mutable_bytes(b->ctx[i]);
@@ -1389,7 +1420,7 @@ opf_status opf_batch_autotune(opf_batch *b, int32_t steps, int32_t *choice, doub
     copy_all(false);
     // as in a call: residuals where a stopping test or an adaptation reads
     // them (past a call's last iteration every iteration would form them)
-    if (e == cudaSuccess && opfk_begin_batch_launch(b->d_params, n, steps + 2, b->stream) != 0) e = cudaErrorUnknown;
+    if (e == cudaSuccess && opfk_begin_batch_launch(b->d_params, b->plan, n, steps + 2, b->stream) != 0) e = cudaErrorUnknown;
     launch_batch_steps(b, 1, &e);                    // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(t0, b->stream);
     launch_batch_steps(b, steps, &e);
@@ -1475,7 +1506,7 @@ opf_status opf_batch_compact(opf_batch *b, int32_t *n_scheduled) {
     if (run[i]) order.push_back(i);
   }
   if ((int)order.size() != b->n_sched) {
-    const opfk::BatchLayout lay{order.data(), b->lay_interleave, b->lay_div, 0.0};
+    const opfk::BatchLayout lay{order.data(), b->lay_interleave, b->lay_div};
     const opf_status st = schedule_batch(b, (int)order.size(), lay);
     if (st != OPF_OK) return st;
   }

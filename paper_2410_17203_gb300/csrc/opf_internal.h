@@ -150,7 +150,7 @@ struct Params {
   // numbering maps (internal -> caller) for import / export
   const int *node_perm, *line_perm;
   // scratch
-  double *partials;  // [node_grid][NSLOT] per-CTA residual partial sums of the node kernel
+  double *partials;  // [node_grid][NSLOT] residual partial sums of the node kernel (one per CTA of its own grid)
   int node_grid;     // CTAs of the node kernel (partial-sum slots)
   unsigned *done;    // CTAs of the node kernel that have finished this iteration (0 between iterations)
   DevScalars *sc;
@@ -239,27 +239,41 @@ struct IterPlan {
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
 };
 
-// A batch of instances: the CTA schedules of each batch kernel, concatenated
-// in one array of (instance, block within the instance, blocks of the
-// instance, 0), in the order of BatchKernel.
-enum BatchKernel { BK_INNER, BK_CLOSED, BK_LINE4, BK_LINE1, BK_NODE4, BK_NODE1, BK_COUNT };
+// A batch of instances: the CTA schedules of the device and line kernels,
+// concatenated in one array of (instance, block within the instance, blocks of
+// the instance, 0), in the order of BatchKernel.
+enum BatchKernel { BK_INNER, BK_CLOSED, BK_LINE4, BK_LINE1, BK_COUNT };
+// The node kernel's CTAs are dealt out on the device, over the instances that
+// run: one wave of them (slots), each instance's share by its items, so that
+// the last running instances of a batch have the GPU to themselves.
+struct NodeShare {
+  int inst;
+  unsigned items;   // node items (of four steps or one)
+  int grid;         // at most this many CTAs (its residual partial sums: Params::node_grid)
+  int pad;
+};
+struct NodeDeal {
+  const NodeShare *share;  // [n]
+  int4 *slot;              // [cap] (instance or -1, block within it, its blocks, 0)
+  int *dirty;              // 1: slot is to be written anew
+  int n, slots, cap;
+};
 struct BatchPlan {
   int count[BK_COUNT];
   int offset[BK_COUNT];
+  NodeDeal deal;           // n, slots and cap; the caller adds the arrays
   size_t inner_smem;
   int inner_c;  // register chunk of the batch's inner-ADMM kernel (0: shared-memory path)
   int relax;   // the instances run over-relaxed (alpha != 1): the node kernels that carry it
 };
 // How a batch schedule lays out CTAs: instances in `order` (NULL: as given),
 // each instance's CTAs of a phase contiguous or dealt round-robin across
-// instances, and `div` times fewer CTAs for the grid-stride phases (devices,
-// node sums), each doing proportionally more work.
+// instances, and `div` times fewer CTAs for the devices, each doing
+// proportionally more work.
 struct BatchLayout {
   const int *order;
   int interleave;
   int div;
-  double node_items;   // of every instance of the batch, scheduled or not (an instance's share of the
-                       // node CTAs, and so its partial sums, does not change when others stop)
 };
 
 }  // namespace opfk
@@ -273,7 +287,8 @@ int opfk_plan(const opfk::Params &p, opfk::IterPlan *plan);
 // Start a call of n iterations: the residuals are formed at its last one;
 // clear_stop restarts a context that stopped (opf_iterate, not batches).
 int opfk_begin_launch(const opfk::Params &p, long long n, int clear_stop, void *stream);
-int opfk_begin_batch_launch(const opfk::Params *d_params, int n_inst, long long n, void *stream);
+int opfk_begin_batch_launch(const opfk::Params *d_params, const opfk::BatchPlan &bp, int n_inst, long long n,
+                            void *stream);
 // Enqueue one iteration: the device kernel (or xs, inner and dsum) and the
 // node kernel (whose last CTA takes the decisions) on main_stream, the line kernel on aux_stream (forked
 // after the previous iteration, joined before the node kernel).  Works under
@@ -283,11 +298,11 @@ int opfk_iteration_enqueue(const opfk::Params &p, const opfk::IterPlan &plan, vo
 // n iterations of a small instance (IterPlan::small) in one launch.
 int opfk_small_launch(const opfk::Params &p, int n, void *stream);
 // Schedules of the batch kernels for n instances (host parameter copies and
-// their plans): fills sched (4 ints per CTA, BatchPlan order) and the plan.
+// their plans): fills sched (4 ints per CTA, BatchPlan order), share [n] (NULL:
+// not wanted) and the plan.
 int opfk_batch_plan(const opfk::Params *hp, const opfk::IterPlan *plans, int n, const opfk::BatchLayout &lay,
-                    int *sched_out, long long sched_cap, long long *sched_len, opfk::BatchPlan *bp);
-// Node items of n instances (BatchLayout::node_items).
-double opfk_batch_node_items(const opfk::Params *hp, int n);
+                    int *sched_out, long long sched_cap, long long *sched_len, opfk::NodeShare *share,
+                    opfk::BatchPlan *bp);
 // Enqueue one iteration of every instance: d_params [n] and d_sched on the
 // device; the same stream and event roles as opfk_iteration_enqueue.
 int opfk_batch_enqueue(const opfk::Params *d_params, const int *d_sched, const opfk::BatchPlan &bp,

@@ -40,6 +40,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "opf_internal.h"
@@ -51,11 +52,6 @@ constexpr int WARPS = BLOCK / 32;
 constexpr int ST_NONFINITE = 5;  // opf_status value set on the device
 constexpr int NODE_VW = 4;       // time steps per node item
 constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is compiled for (64 registers)
-// Waves of node CTAs of a batch (its instances share the resident CTAs out by
-// items): 16 mixed instances of up to 3,000 buses, us per iteration: one wave
-// 81, two 84; every instance with a grid of its own, the two step widths in a
-// launch each, 101.
-constexpr double NODE_WAVES = 1.0;
 // Up to this many node items (four steps / one step each; about what two CTAs
 // per SM hold at once) the pass is latency alone, and a variant with the
 // registers to request all loads of an item together is faster: us per
@@ -63,6 +59,7 @@ constexpr double NODE_WAVES = 1.0;
 // (105k items) 15.5 -> 14.9, 900 buses T = 24 (76k) 16.9 -> 16.4; beyond it
 // the second wave costs more: 500 buses T = 168 (105k items of four) 35.1 -> 36.5.
 constexpr long long NODE_LAT_ITEMS4 = 2 * 152 * BLOCK, NODE_LAT_ITEMS1 = 1 << 17;
+constexpr int NODE_UNITS = 8;    // partial sums that a batch's node CTA forms between barriers
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
@@ -1618,7 +1615,8 @@ __device__ __forceinline__ void advance(const Params &p) {
   p.sc->v_fresh = 0;
 }
 
-__device__ __forceinline__ void decide_body(const Params &p, int n_part, double (*red)[NSLOT]) {
+// (dirty: told of a stop)
+__device__ __forceinline__ void decide_body(const Params &p, int n_part, double (*red)[NSLOT], int *dirty = nullptr) {
   double tot[NSLOT];
   if (p.slice) {
     // a contingency slice: the residual sums of every slice, exchanged
@@ -1701,6 +1699,7 @@ __device__ __forceinline__ void decide_body(const Params &p, int n_part, double 
   sc.v_fresh = 0;
   set_iter(p, sc);
   *p.sc = sc;
+  if (dirty && (sc.cur.flags & ITF_SKIP)) *dirty = 1;
 }
 
 // the CTA's residual partial sums, FP32 per thread and FP64 across warps, as
@@ -1723,6 +1722,76 @@ __device__ __forceinline__ void write_partials(const Params &p, unsigned part, c
   }
 }
 
+// The warp's FP32 sums of acc, in the order of write_partials (every pair that
+// its shuffles add meets here): at each step a lane keeps half of its sums and
+// hands the others over, 8 shuffles for the five sums instead of 25.
+__device__ __forceinline__ void warp_sums(const float (&acc)[NSLOT], float *out) {
+  static_assert(NSLOT == 5, "the halves below");
+  const int lane = threadIdx.x & 31;
+  const bool h = lane & 16, b = lane & 8, c = lane & 4;
+  auto give = [](float v, int o) { return __shfl_xor_sync(FULL, v, o); };
+  // sums 0 1 2 to the lower half, 3 4 to the upper
+  float x0 = (h ? acc[3] : acc[0]) + give(h ? acc[0] : acc[3], 16);
+  float x1 = (h ? acc[4] : acc[1]) + give(h ? acc[1] : acc[4], 16);
+  float x2 = acc[2] + give(acc[2], 16);   // (unused in the upper half)
+  // the first two to the lower quarters, the third to the upper
+  float y0 = (b ? x2 : x0) + give(b ? x0 : x2, 8);
+  float y1 = x1 + give(x1, 8);            // (unused in the upper quarters)
+  float z = (c ? y1 : y0) + give(c ? y0 : y1, 4);
+  z += give(z, 2);
+  z += give(z, 1);
+  // lanes 0, 4, 8, 16, 20 hold sums 0, 1, 2, 3, 4
+  const int slot = (h ? 3 : 0) + (b ? 2 : 0) + (c ? 1 : 0);
+  if ((lane & 3) == 0 && !(b && c) && slot < NSLOT) out[slot] = z;
+}
+
+// the node kernel's shared memory
+struct NodeMem {
+  double red[WARPS][NSLOT];
+  int last;
+};
+// ... in a batch, once for both step widths: two KB a CTA more and the kernel
+// takes another share of L1
+struct NodeMemB : NodeMem {
+  float wsum[NODE_UNITS][WARPS][NSLOT];
+};
+
+// The pass with residuals of a batch's instance.  Its partial sums are always
+// those of its own grid (p.node_grid, one per CTA there), so that the residuals
+// do not depend on how many CTAs the instance has here: each CTA forms several,
+// NODE_UNITS at a time between barriers (one at a time cost 64 mixed instances
+// 24 us per step, though one iteration in ten forms them).  Out of line: inlined,
+// it took registers from the pass without residuals (16 mixed instances 1.1 us
+// per step).
+template <int VW, bool RELAX>
+__device__ __noinline__ void node_units(const Params &p, unsigned bid, unsigned nblk, NodeMemB &mem) {
+  const int TV = p.T / VW, Kp = p.Kp;
+  const unsigned n = (unsigned)Kp * (unsigned)p.N * (unsigned)TV;
+  const unsigned parts = (unsigned)p.node_grid, ustride = parts * BLOCK;
+  const Iter q = load_iter(p);
+  Idx3 ix, dx;
+  dx.set(ustride, Kp, TV);
+  for (unsigned u0 = bid; u0 < parts; u0 += nblk * NODE_UNITS) {
+    int units = 0;
+    for (unsigned u = u0; units < NODE_UNITS && u < parts; u += nblk, ++units) {
+      float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      unsigned item = u * BLOCK + threadIdx.x;
+      ix.set(item, Kp, TV);
+      for (; item < n; item += ustride, ix.step(dx, Kp, TV))
+        node_item<VW, RELAX, true, NODE_RES_NB, true, false>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+      warp_sums(acc, mem.wsum[units][threadIdx.x >> 5]);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < units * NSLOT; x += BLOCK) {   // as write_partials
+      const int i = x / NSLOT, s = x - i * NSLOT;
+      double v = 0.0;
+      for (int w = 0; w < WARPS; ++w) v += (double)mem.wsum[i][w][s];
+      p.partials[(size_t)(u0 + i * nblk) * NSLOT + s] = v;
+    }
+    __syncthreads();   // mem.wsum is used again
+  }
+}
+
 // ---------------------------------------------------------------------------
 // node: step 3 for every (contingency, node, VW time steps); where the
 // residuals are read, the CTA's partial sums (FP32 per thread, FP64 across
@@ -1734,10 +1803,12 @@ __device__ __forceinline__ void write_partials(const Params &p, unsigned part, c
 // its 36 us on their launches.  At 64 registers (four CTAs per SM, what the
 // residual-free pass wants) the general pass gathers one terminal at a time.
 // ---------------------------------------------------------------------------
-template <int VW, bool RELAX, bool ILD, bool LAT = false>
-__device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk) {
-  __shared__ double red[WARPS][NSLOT];
-  __shared__ int s_last;
+// UNITS (batches): an instance's CTAs are fewer than its residual partial sums
+// (node_units).
+template <int VW, bool RELAX, bool ILD, bool LAT = false, bool UNITS = false>
+__device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk,
+                                          std::conditional_t<UNITS, NodeMemB, NodeMem> &mem, int *dirty = nullptr) {
+  double(*red)[NSLOT] = mem.red;
   const int N = p.N, TV = p.T / VW, Kp = p.Kp;
   const unsigned n = (unsigned)Kp * (unsigned)N * (unsigned)TV;
   const unsigned stride = nblk * BLOCK;
@@ -1752,14 +1823,17 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   if (q.flags & ITF_SKIP) return;
   const bool res = q.flags & ITF_RES;
   float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  if (res) {
+  if constexpr (UNITS) {
+    if (res) node_units<VW, RELAX>(p, bid, nblk, mem);
+  }
+  if (!UNITS && res) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
       node_item<VW, RELAX, true, LAT ? 4 : NODE_RES_NB, ILD, LAT>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
-  } else {
+  } else if (!res) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
       node_item<VW, RELAX, false, LAT ? 4 : NODE_LEAN_NB, ILD, LAT>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
   }
-  if (res) write_partials(p, bid, acc, red);
+  if (res && !UNITS) write_partials(p, bid, acc, red);
   if (p.slice) return;
   // the count is taken after every thread of the CTA has read the scalars and
   // (res) its partial sums are written; the last CTA alone goes on
@@ -1767,7 +1841,7 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   if (threadIdx.x == 0) {
     if (res) __threadfence();
     const bool last = atomicAdd(p.done, 1u) == nblk - 1;
-    s_last = last;
+    mem.last = last;
     if (last) {
       *p.done = 0;
       if (!res) advance(p);
@@ -1775,9 +1849,9 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   }
   if (!res) return;
   __syncthreads();
-  if (!s_last) return;
+  if (!mem.last) return;
   __threadfence();
-  decide_body(p, (int)nblk, red);
+  decide_body(p, UNITS ? p.node_grid : (int)nblk, red, dirty);
 }
 
 // ---------------------------------------------------------------------------
@@ -1818,7 +1892,8 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel(Params p, int ipt) {
 // every iteration carried the residual sums).  ILD: device sums in the pass.
 template <int VW, bool RELAX, bool ILD, bool LAT>
 __global__ void __launch_bounds__(BLOCK, LAT ? 2 : RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel(Params p) {
-  node_body<VW, RELAX, ILD, LAT>(p, blockIdx.x, gridDim.x);
+  __shared__ NodeMem mem;
+  node_body<VW, RELAX, ILD, LAT>(p, blockIdx.x, gridDim.x, mem);
 }
 
 // ---------------------------------------------------------------------------
@@ -1946,11 +2021,10 @@ __global__ void __launch_bounds__(BLOCK) slice_sums_kernel(Params p, int prime) 
   }
 }
 
-// the instance of this CTA: its parameters copied to shared memory, and
-// (block, blocks) within the instance
-__device__ __forceinline__ const Params &batch_params(const Params *ps, const int4 *sched, Params &sp,
+// the instance of this CTA, from its schedule entry e: its parameters copied
+// to shared memory, and (block, blocks) within the instance
+__device__ __forceinline__ const Params &batch_params(const Params *ps, const int4 e, Params &sp,
                                                       unsigned &bid, unsigned &nblk) {
-  const int4 e = sched[blockIdx.x];
   static_assert(sizeof(Params) % 4 == 0, "Params is copied as 32-bit words");
   const int *src = reinterpret_cast<const int *>(ps + e.x);
   int *dst = reinterpret_cast<int *>(&sp);
@@ -1961,38 +2035,98 @@ __device__ __forceinline__ const Params &batch_params(const Params *ps, const in
   return sp;
 }
 
+// The node kernel's CTAs shared out over the running instances, by the device
+// kernel's first CTA in front of its devices, in the iterations that follow the
+// start of a call or an instance's stop: floor(slots x items / all running
+// items) CTAs each, at least one and at most its grid.  64 mixed instances, us
+// per step as given: all running 721 with a grid of its own for each (in
+// seven launches), 570 with shares that stay when others stop, 576 with these;
+// the last one running, the others compacted away, 34 to 90, 92 to 142 and 16
+// to 67; four running 106, 177 and 65.
+// (mem: the CTA's shared memory for an instance's parameters, not in use yet.
+// More would change the kernel's share of L1, which the concurrent line kernel's
+// CTAs cannot follow: with arrays of its own 16 mixed instances took 3 us more
+// per step.)
+struct DealMem {
+  static constexpr int N = 64;   // instances at a time
+  unsigned long long sum[DEV_WARPS];
+  int m[N], inst[N];
+};
+__device__ void deal_nodes(const Params *ps, const NodeDeal &d, DealMem &mem) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  auto runs = [&](const NodeShare &s) { return !(ps[s.inst].sc->cur.flags & ITF_SKIP); };
+  unsigned long long sum = 0;
+  for (int i = tid; i < d.n; i += DEVB) {
+    const NodeShare s = d.share[i];
+    if (runs(s)) sum += s.items;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+  if (lane == 0) mem.sum[w] = sum;
+  __syncthreads();
+  sum = 0;
+#pragma unroll
+  for (int i = 0; i < DEV_WARPS; ++i) sum += mem.sum[i];
+  int at = 0;   // entries written
+  for (int i0 = 0; i0 < d.n; i0 += DealMem::N) {
+    const int i = i0 + tid;
+    if (tid < DealMem::N && i < d.n) {
+      const NodeShare s = d.share[i];
+      mem.m[tid] = runs(s) ? min(s.grid, max(1, (int)((unsigned long long)d.slots * s.items / sum))) : 0;
+      mem.inst[tid] = s.inst;
+    }
+    __syncthreads();
+    for (int j = 0; j < DealMem::N && i0 + j < d.n; ++j) {
+      const int mj = mem.m[j];
+      for (int r = tid; r < mj; r += DEVB) d.slot[at + r] = make_int4(mem.inst[j], r, mj, 0);
+      at += mj;
+    }
+    __syncthreads();
+  }
+  for (int b = at + tid; b < d.cap; b += DEVB) d.slot[b] = make_int4(-1, 0, 0, 0);
+  if (tid == 0) *d.dirty = 0;
+}
+
 // the devices of every instance: the first inner_blocks CTAs of the schedule
 // take inner-ADMM devices, the others closed-form ones.  C: the largest
 // register chunk of the batch's instances (0: every horizon beyond
 // BATCH_REG_T), any longer horizon on the shared-memory path (the same bits)
 template <int C>
-__global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks) {
+__global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
   extern __shared__ float smem[];
   __shared__ Params sp;
+  if (blockIdx.x == 0) {
+    static_assert(sizeof(DealMem) <= sizeof(Params) && alignof(DealMem) <= alignof(Params), "shared by turns");
+    if (*deal.dirty) deal_nodes(ps, deal, *reinterpret_cast<DealMem *>(&sp));
+    if (blocks == 0) return;   // no device in any instance
+  }
   unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
+  const Params &p = batch_params(ps, sched[blockIdx.x], sp, bid, nblk);
   if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true, DEV_WARPS, false);
   else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), bid, nblk);
   else closed_body<1>(p, load_iter(p), bid, nblk);
 }
 
 // the lines of every instance: the first n4 CTAs of the schedule take those
-// whose horizon is whole 4-step blocks, the others the rest; the nodes alike
+// whose horizon is whole 4-step blocks, the others the rest
 __global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, const int4 *sched, int n4) {
   __shared__ Params sp;
   unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
+  const Params &p = batch_params(ps, sched[blockIdx.x], sp, bid, nblk);
   if ((int)blockIdx.x < n4) line_body<4>(p, bid, LINE_IPT);
   else line_body<1>(p, bid, LINE_IPT);
 }
 
 template <bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *sched, int n4) {
+__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *slot, int *dirty) {
   __shared__ Params sp;
+  __shared__ NodeMemB mem;
+  const int4 e = slot[blockIdx.x];   // dealt out by deal_nodes
+  if (e.x < 0) return;
   unsigned bid, nblk;
-  const Params &p = batch_params(ps, sched, sp, bid, nblk);
-  if ((int)blockIdx.x < n4) node_body<4, RELAX, true>(p, bid, nblk);
-  else node_body<1, RELAX, true>(p, bid, nblk);
+  const Params &p = batch_params(ps, e, sp, bid, nblk);
+  if (p.T % NODE_VW == 0) node_body<NODE_VW, RELAX, true, false, true>(p, bid, nblk, mem, dirty);
+  else node_body<1, RELAX, true, false, true>(p, bid, nblk, mem, dirty);
 }
 
 // A line's terminal values from its stored (p, mid) at contingency k:
@@ -2273,8 +2407,9 @@ __global__ void begin_kernel(Params p, long long n, int clear_stop) {
   *p.sc = sc;
 }
 
-__global__ void begin_batch_kernel(const Params *ps, int n_inst, long long n) {
+__global__ void begin_batch_kernel(const Params *ps, int n_inst, long long n, int *dirty) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *dirty = 1;   // instances may have been reset since the last call
   if (i >= n_inst) return;
   DevScalars sc = *ps[i].sc;
   sc.it_last = sc.it + n;
@@ -2493,17 +2628,8 @@ int opfk_slice_prime_launch(const Params &p, void *stream) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// node items (of four steps or one) of an instance
-static double node_items(const Params &p) { return (double)p.Kp * p.N * (p.T % NODE_VW == 0 ? p.T / NODE_VW : p.T); }
-
-double opfk_batch_node_items(const Params *hp, int n) {
-  double s = 0.0;
-  for (int i = 0; i < n; ++i) s += node_items(hp[i]);
-  return s;
-}
-
 int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchLayout &lay, int *sched_out,
-                    long long sched_cap, long long *sched_len, BatchPlan *bp) {
+                    long long sched_cap, long long *sched_len, NodeShare *share, BatchPlan *bp) {
   long long len = 0;
   size_t ism = 0;
   int ic_max = 0;
@@ -2520,8 +2646,6 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     return true;
   };
   const int div = std::max(1, lay.div);
-  const int slots = resident_grid(node_kernel_b<false>, 0);
-  if (slots < 1) return -1;
   std::vector<long long> nb(n);
   for (int kind = 0; kind < BK_COUNT; ++kind) {
     bp->offset[kind] = (int)len;
@@ -2529,7 +2653,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     for (int j = 0; j < n; ++j) {
       const int i = lay.order ? lay.order[j] : j;
       const Params &p = hp[i];
-      const bool v4 = (p.T % 4 == 0), vn = (p.T % NODE_VW == 0);
+      const bool v4 = (p.T % 4 == 0);
       const long long tv4 = p.T / (v4 ? 4 : 1);
       const int n_inner = inner_units(p);
       long long blocks = 0;
@@ -2549,17 +2673,9 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           if ((kind == BK_LINE4) == v4 && p.L > 0)
             blocks = ((long long)p.Kp * p.L * tv4 + (long long)BLOCK * LINE_IPT - 1) / ((long long)BLOCK * LINE_IPT);
           break;
-        case BK_NODE4: case BK_NODE1:
-          // the resident CTAs shared out by items, so that one wave of CTAs, each
-          // walking as many items as the others, serves the batch
-          if ((kind == BK_NODE4) == vn)
-            blocks = std::min<long long>(plans[i].node_grid,
-                                         std::max<long long>(1, (long long)(node_items(p) * NODE_WAVES * slots / lay.node_items)));
-          break;
       }
-      // the grid-stride phases take any block count: `div` puts more work in
-      // each CTA
-      if (blocks > 0 && (kind == BK_INNER || kind == BK_CLOSED || kind == BK_NODE4 || kind == BK_NODE1))
+      // the devices take any block count: `div` puts more work in each CTA
+      if (blocks > 0 && (kind == BK_INNER || kind == BK_CLOSED))
         blocks = (blocks + div - 1) / div;
       nb[j] = blocks;
       most = std::max(most, blocks);
@@ -2576,12 +2692,25 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     }
     bp->count[kind] = (int)(len - bp->offset[kind]);
   }
-  static_assert(NODE_VW == 4, "the batch node kernels are instantiated for widths 4 and 1");
   bp->inner_c = ic_max;
   bp->inner_smem = ism;
   bp->relax = (n > 0 && hp[0].alpha != 1.f) ? 1 : 0;
   for (int i = 0; i < n; ++i)
     if ((hp[i].alpha != 1.f) != (bp->relax != 0)) return -2;   // one node kernel for every instance
+  bp->deal = NodeDeal{};
+  bp->deal.n = n;
+  bp->deal.slots = bp->relax ? resident_grid(node_kernel_b<true>, 0) : resident_grid(node_kernel_b<false>, 0);
+  if (bp->deal.slots < 1) return -1;
+  // the shares round down and are at least one each, at most the grid
+  long long grids = 0;
+  for (int j = 0; j < n; ++j) {
+    const int i = lay.order ? lay.order[j] : j;
+    const Params &p = hp[i];
+    const int tv = p.T % NODE_VW == 0 ? p.T / NODE_VW : p.T;
+    if (share) share[j] = NodeShare{i, (unsigned)p.Kp * (unsigned)p.N * (unsigned)tv, plans[i].node_grid, 0};
+    grids += plans[i].node_grid;
+  }
+  bp->deal.cap = (int)std::min<long long>(grids, (long long)bp->deal.slots + n);
   if (!allow_smem(dev_kernel_b<0>, ism) || !allow_smem(dev_kernel_b<1>, ism) || !allow_smem(dev_kernel_b<2>, ism) ||
       !allow_smem(dev_kernel_b<3>, ism) || !allow_smem(dev_kernel_b<4>, ism))
     return -1;
@@ -2596,26 +2725,29 @@ int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPl
   auto at = [&](int kind) { return sched + bp.offset[kind]; };
   if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
   if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
-  static_assert(BK_LINE1 == BK_LINE4 + 1 && BK_NODE1 == BK_NODE4 + 1, "one launch over both widths' schedules");
+  // the devices first: a graph's first iteration starts its kernels in this
+  // order, and line CTAs that fill the GPU hold up the longer device chain
+  // (16 instances of T = 128, calls of 9 steps: 172 -> 140 us per step)
+  static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
+  const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED];
+  if (bp.deal.n > 0) {
+    const int4 *si = at(BK_INNER);
+    switch (bp.inner_c) {
+      case 1: dev_kernel_b<1><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
+      case 2: dev_kernel_b<2><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
+      case 3: dev_kernel_b<3><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
+      case 4: dev_kernel_b<4><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
+      default: dev_kernel_b<0><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
+    }
+  }
+  static_assert(BK_LINE1 == BK_LINE4 + 1, "one launch over both widths' schedules");
   const int l4 = bp.count[BK_LINE4], nl = l4 + bp.count[BK_LINE1];
   if (nl) line_kernel_b<<<nl, BLOCK, 0, sa>>>(d_params, at(BK_LINE4), l4);
   if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
-  static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
-  const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED];
-  if (nd) {
-    const int4 *si = at(BK_INNER);
-    switch (bp.inner_c) {
-      case 1: dev_kernel_b<1><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
-      case 2: dev_kernel_b<2><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
-      case 3: dev_kernel_b<3><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
-      case 4: dev_kernel_b<4><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
-      default: dev_kernel_b<0><<<nd, DEVB, bp.inner_smem, sm>>>(d_params, si, ni); break;
-    }
-  }
   if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
-  const int n4 = bp.count[BK_NODE4], nn = n4 + bp.count[BK_NODE1];
-  if (nn && bp.relax) node_kernel_b<true><<<nn, BLOCK, 0, sm>>>(d_params, at(BK_NODE4), n4);
-  else if (nn) node_kernel_b<false><<<nn, BLOCK, 0, sm>>>(d_params, at(BK_NODE4), n4);
+  const int nn = bp.deal.cap;
+  if (nn && bp.relax) node_kernel_b<true><<<nn, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
+  else if (nn) node_kernel_b<false><<<nn, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -2672,8 +2804,8 @@ int opfk_begin_launch(const Params &p, long long n, int clear_stop, void *stream
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int opfk_begin_batch_launch(const Params *d_params, int n_inst, long long n, void *stream) {
-  begin_batch_kernel<<<(n_inst + 255) / 256, 256, 0, (cudaStream_t)stream>>>(d_params, n_inst, n);
+int opfk_begin_batch_launch(const Params *d_params, const BatchPlan &bp, int n_inst, long long n, void *stream) {
+  begin_batch_kernel<<<(n_inst + 255) / 256, 256, 0, (cudaStream_t)stream>>>(d_params, n_inst, n, bp.deal.dirty);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

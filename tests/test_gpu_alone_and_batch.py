@@ -94,3 +94,57 @@ def test_batch_at_the_edge_of_48_kb(T):
         opf_batch_destroy(b)
         single.close()
         member.close()
+
+
+@pytest.mark.parametrize("alpha", [1.0, 1.5])
+def test_members_equal_contexts_alone_in_every_bit(alpha):
+    """Iterates, residuals, penalties and histories of a batch's instances are
+    those of each context alone, whatever CTAs the node kernel deals them: with
+    every instance running, after some have stopped (on tolerances of their
+    own), after compaction, after a reset, and in every layout.  The largest
+    has more node items than its grid has threads, the smallest less than one
+    CTA's worth; eleven are more than half of what stops."""
+    from paper_2410_17203_gb300 import (Solver, opf_batch_autotune, opf_batch_compact, opf_batch_create,
+                                        opf_batch_destroy, opf_batch_iterate, opf_reset)
+    sizes = [(3000, 24, 10), (5, 1, 0), (300, 24, 4), (60, 7, 22), (200, 1, 9), (90, 31, 2), (40, 12, 3),
+             (700, 48, 1), (25, 128, 1), (50, 24, 20), (30, 300, 0)]
+    cases = [make_case(scale_case(n, T, K, seed=70 + i, n_hvdc=i % 2 if n > 20 else 0))
+             for i, (n, T, K) in enumerate(sizes)]
+    # all but three stop at the first stopping test that finds residuals below a generous tolerance
+    opts = [dict(adapt_every=5, check_every=4, alpha=alpha, history_len=64, eps=1e-9 if i in (0, 3, 7) else 1.0)
+            for i in range(len(sizes))]
+    alone = [Solver(c, o) for c, o in zip(cases, opts)]
+    member = [Solver(c, o) for c, o in zip(cases, opts)]
+
+    def check():
+        for a, m in zip(alone, member):
+            _assert_same_state(m, a)
+            np.testing.assert_array_equal(m.residuals(), a.residuals())
+            np.testing.assert_array_equal(m.history(), a.history())
+            i, j = a.get_info(), m.get_info()
+            assert [i[k] for k in ("iterations", "converged", "rho_p", "rho_theta")] == \
+                   [j[k] for k in ("iterations", "converged", "rho_p", "rho_theta")]
+
+    def both(n):
+        for a in alone:
+            if not a.get_info()["converged"]:
+                a.iterate(n)
+        opf_batch_iterate(b, n)
+        check()
+
+    b = opf_batch_create([m.h for m in member])
+    try:
+        for n in (3, 9, 20):
+            both(n)
+        left = sum(not a.get_info()["converged"] for a in alone)
+        assert left == opf_batch_compact(b)
+        both(7)
+        for h in [a.h for a in alone] + [m.h for m in member]:
+            opf_reset(h)
+        opf_batch_autotune(b, steps=2)
+        for n in (2, 17):
+            both(n)
+    finally:
+        opf_batch_destroy(b)
+        for s in alone + member:
+            s.close()
