@@ -2425,10 +2425,13 @@ opf_status opf_diff_create(const opf_network *net, int32_t T, const opf_continge
     delete d;
     return dfail(OPF_EINVAL, "diff: the horizon is too long for one inner-ADMM device per CTA");
   }
-  if (e == cudaSuccess && d->smem_fwd)
-    e = cudaFuncSetAttribute(fwd_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem_fwd);
-  if (e == cudaSuccess && d->smem_bwd)
-    e = cudaFuncSetAttribute(bwd_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem_bwd);
+  // the limit is the function's, not this context's: always the same value
+  // (neither kernel has static shared memory), so that no context lowers
+  // another's
+  if (e == cudaSuccess && T > DREG_T && d->smem_fwd) {
+    e = cudaFuncSetAttribute(fwd_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(bwd_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+  }
   DP &p = d->p;
   p.N = N;
   p.L = L;
