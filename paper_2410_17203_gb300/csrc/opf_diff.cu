@@ -1927,9 +1927,11 @@ struct opf_diff {
   // The launches of a call's forward and reverse pass as CUDA graphs, kept
   // for the next calls of the same shape (PassKey): a graph starts a small
   // kernel every 0.7 us, a stream every 2 us, and an iteration has seven.
-  // They are built by the second call of a shape in a row (a first call
-  // launches directly: capture and instantiation take about 2 us a kernel),
-  // up to GRAPH_MAX_K iterations, captured on `cap`.
+  // Capture and instantiation take about 2 us a kernel, so the calls of a run
+  // share them: the first launches directly, the second builds the forward
+  // pass's, the third the reverse pass's (ms per call, 151 buses T = 31 x 60:
+  // both in the second call 3.05, 3.70, 2.05, 2.05, shared 3.06, 3.25, 2.90, 2.05; without
+  // graphs 3.05).  Up to GRAPH_MAX_K iterations, captured on `cap`.
   cudaStream_t cap = nullptr;
   cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
   PassKey key{};
@@ -2794,8 +2796,9 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   if (!same) {
     drop_graphs(d);
     d->key = key;
-  } else if (!d->g_fwd && K <= GRAPH_MAX_K) {
-    if (!build_graph(d, forward, &d->g_fwd) || (grads && !build_graph(d, reverse, &d->g_bwd))) drop_graphs(d);
+  } else if (K <= GRAPH_MAX_K) {
+    if (!d->g_fwd) build_graph(d, forward, &d->g_fwd);
+    else if (grads && !d->g_bwd) build_graph(d, reverse, &d->g_bwd);
   }
   e = d->g_fwd ? cudaGraphLaunch(d->g_fwd, d->stream) : forward(d->stream);
   // the cost's inputs to the host, where it is summed while the reverse pass runs
