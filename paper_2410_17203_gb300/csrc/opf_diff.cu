@@ -1935,6 +1935,7 @@ struct opf_diff {
   cudaStream_t cap = nullptr;
   cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
   PassKey key{};
+  bool no_graph = false;   // a build failed at this key: not tried again
   // host staging of the cost's inputs (pinned), read while the reverse pass runs
   cudaEvent_t ev_cost = nullptr;
   float *stage_host = nullptr;
@@ -2796,9 +2797,10 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   if (!same) {
     drop_graphs(d);
     d->key = key;
-  } else if (K <= GRAPH_MAX_K) {
-    if (!d->g_fwd) build_graph(d, forward, &d->g_fwd);
-    else if (grads && !d->g_bwd) build_graph(d, reverse, &d->g_bwd);
+    d->no_graph = false;
+  } else if (K <= GRAPH_MAX_K && !d->no_graph) {
+    if (!d->g_fwd) d->no_graph = !build_graph(d, forward, &d->g_fwd);
+    else if (grads && !d->g_bwd) d->no_graph = !build_graph(d, reverse, &d->g_bwd);
   }
   e = d->g_fwd ? cudaGraphLaunch(d->g_fwd, d->stream) : forward(d->stream);
   // the cost's inputs to the host, where it is summed while the reverse pass runs
