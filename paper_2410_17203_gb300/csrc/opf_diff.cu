@@ -58,7 +58,7 @@ struct DP {
   int N, L, T, Kp, G, D, B, H, S;       // H HVDC links, terminals H0 + 2h and H0 + 2h + 1 (H0 = G + D + B)
   float rp, rt, rd;                    // rho_p, rho_theta, (K+1) rho_p (= omega of the inner ADMM)
   const int *n1, *n2;                  // line ends (terminal 1 at n1 carries -p)
-  const float *b;                      // susceptance [L]
+  const float4 *ldiv;                  // [L] divisors of the line prox (line_div)
   const int *out;                      // [Kp] outaged line, -1 = none
   const int *lptr, *lcode;             // node -> line terminal codes 2 l + end (end 1: terminal 2)
   const int4 *lcode4;                  // each node's first four codes (-1: none)
@@ -364,15 +364,10 @@ __device__ __forceinline__ LineIn line_inputs(const DP &p, const St &s, int k, i
 // The prox inputs that decide a clip, each rounding written out, so that the
 // reverse pass's recomputation (without a record) takes the forward's
 // decisions whatever the compiler contracts elsewhere: the line prox's
-// denominator 2 rho_p + rho_theta / (2 b^2) and unclipped flow (Section 4.2),
-// a generator's and a curtailable load's unclipped power (Section 4.1)
-__device__ __forceinline__ float line_den(const DP &p, float b, float tb) {
-  return __fadd_rn(__fmul_rn(2.f, p.rp), p.rt / (tb * b));
-}
-// (rtb = 1 / tb, rden = 1 / den: the quotients by the rounded reciprocals and
-// one correction each, as the division rounds them)
-__device__ __forceinline__ float line_z(const DP &p, const LineIn &in, float tb, float rtb, float den, float rden) {
-  return qdiv(__fadd_rn(__fmul_rn(p.rp, in.x2 - in.x1), qdiv(__fmul_rn(p.rt, in.y1 - in.y2), tb, rtb)), den, rden);
+// unclipped flow (Section 4.2, d: line_div), a generator's and a curtailable
+// load's unclipped power (Section 4.1)
+__device__ __forceinline__ float line_z(const DP &p, const LineIn &in, const float4 &d) {
+  return qdiv(__fadd_rn(__fmul_rn(p.rp, in.x2 - in.x1), qdiv(__fmul_rn(p.rt, in.y1 - in.y2), d.x, d.y)), d.z, d.w);
 }
 __device__ __forceinline__ float gen_den(const DP &p, int d) { return __fadd_rn(__fmul_rn(2.f, p.ga[d]), p.rd); }
 __device__ __forceinline__ float gen_z(const DP &p, int d, float X) {
@@ -403,19 +398,19 @@ __global__ void __launch_bounds__(TB, VW == 4 ? VW4_CTAS : 8) fwd_line(DP p, St 
     const Vf<VW> TB2 = ldv<VW>(s.TBR + o2), V1 = ldv<VW>(s.V1 + o), V2 = ldv<VW>(s.V2 + o);
     Vf<VW> np, t1, t2;
     if (p.out[k] != l) {
-      const float b = p.b[l], tb = 2.f * b, u = p.lu[l], den = line_den(p, b, tb);
-      const float rtb = __frcp_rn(tb), rden = __frcp_rn(den);
+      const float u = p.lu[l];
+      const float4 dv = p.ldiv[l];
       Vb<VW> code;
 #pragma unroll
       for (int e = 0; e < VW; ++e) {
         // the prox inputs as line_inputs forms them
         const LineIn in{-P.x[e] - PB1.x[e] - U1.x[e], P.x[e] - PB2.x[e] - U2.x[e], TB1.x[e] - V1.x[e],
                         TB2.x[e] - V2.x[e]};
-        const float z = line_z(p, in, tb, rtb, den, rden);
+        const float z = line_z(p, in, dv);
         code.x[e] = clip_code(z, -u, u);
         const float p2 = fminf(fmaxf(z, -u), u);
         const float mid = 0.5f * (in.y1 + in.y2);
-        const float h = qdiv(p2, tb, rtb);
+        const float h = qdiv(p2, dv.x, dv.y);
         np.x[e] = p2;
         t1.x[e] = mid + h;
         t2.x[e] = mid - h;
@@ -778,12 +773,9 @@ __device__ __forceinline__ void line_back(const DP &p, const St &s, const Adj &a
     const float lt2 = fmaf(B2.x[e], ih2, __fadd_rn(lt20.x[e], LV2.x[e]));
     float lx1 = 0.f, lx2 = 0.f, ly1, ly2;
     if (act) {
-      const float b = p.b[l], tb = 2.f * b, u = p.lu[l];
+      const float u = p.lu[l];
       unsigned char cd = code.x[e];
-      if (!lmask) {
-        const float den = line_den(p, b, tb);
-        cd = clip_code(line_z(p, line_inputs(p, s, k, l, it.t0 + e), tb, __frcp_rn(tb), den, __frcp_rn(den)), -u, u);
-      }
+      if (!lmask) cd = clip_code(line_z(p, line_inputs(p, s, k, l, it.t0 + e), p.ldiv[l]), -u, u);
       const float lpt = fmaf(lt1 - lt2, p.lfac[l], lp);     // theta_{1,2} = mid +- p / (2b)
       const float half = __fmul_rn(0.5f, lt1 + lt2);
       ly1 = ly2 = half;
@@ -2124,6 +2116,17 @@ void stor_factor(int T, double rd, double eta, std::vector<float> &out) {
   tri_pivots(T + 1, 3.0 * om + gam, 2.0 * om + 2.0 * gam, -gam, out);
 }
 
+// A line's tb = 2 b and prox denominator 2 rho_p + rho_theta / (2 b^2), each with
+// its rounded reciprocal (qdiv).  An infinite one -- a line of infinite
+// susceptance, the denominator of a line whose susceptance squared underflows --
+// is 1 with the reciprocal 0, so that it divides to 0 and not to NaN, which the
+// clamp would make the negative limit.
+float4 line_div(float rp, float rt, float b) {
+  const float tb = 2.f * b, den = 2.f * rp + rt / (tb * b);
+  const bool ti = std::isinf(tb), di = std::isinf(den);
+  return make_float4(ti ? 1.f : tb, ti ? 0.f : 1.f / tb, di ? 1.f : den, di ? 0.f : 1.f / den);
+}
+
 St carve_state(const opf_diff *d, float *base) {
   const size_t KLT = (size_t)d->Kp * d->L * d->T, KNT = (size_t)d->Kp * d->N * d->T, ST = (size_t)d->S * d->T;
   St s;
@@ -2455,7 +2458,11 @@ opf_status opf_diff_create(const opf_network *net, int32_t T, const opf_continge
   };
   U(&p.n1, n1);
   U(&p.n2, n2);
-  U(&p.b, b);
+  {
+    std::vector<float4> ld(L);
+    for (int l = 0; l < L; ++l) ld[l] = line_div(p.rp, p.rt, b[l]);
+    U(&p.ldiv, ld);
+  }
   U(&p.out, outl);
   U(&p.lptr, lptr);
   U(&p.lcode, lcode);

@@ -16,11 +16,15 @@ __device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b)
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// x / q by the rounded reciprocal rq = 1 / q and one residual correction
-// (Markstein 1990): the correctly rounded quotient for the operands of these
-// solves (2e8 random pairs over 2^-40 .. 2^20 by 2^-10 .. 2^12: every result
-// equal to the division's), in three dependent operations.  The inner
-// iterations divide by pivots and constants that do not change between them.
+// x / q by the rounded reciprocal rq = 1 / q and one residual correction, in
+// three dependent operations: the division's result, correctly rounded, while
+// q, x and the quotient are normal numbers with room for the residual (|q| <=
+// 2^126, |x| >= 2^-100 or 0).  rq is within half an ulp of 1 / q and q0 within
+// 1.5 ulp of x / q, the residual is exact, so the sum rounds wrongly only if
+// x / q lies within 1.5 * 2^-24 ulp of a rounding boundary: |x 2^k - M q| <= 3
+// for a boundary M and significands x, q < 2^24.  All pairs with |...| <= 16
+// round as the division does (8e8 of them, enumerated; the test samples them).
+// Smaller x: within one ulp.  An infinite q, x or quotient gives NaN.
 __device__ __forceinline__ float qdiv(float x, float q, float rq) {
   const float q0 = rmul(x, rq);
   return rfma(rfma(-q0, q, x), rq, q0);
