@@ -1151,11 +1151,12 @@ opf_status opf_solution(opf_ctx *c, int32_t on_device, double *objective, float 
 struct opf_batch {
   std::vector<opf_ctx *> ctx;
   int device = 0;
-  // the batch kernels run on these two streams (main: devices, node sums,
-  // decisions; aux: line proxes); every instance's parameters and the CTA
-  // schedules of the batch kernels live in device memory
-  cudaStream_t stream = nullptr, s_aux = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_done = nullptr;
+  // the batch kernels run on these streams (main: devices, node sums,
+  // decisions; aux: line proxes; dev: devices that solve in shared memory);
+  // every instance's parameters and the CTA schedules of the batch kernels live
+  // in device memory
+  cudaStream_t stream = nullptr, s_aux = nullptr, s_dev = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_dev = nullptr, ev_done = nullptr;
   opfk::Params *d_params = nullptr;
   int *d_sched = nullptr;
   // the deal of the node kernel's CTAs (opfk::NodeDeal)
@@ -1178,10 +1179,11 @@ namespace {
 void release_batch(opf_batch *b) {
   if (b->g_one) cudaGraphExecDestroy(b->g_one);
   if (b->g_many) cudaGraphExecDestroy(b->g_many);
-  for (cudaEvent_t e : {b->ev_fork, b->ev_join, b->ev_done})
+  for (cudaEvent_t e : {b->ev_fork, b->ev_join, b->ev_dev, b->ev_done})
     if (e) cudaEventDestroy(e);
   if (b->stream) cudaStreamDestroy(b->stream);
   if (b->s_aux) cudaStreamDestroy(b->s_aux);
+  if (b->s_dev) cudaStreamDestroy(b->s_dev);
   if (b->d_params) cudaFree(b->d_params);
   if (b->d_sched) cudaFree(b->d_sched);
   if (b->d_share) cudaFree(b->d_share);
@@ -1195,7 +1197,8 @@ opf_status build_batch_graph(opf_batch *b, int iters, cudaGraphExec_t *out) {
   CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   bool ok = true;
   for (int it = 0; ok && it < iters; ++it)
-    ok = opfk_batch_enqueue(b->d_params, b->d_sched, b->plan, b->stream, b->s_aux, b->ev_fork, b->ev_join) == 0;
+    ok = opfk_batch_enqueue(b->d_params, b->d_sched, b->plan,
+                            {b->stream, b->s_aux, b->s_dev, b->ev_fork, b->ev_join, b->ev_dev}) == 0;
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(b->stream, &g);
   if (!ok || e != cudaSuccess) {
@@ -1324,7 +1327,8 @@ opf_status opf_batch_create(opf_ctx *const *ctxs, int32_t n, opf_batch **out) {
   if (st == OPF_OK) {
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->stream, cudaStreamNonBlocking, hi);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->s_aux, cudaStreamNonBlocking, lo);
-    for (cudaEvent_t *ev : {&b->ev_fork, &b->ev_join, &b->ev_done})
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->s_dev, cudaStreamNonBlocking, hi);
+    for (cudaEvent_t *ev : {&b->ev_fork, &b->ev_join, &b->ev_dev, &b->ev_done})
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_params, n * sizeof(Params));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_sched, sched.size() * sizeof(int));

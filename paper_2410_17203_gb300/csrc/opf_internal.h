@@ -239,10 +239,18 @@ struct IterPlan {
   int inner_c;     // register chunk of the inner-ADMM kernel (0: shared-memory path)
 };
 
+// The streams of a batch's phases and the events between them: devices and
+// node sums on main, line proxes on aux, and on dev the devices that solve in
+// shared memory.
+struct Lanes {
+  void *main, *aux, *dev;
+  void *ev_fork, *ev_join, *ev_dev;
+};
+
 // A batch of instances: the CTA schedules of the device and line kernels,
 // concatenated in one array of (instance, block within the instance, blocks of
 // the instance, 0), in the order of BatchKernel.
-enum BatchKernel { BK_INNER, BK_CLOSED, BK_LINE4, BK_LINE1, BK_COUNT };
+enum BatchKernel { BK_SMEM, BK_INNER, BK_CLOSED, BK_LINE4, BK_LINE1, BK_COUNT };
 // The node kernel's CTAs are dealt out on the device, over the instances that
 // run: one wave of them (slots), each instance's share by its items, so that
 // the last running instances of a batch have the GPU to themselves.
@@ -262,8 +270,8 @@ struct BatchPlan {
   int count[BK_COUNT];
   int offset[BK_COUNT];
   NodeDeal deal;           // n, slots and cap; the caller adds the arrays
-  size_t inner_smem;
-  int inner_c;  // register chunk of the batch's inner-ADMM kernel (0: shared-memory path)
+  size_t inner_smem;       // of the kernel that solves in shared memory (BK_SMEM)
+  int inner_c;             // the largest register chunk of the batch's instances
   int relax;   // the instances run over-relaxed (alpha != 1): the node kernels that carry it
 };
 // How a batch schedule lays out CTAs: instances in `order` (NULL: as given),
@@ -304,9 +312,9 @@ int opfk_batch_plan(const opfk::Params *hp, const opfk::IterPlan *plans, int n, 
                     int *sched_out, long long sched_cap, long long *sched_len, opfk::NodeShare *share,
                     opfk::BatchPlan *bp);
 // Enqueue one iteration of every instance: d_params [n] and d_sched on the
-// device; the same stream and event roles as opfk_iteration_enqueue.
+// device.
 int opfk_batch_enqueue(const opfk::Params *d_params, const int *d_sched, const opfk::BatchPlan &bp,
-                       void *main_stream, void *aux_stream, void *ev_fork, void *ev_join);
+                       const opfk::Lanes &on);
 // State import / export between internal and caller numbering; `cur` selects
 // the node buffer holding the current state.
 int opfk_import_launch(const opfk::Params &p, int cur, const float *p_line, const float *th1,

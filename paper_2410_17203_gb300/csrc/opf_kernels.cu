@@ -81,8 +81,14 @@ constexpr int BATCH_C = 4;         // the same in batches, whose kernels hold ev
 constexpr int BATCH_REG_T = 32 * BATCH_C - 1;
 
 // shared floats per warp of the shared-memory inner ADMM: 3 (T+1) for the
-// work arrays and, staged, one device's (lam, beta)
-__host__ __device__ inline int warp_smem_floats(int T, bool staged) { return (T + 1) * (staged ? 3 + 2 * SG_N : 3); }
+// work arrays and one device's (lam, beta)
+__host__ __device__ inline int warp_smem_floats(int T) { return (T + 1) * (3 + 2 * SG_N); }
+// warps of a CTA with `bytes` of shared memory that can each hold a device
+__host__ __device__ inline int smem_warps(int T, size_t bytes) {
+  int nw = DEV_WARPS;
+  while (nw > 1 && nw * (size_t)warp_smem_floats(T) * sizeof(float) > bytes) nw /= 2;
+  return nw;
+}
 
 // warps' worth of work of the inner kernels: a device each, a link one per 32 steps
 __host__ __device__ inline int inner_units(const Params &p) { return p.n_stor + p.n_ramp + p.n_hvdc * ((p.T + 31) >> 5); }
@@ -1439,47 +1445,29 @@ __device__ __forceinline__ void ramp_r(const Params &p, int r, int lane, int cr,
 // ---------------------------------------------------------------------------
 // inner: one warp per battery, then per ramp-limited generator (Appendix D),
 // then per HVDC link and 32 steps.  C > 0: the register path, for horizons of at most
-// REG_T steps (chunks of at most C); C = 0: the shared-memory path.  MIXED
-// (batches): the instance's horizon chooses, beyond BATCH_REG_T the
-// shared-memory path.  avg: each warp forms its node's average over
-// contingencies (else it is in XS).  nw: the CTA's warps that take devices.  staged: the
+// REG_T steps (ONLY: chunks of C, else of at most C, by the instance's horizon);
+// C = 0: the shared-memory path.  avg: each warp forms its node's average over
+// contingencies (else it is in XS).  nw: the CTA's warps that take devices.  The
 // shared-memory path holds the device's state there through the ten inner
 // iterations; in global memory each row's read, step and write is a round trip
-// to L2 (30 buses, T = 1000: 1005 -> 352 us per iteration; 40 buses, T = 300,
-// where L1 holds it: 103 -> 108).  Batches, whose instances share one launch's shared memory, do not stage.
+// to L2, or L1 while it holds them (30 buses, T = 1000: 1005 -> 352 us per
+// iteration; 40 buses, T = 300: 103 -> 108).
 // ---------------------------------------------------------------------------
-template <int C, bool MIXED>
-__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem, bool avg, int nw,
-                                           bool staged) {
+template <int C, bool ONLY>
+__device__ __forceinline__ void inner_body(const Params &p, unsigned bid, unsigned nblk, float *smem, bool avg, int nw) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (wib >= nw) return;
-  const int T = p.T;
-  const int n_inner = inner_units(p);
-  constexpr bool HAS_SMEM = C == 0 || MIXED, HAS_REG = C > 0;
-  const bool reg = HAS_REG && (!HAS_SMEM || T <= BATCH_REG_T);
-  float *wsm = nullptr, *state_sh = nullptr;
-  if (HAS_SMEM && !reg) {
-    wsm = smem + (size_t)wib * warp_smem_floats(T, staged);
-    state_sh = staged ? wsm + 3 * (T + 1) : nullptr;
-  }
+  const int T = p.T, n_inner = inner_units(p);
+  float *wsm = C == 0 ? smem + (size_t)wib * warp_smem_floats(T) : nullptr;
+  float *state_sh = C == 0 ? wsm + 3 * (T + 1) : nullptr;
   const int cs = (T + 32) >> 5, cr = (T + 31) >> 5;   // chunks of T + 1 and T elements
   for (int w = bid * nw + wib; w < n_inner; w += nblk * nw) {
     if (w < p.n_stor) {
-      if constexpr (HAS_REG) {
-        if (reg) {
-          stor_r<C, !MIXED>(p, w, lane, cs, avg);
-          continue;
-        }
-      }
-      if constexpr (HAS_SMEM) stor_prox(p, w, wsm, state_sh, lane, avg);
+      if constexpr (C > 0) stor_r<C, ONLY>(p, w, lane, cs, avg);
+      else stor_prox(p, w, wsm, state_sh, lane, avg);
     } else if (w < p.n_stor + p.n_ramp) {
-      if constexpr (HAS_REG) {
-        if (reg) {
-          ramp_r<C, !MIXED>(p, w - p.n_stor, lane, cr, avg);
-          continue;
-        }
-      }
-      if constexpr (HAS_SMEM) ramp_prox(p, w - p.n_stor, wsm, state_sh, lane, avg);
+      if constexpr (C > 0) ramp_r<C, ONLY>(p, w - p.n_stor, lane, cr, avg);
+      else ramp_prox(p, w - p.n_stor, wsm, state_sh, lane, avg);
     } else {
       hvdc_prox(p, w - p.n_stor - p.n_ramp, lane, avg);
     }
@@ -1873,7 +1861,7 @@ __global__ void __launch_bounds__(BLOCK) xs_kernel(Params p) { xs_body<VW>(p, bl
 template <int C>
 __global__ void __launch_bounds__(DEVB) dev_kernel(Params p, int inner_blocks, bool avg, int nw) {
   extern __shared__ float smem[];
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, blockIdx.x, inner_blocks, smem, avg, nw, true);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, true>(p, blockIdx.x, inner_blocks, smem, avg, nw);
   else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
   else closed_body<1>(p, load_iter(p), blockIdx.x - inner_blocks, gridDim.x - inner_blocks);
 }
@@ -2087,13 +2075,11 @@ __device__ void deal_nodes(const Params *ps, const NodeDeal &d, DealMem &mem) {
   if (tid == 0) *d.dirty = 0;
 }
 
-// the devices of every instance: the first inner_blocks CTAs of the schedule
-// take inner-ADMM devices, the others closed-form ones.  C: the largest
-// register chunk of the batch's instances (0: every horizon beyond
-// BATCH_REG_T), any longer horizon on the shared-memory path (the same bits)
+// The devices of every instance: the first inner_blocks CTAs of the schedule
+// take links and inner-ADMM devices of up to BATCH_REG_T steps, the others
+// closed-form ones.  C: the largest register chunk of the batch's instances.
 template <int C>
 __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
-  extern __shared__ float smem[];
   __shared__ Params sp;
   if (blockIdx.x == 0) {
     static_assert(sizeof(DealMem) <= sizeof(Params) && alignof(DealMem) <= alignof(Params), "shared by turns");
@@ -2102,9 +2088,22 @@ __global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int
   }
   unsigned bid, nblk;
   const Params &p = batch_params(ps, sched[blockIdx.x], sp, bid, nblk);
-  if ((int)blockIdx.x < inner_blocks) inner_body<C, (C > 0)>(p, bid, nblk, smem, true, DEV_WARPS, false);
+  if ((int)blockIdx.x < inner_blocks) inner_body<C, false>(p, bid, nblk, nullptr, true, DEV_WARPS);
   else if (p.T % 4 == 0) closed_body<4>(p, load_iter(p), bid, nblk);
   else closed_body<1>(p, load_iter(p), bid, nblk);
+}
+
+// The inner-ADMM devices of the instances beyond BATCH_REG_T steps, staged in
+// shared memory, on a stream of their own: their chains are the longest of the
+// phase, and the other devices' CTAs are not held to the room that they leave
+// (one launch for all, unstaged: 15 instances of T = 24 with one of T = 1000
+// took 771 us per step, now 340; 16 instances of T = 168 165 -> 138).
+__global__ void __launch_bounds__(DEVB) smem_kernel_b(const Params *ps, const int4 *sched, unsigned bytes) {
+  extern __shared__ float smem[];
+  __shared__ Params sp;
+  unsigned bid, nblk;
+  const Params &p = batch_params(ps, sched[blockIdx.x], sp, bid, nblk);
+  inner_body<0, true>(p, bid, nblk, smem, true, smem_warps(p.T, bytes));
 }
 
 // the lines of every instance: the first n4 CTAs of the schedule take those
@@ -2429,9 +2428,7 @@ __global__ void set_rho_kernel(Params p, double rho) {
   *p.sc = s;
 }
 
-static size_t inner_smem(int T, int warps, bool staged) {
-  return (size_t)warps * warp_smem_floats(T, staged) * sizeof(float);
-}
+static size_t inner_smem(int T, int warps) { return (size_t)warps * warp_smem_floats(T) * sizeof(float); }
 
 }  // namespace opfk
 
@@ -2506,14 +2503,12 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // device kernel would take it, the closed-form ones too, and run one or two
   // to an SM)
   const bool admm = p.n_stor + p.n_ramp > 0;
-  int nw = DEV_WARPS;
-  if (!ic && admm)
-    for (const size_t m = max_smem(); nw > 1 && inner_smem(p.T, nw, true) > m;) nw /= 2;
+  const int nw = !ic && admm ? smem_warps(p.T, max_smem()) : DEV_WARPS;
   plan->inner_warps = nw;
   const int one_round = (n_inner + nw - 1) / nw;
   const double round_us = ic ? 5.0 + 0.08 * p.T : 0.45 * p.T;
   const int max_rounds = (int)std::floor((ic ? 0.5 : 0.7) * line_us / round_us);
-  const size_t ism = ic || !admm ? 0 : inner_smem(p.T, nw, true);
+  const size_t ism = ic || !admm ? 0 : inner_smem(p.T, nw);
   if (!allow_smem(dev_kernel<0>, ism)) return -1;
   plan->inner_smem = ism;
   // Without inner-ADMM devices the chain is averages and closed forms alone,
@@ -2631,8 +2626,11 @@ int opfk_slice_prime_launch(const Params &p, void *stream) {
 int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchLayout &lay, int *sched_out,
                     long long sched_cap, long long *sched_len, NodeShare *share, BatchPlan *bp) {
   long long len = 0;
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, smem_kernel_b) != cudaSuccess) return -1;
+  const size_t smem_max = max_smem() - fa.sharedSizeBytes;
   size_t ism = 0;
-  int ic_max = 0;
+  int ic_max = 1;
   auto put = [&](int inst, long long b, long long blocks) -> bool {
     if (sched_out) {
       if (len >= sched_cap) return false;
@@ -2658,12 +2656,13 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
       const int n_inner = inner_units(p);
       long long blocks = 0;
       switch (kind) {
-        case BK_INNER:
-          blocks = (n_inner + DEV_WARPS - 1) / DEV_WARPS;
-          if (blocks) {
-            const int ic = inner_chunk(p.T, BATCH_REG_T);
-            if (ic) ic_max = std::max(ic_max, ic);
-            else ism = std::max(ism, inner_smem(p.T, DEV_WARPS, false));   // the shared-memory path
+        case BK_SMEM: case BK_INNER:
+          // by the form that the instance's horizon takes (links alone need none)
+          if ((kind == BK_SMEM) == (p.T > BATCH_REG_T && p.n_stor + p.n_ramp > 0)) {
+            const int nw = kind == BK_SMEM ? smem_warps(p.T, smem_max) : DEV_WARPS;
+            blocks = (n_inner + nw - 1) / nw;
+            if (kind == BK_SMEM) ism = std::max(ism, inner_smem(p.T, nw));
+            else if (p.n_stor + p.n_ramp > 0) ic_max = std::max(ic_max, inner_chunk(p.T));
           }
           break;
         case BK_CLOSED:
@@ -2675,7 +2674,7 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
           break;
       }
       // the devices take any block count: `div` puts more work in each CTA
-      if (blocks > 0 && (kind == BK_INNER || kind == BK_CLOSED))
+      if (blocks > 0 && (kind == BK_SMEM || kind == BK_INNER || kind == BK_CLOSED))
         blocks = (blocks + div - 1) / div;
       nb[j] = blocks;
       most = std::max(most, blocks);
@@ -2711,43 +2710,46 @@ int opfk_batch_plan(const Params *hp, const IterPlan *plans, int n, const BatchL
     grids += plans[i].node_grid;
   }
   bp->deal.cap = (int)std::min<long long>(grids, (long long)bp->deal.slots + n);
-  if (!allow_smem(dev_kernel_b<0>, ism) || !allow_smem(dev_kernel_b<1>, ism) || !allow_smem(dev_kernel_b<2>, ism) ||
-      !allow_smem(dev_kernel_b<3>, ism) || !allow_smem(dev_kernel_b<4>, ism))
-    return -1;
+  if (!allow_smem(smem_kernel_b, ism)) return -1;
   *sched_len = len;
   return 0;
 }
 
-int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPlan &bp, void *main_stream,
-                       void *aux_stream, void *ev_fork, void *ev_join) {
-  cudaStream_t sm = (cudaStream_t)main_stream, sa = (cudaStream_t)aux_stream;
+int opfk_batch_enqueue(const Params *d_params, const int *d_sched, const BatchPlan &bp, const Lanes &on) {
+  cudaStream_t sm = (cudaStream_t)on.main, sa = (cudaStream_t)on.aux, sd = (cudaStream_t)on.dev;
+  if (bp.deal.n == 0) return 0;
   const int4 *sched = reinterpret_cast<const int4 *>(d_sched);
   auto at = [&](int kind) { return sched + bp.offset[kind]; };
-  if (cudaEventRecord((cudaEvent_t)ev_fork, sm) != cudaSuccess) return -1;
-  if (cudaStreamWaitEvent(sa, (cudaEvent_t)ev_fork, 0) != cudaSuccess) return -1;
-  // the devices first: a graph's first iteration starts its kernels in this
-  // order, and line CTAs that fill the GPU hold up the longer device chain
-  // (16 instances of T = 128, calls of 9 steps: 172 -> 140 us per step)
-  static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
-  const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED];
-  if (bp.deal.n > 0) {
-    const int4 *si = at(BK_INNER);
-    switch (bp.inner_c) {
-      case 1: dev_kernel_b<1><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
-      case 2: dev_kernel_b<2><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
-      case 3: dev_kernel_b<3><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
-      case 4: dev_kernel_b<4><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
-      default: dev_kernel_b<0><<<std::max(nd, 1), DEVB, bp.inner_smem, sm>>>(d_params, si, ni, nd, bp.deal); break;
-    }
+  if (cudaEventRecord((cudaEvent_t)on.ev_fork, sm) != cudaSuccess) return -1;
+  if (cudaStreamWaitEvent(sa, (cudaEvent_t)on.ev_fork, 0) != cudaSuccess) return -1;
+  // the devices first, the longest chains ahead: a graph's first iteration
+  // starts its kernels in this order, and line CTAs that fill the GPU hold up
+  // the device chain (16 instances of T = 128, calls of 9 steps: 172 -> 140 us
+  // per step)
+  const int ns = bp.count[BK_SMEM];
+  if (ns) {
+    if (cudaStreamWaitEvent(sd, (cudaEvent_t)on.ev_fork, 0) != cudaSuccess) return -1;
+    smem_kernel_b<<<ns, DEVB, bp.inner_smem, sd>>>(d_params, at(BK_SMEM), (unsigned)bp.inner_smem);
+    if (cudaEventRecord((cudaEvent_t)on.ev_dev, sd) != cudaSuccess) return -1;
   }
+  static_assert(BK_CLOSED == BK_INNER + 1, "one launch over both parts of the schedule");
+  const int ni = bp.count[BK_INNER], nd = ni + bp.count[BK_CLOSED], gd = std::max(nd, 1);
+  const int4 *si = at(BK_INNER);
+  switch (bp.inner_c) {
+    case 1: dev_kernel_b<1><<<gd, DEVB, 0, sm>>>(d_params, si, ni, nd, bp.deal); break;
+    case 2: dev_kernel_b<2><<<gd, DEVB, 0, sm>>>(d_params, si, ni, nd, bp.deal); break;
+    case 3: dev_kernel_b<3><<<gd, DEVB, 0, sm>>>(d_params, si, ni, nd, bp.deal); break;
+    default: dev_kernel_b<4><<<gd, DEVB, 0, sm>>>(d_params, si, ni, nd, bp.deal); break;
+  }
+  static_assert(BATCH_C == 4, "the chunks launched above");
   static_assert(BK_LINE1 == BK_LINE4 + 1, "one launch over both widths' schedules");
   const int l4 = bp.count[BK_LINE4], nl = l4 + bp.count[BK_LINE1];
   if (nl) line_kernel_b<<<nl, BLOCK, 0, sa>>>(d_params, at(BK_LINE4), l4);
-  if (cudaEventRecord((cudaEvent_t)ev_join, sa) != cudaSuccess) return -1;
-  if (cudaStreamWaitEvent(sm, (cudaEvent_t)ev_join, 0) != cudaSuccess) return -1;
-  const int nn = bp.deal.cap;
-  if (nn && bp.relax) node_kernel_b<true><<<nn, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
-  else if (nn) node_kernel_b<false><<<nn, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
+  if (cudaEventRecord((cudaEvent_t)on.ev_join, sa) != cudaSuccess) return -1;
+  if (cudaStreamWaitEvent(sm, (cudaEvent_t)on.ev_join, 0) != cudaSuccess) return -1;
+  if (ns && cudaStreamWaitEvent(sm, (cudaEvent_t)on.ev_dev, 0) != cudaSuccess) return -1;
+  if (bp.relax) node_kernel_b<true><<<bp.deal.cap, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
+  else node_kernel_b<false><<<bp.deal.cap, BLOCK, 0, sm>>>(d_params, bp.deal.slot, bp.deal.dirty);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

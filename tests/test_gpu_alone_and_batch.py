@@ -148,3 +148,32 @@ def test_members_equal_contexts_alone_in_every_bit(alpha):
         opf_batch_destroy(b)
         for s in alone + member:
             s.close()
+
+
+@pytest.mark.parametrize("T", [256, 700, 1400])
+def test_staged_horizons_match_oracle(T):
+    """Batteries and ramp-limited generators staged in shared memory by four,
+    two and one warps to a CTA, over a change of the penalty, alone and in a
+    batch beside a short instance."""
+    from helpers import compare_states
+    from oracle import Oracle, OracleOptions
+    from paper_2410_17203_gb300 import Solver, opf_batch_create, opf_batch_destroy, opf_batch_iterate
+    case = make_case(scale_case(6, T, 1, seed=T, stor_per_node=0.2, lines_per_node=1.2))
+    short = make_case(scale_case(30, 24, 2, seed=5))
+    opts = dict(adapt_every=5, eps=0.0)
+    single, member, beside, ref = Solver(case, opts), Solver(case, opts), Solver(short, opts), Solver(short, opts)
+    single.iterate(7)
+    ref.iterate(7)
+    b = opf_batch_create([beside.h, member.h])
+    try:
+        opf_batch_iterate(b, 7)
+        _assert_same_state(member, single)
+        _assert_same_state(beside, ref)
+        o = Oracle(case, OracleOptions(**opts))
+        o.iterate(7, stop=False)
+        assert o.rho_p != OracleOptions(**opts).rho_p
+        compare_states(single.state(), o)
+    finally:
+        opf_batch_destroy(b)
+        for s in (single, member, beside, ref):
+            s.close()
