@@ -52,13 +52,14 @@ constexpr int WARPS = BLOCK / 32;
 constexpr int ST_NONFINITE = 5;  // opf_status value set on the device
 constexpr int NODE_VW = 4;       // time steps per node item
 constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is compiled for (64 registers)
-// Up to this many node items (four steps / one step each; about what two CTAs
-// per SM hold at once) the pass is latency alone, and a variant with the
-// registers to request all loads of an item together is faster: us per
-// iteration, 30 buses 9.0 -> 8.6, 301 buses T = 31 14.4 -> 13.8, 5k buses T = 1
-// (105k items) 15.5 -> 14.9, 900 buses T = 24 (76k) 16.9 -> 16.4; beyond it
-// the second wave costs more: 500 buses T = 168 (105k items of four) 35.1 -> 36.5.
-constexpr long long NODE_LAT_ITEMS4 = 2 * 152 * BLOCK, NODE_LAT_ITEMS1 = 1 << 17;
+// A node pass of few items is latency alone, and a variant with the registers
+// to request all loads of an item together (two CTAs per SM) is faster.  Items
+// of four steps: while that variant's CTAs are one wave, half of the node
+// grid's threads (us per iteration, 30 buses 9.0 -> 8.6, 900 buses T = 24, 76k
+// items, 16.9 -> 16.4; with a second wave, 500 buses T = 168, 105k, 35.1 ->
+// 36.5).  Items of one step, whose loads are shorter: measured, up to this many
+// (301 buses T = 31 14.4 -> 13.8, 5k buses T = 1, 105k, 15.5 -> 14.9).
+constexpr long long NODE_LAT_ITEMS1 = 1 << 17;
 constexpr int NODE_UNITS = 8;    // partial sums that a batch's node CTA forms between barriers
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
@@ -2519,7 +2520,7 @@ int opfk_plan(const Params &p, IterPlan *plan) {
   // links 15.9 us 39.3 / 42.0, 2k T = 96 K = 10 16.6 us 43.1 / 39.3, 2k T = 252
   // K = 4 19.8 us 59.1 / 49.5).
   plan->fused = !p.slice && (admm ? max_rounds < 2 : line_us < HIDE_US);
-  plan->node_lat = plan->fused && nn <= (vn ? NODE_LAT_ITEMS4 : NODE_LAT_ITEMS1);
+  plan->node_lat = plan->fused && nn <= (vn ? (long long)gn * BLOCK / 2 : NODE_LAT_ITEMS1);
   // A small instance without inner-ADMM devices runs on one CTA (small_kernel)
   // where its rounds of 256 line, closed-form and node items are estimated to
   // take less than the kernels' 8.3 us: 30 buses, T = 1, K = 5 8.35 -> 5.1 us,
