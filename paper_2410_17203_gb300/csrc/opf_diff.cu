@@ -1303,12 +1303,31 @@ __device__ __forceinline__ void lane_x(const DP &p, const St &s, int d, int t0, 
   }
 }
 
+// the same where most lanes have no step (C = 1, up to SPLIT_T steps) and the
+// sums over many contingencies would be one lane's chain: eight lanes share a
+// step's (us per iteration, cost alone, 500 buses T = 8 K = 100 38 -> 26, 2k buses
+// T = 1 K = 400 174 -> 132)
+constexpr int SPLIT_T = 8;
+__device__ __forceinline__ void split_x(const DP &p, const St &s, int d, int lane, float (&x)[1]) {
+  constexpr int ST = 32 / KL;   // steps at a time
+  const int n = p.dnode[d], T = p.T;
+  float sum = 0.f;
+  for (int b = 0; b < T; b += ST) {
+    const int t = b + lane / KL;
+    float v = 0.f;
+    if (t < T) v = ksumv<1>(p, s.PB, s.U, n, t).x[0];   // the same t in all KL lanes
+    v = __shfl_sync(FULLM, v, ((lane - b) & (ST - 1)) * KL);
+    if (lane >= b && lane < b + ST) sum = v;
+  }
+  x[0] = lane < T ? s.PD[(size_t)d * T + lane] - sum / (float)p.Kp : 0.f;
+}
+
 // step 2 from registers in one launch (it runs beside fwd_line): the first
 // inner_blocks blocks take the inner-ADMM devices, one warp each, which form
 // their inputs themselves, the others the closed-form devices.  As two
 // kernels in a row, behind the line prox, the phase took 28 us of a 2k
 // iteration's 44.
-template <int C, int VW>
+template <int C, int VW, bool SPLIT>
 __global__ void __launch_bounds__(TB, 1) fwd_devs(DP p, St s, St nx, float *DEL, unsigned long long *grec,
                                                   unsigned char *dmask, int inner_blocks) {
   if ((int)blockIdx.x >= inner_blocks) {
@@ -1322,7 +1341,8 @@ __global__ void __launch_bounds__(TB, 1) fwd_devs(DP p, St s, St nx, float *DEL,
   float *Bo = nx.INS + dv.h, *Lo = nx.INS + p.Mtot + dv.h;
   float x[C], xd[C];
   TriFac<C> tf;
-  lane_x<C>(p, s, dv.dev, t0, xd);
+  if constexpr (SPLIT) split_x(p, s, dv.dev, lane, xd);
+  else lane_x<C>(p, s, dv.dev, t0, xd);
   if (dv.bat < 0) {
     float hU[C], hL[C], hRU[C], hRD[C], bU[C], lU[C], bL[C], lL[C], bRU[C], lRU[C], bRD[C], lRD[C], z[C];
     ramp_load<C>(p, s, dv, T, lane, x, tf, hU, hL, hRU, hRD, bU, lU, bL, lL, bRU, lRU, bRD, lRD, nullptr);
@@ -2168,10 +2188,14 @@ cudaError_t forward_step(const opf_diff *d, cudaStream_t sm, cudaStream_t sa, co
     const int ni = (p.n_inner + RWARPS - 1) / RWARPS, g = ni + dg;
 #define DEVS_LAUNCH(C)                                                                     \
   case C:                                                                                  \
-    if (v4) fwd_devs<C, 4><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);              \
-    else fwd_devs<C, 1><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);                 \
+    if (v4) fwd_devs<C, 4, false><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);       \
+    else fwd_devs<C, 1, false><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);          \
     break
-    switch (p.reg_c) {
+    static_assert(SPLIT_T < 32, "one step per lane");
+    if (p.T <= SPLIT_T) {
+      if (v4) fwd_devs<1, 4, true><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);
+      else fwd_devs<1, 1, true><<<g, TB, 0, sm>>>(p, s, nx, DEL, rrec, dmask, ni);
+    } else switch (p.reg_c) {
       DEVS_LAUNCH(1);
       DEVS_LAUNCH(2);
       DEVS_LAUNCH(3);
