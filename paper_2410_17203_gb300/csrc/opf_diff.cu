@@ -2673,13 +2673,18 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   // forward pass in place: the line prox, the devices and the node averages
   // each read their own entries before they write them, and the node values
   // (read at other items) are written by the averages alone, after everything
-  // that reads them.  Only the device powers alternate between two arrays (an
-  // HVDC terminal reads its partner's).  At 2k buses the forward pass then
-  // works on 44 MB, which stays in L2, instead of two states and the
-  // checkpoints between them: cost alone 35.9 -> 34.4 us per iteration.
+  // that reads them.  At 2k buses the forward pass then works on some 57 MB,
+  // which stay in L2, instead of two states and the checkpoints between them:
+  // cost alone 35.9 -> 33 us per iteration.  Two alternate between two arrays:
+  // the device powers (an HVDC terminal reads its partner's), and the phase
+  // duals, which the averages gather and write line by line: in place, a
+  // thread's store to a sector took it from its neighbours' reads (us per
+  // iteration, cost alone, 2k buses T = 1 K = 400 132 -> 66, fwd_avg 103 -> 39;
+  // 1k T = 7 K = 100 50 -> 40, 2k T = 24 K = 20 35 -> 34).
+  const size_t STp = (ST + 63) & ~size_t(63);
   const bool ckpt = grads && !rec;
   cudaError_t e = ckpt ? ensure(&d->ck, &d->ck_cap, (size_t)n_ck * SF) : cudaSuccess;
-  if (e == cudaSuccess) e = ensure(&d->seg, &d->seg_cap, ckpt ? (size_t)std::max(C, 2) * SF : SF + ST);
+  if (e == cudaSuccess) e = ensure(&d->seg, &d->seg_cap, ckpt ? (size_t)std::max(C, 2) * SF : SF + STp + 2 * KLT);
   if (e == cudaSuccess) e = ensure(&d->adj, &adj_cap, adj_floats);
   if (e == cudaSuccess) e = ensure(&d->work, &work_cap, work_floats);
   if (e == cudaSuccess) e = ensure(&d->gline, &gl_cap, L);
@@ -2710,7 +2715,11 @@ opf_status cost_grad(opf_diff *d, int32_t K, int on_device, const float *load_p,
   auto fwdst = [&](int i) {
     if (ckpt) return i % C == 0 ? ckst(i / C) : carve_state(d, seg + (size_t)(i & 1) * SF);
     St st = carve_state(d, seg);
-    if (i & 1) st.PD = seg + SF;
+    if (i & 1) {
+      st.PD = seg + SF;
+      st.V1 = st.PD + STp;
+      st.V2 = st.V1 + KLT;
+    }
     return st;
   };
   // state K (the reverse pass may overwrite it; its cost inputs are copied first)
