@@ -2079,8 +2079,11 @@ __device__ void deal_nodes(const Params *ps, const NodeDeal &d, DealMem &mem) {
 // The devices of every instance: the first inner_blocks CTAs of the schedule
 // take links and inner-ADMM devices of up to BATCH_REG_T steps, the others
 // closed-form ones.  C: the largest register chunk of the batch's instances.
+// Registers are held to 80, 128, 128 and 168: left to the compiler, C = 1 took
+// 93 and five CTAs per SM instead of six (40 instances of T = 7 and 31 60.0
+// against 57.0 us per step, 256 of T = 1 and 24 57.3 against 55.9).
 template <int C>
-__global__ void __launch_bounds__(DEVB) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
+__global__ void __launch_bounds__(DEVB, C == 1 ? 6 : C == 4 ? 3 : 4) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
   __shared__ Params sp;
   if (blockIdx.x == 0) {
     static_assert(sizeof(DealMem) <= sizeof(Params) && alignof(DealMem) <= alignof(Params), "shared by turns");
