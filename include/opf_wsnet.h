@@ -21,8 +21,12 @@
  * even) and accumulate in FP32; gradients treat the rounding as the identity.
  * Training uses Adam (beta1 0.9, beta2 0.999, eps 1e-8) on the FP32 vector.
  *
- * All GPU work is enqueued on the stream given at creation; functions that
- * return host data synchronize it.  Device pointers are of the current device.
+ * A network keeps about 4.2 KB of device memory per row (activations, their
+ * adjoints and the partial weight gradients).
+ *
+ * All GPU work is enqueued on the stream given at creation (weight gradients on
+ * a second one, forked from it and joined to it); functions that return host
+ * data synchronize it.  Device pointers are of the current device.
  */
 #ifndef OPF_WSNET_H_
 #define OPF_WSNET_H_

@@ -30,7 +30,9 @@
 // There is no spin-wait on the device: ordering comes from kernel boundaries
 // and graph edges.  Every kernel body also serves a batch of independent
 // instances: the batch entry points take the instances' parameters and a
-// CTA schedule, so one launch per phase covers all instances.
+// CTA schedule, so one launch per phase covers all instances (devices that
+// solve in shared memory have one of their own), and the node phase's CTAs are
+// dealt out on the device over the instances that still run.
 //
 // Memory layout (line- and node-major), numbering and the deferred v
 // update: opf_internal.h.

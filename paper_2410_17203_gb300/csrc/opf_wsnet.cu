@@ -15,9 +15,14 @@
 //
 // A training pass over 48,000 rows (2k buses, T = 24) moves about 0.35 GB and
 // does 7.3 GFLOP outside the tensor cores (the FP32 activations keep their
-// precision): bound by the FP32 pipes.  As fifty launches (averages, layers,
-// relu masks and each weight gradient apart) it took 0.97 ms, as sixteen
-// (weight gradients beside the chain of layers) 0.37 ms.
+// precision), 0.1 ms of the FP32 pipes.  Its layer kernels are bound by neither
+// pipes nor memory: they issue in half of their cycles (12 warps per SM), the
+// rest waits for the gather of a tile's rows, which does not overlap its
+// products, and 750 tiles on 608 CTAs leave the second round mostly empty.  As
+// fifty launches (averages, layers, relu masks and each weight gradient apart)
+// a pass took 0.97 ms, as sixteen (weight gradients beside the chain of layers)
+// 0.37 ms.  Device memory: about 4.2 KB per row (fifteen arrays of 64 floats,
+// and per 256 rows a partial sum of every parameter).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -112,8 +117,8 @@ __device__ __forceinline__ float4 weights4(const __nv_bfloat16 *p) {
                      __uint_as_float(v.y & 0xffff0000u));
 }
 
-// acc[i][c] += sum_k at[RT ty + i][k] ws[k][4 tx + c], k in order.  Shared
-// memory bounds this loop, not the FP32 pipes: rows are read four k at a time
+// acc[i][c] += sum_k at[RT ty + i][k] ws[k][4 tx + c], k in order.  Within the
+// products shared memory is the limit, not the FP32 pipes: rows are read four k at a time
 // (one 16-byte read serves 16 lanes), weights as bfloat16 (a warp's 16 columns
 // groups are one 128-byte wavefront), and eight rows share a weight, so that
 // four k are 12 wavefronts for 128 products per lane (FP32 weights and 4 x 4
