@@ -16,8 +16,8 @@
 //   devices PD, DPD                         [S][T]         float
 //   inner ADMM state of ramp generators     lam, beta [n_ramp][4][T],  q [n_ramp][3][T]
 //   inner ADMM state of batteries           lam, beta [n_stor][9][T+1], q [n_stor][3][T+1]
-// (q: pivots; 1 / q and -off / q beside them beyond 127 steps, where a batch or
-// both forms solve from shared memory)
+// (q: pivots; 1 / q and -off / q beside them where the shared-memory form
+// solved last or since they were factored, else 0 for the first 1 / q)
 // Buffer (it & 1) holds the state after `it` iterations; an iteration reads
 // the old buffers and writes the other ones, because both ends of a line
 // evaluate its prox from the old line and node values.

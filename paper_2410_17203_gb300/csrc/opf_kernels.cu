@@ -489,6 +489,8 @@ __device__ void ramp_prox(const Params &p, int r, float *sm, float *state_sh, in
       p.ramp_rho[r] = rho;
     }
     tri_tables(mf, T, -om2, lane);
+  } else if (mf[T] == 0.f) {   // no_tables
+    tri_tables(mf, T, -om2, lane);
   }
   device_x(p, q, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
   for (int itn = 0; itn < p.inner_iters; ++itn) {
@@ -600,6 +602,8 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
       p.stor_rho[sidx] = rho;
     }
     tri_tables(mf, Tp, -gam, lane);
+  } else if (mf[Tp] == 0.f) {   // no_tables
+    tri_tables(mf, Tp, -gam, lane);
   }
   device_x(p, it, n, pd, X, lane, avg);   // p_d - avg_k(pbar + u)
 #define LAM(g, t) lam[(g) * Tp + (t)]
@@ -680,13 +684,13 @@ __device__ void stor_prox(const Params &p, int sidx, float *sm, float *state_sh,
 // instance, a batch) computes the same bits.
 // ---------------------------------------------------------------------------
 
-// Whether a batch solves a device of this horizon from shared memory: it then
-// reads the tables of tri_tables, which are written with the pivots, under the
-// same record of the penalty they belong to (ramp_rho, stor_rho), whichever
-// form factors.
+// Pivots written without the tables that the shared-memory form reads beside
+// them (a batch solves devices beyond BATCH_REG_T steps that way): the first
+// reciprocal, never 0 otherwise, says so, and that form makes them when it
+// comes to the device.  (Writing them here too cost a week of 500 buses 0.4 %.)
 template <int C>
-__device__ __forceinline__ bool tables_too(int T) {
-  return 32 * C > BATCH_REG_T && T > BATCH_REG_T;   // a chunk of C holds up to 32 C elements
+__device__ __forceinline__ void no_tables(float *mf, int n) {
+  if (32 * C > BATCH_REG_T) mf[n] = 0.f;
 }
 
 // Lanes beyond the horizon run along (right-hand side 0, nothing of theirs is
@@ -740,10 +744,10 @@ __device__ void ramp_prox_r(const Params &p, int r, int lane, bool avg) {
     if (lane == 0) {
       const float base = radd(rmul(2.f, a), rho);
       tri_factor(mf, T, radd(base, rmul(4.f, om)), radd(base, rmul(6.f, om)), -om2);
+      no_tables<C>(mf, T);
       p.ramp_rho[r] = rho;
     }
     __syncwarp();
-    if (tables_too<C>(T)) tri_tables(mf, T, -om2, lane);
 #pragma unroll
     for (int j = 0; j < C; ++j) {
 #pragma unroll
@@ -856,10 +860,10 @@ __device__ void stor_prox_r(const Params &p, int sidx, int lane, bool avg) {
     const float ls = (rho_old == 0.f) ? 1.f : rdiv(fabsf(rho_old), rho);
     if (lane == 0) {
       tri_factor(mf, Tp, radd(gam, rmul(3.f, om)), radd(rmul(2.f, gam), om2), -gam);
+      no_tables<C>(mf, Tp);
       p.stor_rho[sidx] = rho;
     }
     __syncwarp();
-    if (tables_too<C>(T)) tri_tables(mf, Tp, -gam, lane);
     e3a = rmul(e3a, ls);
     e3b = rmul(e3b, ls);
 #pragma unroll
