@@ -2089,7 +2089,8 @@ __device__ void deal_nodes(const Params *ps, const NodeDeal &d, DealMem &mem) {
 // 93 and five CTAs per SM instead of six (40 instances of T = 7 and 31 60.0
 // against 57.0 us per step, 256 of T = 1 and 24 57.3 against 55.9).
 template <int C>
-__global__ void __launch_bounds__(DEVB, C == 1 ? 6 : C == 4 ? 3 : 4) dev_kernel_b(const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
+__global__ void __launch_bounds__(DEVB, C == 1 ? 6 : C == 4 ? 3 : 4) dev_kernel_b(
+    const Params *ps, const int4 *sched, int inner_blocks, int blocks, NodeDeal deal) {
   __shared__ Params sp;
   if (blockIdx.x == 0) {
     static_assert(sizeof(DealMem) <= sizeof(Params) && alignof(DealMem) <= alignof(Params), "shared by turns");
@@ -2127,7 +2128,8 @@ __global__ void __launch_bounds__(BLOCK, 4) line_kernel_b(const Params *ps, cons
 }
 
 template <bool RELAX>
-__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(const Params *ps, const int4 *slot, int *dirty) {
+__global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(
+    const Params *ps, const int4 *slot, int *dirty) {
   __shared__ Params sp;
   __shared__ NodeMemB mem;
   const int4 e = slot[blockIdx.x];   // dealt out by deal_nodes
