@@ -364,6 +364,7 @@ void carve(opf_ctx *c, Arena &a) {
   p.DSM = a.take<float>((size_t)c->N * T);
   p.DSQ = a.take<float>((size_t)c->N * T);
   p.partials = a.take<double>((size_t)c->plan.node_grid * opfk::NSLOT);
+  p.wsums = a.take<float>((size_t)c->plan.node_grid * (opfk::BLOCK / 32) * opfk::NSLOT);
   p.done = a.take<unsigned>(1);
   p.xsum = c->slice ? a.take<double>(slice_exchange_len(c)) : nullptr;
 }

@@ -152,6 +152,7 @@ struct Params {
   // scratch
   double *partials;  // [node_grid][NSLOT] residual partial sums of the node kernel (one per CTA of its own grid)
   int node_grid;     // CTAs of the node kernel (partial-sum slots)
+  float *wsums;      // [node_grid][BLOCK / 32][NSLOT] in a batch: their parts by warp
   unsigned *done;    // CTAs of the node kernel that have finished this iteration (0 between iterations)
   DevScalars *sc;
   // options

@@ -42,7 +42,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
 #include <vector>
 
 #include "opf_internal.h"
@@ -62,7 +61,6 @@ constexpr int NODE_CTAS = 4;     // resident CTAs per SM the node kernel is comp
 // 36.5).  Items of one step, whose loads are shorter: measured, up to this many
 // (301 buses T = 31 14.4 -> 13.8, 5k buses T = 1, 105k, 15.5 -> 14.9).
 constexpr long long NODE_LAT_ITEMS1 = 1 << 17;
-constexpr int NODE_UNITS = 8;    // partial sums that a batch's node CTA forms between barriers
 constexpr int NODE_RX_CTAS = 3;  // ... its over-relaxed variant (80 registers)
 constexpr int NODE_RES_NB = 1;   // line terminals gathered together where residuals are formed ...
 constexpr int NODE_LEAN_NB = 2;  // ... and where they are not
@@ -1745,45 +1743,39 @@ struct NodeMem {
   double red[WARPS][NSLOT];
   int last;
 };
-// ... in a batch, once for both step widths: two KB a CTA more and the kernel
-// takes another share of L1
-struct NodeMemB : NodeMem {
-  float wsum[NODE_UNITS][WARPS][NSLOT];
-};
-
 // The pass with residuals of a batch's instance.  Its partial sums are always
 // those of its own grid (p.node_grid, one per CTA there), so that the residuals
-// do not depend on how many CTAs the instance has here: each CTA forms several,
-// NODE_UNITS at a time between barriers (one at a time cost 64 mixed instances
-// 24 us per step, though one iteration in ten forms them).  Out of line: inlined,
-// it took registers from the pass without residuals (16 mixed instances 1.1 us
-// per step).
+// do not depend on how many CTAs the instance has here: each CTA forms several.
+// A warp leaves its sums of each in p.wsums and goes on; one barrier later the
+// CTA adds them up by partial sum (a barrier for each cost 64 mixed instances 24
+// us per step, though one iteration in ten forms them; one for every eight, in
+// shared memory, 40 instances of T = 7 and 31 0.9 us).  Out of line: inlined, it took registers
+// from the pass without residuals (16 mixed instances 1.1 us per step).
 template <int VW, bool RELAX>
-__device__ __noinline__ void node_units(const Params &p, unsigned bid, unsigned nblk, NodeMemB &mem) {
+__device__ __noinline__ void node_units(const Params &p, unsigned bid, unsigned nblk) {
   const int TV = p.T / VW, Kp = p.Kp;
   const unsigned n = (unsigned)Kp * (unsigned)p.N * (unsigned)TV;
   const unsigned parts = (unsigned)p.node_grid, ustride = parts * BLOCK;
   const Iter q = load_iter(p);
   Idx3 ix, dx;
   dx.set(ustride, Kp, TV);
-  for (unsigned u0 = bid; u0 < parts; u0 += nblk * NODE_UNITS) {
-    int units = 0;
-    for (unsigned u = u0; units < NODE_UNITS && u < parts; u += nblk, ++units) {
-      float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
-      unsigned item = u * BLOCK + threadIdx.x;
-      ix.set(item, Kp, TV);
-      for (; item < n; item += ustride, ix.step(dx, Kp, TV))
-        node_item<VW, RELAX, true, NODE_RES_NB, true, false>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
-      warp_sums(acc, mem.wsum[units][threadIdx.x >> 5]);
-    }
-    __syncthreads();
-    for (int x = threadIdx.x; x < units * NSLOT; x += BLOCK) {   // as write_partials
-      const int i = x / NSLOT, s = x - i * NSLOT;
-      double v = 0.0;
-      for (int w = 0; w < WARPS; ++w) v += (double)mem.wsum[i][w][s];
-      p.partials[(size_t)(u0 + i * nblk) * NSLOT + s] = v;
-    }
-    __syncthreads();   // mem.wsum is used again
+  for (unsigned u = bid; u < parts; u += nblk) {
+    float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    unsigned item = u * BLOCK + threadIdx.x;
+    ix.set(item, Kp, TV);
+    for (; item < n; item += ustride, ix.step(dx, Kp, TV))
+      node_item<VW, RELAX, true, NODE_RES_NB, true, false>(p, q.old, q.old ^ 1, ix.b, ix.a, ix.c * VW, q.fsu, acc);
+    warp_sums(acc, p.wsums + ((size_t)u * WARPS + (threadIdx.x >> 5)) * NSLOT);
+  }
+  __syncthreads();
+  const unsigned units = (parts - bid + nblk - 1) / nblk;   // bid < nblk <= parts
+  for (unsigned x = threadIdx.x; x < units * NSLOT; x += BLOCK) {   // as write_partials
+    const unsigned u = bid + x / NSLOT * nblk, s = x % NSLOT;
+    const float *f = p.wsums + (size_t)u * WARPS * NSLOT + s;
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) v += (double)f[w * NSLOT];
+    p.partials[(size_t)u * NSLOT + s] = v;
   }
 }
 
@@ -1801,8 +1793,8 @@ __device__ __noinline__ void node_units(const Params &p, unsigned bid, unsigned 
 // UNITS (batches): an instance's CTAs are fewer than its residual partial sums
 // (node_units).
 template <int VW, bool RELAX, bool ILD, bool LAT = false, bool UNITS = false>
-__device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk,
-                                          std::conditional_t<UNITS, NodeMemB, NodeMem> &mem, int *dirty = nullptr) {
+__device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigned nblk, NodeMem &mem,
+                                          int *dirty = nullptr) {
   double(*red)[NSLOT] = mem.red;
   const int N = p.N, TV = p.T / VW, Kp = p.Kp;
   const unsigned n = (unsigned)Kp * (unsigned)N * (unsigned)TV;
@@ -1819,7 +1811,7 @@ __device__ __forceinline__ void node_body(const Params &p, unsigned bid, unsigne
   const bool res = q.flags & ITF_RES;
   float acc[NSLOT] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if constexpr (UNITS) {
-    if (res) node_units<VW, RELAX>(p, bid, nblk, mem);
+    if (res) node_units<VW, RELAX>(p, bid, nblk);
   }
   if (!UNITS && res) {
     for (; item < n; item += stride, ix.step(dx, Kp, TV))
@@ -2131,7 +2123,7 @@ template <bool RELAX>
 __global__ void __launch_bounds__(BLOCK, RELAX ? NODE_RX_CTAS : NODE_CTAS) node_kernel_b(
     const Params *ps, const int4 *slot, int *dirty) {
   __shared__ Params sp;
-  __shared__ NodeMemB mem;
+  __shared__ NodeMem mem;
   const int4 e = slot[blockIdx.x];   // dealt out by deal_nodes
   if (e.x < 0) return;
   unsigned bid, nblk;
